@@ -41,7 +41,7 @@ struct qmc_system {
     float *d_C32 = nullptr, *d_ptrig32 = nullptr;
     int4* d_kvec = nullptr;
     double2 *d_eikR = nullptr, *d_rhop = nullptr;
-    double *d_vconst = nullptr, *d_dvpp = nullptr;
+    double *d_vconst = nullptr, *d_dvpp = nullptr, *d_vpp = nullptr;
     float *d_R32 = nullptr, *d_kw32 = nullptr, *d_zeta32 = nullptr;
     void* d_ptp = nullptr;     // (sin, cos)(pi x'/L) of the proposals of the current sweep
     float2* d_eikR32 = nullptr;
@@ -201,7 +201,7 @@ size_t footprint(const qmc_params* p) {
             }
     const size_t nk = nkc;
     size_t b = 0;
-    b += 8 * (3 * N + G + B * n + 6 * N + 3 * N + 2) + 4 * (B * n + 6 * N) + 16 * nk + 8 * nk + 16 * (N * nk + nk);
+    b += 8 * (3 * N + G + B * n + 6 * N + 4 * N + 2) + 4 * (B * n + 6 * N) + 16 * nk + 8 * nk + 16 * (N * nk + nk);
     b += 4 * (3 * N + G + nk) + 8 * N * nk + 4;      // FP32 copies of R, zeta, kw, exp(i k.R); error word
     b += t * W * N * 6;                              // proposal trig
     b += 8 * 2 * W * 3 * N;                          // X, Xp
@@ -274,13 +274,10 @@ SysView<T> view(qmc_system* h, int W) {
 }
 
 void setup_tables(qmc_system* h) {
-    h->nlaunch += 5;
+    h->nlaunch += 2;
     launch_setup(h->N, h->p.L, h->p.ewald_kappa, h->nk, h->d_kvec, h->d_R, h->d_kw, h->d_ptrig64, h->d_ptrig32,
-                 h->d_eikR, h->d_rhop, h->d_vconst, h->d_dvpp, h->d_R32, h->d_eikR32, h->d_kw32, h->stream);
-    if (h->d_Trec) {
-        h->nlaunch += 1;
-        launch_recforce_table(h->N, h->nk, h->p.L, h->d_kvec, h->d_kw, h->d_eikR, h->d_Trec, h->stream);
-    }
+                 h->d_eikR, h->d_rhop, h->d_vconst, h->d_dvpp, h->d_vpp, h->d_R32, h->d_eikR32, h->d_kw32, h->d_Trec,
+                 h->stream);
 }
 
 // Orbital rows at `pos`: tensor-core kernel in the mixed form, SIMT otherwise.
@@ -584,6 +581,7 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
     h->d_rhop = dalloc<double2>(h, nk, &rc);
     h->d_vconst = dalloc<double>(h, 1, &rc);
     h->d_dvpp = dalloc<double>(h, 3 * N, &rc);
+    h->d_vpp = dalloc<double>(h, N, &rc);
     h->d_R32 = dalloc<float>(h, 3 * N, &rc);
     h->d_zeta32 = dalloc<float>(h, h->G, &rc);
     h->d_ptp = dalloc<unsigned char>(h, t * (size_t)W * N * 6, &rc);

@@ -52,14 +52,12 @@ void launch_measure(const SysView<T>& s, const double* X, const T* D, const T* L
 template <typename T>
 size_t measure_smem_bytes(int N, int n, int nk, int mmax, bool split);
 
-// k_setup.cu: per-R tables (proton trig, structure factors, p-p Ewald terms).
+// k_setup.cu: per-R tables (proton trig, structure factors, p-p Ewald terms; vpp is
+// work space [N]) and, with Trec, the reciprocal-space force as a [3N][2 nk]
+// matrix on rho(k) (split measure path).
 void launch_setup(int N, double L, double kappa, int nk, const int4* kvec, const double* R, double* kw,
                   double* ptrig64, float* ptrig32, double2* eikR, double2* rho_p, double* vconst, double* dvpp,
-                  float* R32, float2* eikR32, float* kw32, cudaStream_t st);
-
-// k_setup.cu: the reciprocal-space force as a [3N][2 nk] matrix on rho(k) (split measure path).
-void launch_recforce_table(int N, int nk, double L, const int4* kvec, const double* kw, const double2* eikR, float* T,
-                           cudaStream_t st);
+                  double* vpp, float* R32, float2* eikR32, float* kw32, float* Trec, cudaStream_t st);
 
 // k_recforce.cu: F[W][M] = rho[W][K] . T[K][M] (reciprocal-space force of every walker sample).
 void launch_recforce_gemm(int W, int M, int K, const float* rho, const float* T, float* F, cudaStream_t st);
