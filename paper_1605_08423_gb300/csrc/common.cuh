@@ -65,12 +65,42 @@ __device__ __forceinline__ double qexp(double x) { return exp(x); }
 __device__ __forceinline__ float qexp(float x) { return expf(x); }
 __device__ __forceinline__ double qsqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ float qsqrt(float x) { return sqrtf(x); }
-// Reciprocal and square root of the pair loops: IEEE in FP64; in FP32 the
-// hardware approximations (a few ulp), well inside the FP32-level tolerance of
-// the mixed form.
-__device__ __forceinline__ double qrcp(double x) { return 1.0 / x; }
+// Reciprocal and square root of the pair loops.  FP32: the hardware
+// approximations (a few ulp), well inside the FP32-level tolerance of the mixed
+// form.  FP64: the FP64 pipe issues two multiply-adds a clock and SM, so the
+// pair loops are bound by their FP64 operation count; a hardware seed (about
+// 20 bits, PTX rcp / rsqrt.approx.ftz.f64) followed by one third-order
+// Householder step (Householder 1970; error of the seed cubed, below 2^-57)
+// takes 3 and 5 FP64 operations with no slow path:
+//   1/x:       e = 1 - x y,    y (1 + e + e^2)
+//   1/sqrt x:  e = 1 - x y^2,  y (1 + e/2 + 3 e^2 / 8)
+// Arguments are normal and positive in the pair loops (1 + b r, t > 0).
+__device__ __forceinline__ double rcp_seed(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return y;
+}
+__device__ __forceinline__ double rsqrt_seed(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return y;
+}
+__device__ __forceinline__ double qrcp(double x) {
+    const double y = rcp_seed(x);
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
 __device__ __forceinline__ float qrcp(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double qsqrt_pair(double x) { return sqrt(x); }
+__device__ __forceinline__ double qrsqrt(double x) {
+    const double y = rsqrt_seed(x);
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+__device__ __forceinline__ double qsqrt_pair(double x) {
+    // x = 0 (coincident points) gives 0: the sign-and-magnitude word of a
+    // non-negative double is zero only there, so no FP64 compare is needed
+    return __double_as_longlong(x) > 0 ? x * qrsqrt(x) : 0.0;
+}
 __device__ __forceinline__ float qsqrt_pair(float x) { return x > 0.f ? x * rsqrtf(x) : 0.f; }
 __device__ __forceinline__ double qerfc(double x) { return erfc(x); }
 __device__ __forceinline__ float qerfc(float x) { return erfcf(x); }

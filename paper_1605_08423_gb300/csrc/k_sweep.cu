@@ -1,56 +1,42 @@
 // k_sweep.cu -- one Metropolis sweep of every walker (single-electron moves).
 //
-// One warp per walker.  For electron i (up block first, then down) with
-// proposal r'_i (precomputed by the proposal kernel) and its orbital row
-// phi'_j = phi_j(r'_i) (precomputed by the orbital kernel for the whole sweep):
+// For electron i (up block first, then down) with proposal r'_i (precomputed
+// by the proposal kernel) and its orbital row phi'_j = phi_j(r'_i) (precomputed
+// by the orbital kernel for the whole sweep):
 //   ratio   R  = sum_j phi'_j G_{j,i}                     (determinant ratio)
 //   Jastrow dU = sum_{j != i} [u_ee(r'_i,r_j) - u_ee(r_i,r_j)] + sum_a [u_en(r'_i,R_a) - u_en(r_i,R_a)]
 //   accept if u < R^2 exp(2 dU)
 // and on acceptance the Sherman-Morrison rank-1 update of the inverse of the
 // spin block:  G' = G - G_{:,i} (phi'^T G - e_i^T) / R.
-// The inverse of the moving spin block is staged in shared memory (row stride
-// n+1: conflict-free per-lane rows) for the n moves of that block.
+// The electron's own e-n sum V_i = sum_a u_en(r_i, R_a) is carried between the
+// moves and the sweeps of a call (an accepted move replaces it by the sum at
+// the proposal), so a move evaluates the e-n terms at the proposal only.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.cuh"
 
 namespace qmc {
 
-template <typename T>
+// FP64 form, one warp per walker; the inverse of the moving spin block is
+// staged in shared memory for the n moves of that block.
 struct SweepSmem {
     // Rows of the staged inverse are 16-byte vectors: nv = n rounded up to a
     // whole vector (zero padded), row stride ld = nv + one vector, so that the
     // 16-byte accesses of 8 consecutive lanes (one per row) hit distinct banks.
-    static constexpr int VE = 16 / sizeof(T);   // elements per 16-byte vector
+    static constexpr int VE = 2;   // doubles per 16-byte vector
     __host__ __device__ static int nv(int n) { return (n + VE - 1) / VE * VE; }
     __host__ __device__ static int ld(int n) { return nv(n) + VE; }
-    // per warp: G^T [n][ld], old row [nv], phi' [nv], trig [6N], and only with
-    // the e-e-n-n Jastrow term (j34) three [N] vectors (sum over electrons of
-    // chi_a, chi_a at the moving electron and at its proposal)
+    // per warp: G^T [n][ld], old row [nv], phi' [nv], proposal trig [6], trig
+    // [6N], V [N], and only with the e-e-n-n Jastrow term (j34) three [N]
+    // vectors (sum over electrons of chi_a, chi_a at the moving electron and
+    // at its proposal)
     __host__ __device__ static size_t warp_bytes(int N, int n, bool j34) {
-        size_t b = ((size_t)n * ld(n) + 2 * (size_t)nv(n)) * sizeof(T);
-        b += (size_t)(j34 ? 9 : 6) * N * sizeof(T);
+        size_t b = ((size_t)n * ld(n) + 2 * (size_t)nv(n) + 6) * sizeof(double);
+        b += (size_t)(j34 ? 10 : 7) * N * sizeof(double);
         return (b + 15) & ~size_t(15);
     }
 };
-
-template <typename T> struct Vec16;
-template <> struct Vec16<float> { using type = float4; };
-template <> struct Vec16<double> { using type = double2; };
-
-__device__ __forceinline__ float vdot(float4 a, float4 b, float acc[4]) {
-    acc[0] += a.x * b.x; acc[1] += a.y * b.y; acc[2] += a.z * b.z; acc[3] += a.w * b.w;
-    return 0.f;
-}
-__device__ __forceinline__ double vdot(double2 a, double2 b, double acc[4]) {
-    acc[0] += a.x * b.x; acc[1] += a.y * b.y;
-    return 0.0;
-}
-__device__ __forceinline__ float4 vaxpy(float4 g, float c, float4 r) {
-    return make_float4(g.x - c * r.x, g.y - c * r.y, g.z - c * r.z, g.w - c * r.w);
-}
-__device__ __forceinline__ double2 vaxpy(double2 g, double c, double2 r) {
-    return make_double2(g.x - c * r.x, g.y - c * r.y);
-}
 
 // exp(-zeta |d|^2) for the periodised displacement between two points given
 // by their (sin, cos)(pi x / L) triples (e-e-n-n Jastrow orbital)
@@ -78,160 +64,170 @@ __device__ __forceinline__ T pair_dist(const T* a, const T* b, T ell) {
     return ell * qsqrt_pair(t);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(512) sweep_kernel(SysView<T> s, double* __restrict__ X, const double* __restrict__ Xp,
-                                                    const T* __restrict__ ptp, const T* __restrict__ uacc,
-                                                    const T* __restrict__ Phi,
-                                                    T* __restrict__ Gt, unsigned long long* __restrict__ nacc) {
+// Pade pair term c r / (1 + b r) of two points' trig triples (c = 1/2: e-e, c = -Zj: e-n).
+__device__ __forceinline__ double pade_u(const double* a, const double* b, double ell, double cb, double cu) {
+    const double r = pair_dist(a, b, ell);
+    return cu * r * qrcp(fma(cb, r, 1.0));
+}
+
+// FP64 form.  Bound by the FP64 pipe (two multiply-adds a clock and SM, so a
+// warp instruction occupies it for 16 clocks however many lanes are on): a move
+// of N = 64 costs 3 N Pade pairs of 22 operations and the rank-1 update.  The
+// new and old e-e terms share one lane loop of 2 N items, so that small N
+// fills the warp; walkers are spread evenly over the SMs by the launcher.
+__global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* __restrict__ X,
+                                                    const double* __restrict__ Xp, const double* __restrict__ ptp,
+                                                    const double* __restrict__ uacc, const double* __restrict__ Phi,
+                                                    double* __restrict__ Gt, unsigned long long* __restrict__ nacc,
+                                                    double* __restrict__ Vep, int vep_init) {
     extern __shared__ __align__(16) unsigned char smraw[];
-    using V = typename Vec16<T>::type;
-    constexpr int VE = SweepSmem<T>::VE;
-    const int N = s.N, n = s.n, nv = SweepSmem<T>::nv(n), ld = SweepSmem<T>::ld(n), nvv = nv / VE;
+    constexpr int VE = SweepSmem::VE;
+    const int N = s.N, n = s.n, nv = SweepSmem::nv(n), ld = SweepSmem::ld(n), nvv = nv / VE;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    T* ptr_s = (T*)smraw;                                    // [N][6] proton trig
-    size_t off = ((size_t)6 * N * sizeof(T) + 15) & ~size_t(15);
-    const bool j34 = sizeof(T) == 8 && s.fjt != nullptr;
-    unsigned char* mine = smraw + off + (size_t)warp * SweepSmem<T>::warp_bytes(N, n, j34);
-    T* Gs = (T*)mine;
-    T* rowb = Gs + (size_t)n * ld;
-    T* phi = rowb + nv;
-    T* et = phi + nv;
-    T* c34 = et + 6 * N;     // [N] sum over electrons of chi_a (e-e-n-n Jastrow term, FP64 form)
-    T* cho = c34 + N;        // [N] chi_a at the moving electron
-    T* chn = cho + N;        // [N] chi_a at its proposal
+    double* ptr_s = (double*)smraw;                          // [N][6] proton trig
+    const size_t off = ((size_t)6 * N * sizeof(double) + 15) & ~size_t(15);
+    const bool j34 = s.fjt != nullptr;
+    unsigned char* mine = smraw + off + (size_t)warp * SweepSmem::warp_bytes(N, n, j34);
+    double* Gs = (double*)mine;
+    double* rowb = Gs + (size_t)n * ld;
+    double* phi = rowb + nv;
+    double* ptb = phi + nv;       // [6] the proposal's trig
+    double* et = ptb + 6;
+    double* vj = et + 6 * N;      // [N] V_i
+    double* c34 = vj + N;         // [N] sum over electrons of chi_a (e-e-n-n Jastrow term)
+    double* cho = c34 + N;        // [N] chi_a at the moving electron
+    double* chn = cho + N;        // [N] chi_a at its proposal
 
     for (int idx = threadIdx.x; idx < 6 * N; idx += blockDim.x) ptr_s[idx] = s.ptrig[idx];
     __syncthreads();
     const int w = blockIdx.x * wpb + warp;
     if (w >= s.W) return;
 
-    const T ell = (T)s.ell, bee = (T)s.b_ee, bep = (T)s.b_ep, Zj = (T)s.Zj;
-    const double L = s.L;
+    const double ell = s.ell, bee = s.b_ee, bep = s.b_ep, Zj = s.Zj;
+    const double L = s.L, iL = s.iL;
     double* Xw = X + (size_t)w * 3 * N;   // positions stay in HBM; accepted moves are written through
-    const double iL = 1.0 / L;
     for (int idx = lane; idx < 3 * N; idx += 32) {
         const int i = idx / 3, mu = idx % 3;
-        T sn, cs;
-        qsincospi((T)(Xw[idx] * iL), &sn, &cs);
+        double sn, cs;
+        sincospi(Xw[idx] * iL, &sn, &cs);
         et[6 * i + mu] = sn;
         et[6 * i + 3 + mu] = cs;
     }
     __syncwarp();
-    const T zj = (T)s.zeta_j;
+    for (int i = lane; i < N; i += 32) {
+        double v = 0;
+        if (vep_init)
+            for (int a = 0; a < N; ++a) v += pade_u(et + 6 * i, ptr_s + 6 * a, ell, bep, -Zj);
+        else
+            v = Vep[(size_t)w * N + i];
+        vj[i] = v;
+    }
+    const double zj = s.zeta_j;
     if (j34) {
         for (int a = lane; a < N; a += 32) {
-            T c = 0;
+            double c = 0;
             for (int j = 0; j < N; ++j) c += jas_orbital(et + 6 * j, ptr_s + 6 * a, ell, zj);
             c34[a] = c;
         }
-        __syncwarp();
     }
-    for (int j = n + lane; j < nv; j += 32) phi[j] = T(0);   // padding stays zero
+    __syncwarp();
+    for (int j = n + lane; j < nv; j += 32) phi[j] = 0.0;   // padding stays zero
     unsigned long long naccept = 0;
-    // the next move's proposal trig, orbital row (n <= 64: two per lane) and
-    // uniform are loaded one move ahead, so their HBM latency overlaps a move
-    T pt_nx[6], ph_nx[2], u_nx;
+    // the next move's proposal trig (lanes 0-5), orbital row (n <= 64: two per
+    // lane) and uniform are loaded one move ahead, so their HBM latency
+    // overlaps a move
+    double pt_nx, ph_nx[2], u_nx;
     auto fetch = [&](int i) {
         const size_t row = (size_t)w * N + i;
+        pt_nx = lane < 6 ? ptp[row * 6 + lane] : 0.0;
 #pragma unroll
-        for (int mu = 0; mu < 6; ++mu) pt_nx[mu] = ptp[row * 6 + mu];
-#pragma unroll
-        for (int k = 0; k < 2; ++k) ph_nx[k] = (lane + 32 * k < n) ? Phi[row * n + lane + 32 * k] : T(0);
+        for (int k = 0; k < 2; ++k) ph_nx[k] = (lane + 32 * k < n) ? Phi[row * n + lane + 32 * k] : 0.0;
         u_nx = uacc[row];
     };
     fetch(0);
     for (int sp = 0; sp < 2; ++sp) {
-        T* G = Gt + ((size_t)w * 2 + sp) * n * n;
+        double* G = Gt + ((size_t)w * 2 + sp) * n * n;
         for (int idx = lane; idx < n * nv; idx += 32) {
             const int r = idx / nv, c = idx - r * nv;
-            Gs[r * ld + c] = c < n ? G[r * n + c] : T(0);
+            Gs[r * ld + c] = c < n ? G[r * n + c] : 0.0;
         }
         __syncwarp();
         for (int il = 0; il < n; ++il) {
             const int i = sp * n + il;
             const size_t row = (size_t)w * N + i;
-            T pt[6];
-#pragma unroll
-            for (int mu = 0; mu < 6; ++mu) pt[mu] = pt_nx[mu];
+            if (lane < 6) ptb[lane] = pt_nx;
 #pragma unroll
             for (int k = 0; k < 2; ++k)
                 if (lane + 32 * k < n) phi[lane + 32 * k] = ph_nx[k];
-            const T u = u_nx;
+            const double u = u_nx;
             if (i + 1 < N) fetch(i + 1);
             __syncwarp();
-            T part = 0;
+            double part = 0;
             for (int j = lane; j < n; j += 32) part += phi[j] * Gs[il * ld + j];
-            const T ratio = warp_sum(part);
-            T du = 0;
-            const T* ei = et + 6 * i;
-#pragma unroll 4
-            for (int j = lane; j < N; j += 32) {
-                const T* ej = et + 6 * j;
-                T u1, u0, d1, d2;
-                pade_ee(bee, pair_dist(pt, ej, ell), u1, d1, d2);
-                pade_ee(bee, pair_dist(ei, ej, ell), u0, d1, d2);
-                du += (j != i) ? u1 - u0 : T(0);
+            const double ratio = warp_sum(part);
+            const double* ei = et + 6 * i;
+            // items 0..N-1: u_ee at the proposal, N..2N-1: minus u_ee at the old position
+            double du = 0, vnew = 0;
+            for (int k = lane; k < 2 * N; k += 32) {
+                const bool old = k >= N;
+                const int j = old ? k - N : k;
+                const double v = pade_u(old ? ei : ptb, et + 6 * j, ell, bee, old ? -0.5 : 0.5);
+                du += j != i ? v : 0.0;
             }
-#pragma unroll 4
-            for (int a = lane; a < N; a += 32) {
-                const T* pa = ptr_s + 6 * a;
-                T u1, u0, d1, d2, d3;
-                pade_ep(bep, Zj, pair_dist(pt, pa, ell), u1, d1, d2, d3);
-                pade_ep(bep, Zj, pair_dist(ei, pa, ell), u0, d1, d2, d3);
-                du += u1 - u0;
-            }
+            for (int a = lane; a < N; a += 32) vnew += pade_u(ptb, ptr_s + 6 * a, ell, bep, -Zj);
             if (j34) {
                 // e-e-n-n term: the pairs (i, j != i) change by
                 // sum_a (chi_a(r'_i) - chi_a(r_i)) sum_b f_ab (c_b - chi_b(r_i))
                 for (int a = lane; a < N; a += 32) {
-                    chn[a] = jas_orbital(pt, ptr_s + 6 * a, ell, zj);
+                    chn[a] = jas_orbital(ptb, ptr_s + 6 * a, ell, zj);
                     cho[a] = jas_orbital(ei, ptr_s + 6 * a, ell, zj);
                 }
                 __syncwarp();
                 for (int a = lane; a < N; a += 32) {
                     // f is symmetric (checked at qmc_init): column a = row a,
                     // and the lanes' loads of a column element are consecutive
-                    const T* fa = s.fjt + a;
-                    T wa = 0;
+                    const double* fa = s.fjt + a;
+                    double wa = 0;
                     for (int b = 0; b < N; ++b) wa += fa[(size_t)b * N] * (c34[b] - cho[b]);
                     du += (chn[a] - cho[a]) * wa;
                 }
             }
-            du = warp_sum(du);
-            const T prob = ratio * ratio * qexp(T(2) * du);
+            // both warp sums in five additions: lanes 0-15 reduce du, 16-31 vnew
+            double x = lane < 16 ? du : vnew;
+            x += __shfl_xor_sync(0xffffffffu, lane < 16 ? vnew : du, 16);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            vnew = __shfl_sync(0xffffffffu, x, 16);
+            du = __shfl_sync(0xffffffffu, x, 0) + (vnew - vj[i]);
+            const double prob = ratio * ratio * exp(2.0 * du);
             if (u < prob) {
                 for (int j = lane; j < nv; j += 32) rowb[j] = Gs[il * ld + j];
                 __syncwarp();
-                const T ir = T(1) / ratio;
-                const V* phv = (const V*)phi;
-                const V* rbv = (const V*)rowb;
+                const double ir = 1.0 / ratio;
+                const double2* phv = (const double2*)phi;
+                const double2* rbv = (const double2*)rowb;
                 for (int l = lane; l < n; l += 32) {
-                    V* gl = (V*)(Gs + l * ld);
-                    T w4[4] = {0, 0, 0, 0};   // partial sums per vector component: short chains
-                    for (int jv = 0; jv < nvv; ++jv) vdot(phv[jv], gl[jv], w4);
-                    const T wl = (w4[0] + w4[1]) + (w4[2] + w4[3]);
-                    const T coef = (wl - (l == il ? T(1) : T(0))) * ir;
-                    for (int jv = 0; jv < nvv; ++jv) gl[jv] = vaxpy(gl[jv], coef, rbv[jv]);
-                }
-                if (lane < 3) {
-                    // FP64 form: wrap into [0, L) at once (as the reference chain does).
-                    // Mixed form: keep the proposal as is (every function of the
-                    // positions is periodic; the next proposal pass wraps), so no
-                    // FP64 arithmetic runs per move.
-                    const double xpl = Xp[row * 3 + lane];
-                    if (sizeof(T) == 8) {
-                        const double x = xpl - L * floor(xpl / L);
-                        Xw[3 * i + lane] = x;
-                        T sn, cs;
-                        qsincospi((T)(x / L), &sn, &cs);
-                        et[6 * i + lane] = sn;
-                        et[6 * i + 3 + lane] = cs;
-                    } else {
-                        Xw[3 * i + lane] = xpl;
-                        et[6 * i + lane] = pt[lane];
-                        et[6 * i + 3 + lane] = pt[3 + lane];
+                    double2* gl = (double2*)(Gs + l * ld);
+                    double w0 = 0, w1 = 0;   // two partial sums: short chains
+                    for (int jv = 0; jv < nvv; ++jv) {
+                        const double2 p = phv[jv], g = gl[jv];
+                        w0 += p.x * g.x; w1 += p.y * g.y;
+                    }
+                    const double coef = ((w0 + w1) - (l == il ? 1.0 : 0.0)) * ir;
+                    for (int jv = 0; jv < nvv; ++jv) {
+                        const double2 g = gl[jv], r = rbv[jv];
+                        gl[jv] = make_double2(g.x - coef * r.x, g.y - coef * r.y);
                     }
                 }
+                if (lane < 3) {   // wrap into [0, L) at once (as the reference chain does)
+                    const double xpl = Xp[row * 3 + lane];
+                    Xw[3 * i + lane] = xpl - L * floor(xpl / L);
+                }
+                // the trig triple of the unwrapped proposal: wrapping flips the
+                // signs of a component's sine and cosine together, and every use
+                // is even in that sign
+                if (lane < 6) et[6 * i + lane] = ptb[lane];
+                if (lane == 0) vj[i] = vnew;
                 if (j34)
                     for (int a = lane; a < N; a += 32) c34[a] += chn[a] - cho[a];
                 ++naccept;
@@ -239,9 +235,9 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<T> s, double* __rest
             __syncwarp();
         }
         for (int idx = lane; idx < n * n; idx += 32) G[idx] = Gs[(idx / n) * ld + idx % n];
-        (void)VE;
         __syncwarp();
     }
+    for (int i = lane; i < N; i += 32) Vep[(size_t)w * N + i] = vj[i];
     if (lane == 0) nacc[w] += naccept;
 }
 
@@ -501,44 +497,49 @@ __global__ void __launch_bounds__(64 * kSwWalkers) sweep_reg_kernel(SysView<floa
     if (tw == 0) nacc[w] += naccept;
 }
 
-template <typename T>
-void launch_sweep(const SysView<T>& s, double* X, const double* Xp, const T* ptp, const T* uacc, const T* Phi, T* Gt,
-                  unsigned long long* nacc, float* vep, bool vep_init, cudaStream_t st) {
-    if constexpr (sizeof(T) == 4) {
-        if (s.n <= kSwRow) {   // mixed form: inverse rows in registers
-            const bool j34 = s.fjt != nullptr;
-            const size_t smem = sizeof(float) * (((kTS * s.N + 3) & ~3) + (j34 ? (size_t)s.N * s.N : 0) +
-                                                 kSwWalkers * sweep_reg_walker_floats(s.N, j34));
-            static size_t attr = 0;
-            if (smem > attr &&
-                cudaFuncSetAttribute(sweep_reg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-                    cudaSuccess)
-                attr = smem;
-            sweep_reg_kernel<<<(s.W + kSwWalkers - 1) / kSwWalkers, 64 * kSwWalkers, smem, st>>>(
-                *(const SysView<float>*)&s, X, Xp, (const float*)ptp, (const float*)uacc, (const float*)Phi,
-                (float*)Gt, nacc, vep, vep_init ? 1 : 0);
-            return;
-        }
-    }
-    const size_t wb = SweepSmem<T>::warp_bytes(s.N, s.n, sizeof(T) == 8 && s.fjt != nullptr);
-    const size_t head = ((size_t)6 * s.N * sizeof(T) + 15) & ~size_t(15);
-    // as many walkers per CTA as the shared memory of one SM holds (one CTA per SM)
-    int wpb = (int)((226 * 1024 - head) / wb);
-    if (wpb > 16) wpb = 16;
-    if (wpb < 1) wpb = 1;
-    const size_t smem = head + wpb * wb;
-    static bool attr_set[2] = {false, false};
-    const int which = sizeof(T) == 8;
-    if (!attr_set[which]) {
-        cudaFuncSetAttribute(sweep_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-        attr_set[which] = true;
-    }
-    sweep_kernel<T><<<(s.W + wpb - 1) / wpb, 32 * wpb, smem, st>>>(s, X, Xp, ptp, uacc, Phi, Gt, nacc);
+// Walkers per CTA of a kernel that takes one warp per walker: at most `most`
+// (shared memory), and no more than spreads the walkers evenly over the SMs in
+// the fewest rounds.  With 16 walkers a CTA, 1024 walkers sat on 64 of the 152
+// SMs and a sweep of N = 64 took 2.9 ms (0.9 ms with 7 a CTA on 147 of them).
+int walkers_per_cta(int W, int most) {
+    static const int sms = [] {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        return v > 0 ? v : 1;
+    }();
+    const long long per_round = (long long)sms * most;
+    const long long rounds = (W + per_round - 1) / per_round;
+    return (int)((W + sms * rounds - 1) / (sms * rounds));
 }
 
-template void launch_sweep<double>(const SysView<double>&, double*, const double*, const double*, const double*,
-                                   const double*, double*, unsigned long long*, float*, bool, cudaStream_t);
-template void launch_sweep<float>(const SysView<float>&, double*, const double*, const float*, const float*,
-                                  const float*, float*, unsigned long long*, float*, bool, cudaStream_t);
+void launch_sweep(const SysView<float>& s, double* X, const double* Xp, const float* ptp, const float* uacc,
+                  const float* Phi, float* Gt, unsigned long long* nacc, float* vep, bool vep_init, cudaStream_t st) {
+    const bool j34 = s.fjt != nullptr;
+    const size_t smem = sizeof(float) * (((kTS * s.N + 3) & ~3) + (j34 ? (size_t)s.N * s.N : 0) +
+                                         kSwWalkers * sweep_reg_walker_floats(s.N, j34));
+    static size_t attr = 0;
+    if (smem > attr &&
+        cudaFuncSetAttribute(sweep_reg_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)
+        attr = smem;
+    sweep_reg_kernel<<<(s.W + kSwWalkers - 1) / kSwWalkers, 64 * kSwWalkers, smem, st>>>(s, X, Xp, ptp, uacc, Phi, Gt,
+                                                                                         nacc, vep, vep_init ? 1 : 0);
+}
+
+void launch_sweep(const SysView<double>& s, double* X, const double* Xp, const double* ptp, const double* uacc,
+                  const double* Phi, double* Gt, unsigned long long* nacc, double* vep, bool vep_init,
+                  cudaStream_t st) {
+    const size_t wb = SweepSmem::warp_bytes(s.N, s.n, s.fjt != nullptr);
+    const size_t head = ((size_t)6 * s.N * sizeof(double) + 15) & ~size_t(15);
+    const int fit = (int)((226 * 1024 - head) / wb);
+    const int wpb = walkers_per_cta(s.W, std::max(1, std::min(16, fit)));
+    static bool attr_set = false;
+    if (!attr_set) {
+        cudaFuncSetAttribute(sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        attr_set = true;
+    }
+    sweep_kernel<<<(s.W + wpb - 1) / wpb, 32 * wpb, head + wpb * wb, st>>>(s, X, Xp, ptp, uacc, Phi, Gt, nacc, vep,
+                                                                           vep_init ? 1 : 0);
+}
 
 }  // namespace qmc

@@ -36,13 +36,16 @@ void launch_invert(int W, int N, int n, const T* Phi, T* Gt, double* logdet, int
 // Gauss-Jordan where the carried inverse is too far off).
 void launch_refine(int W, int N, int n, const float* Phi, float* Gt, double* logdet, int* err, cudaStream_t st);
 
-// k_sweep.cu: one Metropolis sweep per walker (warp per walker).
-template <typename T>
+// k_sweep.cu: one Metropolis sweep per walker.
 // vep: [W][N] per-electron e-n Jastrow sums carried between the sweeps of a
-// call by the mixed-form register sweep (computed when vep_init, i.e. in the
-// call's first sweep); unused by the other sweep kernels.
-void launch_sweep(const SysView<T>& s, double* X, const double* Xp, const T* ptp, const T* uacc, const T* Phi, T* Gt,
-                  unsigned long long* nacc, float* vep, bool vep_init, cudaStream_t st);
+// call (computed when vep_init, i.e. in the call's first sweep).
+void launch_sweep(const SysView<float>& s, double* X, const double* Xp, const float* ptp, const float* uacc,
+                  const float* Phi, float* Gt, unsigned long long* nacc, float* vep, bool vep_init, cudaStream_t st);
+void launch_sweep(const SysView<double>& s, double* X, const double* Xp, const double* ptp, const double* uacc,
+                  const double* Phi, double* Gt, unsigned long long* nacc, double* vep, bool vep_init,
+                  cudaStream_t st);
+// Walkers per CTA for a warp-per-walker kernel that holds at most `most` of them.
+int walkers_per_cta(int W, int most);
 
 // k_measure.cu: local energy, d ln psi / dR and dE_L / dR per walker.
 template <typename T>
