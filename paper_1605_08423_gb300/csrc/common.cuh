@@ -179,6 +179,8 @@ struct SysView {
     const double* fj;       // [N][N] e-e-n-n Jastrow coefficients (symmetric), or null
     const T* fjt;           // the same in the working precision, or null
     double zeta_j;          // their Gaussians' exponent
+    const double* ewt;      // real-space Ewald table (FP64 form, kappa L <= kEwMaxKL), or null: see EwTable
+    double ew_h, ew_ih;     // its node spacing in r^2 and the inverse
 };
 
 // Twisted boundary conditions: walker w samples twist t = w / Wk (K contiguous
@@ -290,6 +292,100 @@ __device__ __forceinline__ T ewald_real(T dx, T dy, T dz, T Lt, T kappa, T* grad
             const T s = dphi * ir;
             grad[0] += s * a; grad[1] += s * b; grad[2] += s * e;
         }
+    }
+    return v;
+}
+
+// ---------------------------------------------------------------------------
+// Real-space Ewald terms from a table (FP64 form).  With x = (kappa r)^2,
+//   erf(kappa r)/r  = kappa (2/sqrt pi) F_0(x),   F_n(x) = int_0^1     s^2n exp(-x s^2) ds,
+//   erfc(kappa r)/r = kappa (2/sqrt pi) G_0(x),   G_n(x) = int_1^inf  s^2n exp(-x s^2) ds
+// (F_n: the Boys functions, S. F. Boys, Proc. R. Soc. A 200, 1950), and
+// d/dx F_n = -F_{n+1}, d/dx G_n = -G_{n+1}: the Taylor coefficients about a node
+// are (-1)^n F_n / n! times powers of kappa, filled by stable recurrences
+// (k_setup.cu).  Both are tabulated in r^2 at nodes i h, h = 0.75 L^2 / 511, to
+// degree 7: erf(kappa r)/r for the minimum image (r^2 <= 3/4 L^2, the term
+// 1/r - erf(kappa r)/r), erfc(kappa r)/r for the other images (L^2/4 <= r^2 <
+// L^2).  |x - x_node| <= 0.0264 for kappa L <= 6, so the remainder is below
+// 1e-18 of kappa for the value and 2e-16 kappa^3 for the derivative in r^2,
+// under the rounding of the sums they enter.  A value and its derivative cost
+// 16 FP64 operations, where erfc, exp, a square root and the divisions took
+// about 190; the FP64 pipe is what bounds the pair sums.
+constexpr int kEwNodes = 512, kEwTerms = 8;
+constexpr int kEwFirstB = 170;            // first node of the erfc table: floor(0.25 L^2 / h)
+constexpr double kEwMaxKL = 6.0;
+
+struct EwTable {
+    const double* t;    // [2][kEwNodes][kEwTerms]
+    double h, ih, L, iL, LL;
+};
+
+// Value at r2 (and derivative in r2) of table `which` (0: erf(kappa r)/r, 1: erfc(kappa r)/r).
+template <bool kGrad>
+__device__ __forceinline__ double ew_eval(const EwTable& T, int which, double r2, double* d) {
+    const double magic = 6755399441055744.0;   // 1.5 * 2^52: the sum's low word is the nearest integer
+    const double qm = fma(r2, T.ih, magic);
+    int i = __double2loint(qm) - (which ? kEwFirstB : 0);
+    i = i < 0 ? 0 : (i > kEwNodes - 1 ? kEwNodes - 1 : i);
+    const double t = fma(-T.h, qm - magic, r2);
+    const double2* c = (const double2*)(T.t + ((size_t)which * kEwNodes + i) * kEwTerms);
+    const double2 c67 = c[3], c45 = c[2], c23 = c[1], c01 = c[0];
+    double v = fma(c67.y, t, c67.x);
+    if (kGrad) {
+        double g = fma(c67.y, t, v);
+        v = fma(v, t, c45.y); g = fma(g, t, v);
+        v = fma(v, t, c45.x); g = fma(g, t, v);
+        v = fma(v, t, c23.y); g = fma(g, t, v);
+        v = fma(v, t, c23.x); g = fma(g, t, v);
+        v = fma(v, t, c01.y); g = fma(g, t, v);
+        v = fma(v, t, c01.x);
+        *d = g;
+    } else {
+        v = fma(v, t, c45.y); v = fma(v, t, c45.x); v = fma(v, t, c23.y);
+        v = fma(v, t, c23.x); v = fma(v, t, c01.y); v = fma(v, t, c01.x);
+    }
+    return v;
+}
+
+// ewald_real<double> from the table: sum of phi(r) over the images with r < L,
+// and when kGrad its gradient in g (overwritten).
+template <bool kGrad>
+__device__ __forceinline__ double ewald_table(double dx, double dy, double dz, const EwTable& T, double* g) {
+    const double magic = 6755399441055744.0, L = T.L;
+    dx = fma(-L, fma(dx, T.iL, magic) - magic, dx);
+    dy = fma(-L, fma(dy, T.iL, magic) - magic, dy);
+    dz = fma(-L, fma(dz, T.iL, magic) - magic, dz);
+    const double r0 = dx * dx + dy * dy + dz * dz;
+    // moving component m of the minimum image by L away from zero adds L (L - 2 |d_m|) to r^2
+    const double e0 = fma(-2.0 * L, fabs(dx), T.LL), e1 = fma(-2.0 * L, fabs(dy), T.LL),
+                 e2 = fma(-2.0 * L, fabs(dz), T.LL);
+    const double r1 = r0 + e0, r2 = r0 + e1, r3 = r1 + e1, r4 = r0 + e2;
+    // positive doubles compare as their bit patterns (integer pipe)
+    const long long lim = __double_as_longlong(T.LL);
+    auto in = [&](double r) { return __double_as_longlong(r) < lim; };
+    unsigned mask = (in(r1) ? 2u : 0u) | (in(r2) ? 4u : 0u) | (in(r3) ? 8u : 0u) | (in(r4) ? 16u : 0u) |
+                    (in(r1 + e2) ? 32u : 0u) | (in(r2 + e2) ? 64u : 0u) | (in(r3 + e2) ? 128u : 0u);
+    double v = 0, s = 0, s0 = 0, s1 = 0, s2 = 0, d;
+    if (__double_as_longlong(r0) > 0) {
+        const double ir = qrsqrt(r0);
+        v = ir - ew_eval<kGrad>(T, 0, r0, &d);
+        if (kGrad) s = fma(-ir * ir, 0.5 * ir, -d);    // d phi / d r^2
+    }
+    while (mask) {
+        const int c = __ffs(mask) - 1;
+        mask &= mask - 1;
+        const double ra = (c & 1) ? e0 : 0.0, rb = (c & 2) ? e1 : 0.0, rc = (c & 4) ? e2 : 0.0;
+        v += ew_eval<kGrad>(T, 1, r0 + ra + rb + rc, &d);
+        if (kGrad) {
+            s += d;
+            s0 += (c & 1) ? d : 0.0; s1 += (c & 2) ? d : 0.0; s2 += (c & 4) ? d : 0.0;
+        }
+    }
+    if (kGrad) {   // grad = 2 sum d (x + shift): the shifts collected per component
+        const double s2x = s + s;
+        g[0] = fma(s2x, dx, (dx >= 0.0 ? -2.0 : 2.0) * L * s0);
+        g[1] = fma(s2x, dy, (dy >= 0.0 ? -2.0 : 2.0) * L * s1);
+        g[2] = fma(s2x, dz, (dz >= 0.0 ? -2.0 : 2.0) * L * s2);
     }
     return v;
 }

@@ -40,6 +40,7 @@ struct qmc_system {
     double *d_R = nullptr, *d_zeta = nullptr, *d_C64 = nullptr, *d_kw = nullptr, *d_ptrig64 = nullptr;
     float *d_C32 = nullptr, *d_ptrig32 = nullptr;
     int4* d_kvec = nullptr;
+    double* d_ewt = nullptr;   // real-space Ewald table (FP64 form)
     double2 *d_eikR = nullptr, *d_rhop = nullptr;
     double *d_vconst = nullptr, *d_dvpp = nullptr, *d_vpp = nullptr;
     float *d_R32 = nullptr, *d_kw32 = nullptr, *d_zeta32 = nullptr;
@@ -214,6 +215,7 @@ size_t footprint(const qmc_params* p) {
     b += 8 * (2 * W + 6 * W * N);                    // eval outputs
     b += 8 * (3 * 3 * N + 3 * 9 * N * N);           // Langevin
     b += 8 * (2 * 3 * N + 2 * 9 * N * N);           // first simplified scheme between its halves
+    if (t == 8) b += 8 * 2 * kEwNodes * kEwTerms;    // real-space Ewald table
     if (p->fj) b += (t == 4 ? 12 : 8) * N * N;       // e-e-n-n Jastrow coefficients (+ FP32 copy)
     if (p->n_twist > 0) {
         // twists, phase table, real D' / Lp' / unit rows / zero coefficients, E_L and ln|psi|, per-twist results
@@ -268,6 +270,7 @@ SysView<T> view(qmc_system* h, int W) {
     s.nk = h->nk; s.mmax = h->mmax;
     s.kvec = h->d_kvec; s.kw = h->d_kw; s.eikR = h->d_eikR; s.rho_p = h->d_rhop;
     s.vconst = h->d_vconst; s.dvpp = h->d_dvpp; s.err = h->d_err; s.vacc = h->d_vacc;
+    s.ewt = h->d_ewt; s.ew_h = 0.75 * h->p.L * h->p.L / (kEwNodes - 1); s.ew_ih = 1.0 / s.ew_h;
     s.fj = h->d_fj; s.zeta_j = h->p.zeta_j;
     s.fjt = (const T*)(sizeof(T) == 8 ? (const void*)h->d_fj : (const void*)h->d_fj32);
     return s;
@@ -662,6 +665,7 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
             h->use_tc_adj = true;
         }
     }
+    if (!h->mixed && p->ewald_kappa * p->L <= kEwMaxKL) h->d_ewt = dalloc<double>(h, 2 * kEwNodes * kEwTerms, &rc);
     if (rc != QMC_OK) { qmc_destroy(h); return rc; }
     std::vector<float> c32(h->coeff_h.begin(), h->coeff_h.end());
     std::vector<float> z32(h->zeta_h.begin(), h->zeta_h.end());
@@ -687,6 +691,7 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
     cudaMemsetAsync(h->d_nacc, 0, sizeof(unsigned long long) * W, st);
     if (h->d_chat) prepare_tc_coeff(h->d_C32, B, n, h->d_chat, st);
     if (h->d_ahat) prepare_tc_adjoint_coeff(h->d_C32, N, h->G, n, h->d_ahat, st);
+    if (h->d_ewt) launch_ewald_table(p->ewald_kappa, 0.75 * p->L * p->L / (kEwNodes - 1), h->d_ewt, st);
     setup_tables(h);
     launch_init_walkers(W, N, p->L, h->d_R, h->d_X, make_key(p->seed), 0u, st);
     h->emp_lambda = thomas_fermi_length(N, p->L);

@@ -136,30 +136,6 @@ __device__ __forceinline__ void ep_jastrow(const S sd[3], const S cd[3], S ell, 
     for (int mu = 0; mu < 3; ++mu) { dl[mu] = -rd.g[mu]; de[mu] = hv[mu] + S(0.5) * rd.tl[mu]; }
 }
 
-template <typename S>
-__device__ __forceinline__ void ep_pair(const S sd[3], const S cd[3], S ell, S k2, S bep, S Zj, S dx, S dy, S dz, S L,
-                                        S kap, const S vv[3], S& v, S g[3], S dl[3], S de[3]) {
-    S p[3], q[3], t = 0;
-#pragma unroll
-    for (int mu = 0; mu < 3; ++mu) {
-        p[mu] = ell * sd[mu] * cd[mu];
-        q[mu] = cd[mu] * cd[mu] - sd[mu] * sd[mu];
-        t += sd[mu] * sd[mu];
-    }
-    t *= ell * ell;
-    const S r = qsqrt_pair(t);
-    S u, u1, u2, u3, f1, f2, f3;
-    pade_ep(bep, Zj, r, u, u1, u2, u3);
-    rho_to_t(r, u1, u2, u3, f1, f2, f3);
-    RadialDerivs<S> rd;
-    radial_chain(p, q, f1, f2, f3, k2, rd);
-    S hv[3];
-    hess_mul(rd.h, vv, hv);
-#pragma unroll
-    for (int mu = 0; mu < 3; ++mu) { dl[mu] = -rd.g[mu]; de[mu] = hv[mu] + S(0.5) * rd.tl[mu]; }
-    v = ewald_real<S>(dx, dy, dz, L, kap, g);
-}
-
 // e-e-n-n Jastrow orbital chi_a(r_i) = exp(-zeta |d|^2) of electron trig ei and
 // nucleus trig pa with its gradient, Hessian, Laplacian and gradient of the
 // Laplacian in the electron coordinate (radial chain of f(t) = exp(-zeta t)).
@@ -525,6 +501,7 @@ __global__ void __launch_bounds__(256, kSplit ? 3 : 1) measure_kernel(SysView<T>
     // ---- P4a: electron-electron real-space Ewald
     double vee_p = 0.0;
     const T Lt = (T)L;
+    const EwTable ewt{s.ewt, s.ew_h, s.ew_ih, L, iL, L * L};
     const float iLt = 1.f / (float)Lt, rc2 = kRealCut2Mixed * (float)Lt * (float)Lt;
     // balanced cyclic pairing: electron i with i+d (mod N), d = 1..N/2 (d = N/2 only for i < N/2),
     // the distance range split into nparts slices
@@ -539,10 +516,13 @@ __global__ void __launch_bounds__(256, kSplit ? 3 : 1) measure_kernel(SysView<T>
             if constexpr (sizeof(T) == 4) {
                 v += ewald_real_cut<false>(xt[3 * i] - xt[3 * j], xt[3 * i + 1] - xt[3 * j + 1],
                                            xt[3 * i + 2] - xt[3 * j + 2], false, Lt, iLt, rc2, kap, nullptr);
-                continue;
             }
-            v += ewald_real<T>(xt[3 * i] - xt[3 * j], xt[3 * i + 1] - xt[3 * j + 1], xt[3 * i + 2] - xt[3 * j + 2], Lt,
-                               kap, nullptr);
+            else {
+                const double dx = xs[3 * i] - xs[3 * j], dy = xs[3 * i + 1] - xs[3 * j + 1],
+                             dz = xs[3 * i + 2] - xs[3 * j + 2];
+                v += ewt.t ? ewald_table<false>(dx, dy, dz, ewt, nullptr)
+                           : ewald_real<double>(dx, dy, dz, L, kap, nullptr);
+            }
         }
         vee_p += (double)v;
     }
@@ -581,20 +561,16 @@ __global__ void __launch_bounds__(256, kSplit ? 3 : 1) measure_kernel(SysView<T>
                 }
                 v += ewald_real_cut<true>(xt[3 * i] - ra[0], xt[3 * i + 1] - ra[1], xt[3 * i + 2] - ra[2], close, Lt,
                                           iLt, rc2, kap, gv);
-                continue;
             }
-            if (close) {   // only the images other than the nearest one here
-                T pg[3] = {0, 0, 0};
-                v += ewald_real<T>(xt[3 * i] - ra[0], xt[3 * i + 1] - ra[1], xt[3 * i + 2] - ra[2], Lt, kap, pg, true);
-                for (int mu = 0; mu < 3; ++mu) gv[mu] += pg[mu];
-                continue;
+            else {
+                double vv[3], pg[3], pl[3], pe[3];
+                for (int mu = 0; mu < 3; ++mu) vv[mu] = vvs[3 * i + mu];
+                ep_jastrow<double>(sd, cd, ell, k2, bep, Zj, vv, pl, pe);
+                const double dx = xs[3 * i] - s.R[3 * a], dy = xs[3 * i + 1] - s.R[3 * a + 1],
+                             dz = xs[3 * i + 2] - s.R[3 * a + 2];
+                v += ewt.t ? ewald_table<true>(dx, dy, dz, ewt, pg) : ewald_real<double>(dx, dy, dz, L, kap, pg);
+                for (int mu = 0; mu < 3; ++mu) { gv[mu] += pg[mu]; dl[mu] += pl[mu]; de[mu] += pe[mu]; }
             }
-            T vv[3], pv, pg[3], pl[3], pe[3];
-            for (int mu = 0; mu < 3; ++mu) vv[mu] = gi[3 * i + mu] + gU[3 * i + mu];
-            ep_pair<T>(sd, cd, ell, k2, bep, Zj, xt[3 * i] - ra[0], xt[3 * i + 1] - ra[1], xt[3 * i + 2] - ra[2],
-                       Lt, kap, vv, pv, pg, pl, pe);
-            v += pv;
-            for (int mu = 0; mu < 3; ++mu) { gv[mu] += pg[mu]; dl[mu] += pl[mu]; de[mu] += pe[mu]; }
         }
         v = warp_sum(v);
 #pragma unroll

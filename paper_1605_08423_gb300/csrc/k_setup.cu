@@ -134,4 +134,39 @@ void launch_setup(int N, double L, double kappa, int nk, const int4* kvec, const
     setup_sum_kernel<<<1 + bRho + bRec, 128, 0, st>>>(N, nk, bRho, L, kappa, kvec, kw, eikR, vpp, rho_p, vconst, Trec);
 }
 
+// Taylor coefficients of the real-space Ewald table (EwTable in common.cuh),
+// once per handle: one thread per node.  F_7 from its (all-positive) series
+//   F_n(x) = exp(-x) sum_i (2x)^i / ((2n+1)(2n+3)...(2n+2i+1)),
+// F_6..F_0 by F_{n-1} = (2x F_n + exp(-x)) / (2n-1); G_0 from erfc and
+// G_n = (exp(-x) + (2n-1) G_{n-1}) / 2x: every term positive, no cancellation.
+__global__ void ewald_table_kernel(double kappa, double h, double* __restrict__ t) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= 2 * kEwNodes) return;
+    const int which = k / kEwNodes, i = k - which * kEwNodes + (which ? kEwFirstB : 0);
+    const double x = kappa * kappa * (h * i), ex = exp(-x);
+    double f[kEwTerms];
+    if (which == 0) {
+        double term = 1.0 / (2 * kEwTerms - 1), sum = 0.0;
+        for (int j = 1; j < 400 && term > 1e-18 * sum; ++j) {
+            sum += term;
+            term *= 2.0 * x / (2 * kEwTerms - 1 + 2 * j);
+        }
+        f[kEwTerms - 1] = ex * sum;
+        for (int n = kEwTerms - 1; n > 0; --n) f[n - 1] = (2.0 * x * f[n] + ex) / (2 * n - 1);
+    } else {
+        const double r = sqrt(x);
+        f[0] = 0.88622692545275801365 * erfc(r) / r;   // sqrt(pi) / 2
+        for (int n = 1; n < kEwTerms; ++n) f[n] = (ex + (2 * n - 1) * f[n - 1]) / (2.0 * x);
+    }
+    double c = 1.1283791670955125739 * kappa;          // 2 / sqrt(pi)
+    for (int n = 0; n < kEwTerms; ++n) {
+        t[(size_t)k * kEwTerms + n] = c * f[n];
+        c *= -kappa * kappa / (n + 1);
+    }
+}
+
+void launch_ewald_table(double kappa, double h, double* t, cudaStream_t st) {
+    ewald_table_kernel<<<(2 * kEwNodes + 63) / 64, 64, 0, st>>>(kappa, h, t);
+}
+
 }  // namespace qmc

@@ -62,6 +62,9 @@ void launch_setup(int N, double L, double kappa, int nk, const int4* kvec, const
                   double* ptrig64, float* ptrig32, double2* eikR, double2* rho_p, double* vconst, double* dvpp,
                   double* vpp, float* R32, float2* eikR32, float* kw32, float* Trec, cudaStream_t st);
 
+// k_setup.cu: real-space Ewald table of the FP64 form (EwTable), once per handle.
+void launch_ewald_table(double kappa, double h, double* t, cudaStream_t st);
+
 // k_recforce.cu: F[W][M] = rho[W][K] . T[K][M] (reciprocal-space force of every walker sample).
 void launch_recforce_gemm(int W, int M, int K, const float* rho, const float* T, float* F, cudaStream_t st);
 
