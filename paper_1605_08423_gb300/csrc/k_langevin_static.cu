@@ -28,27 +28,27 @@ namespace qmc {
 static __device__ __align__(256) double g_langevin_scratch[QMC_STATIC_MAX_N3 * QMC_STATIC_MAX_N3];
 static __device__ __align__(256) int g_langevin_err;
 
-// The step of langevin_kernel (same device code, cta_langevin_step), with the
-// previous pair (R_prev, S_prev) given by the caller (nothing is stored) and
-// the result written to Rout.  Rout may be R itself (the entry point passes
-// the same buffer): R, Rprev and Rout are therefore not __restrict__, and every
-// read of R and Rprev is done before the barrier that precedes the store.
-__global__ void __launch_bounds__(1024) langevin_static_kernel(int n, const double* R, const double* Rprev,
-                                                               const double* __restrict__ f,
-                                                               const double* __restrict__ S,
-                                                               const double* __restrict__ Sprev, double* Lc,
-                                                               double* Rout, double T, double delta, double alpha,
-                                                               Key key, uint32_t md, double box, int identity,
-                                                               int* err) {
+// The step of langevin_kernel (same device code, lv_step), with the previous
+// pair (R_prev, S_prev) given by the caller (nothing is stored) and the result
+// written to Rout.  Rout may be R itself (the entry point passes the same
+// buffer): R, Rprev and Rout are therefore not __restrict__, and every read of
+// R and Rprev is done before the step returns.
+__global__ void __launch_bounds__(kLvThreads) langevin_static_kernel(int n, const double* R, const double* Rprev,
+                                                                     const double* f, const double* S,
+                                                                     const double* Sprev, double* Lc, double* Rout,
+                                                                     double T, double delta, double alpha, Key key,
+                                                                     uint32_t md, double box, int identity, int* err) {
     extern __shared__ double v[];
-    __shared__ double red[32];
-    double* r1 = nullptr;
-    if (!cta_langevin_step(n, R, Rprev, f, S, Sprev, Lc, T, delta, alpha, key, md, box, identity, kLvAdopted, v, red,
-                           &r1)) {
-        if (threadIdx.x == 0) atomicOr(err, kErrNotPD);
+    __shared__ LvSmem sm;
+    cg::cluster_group cl = cg::this_cluster();
+    double *r0 = nullptr, *r1 = nullptr;
+    if (!lv_step(cl, n, R, Rprev, f, S, Sprev, Lc, T, delta, alpha, key, md, box, identity, kLvAdopted, v, sm, &r0,
+                 &r1)) {
+        if (threadIdx.x == 0 && cl.block_rank() == 0) atomicOr(err, kErrNotPD);
         return;
     }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) Rout[i] = r1[i];
+    if (r1)
+        for (int i = threadIdx.x; i < n; i += kLvThreads) Rout[i] = r1[i];
 }
 
 namespace {
@@ -102,9 +102,12 @@ extern "C" int qmc_langevin_step_static(int n3, double* R, const double* Rprev, 
     const int identity = s_mode == QMC_S_IDENTITY;
     if (cudaMemsetAsync(a.err, 0, sizeof(int), st) != cudaSuccess) return QMC_ERR_CUDA;
     const size_t smem = 5 * (size_t)n3 * sizeof(double);
-    langevin_static_kernel<<<1, 1024, smem, st>>>(n3, R, Rprev, f, S, Sprev, a.scratch, R,
-                                                   T_kelvin * 3.166811563e-6, delta, identity ? 0.0 : alpha,
-                                                   make_key(seed), step, box, identity, a.err);
+    if (lv_launch(langevin_static_kernel, identity ? 1 : langevin_cluster(n3), smem, st, n3, R, Rprev, f, S, Sprev,
+                  a.scratch, R, T_kelvin * 3.166811563e-6, delta, identity ? 0.0 : alpha, make_key(seed), step, box,
+                  identity, a.err) != cudaSuccess) {
+        cudaGetLastError();
+        return QMC_ERR_CUDA;
+    }
     if (cudaGetLastError() != cudaSuccess) return QMC_ERR_CUDA;
     int e = 0;
     if (cudaMemcpyAsync(&e, a.err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess) return QMC_ERR_CUDA;

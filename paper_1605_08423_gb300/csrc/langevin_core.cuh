@@ -1,62 +1,253 @@
-// langevin_core.cuh -- one-CTA FP64 building blocks of the accelerated
-// first-order Langevin step (SI, integration schemes), shared by the handle's
-// kernel (k_langevin.cu) and the allocation-free entry point
-// (k_langevin_static.cu), so that both compute the step with the same code.
+// langevin_core.cuh -- FP64 building blocks of the accelerated first-order
+// Langevin step (SI, integration schemes), shared by the handle's kernels
+// (k_langevin.cu) and the allocation-free entry point (k_langevin_static.cu),
+// so that all compute the step with the same code.
+//
+// One thread-block cluster of P CTAs (P = 1 for small n) takes the step.  The
+// Cholesky factorisation is blocked: per block column of 32, one warp factors
+// the diagonal tile in registers (shuffles, L D L^T order so that one
+// reciprocal and no square root is on the chain), the rows below are solved
+// against it (a row per lane), and the trailing 32 x 32 tiles are updated by
+// all CTAs; the first CTA updates the next diagonal tile first and factors it
+// while the others work on the rest.  The matrix stays in L2 (Lc, read and
+// written with .cg accesses); the cluster barrier orders the phases.
+//
+// What bounds it: an SM issues two FP64 multiply-adds a clock, so the n^3/6 of
+// n = 384 take 2.3 ms on one SM; 16 SMs bring that under the chain of diagonal
+// tiles and barriers.  One CTA, column by column, took 11.5 ms at n = 384 and
+// 0.77 ms at n = 48 (1.03 and 0.15 ms in this form).
 #pragma once
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "kernels.cuh"
 
 namespace qmc {
 
-// Cholesky S = L L^T of an n x n SPD matrix (row-major) by one CTA,
-// left-looking, column by column, into the lower triangle of Lc.  Returns
-// false on every thread if S is not positive definite (the pivot test uses a
-// block-wide sum, so all threads see the same value).
-__device__ inline bool cta_cholesky(int n, const double* __restrict__ S, double* Lc, double* red) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    for (int j = 0; j < n; ++j) {
-        double p = 0.0;
-        for (int k = tid; k < j; k += nt) p += Lc[(size_t)j * n + k] * Lc[(size_t)j * n + k];
-        p = block_sum(p, red);
-        const double d = S[(size_t)j * n + j] - p;
-        if (!(d > 0.0)) return false;
-        const double ljj = sqrt(d);
-        if (tid == 0) Lc[(size_t)j * n + j] = ljj;
-        for (int i = j + 1 + tid; i < n; i += nt) {
-            double t = S[(size_t)i * n + j];
-            for (int k = 0; k < j; ++k) t -= Lc[(size_t)i * n + k] * Lc[(size_t)j * n + k];
-            Lc[(size_t)i * n + j] = t / ljj;
-        }
-        __syncthreads();
+namespace cg = cooperative_groups;
+
+constexpr int kLvThreads = 256, kLvTb = 32;
+
+struct LvSmem {
+    double D[kLvTb][kLvTb + 1];   // diagonal tile of the current block column
+    double A[kLvTb][kLvTb + 1];   // operand tiles (A also stages a row tile)
+    double B[kLvTb][kLvTb + 1];
+    double inv[kLvTb];            // reciprocal diagonal of D
+    double yk[2][kLvTb];          // solved block of up to two right-hand sides
+    int fail;                     // set by the first CTA: not positive definite
+};
+
+// CTAs of the cluster for an n x n factorisation: about as many as the first
+// block column has trailing tiles to share.
+__host__ inline int langevin_cluster(int n) {
+    const int nt = (n + kLvTb - 1) / kLvTb;
+    return nt <= 2 ? 1 : nt <= 4 ? 4 : nt <= 7 ? 8 : 16;
+}
+
+// Diagonal tile k into sm.D with its reciprocal diagonal (identity beyond n).
+__device__ inline void lv_load_diag(int n, const double* Lc, int k, LvSmem& sm) {
+    const int k0 = k * kLvTb;
+    for (int idx = threadIdx.x; idx < kLvTb * kLvTb; idx += kLvThreads) {
+        const int r = idx >> 5, c = idx & 31, i = k0 + r, j = k0 + c;
+        const double v = (i < n && j <= i) ? __ldcg(Lc + (size_t)i * n + j) : (r == c ? 1.0 : 0.0);
+        sm.D[r][c] = v;
+        if (r == c) sm.inv[r] = 1.0 / v;
+    }
+    __syncthreads();
+}
+
+// One warp: Cholesky factor of diagonal tile k in place (lane = row).  Returns
+// false (on every lane) at a pivot that is not positive.
+__device__ inline bool lv_factor_tile(int n, double* Lc, int k) {
+    const int lane = threadIdx.x & 31, k0 = k * kLvTb, row = k0 + lane;
+    double a[kLvTb];
+#pragma unroll
+    for (int c = 0; c < kLvTb; ++c)
+        a[c] = (c <= lane && row < n) ? __ldcg(Lc + (size_t)row * n + k0 + c) : (c == lane ? 1.0 : 0.0);
+    double dl = 1.0;
+    bool ok = true;
+#pragma unroll
+    for (int c = 0; c < kLvTb; ++c) {
+        const double d = __shfl_sync(0xffffffffu, a[c], c);
+        ok = ok && d > 0.0;
+        const double y = (d > 1e-280 && d < 1e280) ? qrcp(d) : 1.0 / d;
+        if (lane == c) dl = d;
+        const double l = a[c] * y;     // unit-triangular entry; a[c] keeps l d
+#pragma unroll
+        for (int j = c + 1; j < kLvTb; ++j) a[j] -= l * __shfl_sync(0xffffffffu, a[c], j);
+    }
+    if (!ok) return false;
+    const double rs = 1.0 / sqrt(dl);
+#pragma unroll
+    for (int c = 0; c < kLvTb; ++c) {
+        const double v = a[c] * __shfl_sync(0xffffffffu, rs, c);
+        if (c <= lane && row < n) __stcg(Lc + (size_t)row * n + k0 + c, v);
     }
     return true;
 }
 
-// In-place forward solve L w = g (g in shared memory), column oriented.
-__device__ inline void cta_forward(int n, const double* Lc, double* g) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    for (int k = 0; k < n; ++k) {
-        const double wk = g[k] / Lc[(size_t)k * n + k];
+// One warp: row tile I of block column k solved against sm.D, X = A L_kk^-T
+// (lane = row).  st: this warp's staging tile.
+__device__ inline void lv_solve_rows(int n, double* Lc, int k, int I, const LvSmem& sm) {
+    const int lane = threadIdx.x & 31, k0 = k * kLvTb, row = I * kLvTb + lane;
+    if (row >= n) return;
+    double* p = Lc + (size_t)row * n + k0;
+    double b[kLvTb];
+#pragma unroll
+    for (int c = 0; c < kLvTb; ++c) b[c] = __ldcg(p + c);
+#pragma unroll
+    for (int c = 0; c < kLvTb; ++c) {
+        b[c] *= sm.inv[c];
+#pragma unroll
+        for (int j = c + 1; j < kLvTb; ++j) b[j] -= b[c] * sm.D[j][c];
+    }
+#pragma unroll
+    for (int c = 0; c < kLvTb; ++c) __stcg(p + c, b[c]);
+}
+
+// The CTA: tile (I, J) -= L_Ik L_Jk^T.
+__device__ inline void lv_update_tile(int n, double* Lc, int k, int I, int J, LvSmem& sm) {
+    const int tid = threadIdx.x, k0 = k * kLvTb, i0 = I * kLvTb, j0 = J * kLvTb;
+    __syncthreads();
+    for (int idx = tid; idx < kLvTb * kLvTb; idx += kLvThreads) {
+        const int r = idx >> 5, c = idx & 31;
+        sm.A[r][c] = i0 + r < n ? __ldcg(Lc + (size_t)(i0 + r) * n + k0 + c) : 0.0;
+        sm.B[r][c] = j0 + r < n ? __ldcg(Lc + (size_t)(j0 + r) * n + k0 + c) : 0.0;
+    }
+    const int tx = tid & 15, ty = tid >> 4;
+    double v[2][2];
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int i = i0 + ty + 16 * a, j = j0 + tx + 16 * b;
+            v[a][b] = (i < n && j <= i) ? __ldcg(Lc + (size_t)i * n + j) : 0.0;
+        }
+    __syncthreads();
+#pragma unroll 8
+    for (int c = 0; c < kLvTb; ++c) {
+        const double a0 = sm.A[ty][c], a1 = sm.A[ty + 16][c], b0 = sm.B[tx][c], b1 = sm.B[tx + 16][c];
+        v[0][0] -= a0 * b0; v[0][1] -= a0 * b1; v[1][0] -= a1 * b0; v[1][1] -= a1 * b1;
+    }
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int i = i0 + ty + 16 * a, j = j0 + tx + 16 * b;
+            if (i < n && j <= i) __stcg(Lc + (size_t)i * n + j, v[a][b]);
+        }
+}
+
+// The CTA: block k of the forward solve L y = g (g in shared memory, solved in
+// place), sm.D holding diagonal tile k: the block itself by one warp, then the
+// rows below, one per thread.
+__device__ inline void lv_forward_block(int n, const double* Lc, int k, double* g, LvSmem& sm) {
+    const int tid = threadIdx.x, k0 = k * kLvTb;
+    if (tid < 32) {
+        double v = k0 + tid < n ? g[k0 + tid] : 0.0;
+#pragma unroll
+        for (int c = 0; c < kLvTb; ++c) {
+            const double y = __shfl_sync(0xffffffffu, v, c) * sm.inv[c];
+            v = tid == c ? y : (tid > c ? v - sm.D[tid][c] * y : v);
+        }
+        sm.yk[0][tid] = v;
+        if (k0 + tid < n) g[k0 + tid] = v;
+    }
+    __syncthreads();
+    for (int i = k0 + kLvTb + tid; i < n; i += kLvThreads) {
+        const double* p = Lc + (size_t)i * n + k0;
+        double s0 = 0, s1 = 0;
+#pragma unroll 8
+        for (int c = 0; c < kLvTb; c += 2) {
+            s0 += __ldcg(p + c) * sm.yk[0][c];
+            s1 += __ldcg(p + c + 1) * sm.yk[0][c + 1];
+        }
+        g[i] -= s0 + s1;
+    }
+    __syncthreads();
+}
+
+// The CTA: back solve L^T x = w for `nrhs` (1 or 2) right-hand sides w[q] in
+// shared memory, solved in place.
+__device__ inline void lv_backward(int n, const double* Lc, double* const w[2], int nrhs, LvSmem& sm) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int k = (n + kLvTb - 1) / kLvTb - 1; k >= 0; --k) {
+        const int k0 = k * kLvTb;
+        lv_load_diag(n, Lc, k, sm);
+        if (warp < nrhs) {
+            double* g = w[warp];
+            double v = k0 + lane < n ? g[k0 + lane] : 0.0;
+#pragma unroll
+            for (int c = kLvTb - 1; c >= 0; --c) {
+                const double x = __shfl_sync(0xffffffffu, v, c) * sm.inv[c];
+                v = lane == c ? x : (lane < c ? v - sm.D[c][lane] * x : v);
+            }
+            sm.yk[warp][lane] = v;
+            if (k0 + lane < n) g[k0 + lane] = v;
+        }
         __syncthreads();
-        if (tid == 0) g[k] = wk;
-        for (int i = k + 1 + tid; i < n; i += nt) g[i] -= Lc[(size_t)i * n + k] * wk;
+        const int m = n - k0 < kLvTb ? n - k0 : kLvTb;
+        for (int j = tid; j < k0; j += kLvThreads) {   // column j of the block's rows: coalesced over threads
+            double s0 = 0, s1 = 0;
+#pragma unroll 8
+            for (int c = 0; c < m; ++c) {
+                const double l = __ldcg(Lc + (size_t)(k0 + c) * n + j);
+                s0 += l * sm.yk[0][c];
+                if (nrhs > 1) s1 += l * sm.yk[1][c];
+            }
+            w[0][j] -= s0;
+            if (nrhs > 1) w[1][j] -= s1;
+        }
         __syncthreads();
     }
 }
 
-// Back solve L^T x = w (w in shared memory, consumed), column oriented.
-__device__ inline void cta_backward(int n, const double* Lc, double* w, double* x) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    for (int k = n - 1; k >= 0; --k) {
-        const double xk = w[k] / Lc[(size_t)k * n + k];
-        __syncthreads();
-        if (tid == 0) x[k] = xk;
-        for (int i = tid; i < k; i += nt) w[i] -= Lc[(size_t)k * n + i] * xk;
-        __syncthreads();
+// The cluster: S = L L^T (row-major SPD, lower triangle used) into the lower
+// triangle of Lc; where g is set (on the cluster's last CTA only, shared
+// memory), the forward solve L y = g runs along, in place.  Returns false on
+// every thread if S is not positive definite.
+__device__ inline bool lv_cholesky(cg::cluster_group& cl, int n, const double* __restrict__ S, double* Lc, double* g,
+                                   LvSmem& sm) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int P = (int)cl.num_blocks(), rank = (int)cl.block_rank(), nt = (n + kLvTb - 1) / kLvTb;
+    for (int i = rank * (kLvThreads / 32) + warp; i < n; i += P * (kLvThreads / 32))
+        for (int j = lane; j <= i; j += 32) __stcg(Lc + (size_t)i * n + j, S[(size_t)i * n + j]);
+    if (tid == 0) sm.fail = 0;
+    cl.sync();
+    if (rank == 0 && warp == 0 && !lv_factor_tile(n, Lc, 0) && lane == 0) sm.fail = 1;
+    cl.sync();
+    const int* fail = cl.map_shared_rank(&sm.fail, 0);
+    for (int k = 0; k < nt; ++k) {
+        if (*(volatile const int*)fail) return false;   // written before the last barrier: the same for all
+        lv_load_diag(n, Lc, k, sm);
+        const int m = nt - 1 - k;                       // row tiles below
+        for (int q = rank + P * warp; q < m; q += P * (kLvThreads / 32)) lv_solve_rows(n, Lc, k, k + 1 + q, sm);
+        cl.sync();
+        // trailing tiles in column order; the first CTA takes (k+1, k+1) and
+        // its factorisation (about a tile's time), the others go round
+        if (rank == 0 && m > 0) {
+            lv_update_tile(n, Lc, k, k + 1, k + 1, sm);
+            __syncthreads();
+            if (warp == 0 && !lv_factor_tile(n, Lc, k + 1) && lane == 0) sm.fail = 1;
+        }
+        const int total = m * (m + 1) / 2;
+        int t = 1, J = 0, base = 0;                      // tile t of column J starts at base
+        for (; t < total; ++t) {
+            const int slot = t + (t >= P ? 1 : 0);       // slot P (the first CTA's second turn) is the factorisation
+            if (slot % P != rank) continue;
+            while (t >= base + (m - J)) { base += m - J; ++J; }
+            lv_update_tile(n, Lc, k, k + 1 + J + (t - base), k + 1 + J, sm);
+        }
+        if (g) {
+            __syncthreads();
+            lv_forward_block(n, Lc, k, g, sm);
+        }
+        cl.sync();
     }
+    return true;
 }
 
-// One step of the SI's adopted scheme (or a variant) by one CTA:
+// One step of the SI's adopted scheme (or a variant) by one cluster:
 //   R' = R + Dt S^{-1} [f - (S_prev - S)(R_prev - R) / (2 Db)] + sqrt(2 T Db) z,  <z z^T> = S^{-1}
 // with Dt = (1 - e^{-alpha D})/alpha, Db = (1 - e^{-2 alpha D})/(2 alpha) for
 // the adopted scheme with alpha > 0 and Dt = Db = D otherwise; kLvNorogna drops
@@ -67,85 +258,108 @@ __device__ inline void cta_backward(int n, const double* Lc, double* w, double* 
 // jump of one box side).
 // xi ~ N(0, I) from Philox (counter = (component, md, 0, kLangevin)).
 //
-// Aliasing: R, Rprev, f, S and Sprev are read, R' is returned in the shared
-// array r1 and nothing is written to global memory except Lc.  Every read of
-// R and Rprev happens before the barrier that precedes the return, so the
-// caller may write R' over R (or over Rprev) afterwards.  Shared memory v
-// holds 5 n doubles.  Returns false on every thread if S is not positive
-// definite (nothing else is computed then).
-__device__ inline bool cta_langevin_step(int n, const double* R, const double* Rprev, const double* f,
-                                         const double* S, const double* Sprev, double* Lc, double T, double delta,
-                                         double alpha, Key key, uint32_t md, double box, int identity, int scheme,
-                                         double* v, double* red, double** r1_out) {
-    double* g = v;          // [n]
-    double* x = g + n;      // [n]
-    double* z = x + n;      // [n]
+// Aliasing: R, Rprev, f, S and Sprev are read and nothing is written to global
+// memory except Lc.  R' (r1) and R (r0) are returned in the last CTA's shared
+// memory (*owner set there); every CTA's reads of S, Sprev, R, Rprev and f are
+// done when the function returns, so the caller may then overwrite them.
+// Dynamic shared memory v holds 5 n doubles.  Returns false on every thread if
+// S is not positive definite (nothing else is computed then).
+__device__ inline bool lv_step(cg::cluster_group& cl, int n, const double* R, const double* Rprev, const double* f,
+                               const double* S, const double* Sprev, double* Lc, double T, double delta, double alpha,
+                               Key key, uint32_t md, double box, int identity, int scheme, double* v, LvSmem& sm,
+                               double** r0_out, double** r1_out) {
+    double* g = v;          // [n] drift, then x
+    double* dr = g + n;     // [n] R_prev - R
+    double* z = dr + n;     // [n] xi, then z
     double* r0 = z + n;     // [n] R
     double* r1 = r0 + n;    // [n] R'
-    const int tid = threadIdx.x, nt = blockDim.x;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int P = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const bool last = rank == P - 1;
     double Dt = delta, Db = delta;
     if (!identity && scheme == kLvAdopted && alpha > 0.0) {
         Dt = (1.0 - exp(-alpha * delta)) / alpha;
         Db = (1.0 - exp(-2.0 * alpha * delta)) / (2.0 * alpha);
     }
-    if (!identity && !cta_cholesky(n, S, Lc, red)) return false;
     const bool two_time = !identity && scheme != kLvNorogna;
-    if (two_time) {   // R_prev - R (minimum image), kept in r1 until R' is formed
-        for (int j = tid; j < n; j += nt) {
-            double dj = Rprev[j] - R[j];
-            if (box > 0.0) dj -= box * rint(dj / box);
-            r1[j] = dj;
-        }
-        __syncthreads();
+    for (int j = tid; j < n; j += kLvThreads) {
+        const double r = R[j];
+        r0[j] = r;
+        double dj = Rprev[j] - r;
+        if (box > 0.0) dj -= box * rint(dj / box);
+        dr[j] = dj;
     }
-    // g = f - (S_prev - S)(R_prev - R) / (2 Db);  xi;  keep R
-    for (int i = tid; i < n; i += nt) {
-        double t = f[i];
+    if (last)
+        for (int i = tid; i < n; i += kLvThreads)
+            z[i] = Draw<double>::normal(philox((uint32_t)i, md, 0u, kLangevin, key));
+    cl.sync();   // every CTA of the cluster runs before its shared memory is written from another
+    // g = f - (S_prev - S)(R_prev - R) / (2 Db): a warp per row, into the last CTA's g
+    double* gl = cl.map_shared_rank(g, P - 1);
+    for (int i = rank * (kLvThreads / 32) + warp; i < n; i += P * (kLvThreads / 32)) {
+        double s = 0.0;
         if (two_time) {
-            double s = 0.0;
-            for (int j = 0; j < n; ++j) s += (Sprev[(size_t)i * n + j] - S[(size_t)i * n + j]) * r1[j];
-            t -= s / (2.0 * Db);
+            for (int j = lane; j < n; j += 32) s += (Sprev[(size_t)i * n + j] - S[(size_t)i * n + j]) * dr[j];
+            s = warp_sum(s);
         }
-        g[i] = t;
-        const uint4 w = philox((uint32_t)i, md, 0u, kLangevin, key);
-        z[i] = Draw<double>::normal(w);
-        r0[i] = R[i];
+        if (lane == 0) gl[i] = two_time ? f[i] - s / (2.0 * Db) : f[i];
     }
-    __syncthreads();
-    if (!identity) {
-        // forward solve L y = g (column oriented), y stored in g
-        for (int k = 0; k < n; ++k) {
-            const double yk = g[k] / Lc[(size_t)k * n + k];
-            __syncthreads();
-            if (tid == 0) g[k] = yk;
-            for (int i = k + 1 + tid; i < n; i += nt) g[i] -= Lc[(size_t)i * n + k] * yk;
-            __syncthreads();
-        }
-        // back solves L^T x = y and L^T z = xi
-        for (int k = n - 1; k >= 0; --k) {
-            const double xk = g[k] / Lc[(size_t)k * n + k];
-            const double zk = z[k] / Lc[(size_t)k * n + k];
-            __syncthreads();
-            if (tid == 0) { x[k] = xk; z[k] = zk; }
-            for (int i = tid; i < k; i += nt) {
-                g[i] -= Lc[(size_t)k * n + i] * xk;
-                z[i] -= Lc[(size_t)k * n + i] * zk;
-            }
-            __syncthreads();
-        }
+    if (identity) {
+        cl.sync();
     } else {
-        for (int i = tid; i < n; i += nt) x[i] = g[i];
+        if (!lv_cholesky(cl, n, S, Lc, last ? g : nullptr, sm)) {   // its first barrier publishes g
+            cl.sync();      // no CTA leaves while another still reads its shared memory
+            return false;
+        }
+        if (last) {
+            double* const w[2] = {g, z};
+            lv_backward(n, Lc, w, 2, sm);
+        }
+    }
+    if (last) {
+        const double amp = T > 0.0 ? sqrt(2.0 * T * Db) : 0.0;
+        for (int i = tid; i < n; i += kLvThreads) {
+            double r = r0[i] + Dt * g[i] + amp * z[i];
+            if (box > 0.0) r -= box * floor(r / box);
+            r1[i] = r;
+        }
         __syncthreads();
     }
-    const double amp = T > 0.0 ? sqrt(2.0 * T * Db) : 0.0;
-    for (int i = tid; i < n; i += nt) {
-        double r = r0[i] + Dt * x[i] + amp * z[i];
-        if (box > 0.0) r -= box * floor(r / box);
-        r1[i] = r;
-    }
-    __syncthreads();
-    *r1_out = r1;
+    *r0_out = last ? r0 : nullptr;
+    *r1_out = last ? r1 : nullptr;
     return true;
+}
+
+// Launch of a cluster kernel with kLvThreads threads per CTA; 16 CTAs need the
+// non-portable size, and 8 are taken where the device does not offer it.
+template <typename... KArgs, typename... Args>
+inline cudaError_t lv_launch(void (*kern)(KArgs...), int P, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kLvThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (P > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        P = 8;
+    }
+    static int offers16 = -1;   // whether the device can place the non-portable cluster (same for every kernel here)
+    for (;;) {
+        at[0].val.clusterDim.x = P;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(P);
+        int active = 0;
+        if (P > 8 && offers16 < 0)
+            offers16 = cudaOccupancyMaxActiveClusters(&active, kern, &cfg) == cudaSuccess && active > 0;
+        if (P > 8 && !offers16) {
+            cudaGetLastError();
+            P = 8;
+            continue;
+        }
+        return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+    }
 }
 
 }  // namespace qmc
