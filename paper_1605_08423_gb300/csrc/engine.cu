@@ -67,7 +67,7 @@ struct qmc_system {
     double* d_pout = nullptr;    // pressure output [5]
     unsigned long long* d_nacc = nullptr;
     // reductions and output
-    double *d_colsum = nullptr, *d_dev = nullptr, *d_out = nullptr;
+    double *d_colsum = nullptr, *d_dev = nullptr, *d_gws = nullptr, *d_out = nullptr;
     double *d_eval = nullptr;  // eval_config outputs
     // Langevin
     double *d_Rl = nullptr, *d_Rprev = nullptr, *d_f = nullptr, *d_S = nullptr, *d_Sprev = nullptr, *d_Lwork = nullptr;
@@ -211,7 +211,9 @@ size_t footprint(const qmc_params* p) {
     b += t * W * N + tc * (W * N * n + 2 * W * n * n + 3 * W * N * n + W * N * n);   // uacc, Phi, Gt, D, Lp
     b += 8 * 2 * W + 8 * W * (3 + 9 * N) + 8 * W;   // logdet, acc, nacc
     b += 8 * W + 8 * 5;                              // V_L sums, pressure output
-    b += 8 * (4 + 9 * N) + 8 * W * (3 * N + 1) + 8 * (4 + 3 * N + 9 * N * N);   // colsum, dev, out
+    const size_t Kr = p->n_twist > 0 ? p->n_twist : 1;
+    b += 8 * gram_ws_doubles((int)Kr, (int)(W / Kr), (int)N);
+    b += 8 * Kr * (4 + 9 * N) + 8 * W * (3 * N + 1) + 8 * (4 + 3 * N + 9 * N * N);   // colsum, dev, out
     b += 8 * (2 * W + 6 * W * N);                    // eval outputs
     b += 8 * (3 * 3 * N + 3 * 9 * N * N);           // Langevin
     b += 8 * (2 * 3 * N + 2 * 9 * N * N);           // first simplified scheme between its halves
@@ -469,12 +471,10 @@ double run_sampling_twist(qmc_system* h) {
 // Each twist's walker block reduced on its own, then the twist average.
 void reduce_twist(qmc_system* h, double moves) {
     const int K = h->K, Wk = h->W / K, N = h->N;
-    const size_t stride = 3 + 9 * (size_t)N, olen = 4 + 3 * (size_t)N + 9 * (size_t)N * N;
-    for (int t = 0; t < K; ++t)
-        launch_reduce(Wk, N, moves / K, h->d_acc + (size_t)t * Wk * stride, h->d_nacc + (size_t)t * Wk, h->d_colsum,
-                      h->d_dev, h->d_tout + (size_t)t * olen, h->d_err, h->stream);
+    launch_reduce(K, Wk, N, moves / K, h->d_acc, h->d_nacc, h->d_colsum, h->d_dev, h->d_gws, h->d_tout, h->d_err,
+                  h->stream);
     launch_twist_average(K, N, h->d_tout, h->d_out, h->stream);
-    h->nlaunch += 5 * K + 1;
+    h->nlaunch += 6;
 }
 
 template <typename T>
@@ -492,7 +492,8 @@ void run_call(qmc_system* h) {
     EventPair ep;
     prof_begin(h, KC_REDUCE, ep);
     h->nlaunch += 5;
-    launch_reduce(h->W, h->N, moves, h->d_acc, h->d_nacc, h->d_colsum, h->d_dev, h->d_out, h->d_err, h->stream);
+    launch_reduce(1, h->W, h->N, moves, h->d_acc, h->d_nacc, h->d_colsum, h->d_dev, h->d_gws, h->d_out, h->d_err,
+                  h->stream);
     prof_end(h, ep);
     h->last_Nc = (double)h->W * (h->p.n_sweeps / h->p.measure_every);
 }
@@ -603,7 +604,9 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
     h->d_vep = dalloc<unsigned char>(h, t * (size_t)W * N, &rc);
     h->d_pout = dalloc<double>(h, 5, &rc);
     h->d_nacc = dalloc<unsigned long long>(h, W, &rc);
-    h->d_colsum = dalloc<double>(h, 4 + 9 * N, &rc);
+    const int Kr = h->K ? h->K : 1;   // walker blocks reduced on their own
+    h->d_colsum = dalloc<double>(h, (size_t)Kr * (4 + 9 * N), &rc);
+    h->d_gws = dalloc<double>(h, gram_ws_doubles(Kr, W / Kr, N), &rc);
     h->d_dev = dalloc<double>(h, (size_t)W * (3 * N + 1), &rc);
     h->d_out = dalloc<double>(h, 4 + 3 * N + 9 * (size_t)N * N, &rc);
     h->d_eval = dalloc<double>(h, (size_t)W * (2 + 6 * N), &rc);
@@ -803,7 +806,7 @@ int qmc_shard_reduce_device(qmc_system* h, const double* sums_dev, double* out_d
     EventPair ep;
     prof_begin(h, KC_REDUCE, ep);
     h->nlaunch += 4;
-    launch_shard_reduce(h->W, h->N, h->d_acc, sums_dev, h->d_dev, out_dev, gram_dev, h->d_err, h->stream);
+    launch_shard_reduce(h->W, h->N, h->d_acc, sums_dev, h->d_dev, h->d_gws, out_dev, gram_dev, h->d_err, h->stream);
     prof_end(h, ep);
     return check_launch();
 }

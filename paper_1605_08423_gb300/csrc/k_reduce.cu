@@ -20,11 +20,19 @@
 
 namespace qmc {
 
+// The reductions run for a batch of K walker blocks of W walkers each (the
+// twists of a twisted handle; K = 1 otherwise), batch index blockIdx.y (.z in
+// the Gram kernels): one launch sequence for the whole mesh, where one per
+// twist made 320 launches and 2.25 ms of a 64-twist call at N = 64 (0.29 ms batched).
+
 // colsum[c] = sum_w acc[w][c] for c < ncol; colsum[ncol] = sum_w nacc[w].
 __global__ void colsum_kernel(int W, int ncol, const double* __restrict__ acc, const unsigned long long* __restrict__ nacc,
                               double* colsum) {
     __shared__ double red[32];
-    const int c = blockIdx.x;
+    const int c = blockIdx.x, b = blockIdx.y;
+    acc += (size_t)b * W * ncol;
+    nacc += (size_t)b * W;
+    colsum += (size_t)b * (ncol + 1);
     double s = 0.0;
     if (c < ncol)
         for (int w = threadIdx.x; w < W; w += blockDim.x) s += acc[(size_t)w * ncol + c];
@@ -38,6 +46,8 @@ __global__ void colsum_kernel(int W, int ncol, const double* __restrict__ acc, c
 // number of moves from colsum[ncol + 2], as the sharded form stores it).
 __global__ void finalize_kernel(int N, double moves, const double* __restrict__ colsum, double* out, int* err) {
     const int N3 = 3 * N, ncol = 3 + 9 * N;
+    colsum += (size_t)blockIdx.x * (ncol + 1);
+    out += (size_t)blockIdx.x * (4 + N3 + (size_t)N3 * N3);
     const double cnt = colsum[0];
     const double E = colsum[1] / cnt;
     for (int c = threadIdx.x; c < N3; c += blockDim.x) {
@@ -59,6 +69,9 @@ __global__ void deviation_kernel(int W, int N, const double* __restrict__ acc, c
     const int N3 = 3 * N, ncol = 3 + 9 * N;
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (size_t)W * (N3 + 1)) return;
+    acc += (size_t)blockIdx.y * W * ncol;
+    out += (size_t)blockIdx.y * (4 + N3 + (size_t)N3 * N3);
+    dev += (size_t)blockIdx.y * W * (N3 + 1);
     const int w = (int)(t / (N3 + 1)), c = (int)(t - (size_t)w * (N3 + 1));
     const double* a = acc + (size_t)w * ncol;
     const double cnt = a[0], E = out[0];
@@ -70,60 +83,118 @@ __global__ void deviation_kernel(int W, int N, const double* __restrict__ acc, c
     }
 }
 
-// sum_w (E_w - E)^2: written as sqrt(sum / (W (W - 1))) when finish != 0, else as the plain sum.
-__global__ void eerr_kernel(int W, int N, const double* __restrict__ dev, double* dst, int finish) {
+// Gram matrix of the deviations, sum_w dev[w][i] dev[w][j], and sum_w (E_w -
+// E)^2.  The FP64 pipe bounds it (3N (3N + 1) / 2 multiply-adds a walker): only
+// the lower triangle is formed, in 16 x 16 tiles of one output a thread, and
+// the walkers of a tile are cut into nsplit slices so that the chip is filled
+// at every N (32 x 32 tiles of the whole matrix left 144 blocks at N = 128 and
+// 36 at N = 64: the reduction took 5.5 ms for 16384 walkers and 1.3 ms for 4096,
+// now 2.5 and 0.24 ms).  The slices'
+// partial tiles go to ws [K][nsplit][tiles][256], summed in order by
+// gram_sum_kernel.  Tile index blockIdx.x (the last one is the energy's sum),
+// slice blockIdx.y, batch blockIdx.z.
+constexpr int kGramTile = 16, kGramRows = 32;
+__global__ void __launch_bounds__(256) gram_kernel(int W, int N, int tiles, const double* __restrict__ dev, double* ws) {
+    __shared__ double A[kGramRows][kGramTile], Bm[kGramRows][kGramTile];
+    const int N3 = 3 * N, ld = N3 + 1, tid = threadIdx.x;
+    const int t = blockIdx.x, sl = blockIdx.y, ns = gridDim.y;
+    dev += (size_t)blockIdx.z * W * ld;
+    ws += (((size_t)blockIdx.z * ns + sl) * (tiles + 1) + t) * 256;
+    const int w0 = (int)((long long)W * sl / ns), w1 = (int)((long long)W * (sl + 1) / ns);
+    if (t == tiles) {
+        double e = 0.0;
+        for (int w = w0 + tid; w < w1; w += 256) {
+            const double d = dev[(size_t)w * ld + N3];
+            e += d * d;
+        }
+        ws[tid] = e;
+        return;
+    }
+    int I = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+    while ((I + 1) * (I + 2) / 2 <= t) ++I;
+    while (I * (I + 1) / 2 > t) --I;
+    const int i0 = kGramTile * I, j0 = kGramTile * (t - I * (I + 1) / 2);
+    const int tx = tid & 15, ty = tid >> 4;
+    double s0 = 0.0, s1 = 0.0;
+    for (int wb = w0; wb < w1; wb += kGramRows) {
+#pragma unroll
+        for (int r = ty; r < kGramRows; r += 16) {
+            const int w = wb + r;
+            A[r][tx] = (w < w1 && i0 + tx < N3) ? dev[(size_t)w * ld + i0 + tx] : 0.0;
+            Bm[r][tx] = (w < w1 && j0 + tx < N3) ? dev[(size_t)w * ld + j0 + tx] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kGramRows; r += 2) {
+            s0 += A[r][ty] * Bm[r][tx];
+            s1 += A[r + 1][ty] * Bm[r + 1][tx];
+        }
+        __syncthreads();
+    }
+    ws[tid] = s0 + s1;
+}
+
+// dst_S[i][j] = dst_S[j][i] = scale * (sum of the tile's slices); *dst_e gets
+// sqrt(scale * sum_w (E_w - E)^2) when finish != 0, else the plain sum.  Per
+// batch dst_S and dst_e advance by `stride`.
+__global__ void __launch_bounds__(256) gram_sum_kernel(int N, int tiles, int ns, const double* __restrict__ ws,
+                                                       double* dst_e, double* dst_S, size_t stride, double scale,
+                                                       int finish) {
     __shared__ double red[32];
-    const int N3 = 3 * N;
-    double s = 0.0;
-    for (int w = threadIdx.x; w < W; w += blockDim.x) {
-        const double d = dev[(size_t)w * (N3 + 1) + N3];
-        s += d * d;
+    const int N3 = 3 * N, tid = threadIdx.x, t = blockIdx.x;
+    dst_e += blockIdx.z * stride;
+    dst_S += blockIdx.z * stride;
+    ws += ((size_t)blockIdx.z * ns * (tiles + 1) + t) * 256 + tid;
+    double v = 0.0;
+    for (int s = 0; s < ns; ++s) v += ws[(size_t)s * (tiles + 1) * 256];
+    if (t == tiles) {
+        v = block_sum(v, red);
+        if (tid == 0) *dst_e = finish ? sqrt(v * scale) : v;
+        return;
     }
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) dst[0] = finish ? (W > 1 ? sqrt(s / ((double)W * (W - 1))) : 0.0) : s;
+    int I = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+    while ((I + 1) * (I + 2) / 2 <= t) ++I;
+    while (I * (I + 1) / 2 > t) --I;
+    const int i = kGramTile * I + (tid >> 4), j = kGramTile * (t - I * (I + 1) / 2) + (tid & 15);
+    if (i >= N3 || j >= N3) return;
+    v *= scale;
+    dst_S[(size_t)i * N3 + j] = v;
+    dst_S[(size_t)j * N3 + i] = v;
 }
 
-// dst[i][j] = scale * sum_w dev[w][i] dev[w][j]: a 32 x 32 tile per block,
-// 256 threads, 4 outputs each.
-__global__ void __launch_bounds__(256) gram_kernel(int W, int N, const double* __restrict__ dev, double* dst,
-                                                   double scale) {
-    __shared__ double A[32][33], Bm[32][33];
-    const int N3 = 3 * N, ld = N3 + 1;
-    const int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    double acc[4] = {0, 0, 0, 0};
-    for (int w0 = 0; w0 < W; w0 += 32) {
-        for (int r = ty; r < 32; r += 8) {
-            const int w = w0 + r;
-            A[r][tx] = (w < W && i0 + tx < N3) ? dev[(size_t)w * ld + i0 + tx] : 0.0;
-            Bm[r][tx] = (w < W && j0 + tx < N3) ? dev[(size_t)w * ld + j0 + tx] : 0.0;
-        }
-        __syncthreads();
-#pragma unroll 8
-        for (int r = 0; r < 32; ++r) {
-            const double b = Bm[r][tx];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[q] += A[r][ty + 8 * q] * b;
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int i = i0 + ty + 8 * q, j = j0 + tx;
-        if (i < N3 && j < N3) dst[(size_t)i * N3 + j] = acc[q] * scale;
-    }
+static int gram_tiles(int N) {
+    const int nt = (3 * N + kGramTile - 1) / kGramTile;
+    return nt * (nt + 1) / 2;
+}
+// Slices per tile: about six blocks an SM of 152 in all, at least 64 walkers each.
+static int gram_splits(int K, int W, int N) {
+    const int want = (912 + gram_tiles(N) * K - 1) / (gram_tiles(N) * K), most = W / 64;
+    return want < 1 || most < 1 ? 1 : (want < most ? want : most);
+}
+size_t gram_ws_doubles(int K, int W, int N) {
+    return (size_t)K * gram_splits(K, W, N) * (gram_tiles(N) + 1) * 256;
 }
 
-void launch_reduce(int W, int N, double moves, const double* acc, const unsigned long long* nacc, double* colsum,
-                        double* dev, double* out, int* err, cudaStream_t st) {
+static void gram(int K, int W, int N, const double* dev, double* ws, double* dst_e, double* dst_S, size_t stride,
+                 double scale, int finish, cudaStream_t st) {
+    const int tiles = gram_tiles(N), ns = gram_splits(K, W, N);
+    gram_kernel<<<dim3(tiles + 1, ns, K), 256, 0, st>>>(W, N, tiles, dev, ws);
+    gram_sum_kernel<<<dim3(tiles + 1, 1, K), 256, 0, st>>>(N, tiles, ns, ws, dst_e, dst_S, stride, scale, finish);
+}
+
+static void deviations(int K, int W, int N, const double* acc, const double* out, double* dev, cudaStream_t st) {
+    const size_t tot = (size_t)W * (3 * N + 1);
+    deviation_kernel<<<dim3((unsigned)((tot + 255) / 256), K), 256, 0, st>>>(W, N, acc, out, dev);
+}
+
+void launch_reduce(int K, int W, int N, double moves, const double* acc, const unsigned long long* nacc, double* colsum,
+                   double* dev, double* ws, double* out, int* err, cudaStream_t st) {
     const int ncol = 3 + 9 * N, N3 = 3 * N;
-    colsum_kernel<<<ncol + 1, 256, 0, st>>>(W, ncol, acc, nacc, colsum);
-    finalize_kernel<<<1, 256, 0, st>>>(N, moves, colsum, out, err);
-    const size_t tot = (size_t)W * (N3 + 1);
-    deviation_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(W, N, acc, out, dev);
-    eerr_kernel<<<1, 256, 0, st>>>(W, N, dev, out + 1, 1);
-    dim3 g((N3 + 31) / 32, (N3 + 31) / 32);
-    gram_kernel<<<g, 256, 0, st>>>(W, N, dev, out + 4 + N3, W > 1 ? 1.0 / ((double)W * (W - 1)) : 0.0);
+    colsum_kernel<<<dim3(ncol + 1, K), 256, 0, st>>>(W, ncol, acc, nacc, colsum);
+    finalize_kernel<<<K, 256, 0, st>>>(N, moves, colsum, out, err);
+    deviations(K, W, N, acc, out, dev, st);
+    gram(K, W, N, dev, ws, out + 1, out + 4 + N3, 4 + N3 + (size_t)N3 * N3, W > 1 ? 1.0 / ((double)W * (W - 1)) : 0.0, 1,
+         st);
 }
 
 // ---------------------------------------------------------------------------
@@ -199,15 +270,11 @@ void launch_shard_sums(int W, int N, double moves, const double* acc, const unsi
     shard_counts_kernel<<<1, 1, 0, st>>>(N, (double)W, moves, sums);
 }
 
-void launch_shard_reduce(int W, int N, const double* acc, const double* sums, double* dev, double* out, double* gram,
-                         int* err, cudaStream_t st) {
-    const int N3 = 3 * N;
+void launch_shard_reduce(int W, int N, const double* acc, const double* sums, double* dev, double* ws, double* out,
+                         double* gram_out, int* err, cudaStream_t st) {
     finalize_kernel<<<1, 256, 0, st>>>(N, -1.0, sums, out, err);
-    const size_t tot = (size_t)W * (N3 + 1);
-    deviation_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(W, N, acc, out, dev);
-    eerr_kernel<<<1, 256, 0, st>>>(W, N, dev, gram, 0);
-    dim3 g((N3 + 31) / 32, (N3 + 31) / 32);
-    gram_kernel<<<g, 256, 0, st>>>(W, N, dev, gram + 1, 1.0);
+    deviations(1, W, N, acc, out, dev, st);
+    gram(1, W, N, dev, ws, gram_out, gram_out + 1, 0, 1.0, 0, st);
 }
 
 void launch_shard_finish(int N, const double* sums, const double* gram, double* out, cudaStream_t st) {

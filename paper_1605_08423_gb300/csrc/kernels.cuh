@@ -69,8 +69,11 @@ void launch_ewald_table(double kappa, double h, double* t, cudaStream_t st);
 void launch_recforce_gemm(int W, int M, int K, const float* rho, const float* T, float* F, cudaStream_t st);
 
 // k_reduce.cu: walker reductions and the covariance matrix.
-void launch_reduce(int W, int N, double moves, const double* acc, const unsigned long long* nacc,
-                   double* colsum, double* dev, double* out, int* err, cudaStream_t st);
+// K walker blocks of W walkers (the twists; else K = 1), each with its own
+// result out[K][4 + 3N + 9N^2]; colsum [K][4 + 9N], ws gram_ws_doubles(K, W, N).
+void launch_reduce(int K, int W, int N, double moves, const double* acc, const unsigned long long* nacc,
+                   double* colsum, double* dev, double* ws, double* out, int* err, cudaStream_t st);
+size_t gram_ws_doubles(int K, int W, int N);
 // k_reduce.cu: virial pressure of the last call's samples, out [5].
 void launch_pressure(int W, int N, const double* acc, const double* vacc, double omega, double T_nuc, double* out,
                      cudaStream_t st);
@@ -79,8 +82,8 @@ void launch_pressure(int W, int N, const double* acc, const double* vacc, double
 // the summed sums, then E_err and S from the summed gram.
 void launch_shard_sums(int W, int N, double moves, const double* acc, const unsigned long long* nacc, double* sums,
                        cudaStream_t st);
-void launch_shard_reduce(int W, int N, const double* acc, const double* sums, double* dev, double* out, double* gram,
-                         int* err, cudaStream_t st);
+void launch_shard_reduce(int W, int N, const double* acc, const double* sums, double* dev, double* ws, double* out,
+                         double* gram_out, int* err, cudaStream_t st);
 void launch_shard_finish(int N, const double* sums, const double* gram, double* out, cudaStream_t st);
 
 // k_twist.cu: twisted boundary conditions (FP64 form, complex orbitals).
