@@ -41,6 +41,10 @@ struct qmc_system {
     float *d_C32 = nullptr, *d_ptrig32 = nullptr;
     int4* d_kvec = nullptr;
     double* d_ewt = nullptr;   // real-space Ewald table (FP64 form)
+    // FP64 measure kernel: its structure-factor tasks and the reciprocal vectors [3][nk]
+    int nktask = 0;
+    int4* d_ktask = nullptr;
+    double* d_kxyz = nullptr;
     double2 *d_eikR = nullptr, *d_rhop = nullptr;
     double *d_vconst = nullptr, *d_dvpp = nullptr, *d_vpp = nullptr;
     float *d_R32 = nullptr, *d_kw32 = nullptr, *d_zeta32 = nullptr;
@@ -92,16 +96,15 @@ struct qmc_system {
     uint32_t langevin_step_no = 0;
     double last_Nc = 0.0;
     // twisted boundary conditions (FP64 form): K twists, walker blocks of W/K;
-    // the twist vectors and their phase table; the real inputs of the FP64
-    // measure kernel (D', Lp' with Re g, Re l in column 0, unit inverse rows,
-    // zero coefficients); E_L and ln|psi| per walker; the per-twist results
-    // before the average
+    // the twist vectors and their phase table; (Re g, Re l) of every electron
+    // for the FP64 measure kernel; E_L and ln|psi| per walker; the per-twist
+    // results before the average
     int K = 0;
     TwistView tv{};
     std::vector<double> twist_h;
     double* d_theta = nullptr;
     double2* d_tph = nullptr;
-    double *d_Dr = nullptr, *d_Lpr = nullptr, *d_Gtr = nullptr, *d_Czero = nullptr;
+    double* d_gl = nullptr;
     double *d_elt = nullptr, *d_lpt = nullptr, *d_tout = nullptr;
     long long nlaunch = 0;  // kernels launched by this handle
     bool profiling = false;
@@ -143,6 +146,18 @@ void enumerate_kvec(int mmax, std::vector<int4>& kv) {
                 const bool half = mx > 0 || (mx == 0 && my > 0) || (mx == 0 && my == 0 && mz > 0);
                 if (half && mx * mx + my * my + mz * mz <= mmax * mmax) kv.push_back(make_int4(mx, my, mz, 0));
             }
+}
+
+// Structure-factor tasks of the FP64 measure kernel: per (m_x, m_y) of the half
+// space and two consecutive |m_z| from m_z0 (even), (m_x, m_y, m_z0, index in kv
+// of (m_x, m_y, 0), extrapolated where that vector is not in the list).
+void enumerate_ktask(const std::vector<int4>& kv, std::vector<int4>& task) {
+    for (size_t k = 0; k < kv.size();) {
+        const int mx = kv[k].x, my = kv[k].y, base = (int)k - kv[k].z;
+        int top = 0;
+        for (; k < kv.size() && kv[k].x == mx && kv[k].y == my; ++k) top = kv[k].z > top ? kv[k].z : top;
+        for (int z = 0; z <= top; z += 2) task.push_back(make_int4(mx, my, z, base));
+    }
 }
 
 // Images per axis of the Bloch-summed Gaussians (twisted orbitals): every
@@ -208,7 +223,9 @@ size_t footprint(const qmc_params* p) {
     b += 8 * 2 * W * 3 * N;                          // X, Xp
     b += t * W * N;                                  // carried e-n Jastrow sums of the sweep
     const size_t tc = p->n_twist > 0 ? 16 : t;     // complex orbitals of the twisted form
-    b += t * W * N + tc * (W * N * n + 2 * W * n * n + 3 * W * N * n + W * N * n);   // uacc, Phi, Gt, D, Lp
+    b += t * W * N + tc * (W * N * n + 2 * W * n * n);   // uacc, Phi, Gt
+    if (t == 4 || p->n_twist > 0) b += tc * 4 * W * N * n;   // D, Lp
+    if (t == 8) b += (16 + 24) * nk;                   // structure-factor tasks (at most nk), reciprocal vectors
     b += 8 * 2 * W + 8 * W * (3 + 9 * N) + 8 * W;   // logdet, acc, nacc
     b += 8 * W + 8 * 5;                              // V_L sums, pressure output
     const size_t Kr = p->n_twist > 0 ? p->n_twist : 1;
@@ -220,9 +237,9 @@ size_t footprint(const qmc_params* p) {
     if (t == 8) b += 8 * 2 * kEwNodes * kEwTerms;    // real-space Ewald table
     if (p->fj) b += (t == 4 ? 12 : 8) * N * N;       // e-e-n-n Jastrow coefficients (+ FP32 copy)
     if (p->n_twist > 0) {
-        // twists, phase table, real D' / Lp' / unit rows / zero coefficients, E_L and ln|psi|, per-twist results
+        // twists, phase table, Re g and Re l, E_L and ln|psi|, per-twist results
         const size_t K = p->n_twist, M = bloch_images(p);
-        b += 8 * 3 * K + 16 * 3 * K * (2 * M + 1) + 8 * (W * N * 4 * n + 2 * W * n * n + B * n) + 8 * 2 * W +
+        b += 8 * 3 * K + 16 * 3 * K * (2 * M + 1) + 8 * W * N * 4 + 8 * 2 * W +
              8 * K * (4 + 3 * N + 9 * N * N);
     }
     b += (size_t)kPoolAllocs * kPoolAlign;           // alignment slack of a carved handle
@@ -330,30 +347,43 @@ void recompute_in_call(qmc_system* h, int W) {
     recompute<T>(h, W);
 }
 
-template <typename T>
-void measure(qmc_system* h, int W, double* el, double* lnpsi, double* dl, double* de) {
-    SysView<T> s = view<T>(h, W);
+void measure(qmc_system* h, const SysView<float>& s, double* el, double* lnpsi, double* dl, double* de) {
     EventPair ep;
     h->nlaunch += 2;
     prof_begin(h, KC_ORB_MEAS, ep);
-    orbitals<T>(h, s, h->d_X, W * h->N, (T*)h->d_Phi, (T*)h->d_D, (T*)h->d_Lp);
+    orbitals<float>(h, s, h->d_X, s.W * h->N, (float*)h->d_Phi, (float*)h->d_D, (float*)h->d_Lp);
     prof_end(h, ep);
-    const bool split = sizeof(T) == 4 && h->use_tc && h->use_tc_adj;
+    const bool split = h->use_tc && h->use_tc_adj;
     prof_begin(h, KC_MEASURE, ep);
-    launch_measure<T>(s, h->d_X, (const T*)h->d_D, (const T*)h->d_Lp, (const T*)h->d_Gt, h->d_logdet, h->d_acc, el,
-                      lnpsi, dl, de, split ? h->d_Kt : nullptr, split ? h->d_eg : nullptr,
-                      split ? h->d_elw : nullptr, split ? h->d_rk : nullptr, h->stream);
+    launch_measure(s, h->d_X, (const float*)h->d_D, (const float*)h->d_Lp, (const float*)h->d_Gt, h->d_logdet, h->d_acc,
+                   el, lnpsi, dl, de, split ? h->d_Kt : nullptr, split ? h->d_eg : nullptr,
+                   split ? h->d_elw : nullptr, split ? h->d_rk : nullptr, h->stream);
     prof_end(h, ep);
     if (split) {
         h->nlaunch += 1;
         prof_begin(h, KC_ADJOINT, ep);
         // reciprocal-space forces of all walkers: F[W][3N] = rho[W][2nk] . T[2nk][3N]
         h->nlaunch += 1;
-        launch_recforce_gemm(W, 3 * h->N, 2 * h->nk, h->d_rk, h->d_Trec, h->d_frec, h->stream);
-        launch_adjoint_tc(*(const SysView<float>*)&s, h->d_ahat, (const float*)h->d_Gt, h->d_Kt, h->d_eg, h->d_elw,
-                          h->d_frec, h->d_acc, dl, de, h->stream);
+        launch_recforce_gemm(s.W, 3 * h->N, 2 * h->nk, h->d_rk, h->d_Trec, h->d_frec, h->stream);
+        launch_adjoint_tc(s, h->d_ahat, (const float*)h->d_Gt, h->d_Kt, h->d_eg, h->d_elw, h->d_frec, h->d_acc, dl, de,
+                          h->stream);
         prof_end(h, ep);
     }
+}
+
+// FP64 form: one kernel, which needs the inverses but no orbital rows.
+void measure(qmc_system* h, const SysView<double>& s, double* el, double* lnpsi, double* dl, double* de) {
+    EventPair ep;
+    h->nlaunch += 1;
+    prof_begin(h, KC_MEASURE, ep);
+    launch_measure64(s, h->nktask, h->d_ktask, h->d_kxyz, h->d_X, (const double*)h->d_Gt, nullptr, h->d_logdet, h->d_acc,
+                     el, lnpsi, dl, de, h->stream);
+    prof_end(h, ep);
+}
+
+template <typename T>
+void measure(qmc_system* h, int W, double* el, double* lnpsi, double* dl, double* de) {
+    measure(h, view<T>(h, W), el, lnpsi, dl, de);
 }
 
 // Sampling part of one energy/force call (recompute, warm-up and measured
@@ -407,10 +437,9 @@ void recompute_twist(qmc_system* h, int W) {
 }
 
 // Local energy and force sample of every walker: complex orbital rows; Re g and
-// Re l into column 0 of D' and Lp'; the FP64 measure kernel on D', Lp', unit
-// inverse rows and zero coefficients (so it computes E_L = Re(H psi / psi), the
-// Jastrow and Ewald force terms with vv = Re g + grad U, and adds nothing from
-// its orbital force phase); then the complex orbital (Pulay) force terms.
+// Re l; the FP64 measure kernel on them (E_L = Re(H psi / psi), the Jastrow and
+// Ewald force terms with vv = Re g + grad U); then the complex orbital (Pulay)
+// force terms.
 void measure_twist(qmc_system* h, int W, double* el, double* lnpsi, double* dl, double* de) {
     SysView<double> s = view<double>(h, W);
     const int N = h->N, n = h->n;
@@ -419,15 +448,13 @@ void measure_twist(qmc_system* h, int W, double* el, double* lnpsi, double* dl, 
     prof_begin(h, KC_ORB_MEAS, ep);
     launch_twist_orbitals(s, h->tv, h->d_X, W * N, (double2*)h->d_Phi, (double2*)h->d_D, (double2*)h->d_Lp,
                           h->stream);
-    launch_twist_gl(W * N, N, n, (const double2*)h->d_D, (const double2*)h->d_Lp, (const double2*)h->d_Gt, h->d_Dr,
-                    h->d_Lpr, h->stream);
+    launch_twist_gl(W * N, N, n, (const double2*)h->d_D, (const double2*)h->d_Lp, (const double2*)h->d_Gt, h->d_gl,
+                    h->stream);
     prof_end(h, ep);
-    SysView<double> s0 = s;
-    s0.C = h->d_Czero;
     double* elw = el ? el : h->d_elt;
     prof_begin(h, KC_MEASURE, ep);
-    launch_measure<double>(s0, h->d_X, h->d_Dr, h->d_Lpr, h->d_Gtr, h->d_logdet, h->d_acc, elw,
-                           lnpsi ? lnpsi : h->d_lpt, dl, de, nullptr, nullptr, nullptr, nullptr, h->stream);
+    launch_measure64(s, h->nktask, h->d_ktask, h->d_kxyz, h->d_X, nullptr, h->d_gl, h->d_logdet, h->d_acc, elw,
+                     lnpsi ? lnpsi : h->d_lpt, dl, de, h->stream);
     prof_end(h, ep);
     prof_begin(h, KC_ADJOINT, ep);
     launch_twist_pulay(s, h->tv, h->d_X, (const double2*)h->d_D, (const double2*)h->d_Lp, (const double2*)h->d_Gt,
@@ -596,8 +623,10 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
     h->d_uacc = dalloc<unsigned char>(h, t * W * N, &rc);
     h->d_Phi = dalloc<unsigned char>(h, tc * W * N * n, &rc);
     h->d_Gt = dalloc<unsigned char>(h, tc * W * 2 * n * n, &rc);
-    h->d_D = dalloc<unsigned char>(h, tc * W * N * 3 * n, &rc);
-    h->d_Lp = dalloc<unsigned char>(h, tc * W * N * n, &rc);
+    if (h->mixed || h->K) {   // the FP64 form at the Gamma point needs no derivative rows
+        h->d_D = dalloc<unsigned char>(h, tc * W * N * 3 * n, &rc);
+        h->d_Lp = dalloc<unsigned char>(h, tc * W * N * n, &rc);
+    }
     h->d_logdet = dalloc<double>(h, 2 * (size_t)W, &rc);
     h->d_acc = dalloc<double>(h, (size_t)W * (3 + 9 * N), &rc);
     h->d_vacc = dalloc<double>(h, W, &rc);
@@ -630,10 +659,7 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
         const int K = h->K, M = bloch_images(p);
         h->d_theta = dalloc<double>(h, 3 * (size_t)K, &rc);
         h->d_tph = dalloc<double2>(h, (size_t)K * 3 * (2 * M + 1), &rc);
-        h->d_Dr = dalloc<double>(h, (size_t)W * N * 3 * n, &rc);
-        h->d_Lpr = dalloc<double>(h, (size_t)W * N * n, &rc);
-        h->d_Gtr = dalloc<double>(h, (size_t)W * 2 * n * n, &rc);
-        h->d_Czero = dalloc<double>(h, (size_t)B * n, &rc);
+        h->d_gl = dalloc<double>(h, (size_t)W * N * 4, &rc);
         h->d_elt = dalloc<double>(h, W, &rc);
         h->d_lpt = dalloc<double>(h, W, &rc);
         h->d_tout = dalloc<double>(h, (size_t)K * (4 + 3 * N + 9 * (size_t)N * N), &rc);
@@ -668,6 +694,19 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
             h->use_tc_adj = true;
         }
     }
+    std::vector<int4> ktask;
+    std::vector<double> kxyz;
+    if (!h->mixed) {
+        enumerate_ktask(kv, ktask);
+        h->nktask = (int)ktask.size();
+        kxyz.resize(3 * (size_t)nk);
+        for (int k = 0; k < nk; ++k) {
+            const double tp = 2.0 * kPi / p->L;
+            kxyz[k] = tp * kv[k].x; kxyz[nk + k] = tp * kv[k].y; kxyz[2 * nk + k] = tp * kv[k].z;
+        }
+        h->d_ktask = dalloc<int4>(h, ktask.size(), &rc);
+        h->d_kxyz = dalloc<double>(h, kxyz.size(), &rc);
+    }
     if (!h->mixed && p->ewald_kappa * p->L <= kEwMaxKL) h->d_ewt = dalloc<double>(h, 2 * kEwNodes * kEwTerms, &rc);
     if (rc != QMC_OK) { qmc_destroy(h); return rc; }
     std::vector<float> c32(h->coeff_h.begin(), h->coeff_h.end());
@@ -680,16 +719,16 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
     if (h->K) {
         cudaMemcpyAsync(h->d_theta, h->twist_h.data(), sizeof(double) * 3 * h->K, cudaMemcpyHostToDevice, st);
         cudaMemcpyAsync(h->d_tph, tph.data(), sizeof(double2) * tph.size(), cudaMemcpyHostToDevice, st);
-        cudaMemsetAsync(h->d_Dr, 0, sizeof(double) * (size_t)W * N * 3 * n, st);
-        cudaMemsetAsync(h->d_Lpr, 0, sizeof(double) * (size_t)W * N * n, st);
-        cudaMemsetAsync(h->d_Czero, 0, sizeof(double) * (size_t)B * n, st);
-        launch_twist_unit_rows(W, n, h->d_Gtr, st);
     }
     std::vector<float> fj32(h->fj_h.begin(), h->fj_h.end());
     if (h->d_fj32) cudaMemcpyAsync(h->d_fj32, fj32.data(), sizeof(float) * N * N, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(h->d_C32, c32.data(), sizeof(float) * B * n, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(h->d_zeta32, z32.data(), sizeof(float) * h->G, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(h->d_kvec, kv.data(), sizeof(int4) * nk, cudaMemcpyHostToDevice, st);
+    if (!h->mixed) {
+        cudaMemcpyAsync(h->d_ktask, ktask.data(), sizeof(int4) * ktask.size(), cudaMemcpyHostToDevice, st);
+        cudaMemcpyAsync(h->d_kxyz, kxyz.data(), sizeof(double) * kxyz.size(), cudaMemcpyHostToDevice, st);
+    }
     cudaMemsetAsync(h->d_err, 0, sizeof(int), st);
     cudaMemsetAsync(h->d_nacc, 0, sizeof(unsigned long long) * W, st);
     if (h->d_chat) prepare_tc_coeff(h->d_C32, B, n, h->d_chat, st);

@@ -1,4 +1,6 @@
-// k_measure.cu -- local energy and nuclear-force sample of every walker.
+// k_measure.cu -- local energy and nuclear-force sample of every walker, mixed
+// form (FP32 with FP64 where it is needed; the FP64 form's kernel is in
+// k_measure64.cu).
 //
 // One CTA per walker.  From the orbital derivative rows (D = grad phi, Lp =
 // lap phi at the current electrons), the inverse G of each spin block and
@@ -21,7 +23,10 @@
 
 namespace qmc {
 
-template <typename T>
+namespace {
+
+using T = float;   // working precision of this kernel
+
 struct MLayout {
     size_t xs, xt, et, gU, lU, Ui, gi, vv, li, facc, gacc, rhot, red, stage, cmask, uni, total;
     // split: the B x n orbital contractions run in the adjoint kernel, so the
@@ -113,10 +118,10 @@ __device__ __forceinline__ void ep_jastrow_f32(const float sd[3], const float cd
     }
 }
 
-template <typename S>
-__device__ __forceinline__ void ep_jastrow(const S sd[3], const S cd[3], S ell, S k2, S bep, S Zj, const S vv[3],
-                                           S dl[3], S de[3]) {
-    S p[3], q[3], t = 0;
+// The same in FP64, for the close pairs.
+__device__ __forceinline__ void ep_jastrow(const double sd[3], const double cd[3], double ell, double k2, double bep,
+                                           double Zj, const double vv[3], double dl[3], double de[3]) {
+    double p[3], q[3], t = 0;
 #pragma unroll
     for (int mu = 0; mu < 3; ++mu) {
         p[mu] = ell * sd[mu] * cd[mu];
@@ -124,22 +129,21 @@ __device__ __forceinline__ void ep_jastrow(const S sd[3], const S cd[3], S ell, 
         t += sd[mu] * sd[mu];
     }
     t *= ell * ell;
-    const S r = qsqrt_pair(t);
-    S u, u1, u2, u3, f1, f2, f3;
+    const double r = qsqrt_pair(t);
+    double u, u1, u2, u3, f1, f2, f3;
     pade_ep(bep, Zj, r, u, u1, u2, u3);
     rho_to_t(r, u1, u2, u3, f1, f2, f3);
-    RadialDerivs<S> rd;
+    RadialDerivs<double> rd;
     radial_chain(p, q, f1, f2, f3, k2, rd);
-    S hv[3];
+    double hv[3];
     hess_mul(rd.h, vv, hv);
 #pragma unroll
-    for (int mu = 0; mu < 3; ++mu) { dl[mu] = -rd.g[mu]; de[mu] = hv[mu] + S(0.5) * rd.tl[mu]; }
+    for (int mu = 0; mu < 3; ++mu) { dl[mu] = -rd.g[mu]; de[mu] = hv[mu] + 0.5 * rd.tl[mu]; }
 }
 
 // e-e-n-n Jastrow orbital chi_a(r_i) = exp(-zeta |d|^2) of electron trig ei and
 // nucleus trig pa with its gradient, Hessian, Laplacian and gradient of the
 // Laplacian in the electron coordinate (radial chain of f(t) = exp(-zeta t)).
-template <typename T>
 __device__ __forceinline__ T jas34_orbital(const T* ei, const T* pa, T ell, T zeta, T k2, RadialDerivs<T>& rd) {
     T sd[3], cd[3], t;
     disp_trig(ei, pa, ell, sd, cd, t);
@@ -160,11 +164,11 @@ __device__ __forceinline__ T jas34_orbital(const T* ei, const T* pa, T ell, T ze
 // and grad U (eg_out, 9 per electron) and E_L of the sample (elw); the
 // reciprocal-space force, a fixed [3N][2 nk] matrix times rho(k), is left to a
 // GEMM over all walkers, so the structure factor goes out too (rk_out).
-// The FP32 instances ask for three CTAs an SM (80 registers): their phases are
-// latency-bound between barriers.  Without the bound the unsplit one took 143
-// registers, one CTA an SM: 3.14 ms for 4096 walkers of N = 64, now 1.53 ms.
-template <typename T, bool kSplit>
-__global__ void __launch_bounds__(256, kSplit || sizeof(T) == 4 ? 3 : 1) measure_kernel(SysView<T> s, int mmax, const double* __restrict__ X,
+// Three CTAs an SM (80 registers): the phases are latency-bound between barriers.
+// Without the bound the unsplit instance took 143 registers, one CTA an SM:
+// 3.14 ms for 4096 walkers of N = 64, now 1.53 ms.
+template <bool kSplit>
+__global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax, const double* __restrict__ X,
                                                       const T* __restrict__ D, const T* __restrict__ Lp,
                                                       const T* __restrict__ Gt, const double* __restrict__ logdet,
                                                       double* __restrict__ acc, double* __restrict__ out_el,
@@ -174,7 +178,7 @@ __global__ void __launch_bounds__(256, kSplit || sizeof(T) == 4 ? 3 : 1) measure
                                                       float* __restrict__ rk_out) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int N = s.N, n = s.n, G = s.G, nk = s.nk;
-    const MLayout<T> lay(N, n, nk, mmax, kSplit);
+    const MLayout lay(N, n, nk, mmax, kSplit);
     double* xs = (double*)(sm + lay.xs);
     T* xt = (T*)(sm + lay.xt);
     T* et = (T*)(sm + lay.et);
@@ -233,7 +237,7 @@ __global__ void __launch_bounds__(256, kSplit || sizeof(T) == 4 ? 3 : 1) measure
     // 32 J + l's.  A diagonal tile takes steps 1..16 (step 16 on lanes 0-15
     // only).  Each (electron, partner block) has one slot of 5; the slots are
     // summed in block order with the e-n slices below.
-    const bool ee_tiles = sizeof(T) == 4 && (N & 31) == 0 && N >= 64;
+    const bool ee_tiles = (N & 31) == 0 && N >= 64;
     T* eepart = jpart + (size_t)5 * 256;   // [N / 32][N][5]
     for (int tt = tid; tt < nparts * N; tt += nt) {
         const int i = tt % N, pi = tt / N;
@@ -245,14 +249,7 @@ __global__ void __launch_bounds__(256, kSplit || sizeof(T) == 4 ? 3 : 1) measure
             T sd[3], cd[3], t;
             disp_trig(ei, et + 6 * j, ell, sd, cd, t);
             T u, f1, f2;
-            if constexpr (sizeof(T) == 4) {
-                jas_ee_f32(t, bee, u, f1, f2);
-            } else {
-                const T r = qsqrt_pair(t);
-                T u1, u2, f3;
-                pade_ee(bee, r, u, u1, u2);
-                rho_to_t(r, u1, u2, T(0), f1, f2, f3);
-            }
+            jas_ee_f32(t, bee, u, f1, f2);
             T pp = 0, sq = 0;
 #pragma unroll
             for (int mu = 0; mu < 3; ++mu) {
@@ -266,16 +263,8 @@ __global__ void __launch_bounds__(256, kSplit || sizeof(T) == 4 ? 3 : 1) measure
         for (int a = j0; a < j1; ++a) {
             T sd[3], cd[3], t;
             disp_trig(ei, s.ptrig + 6 * a, ell, sd, cd, t);
-            T u, f1, f2;
-            if constexpr (sizeof(T) == 4) {
-                float f3;
-                jas_ep_f32(t, bep, Zj, u, f1, f2, f3);
-            } else {
-                const T r = qsqrt_pair(t);
-                T u1, u2, u3, f3;
-                pade_ep(bep, Zj, r, u, u1, u2, u3);
-                rho_to_t(r, u1, u2, T(0), f1, f2, f3);
-            }
+            T u, f1, f2, f3;
+            jas_ep_f32(t, bep, Zj, u, f1, f2, f3);
             T pp = 0, sq = 0;
 #pragma unroll
             for (int mu = 0; mu < 3; ++mu) {
@@ -289,65 +278,63 @@ __global__ void __launch_bounds__(256, kSplit || sizeof(T) == 4 ? 3 : 1) measure
         T* o = jpart + ((size_t)pi * N + i) * 5;
         o[0] = g[0]; o[1] = g[1]; o[2] = g[2]; o[3] = lp; o[4] = ui;
     }
-    if constexpr (sizeof(T) == 4) {
-        if (ee_tiles) {
-            const int nb = N >> 5, noff = nb * (nb - 1) / 2, ntiles = noff + nb;
-            for (int tile = warp; tile < ntiles; tile += nw) {
-                int I = 0, J = 0;
-                if (tile < noff) {   // off-diagonal tiles, I < J in row-major order
-                    int r = tile;
-                    while (r >= nb - 1 - I) { r -= nb - 1 - I; ++I; }
-                    J = I + 1 + r;
-                } else {
-                    I = J = tile - noff;
-                }
-                const bool diag = I == J;
-                const int i = 32 * I + lane;
-                float ei[6];
+    if (ee_tiles) {
+        const int nb = N >> 5, noff = nb * (nb - 1) / 2, ntiles = noff + nb;
+        for (int tile = warp; tile < ntiles; tile += nw) {
+            int I = 0, J = 0;
+            if (tile < noff) {   // off-diagonal tiles, I < J in row-major order
+                int r = tile;
+                while (r >= nb - 1 - I) { r -= nb - 1 - I; ++I; }
+                J = I + 1 + r;
+            } else {
+                I = J = tile - noff;
+            }
+            const bool diag = I == J;
+            const int i = 32 * I + lane;
+            float ei[6];
 #pragma unroll
-                for (int c = 0; c < 6; ++c) ei[c] = et[6 * i + c];
-                float rg[3] = {0.f, 0.f, 0.f}, rl = 0.f, ru = 0.f, cg[3] = {0.f, 0.f, 0.f}, cl = 0.f;
-                const int k0 = diag ? 1 : 0, k1 = diag ? 17 : 32;
-                for (int k = k0; k < k1; ++k) {
-                    if (!diag || k < 16 || lane < 16) {
-                        const int j = 32 * J + ((lane + k) & 31);
-                        float sd[3], cd[3], t;
-                        disp_trig(ei, et + 6 * j, ell, sd, cd, t);
-                        float u, f1, f2;
-                        jas_ee_f32(t, bee, u, f1, f2);
-                        float pp = 0.f, sq = 0.f;
+            for (int c = 0; c < 6; ++c) ei[c] = et[6 * i + c];
+            float rg[3] = {0.f, 0.f, 0.f}, rl = 0.f, ru = 0.f, cg[3] = {0.f, 0.f, 0.f}, cl = 0.f;
+            const int k0 = diag ? 1 : 0, k1 = diag ? 17 : 32;
+            for (int k = k0; k < k1; ++k) {
+                if (!diag || k < 16 || lane < 16) {
+                    const int j = 32 * J + ((lane + k) & 31);
+                    float sd[3], cd[3], t;
+                    disp_trig(ei, et + 6 * j, ell, sd, cd, t);
+                    float u, f1, f2;
+                    jas_ee_f32(t, bee, u, f1, f2);
+                    float pp = 0.f, sq = 0.f;
 #pragma unroll
-                        for (int mu = 0; mu < 3; ++mu) {
-                            const float pm = ell * sd[mu] * cd[mu], gm = 2.f * f1 * pm;
-                            rg[mu] += gm;
-                            cg[mu] -= gm;   // p is odd under the exchange of the pair
-                            pp += pm * pm;
-                            sq += cd[mu] * cd[mu] - sd[mu] * sd[mu];
-                        }
-                        const float lpv = 4.f * f2 * pp + 2.f * f1 * sq;
-                        rl += lpv;
-                        cl += lpv;
-                        ru += u;
+                    for (int mu = 0; mu < 3; ++mu) {
+                        const float pm = ell * sd[mu] * cd[mu], gm = 2.f * f1 * pm;
+                        rg[mu] += gm;
+                        cg[mu] -= gm;   // p is odd under the exchange of the pair
+                        pp += pm * pm;
+                        sq += cd[mu] * cd[mu] - sd[mu] * sd[mu];
                     }
-                    // the column sums move to the lane that meets their electron next
-                    const int src = (lane + 1) & 31;
-#pragma unroll
-                    for (int mu = 0; mu < 3; ++mu) cg[mu] = __shfl_sync(0xffffffffu, cg[mu], src);
-                    cl = __shfl_sync(0xffffffffu, cl, src);
+                    const float lpv = 4.f * f2 * pp + 2.f * f1 * sq;
+                    rl += lpv;
+                    cl += lpv;
+                    ru += u;
                 }
-                if (diag) {   // lane l holds column (l + 17) mod 32: column l's come from lane (l + 15) mod 32
-                    const int src = (lane + 15) & 31;
+                // the column sums move to the lane that meets their electron next
+                const int src = (lane + 1) & 31;
 #pragma unroll
-                    for (int mu = 0; mu < 3; ++mu) cg[mu] = __shfl_sync(0xffffffffu, cg[mu], src);
-                    cl = __shfl_sync(0xffffffffu, cl, src);
-                    T* o = eepart + ((size_t)I * N + i) * 5;
-                    o[0] = rg[0] + cg[0]; o[1] = rg[1] + cg[1]; o[2] = rg[2] + cg[2]; o[3] = rl + cl; o[4] = ru;
-                } else {
-                    T* o = eepart + ((size_t)J * N + i) * 5;
-                    o[0] = rg[0]; o[1] = rg[1]; o[2] = rg[2]; o[3] = rl; o[4] = ru;
-                    T* oc = eepart + ((size_t)I * N + 32 * J + lane) * 5;
-                    oc[0] = cg[0]; oc[1] = cg[1]; oc[2] = cg[2]; oc[3] = cl; oc[4] = 0.f;
-                }
+                for (int mu = 0; mu < 3; ++mu) cg[mu] = __shfl_sync(0xffffffffu, cg[mu], src);
+                cl = __shfl_sync(0xffffffffu, cl, src);
+            }
+            if (diag) {   // lane l holds column (l + 17) mod 32: column l's come from lane (l + 15) mod 32
+                const int src = (lane + 15) & 31;
+#pragma unroll
+                for (int mu = 0; mu < 3; ++mu) cg[mu] = __shfl_sync(0xffffffffu, cg[mu], src);
+                cl = __shfl_sync(0xffffffffu, cl, src);
+                T* o = eepart + ((size_t)I * N + i) * 5;
+                o[0] = rg[0] + cg[0]; o[1] = rg[1] + cg[1]; o[2] = rg[2] + cg[2]; o[3] = rl + cl; o[4] = ru;
+            } else {
+                T* o = eepart + ((size_t)J * N + i) * 5;
+                o[0] = rg[0]; o[1] = rg[1]; o[2] = rg[2]; o[3] = rl; o[4] = ru;
+                T* oc = eepart + ((size_t)I * N + 32 * J + lane) * 5;
+                oc[0] = cg[0]; oc[1] = cg[1]; oc[2] = cg[2]; oc[3] = cl; oc[4] = 0.f;
             }
         }
     }
@@ -504,7 +491,6 @@ __global__ void __launch_bounds__(256, kSplit || sizeof(T) == 4 ? 3 : 1) measure
     // ---- P4a: electron-electron real-space Ewald
     double vee_p = 0.0;
     const T Lt = (T)L;
-    const EwTable ewt{s.ewt, s.ew_h, s.ew_ih, L, iL, L * L};
     const float iLt = 1.f / (float)Lt, rc2 = kRealCut2Mixed * (float)Lt * (float)Lt;
     // balanced cyclic pairing: electron i with i+d (mod N), d = 1..N/2 (d = N/2 only for i < N/2),
     // the distance range split into nparts slices
@@ -516,22 +502,14 @@ __global__ void __launch_bounds__(256, kSplit || sizeof(T) == 4 ? 3 : 1) measure
             const bool skip = 2 * d == N && i >= half;
             const int j = i + d < N ? i + d : i + d - N;      // (i + d) mod N, d < N
             if (skip) continue;
-            if constexpr (sizeof(T) == 4) {
-                v += ewald_real_cut<false>(xt[3 * i] - xt[3 * j], xt[3 * i + 1] - xt[3 * j + 1],
-                                           xt[3 * i + 2] - xt[3 * j + 2], false, Lt, iLt, rc2, kap, nullptr);
-            }
-            else {
-                const double dx = xs[3 * i] - xs[3 * j], dy = xs[3 * i + 1] - xs[3 * j + 1],
-                             dz = xs[3 * i + 2] - xs[3 * j + 2];
-                v += ewt.t ? ewald_table<false>(dx, dy, dz, ewt, nullptr)
-                           : ewald_real<double>(dx, dy, dz, L, kap, nullptr);
-            }
+            v += ewald_real_cut<false>(xt[3 * i] - xt[3 * j], xt[3 * i + 1] - xt[3 * j + 1],
+                                       xt[3 * i + 2] - xt[3 * j + 2], false, Lt, iLt, rc2, kap, nullptr);
         }
         vee_p += (double)v;
     }
     // ---- P4b: electron-proton pairs (warp per proton, lanes over electrons): the
     // real-space Ewald energy and its R-gradient (Hellmann-Feynman) together with
-    // the e-n Jastrow terms of d ln psi/dR and dE_L/dR.  In the mixed form, pairs
+    // the e-n Jastrow terms of d ln psi/dR and dE_L/dR.  Pairs
     // closer than 0.3 bohr are only flagged here and evaluated afterwards in FP64
     // (one thread per proton, electrons in increasing order): there the 1/r^2
     // Coulomb force and the 1/r^2 part of grad lap u_en cancel (cusp
@@ -551,29 +529,18 @@ __global__ void __launch_bounds__(256, kSplit || sizeof(T) == 4 ? 3 : 1) measure
         for (int i = lane; i < N; i += 32) {
             T sd[3], cd[3], t;
             disp_trig(et + 6 * i, pa, ell, sd, cd, t);
-            const bool close = sizeof(T) == 4 && t < T(0.09);
+            const bool close = t < T(0.09);
             if (close) atomicOr(&cmask[a * nwords + (i >> 5)], 1u << (i & 31));
-            if constexpr (sizeof(T) == 4) {
-                // FP32: Jastrow terms unless close; the Ewald images inside the
-                // FP32-level cutoff (a close pair's nearest image is done in FP64)
-                if (!close) {
-                    T vv[3], pl[3], pe[3];
-                    for (int mu = 0; mu < 3; ++mu) vv[mu] = vvs[3 * i + mu];
-                    ep_jastrow_f32(sd, cd, ell, k2, bep, Zj, vv, pl, pe);
-                    for (int mu = 0; mu < 3; ++mu) { dl[mu] += pl[mu]; de[mu] += pe[mu]; }
-                }
-                v += ewald_real_cut<true>(xt[3 * i] - ra[0], xt[3 * i + 1] - ra[1], xt[3 * i + 2] - ra[2], close, Lt,
-                                          iLt, rc2, kap, gv);
-            }
-            else {
-                double vv[3], pg[3], pl[3], pe[3];
+            // Jastrow terms unless close; the Ewald images inside the FP32-level
+            // cutoff (a close pair's nearest image is done in FP64)
+            if (!close) {
+                T vv[3], pl[3], pe[3];
                 for (int mu = 0; mu < 3; ++mu) vv[mu] = vvs[3 * i + mu];
-                ep_jastrow<double>(sd, cd, ell, k2, bep, Zj, vv, pl, pe);
-                const double dx = xs[3 * i] - s.R[3 * a], dy = xs[3 * i + 1] - s.R[3 * a + 1],
-                             dz = xs[3 * i + 2] - s.R[3 * a + 2];
-                v += ewt.t ? ewald_table<true>(dx, dy, dz, ewt, pg) : ewald_real<double>(dx, dy, dz, L, kap, pg);
-                for (int mu = 0; mu < 3; ++mu) { gv[mu] += pg[mu]; dl[mu] += pl[mu]; de[mu] += pe[mu]; }
+                ep_jastrow_f32(sd, cd, ell, k2, bep, Zj, vv, pl, pe);
+                for (int mu = 0; mu < 3; ++mu) { dl[mu] += pl[mu]; de[mu] += pe[mu]; }
             }
+            v += ewald_real_cut<true>(xt[3 * i] - ra[0], xt[3 * i + 1] - ra[1], xt[3 * i + 2] - ra[2], close, Lt, iLt,
+                                      rc2, kap, gv);
         }
         v = warp_sum(v);
 #pragma unroll
@@ -587,7 +554,7 @@ __global__ void __launch_bounds__(256, kSplit || sizeof(T) == 4 ? 3 : 1) measure
             }
         }
     }
-    if (sizeof(T) == 4) {
+    {
         // Close pairs in FP64, one thread per pair: the e-n Jastrow terms and
         // the nearest-image real-space Coulomb term (the pair's other images
         // were summed in FP32 above).  Pairs are numbered nucleus by nucleus,
@@ -642,7 +609,7 @@ __global__ void __launch_bounds__(256, kSplit || sizeof(T) == 4 ? 3 : 1) measure
                 sincospi(dy * iL, &sdd[1], &cdd[1]);
                 sincospi(dz * iL, &sdd[2], &cdd[2]);
                 for (int mu = 0; mu < 3; ++mu) vv[mu] = (double)gi[3 * i + mu] + (double)gU[3 * i + mu];
-                ep_jastrow<double>(sdd, cdd, s.ell, k2d, s.b_ep, s.Zj, vv, pl, pe);
+                ep_jastrow(sdd, cdd, s.ell, k2d, s.b_ep, s.Zj, vv, pl, pe);
                 const double mx = dx - L * rint(dx * iL), my = dy - L * rint(dy * iL), mz = dz - L * rint(dz * iL);
                 const double r2 = mx * mx + my * my + mz * mz, r = sqrt(r2), ir = 1.0 / r;
                 const double ec = erfc(s.kappa * r);
@@ -1015,48 +982,27 @@ __global__ void __launch_bounds__(256, kSplit || sizeof(T) == 4 ? 3 : 1) measure
     if (bad) raise_err(s.err, kErrNonfinite);
 }
 
-template <typename T>
-size_t measure_smem_bytes(int N, int n, int nk, int mmax, bool split) {
-    return MLayout<T>(N, n, nk, mmax, split).total;
-}
+}  // namespace
 
-template <typename T>
-void launch_measure(const SysView<T>& s, const double* X, const T* D, const T* Lp, const T* Gt, const double* logdet,
-                    double* acc, double* out_el, double* out_lnpsi, double* out_dl, double* out_de, float* kt_out,
-                    float* eg_out, double* elw, float* rk_out, cudaStream_t st) {
-    const bool split = sizeof(T) == 4 && kt_out != nullptr;
-    const size_t smem = measure_smem_bytes<T>(s.N, s.n, s.nk, s.mmax, split);
-    static bool attr_set[3] = {false, false, false};
-    const int which = sizeof(T) == 8 ? 1 : (split ? 2 : 0);
-    if constexpr (sizeof(T) == 4) {
-        if (split) {
-            if (!attr_set[which]) {
-                cudaFuncSetAttribute(measure_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     227 * 1024);
-                attr_set[which] = true;
-            }
-            measure_kernel<T, true><<<s.W, 256, smem, st>>>(s, s.mmax, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi,
-                                                            out_dl, out_de, kt_out, eg_out, elw, rk_out);
-            return;
-        }
+void launch_measure(const SysView<float>& s, const double* X, const float* D, const float* Lp, const float* Gt,
+                    const double* logdet, double* acc, double* out_el, double* out_lnpsi, double* out_dl,
+                    double* out_de, float* kt_out, float* eg_out, double* elw, float* rk_out, cudaStream_t st) {
+    const bool split = kt_out != nullptr;
+    const size_t smem = MLayout(s.N, s.n, s.nk, s.mmax, split).total;
+    static bool attr_set[2] = {false, false};
+    if (!attr_set[split]) {
+        if (split)
+            cudaFuncSetAttribute(measure_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        else
+            cudaFuncSetAttribute(measure_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        attr_set[split] = true;
     }
-    {
-        if (!attr_set[which]) {
-            cudaFuncSetAttribute(measure_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-            attr_set[which] = true;
-        }
-        measure_kernel<T, false><<<s.W, 256, smem, st>>>(s, s.mmax, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi,
-                                                         out_dl, out_de, nullptr, nullptr, nullptr, nullptr);
-    }
+    if (split)
+        measure_kernel<true><<<s.W, 256, smem, st>>>(s, s.mmax, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
+                                                     out_de, kt_out, eg_out, elw, rk_out);
+    else
+        measure_kernel<false><<<s.W, 256, smem, st>>>(s, s.mmax, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
+                                                      out_de, nullptr, nullptr, nullptr, nullptr);
 }
-
-template size_t measure_smem_bytes<double>(int, int, int, int, bool);
-template size_t measure_smem_bytes<float>(int, int, int, int, bool);
-template void launch_measure<double>(const SysView<double>&, const double*, const double*, const double*,
-                                     const double*, const double*, double*, double*, double*, double*, double*,
-                                     float*, float*, double*, float*, cudaStream_t);
-template void launch_measure<float>(const SysView<float>&, const double*, const float*, const float*, const float*,
-                                    const double*, double*, double*, double*, double*, double*, float*, float*,
-                                    double*, float*, cudaStream_t);
 
 }  // namespace qmc

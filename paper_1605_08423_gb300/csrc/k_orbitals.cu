@@ -135,8 +135,10 @@ static void launch_orb(const SysView<T>& s, const double* pos, int nrows, T* val
 
 template <typename T>
 void launch_orbitals(const SysView<T>& s, const double* pos, int nrows, T* val, T* grad, T* lap, cudaStream_t st) {
-    if (grad) launch_orb<T, 5>(s, pos, nrows, val, grad, lap, st);
-    else launch_orb<T, 1>(s, pos, nrows, val, nullptr, nullptr, st);
+    if constexpr (sizeof(T) == 4) {   // the FP64 form needs no derivative rows (k_measure64.cu)
+        if (grad) { launch_orb<T, 5>(s, pos, nrows, val, grad, lap, st); return; }
+    }
+    launch_orb<T, 1>(s, pos, nrows, val, nullptr, nullptr, st);
 }
 
 // ---------------------------------------------------------------------------

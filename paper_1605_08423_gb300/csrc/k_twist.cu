@@ -471,14 +471,12 @@ void launch_twist_sweep(const SysView<double>& s, const TwistView& tv, double* X
 // Their real parts are the only way the complex determinant enters E_L:
 //   Re(H psi / psi) = -1/2 sum_i [ Re l_i + 2 Re g_i . grad_i U + lap_i U + |grad_i U|^2 ] + V,
 // and the e-n Jastrow force terms take vv_i = Re g_i + grad_i U.  The FP64
-// measure kernel computes all of that from real rows D, Lp and inverse rows
-// G^T: it is handed D' and Lp' whose column 0 holds Re g_i and Re l_i (the
-// other columns stay zero) and G'^T rows e_0 (twist_unit_rows), so its
-// sum_j D'_ij G'^T[i][j] is Re g_i exactly.  One warp per electron.
+// measure kernel computes all of that from gl [rows][4] = (Re g_i, Re l_i).  One
+// warp per electron.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) twist_gl_kernel(int rows, int n, const double2* __restrict__ D,
                                                        const double2* __restrict__ Lp, const double2* __restrict__ Gt,
-                                                       int N, double* __restrict__ Dr, double* __restrict__ Lpr) {
+                                                       int N, double* __restrict__ gl) {
     const int lane = threadIdx.x & 31, r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (r >= rows) return;
     const int w = r / N, i = r - w * N, sp = i / n, il = i - sp * n;
@@ -496,34 +494,20 @@ __global__ void __launch_bounds__(256) twist_gl_kernel(int rows, int n, const do
     }
     g0 = warp_sum(g0); g1 = warp_sum(g1); g2 = warp_sum(g2); l = warp_sum(l);
     if (lane == 0) {
-        Dr[(size_t)r * 3 * n] = g0;
-        Dr[((size_t)r * 3 + 1) * n] = g1;
-        Dr[((size_t)r * 3 + 2) * n] = g2;
-        Lpr[(size_t)r * n] = l;
+        double* o = gl + 4 * (size_t)r;
+        o[0] = g0; o[1] = g1; o[2] = g2; o[3] = l;
     }
 }
 
-void launch_twist_gl(int rows, int N, int n, const double2* D, const double2* Lp, const double2* Gt, double* Dr,
-                     double* Lpr, cudaStream_t st) {
-    twist_gl_kernel<<<(rows + 7) / 8, 256, 0, st>>>(rows, n, D, Lp, Gt, N, Dr, Lpr);
-}
-
-// G'^T[w][sp][i][j] = (j == 0) for every walker-spin block (written once per handle).
-__global__ void twist_unit_rows_kernel(size_t total, int n, double* __restrict__ Gtr) {
-    const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < total) Gtr[k] = (k % (size_t)n) == 0 ? 1.0 : 0.0;
-}
-
-void launch_twist_unit_rows(int W, int n, double* Gtr, cudaStream_t st) {
-    const size_t total = (size_t)W * 2 * n * n;
-    twist_unit_rows_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(total, n, Gtr);
+void launch_twist_gl(int rows, int N, int n, const double2* D, const double2* Lp, const double2* Gt, double* gl,
+                     cudaStream_t st) {
+    twist_gl_kernel<<<(rows + 7) / 8, 256, 0, st>>>(rows, n, D, Lp, Gt, N, gl);
 }
 
 // ---------------------------------------------------------------------------
 // Orbital (Pulay) terms of the force estimators with complex orbitals, one CTA
 // per walker, after the measure kernel has accumulated everything else of the
-// sample (the Jastrow and Ewald terms; its own orbital force phase runs on zero
-// coefficients and adds nothing) and written E_L.  grad_i U (the Pade e-e and
+// sample (the Jastrow and Ewald terms) and written E_L.  grad_i U (the Pade e-e and
 // e-n terms of the sin-periodised Jastrow, and with s.fj the e-e-n-n term
 // grad_i U34 = sum_a grad chi_a(r_i) w_ia, w_ia = sum_b f_ab (c_b - chi_b(r_i)),
 // c = sum_j chi(r_j)) is formed here again.  Per spin

@@ -47,13 +47,18 @@ void launch_sweep(const SysView<double>& s, double* X, const double* Xp, const d
 // Walkers per CTA for a warp-per-walker kernel that holds at most `most` of them.
 int walkers_per_cta(int W, int most);
 
-// k_measure.cu: local energy, d ln psi / dR and dE_L / dR per walker.
-template <typename T>
-void launch_measure(const SysView<T>& s, const double* X, const T* D, const T* Lp, const T* Gt,
+// k_measure.cu: local energy, d ln psi / dR and dE_L / dR per walker, mixed form.
+void launch_measure(const SysView<float>& s, const double* X, const float* D, const float* Lp, const float* Gt,
                     const double* logdet, double* acc, double* out_el, double* out_lnpsi, double* out_dl,
                     double* out_de, float* kt_out, float* eg_out, double* elw, float* rk_out, cudaStream_t st);
-template <typename T>
-size_t measure_smem_bytes(int N, int n, int nk, int mmax, bool split);
+
+// k_measure64.cu: the same in the FP64 form, straight from the inverses.  gl [W][N][4]:
+// g_i and l_i given (twisted orbitals; the orbital force terms are then left out), or
+// null.  ktask [ntask]: (m_x, m_y, first of two |m_z|, index of (m_x, m_y, 0)); kxyz
+// [3][nk]: the reciprocal vectors.
+void launch_measure64(const SysView<double>& s, int ntask, const int4* ktask, const double* kxyz, const double* X,
+                      const double* Gt, const double* gl, const double* logdet, double* acc, double* out_el,
+                      double* out_lnpsi, double* out_dl, double* out_de, cudaStream_t st);
 
 // k_setup.cu: per-R tables (proton trig, structure factors, p-p Ewald terms; vpp is
 // work space [N]) and, with Trec, the reciprocal-space force as a [3N][2 nk]
@@ -94,9 +99,8 @@ void launch_twist_invert(int W, int N, int n, const double2* Phi, double2* Gt, d
 void launch_twist_sweep(const SysView<double>& s, const TwistView& tv, double* X, const double* Xp, const double* ptp,
                         const double* uacc, const double2* Phi, double2* Gt, unsigned long long* nacc,
                         cudaStream_t st);
-void launch_twist_gl(int rows, int N, int n, const double2* D, const double2* Lp, const double2* Gt, double* Dr,
-                     double* Lpr, cudaStream_t st);
-void launch_twist_unit_rows(int W, int n, double* Gtr, cudaStream_t st);
+void launch_twist_gl(int rows, int N, int n, const double2* D, const double2* Lp, const double2* Gt, double* gl,
+                     cudaStream_t st);
 void launch_twist_pulay(const SysView<double>& s, const TwistView& tv, const double* X, const double2* D,
                         const double2* Lp, const double2* Gt, const double* elw, double* acc, double* out_dl,
                         double* out_de, cudaStream_t st);
