@@ -442,39 +442,87 @@ __device__ __forceinline__ float rint_fma(float x) {
     return __fsub_rn(__fadd_rn(x, m), m);
 }
 
+// exp(y) / t times erfc(sqrt y)/sqrt y and times minus its derivative in y, t = 1/y,
+// 4 <= y <= 30: polynomials of degree 5 and 4, relative error 3e-7 and 3.5e-7
+// (fitted by fit_erfc.py, fit_image).
+__device__ __forceinline__ float erfc_image_p0(float t) {
+    float p = -1.099364281e+00f;
+    p = p * t + 1.300195098e+00f;
+    p = p * t - 7.889494300e-01f;
+    p = p * t + 4.046300352e-01f;
+    p = p * t - 2.814249396e-01f;
+    p = p * t + 5.641801357e-01f;
+    return p;
+}
+__device__ __forceinline__ float erfc_image_p1(float t) {
+    float p = -1.091428846e-01f;
+    p = p * t + 1.425238252e-01f;
+    p = p * t - 1.344549805e-01f;
+    p = p * t + 2.817852199e-01f;
+    p = p * t + 5.641948581e-01f;
+    return p;
+}
+constexpr float kImageKLMin = 4.0f, kImageKLMax = 6.8f;   // kappa L with every image in the polynomials' range
+
 // Mixed-form real-space Ewald sum of one pair: the images of the minimum-image
 // vector inside the FP32-level cutoff (skip_min: leave out the minimum image),
-// phi(r) = erfc(kappa r) / r and, when grad, its gradient added to grad.
+// phi(r) = erfc(kappa r) / r and, when kGrad, its gradient added to grad.
 // iL = 1/Lt and rc2 = kRealCut2Mixed Lt^2 come from the caller (loop invariants).
+// Nearly every pair has its minimum image inside the cutoff, so that one is
+// evaluated outside the lane loop; the other images (r >= L/2, a warp's loop runs
+// to its largest lane count) take the short polynomials above where kappa L
+// allows it (`fast`), and their gradients are collected as sum of d phi / d r^2
+// with the shifted components' parts apart.
 template <bool kGrad>
-__device__ __forceinline__ float ewald_real_cut(float dx, float dy, float dz, bool skip_min, float Lt, float iL,
-                                                float rc2, float kappa, float* grad) {
+__device__ __forceinline__ float ewald_real_cut(float dx, float dy, float dz, bool skip_min, bool fast, float Lt,
+                                                float iL, float rc2, float kappa, float* grad) {
     dx -= Lt * rint_fma(dx * iL); dy -= Lt * rint_fma(dy * iL); dz -= Lt * rint_fma(dz * iL);
     // moving component m of the minimum image by L away from zero adds
     // L (L - 2 |d_m|) > 0 to r^2 (so only the minimum image can sit at r = 0)
     const float r0 = dx * dx + dy * dy + dz * dz;
     const float e0 = Lt * (Lt - 2.f * fabsf(dx)), e1 = Lt * (Lt - 2.f * fabsf(dy)), e2 = Lt * (Lt - 2.f * fabsf(dz));
     const float r1 = r0 + e0, r2_ = r0 + e1, r3 = r1 + e1, r4 = r0 + e2;
-    unsigned mask = (r0 < rc2 && r0 > 0.f && !skip_min) ? 1u : 0u;
-    mask |= (r1 < rc2 ? 2u : 0u) | (r2_ < rc2 ? 4u : 0u) | (r3 < rc2 ? 8u : 0u) | (r4 < rc2 ? 16u : 0u) |
-            (r1 + e2 < rc2 ? 32u : 0u) | (r2_ + e2 < rc2 ? 64u : 0u) | (r3 + e2 < rc2 ? 128u : 0u);
-    const float sx = dx >= 0.f ? -Lt : Lt, sy = dy >= 0.f ? -Lt : Lt, sz = dz >= 0.f ? -Lt : Lt;
+    unsigned mask = (r1 < rc2 ? 2u : 0u) | (r2_ < rc2 ? 4u : 0u) | (r3 < rc2 ? 8u : 0u) | (r4 < rc2 ? 16u : 0u) |
+                    (r1 + e2 < rc2 ? 32u : 0u) | (r2_ + e2 < rc2 ? 64u : 0u) | (r3 + e2 < rc2 ? 128u : 0u);
     const float c2k = 1.1283791670955126f * kappa;      // 2 kappa / sqrt(pi)
     const float nk2 = -1.4426950408889634f * kappa * kappa;   // -kappa^2 log2(e)
-    float v = 0.f;
-    while (mask) {
-        const int c = __ffs(mask) - 1;
-        mask &= mask - 1;
-        const float a = dx + ((c & 1) ? sx : 0.f), b = dy + ((c & 2) ? sy : 0.f), e = dz + ((c & 4) ? sz : 0.f);
-        const float r2 = a * a + b * b + e * e;
+    float v = 0.f, s = 0.f, s0 = 0.f, s1 = 0.f, s2 = 0.f;     // s: phi'(r) / r
+    auto direct = [&](float r2, float& sr) {
         const float ir = rsqrtf(r2), r = r2 * ir;
         const float ex = ex2_fast(nk2 * r2);              // exp(-kappa^2 r^2)
         const float ec = erfc_scaled_fit(kappa * r, ex);
-        v += ec * ir;
-        if (kGrad) {
-            const float s = -(ec * ir + c2k * ex) * ir * ir;   // phi'(r) / r
-            grad[0] += s * a; grad[1] += s * b; grad[2] += s * e;
+        sr = -(ec * ir + c2k * ex) * ir * ir;
+        return ec * ir;
+    };
+    if (r0 < rc2 && r0 > 0.f && !skip_min) v = direct(r0, s);
+    const float ik2 = __fdividef(1.f, kappa * kappa), kd = -2.f * kappa * kappa;
+    while (mask) {
+        const int c = __ffs(mask) - 1;
+        mask &= mask - 1;
+        float r2 = r0;
+        if (c & 1) r2 += e0;
+        if (c & 2) r2 += e1;
+        if (c & 4) r2 += e2;
+        float sr;
+        if (fast) {
+            const float ir = rsqrtf(r2), t = ir * ir * ik2;
+            const float kt = kappa * t * ex2_fast(nk2 * r2);
+            v += kt * erfc_image_p0(t);
+            sr = kGrad ? kd * kt * erfc_image_p1(t) : 0.f;
+        } else {
+            v += direct(r2, sr);
         }
+        if (kGrad) {
+            s += sr;
+            if (c & 1) s0 += sr;
+            if (c & 2) s1 += sr;
+            if (c & 4) s2 += sr;
+        }
+    }
+    if (kGrad) {
+        grad[0] += s * dx + s0 * (dx >= 0.f ? -Lt : Lt);
+        grad[1] += s * dy + s1 * (dy >= 0.f ? -Lt : Lt);
+        grad[2] += s * dz + s2 * (dz >= 0.f ? -Lt : Lt);
     }
     return v;
 }

@@ -41,7 +41,7 @@ struct qmc_system {
     float *d_C32 = nullptr, *d_ptrig32 = nullptr;
     int4* d_kvec = nullptr;
     double* d_ewt = nullptr;   // real-space Ewald table (FP64 form)
-    // FP64 measure kernel: its structure-factor tasks and the reciprocal vectors [3][nk]
+    // structure-factor tasks of the measure kernels; reciprocal vectors [3][nk] (FP64 form)
     int nktask = 0;
     int4* d_ktask = nullptr;
     double* d_kxyz = nullptr;
@@ -148,7 +148,7 @@ void enumerate_kvec(int mmax, std::vector<int4>& kv) {
             }
 }
 
-// Structure-factor tasks of the FP64 measure kernel: per (m_x, m_y) of the half
+// Structure-factor tasks of the measure kernels: per (m_x, m_y) of the half
 // space and two consecutive |m_z| from m_z0 (even), (m_x, m_y, m_z0, index in kv
 // of (m_x, m_y, 0), extrapolated where that vector is not in the list).
 void enumerate_ktask(const std::vector<int4>& kv, std::vector<int4>& task) {
@@ -225,7 +225,7 @@ size_t footprint(const qmc_params* p) {
     const size_t tc = p->n_twist > 0 ? 16 : t;     // complex orbitals of the twisted form
     b += t * W * N + tc * (W * N * n + 2 * W * n * n);   // uacc, Phi, Gt
     if (t == 4 || p->n_twist > 0) b += tc * 4 * W * N * n;   // D, Lp
-    if (t == 8) b += (16 + 24) * nk;                   // structure-factor tasks (at most nk), reciprocal vectors
+    b += 16 * nk + (t == 8 ? 24 * nk : 0);           // structure-factor tasks (at most nk), reciprocal vectors
     b += 8 * 2 * W + 8 * W * (3 + 9 * N) + 8 * W;   // logdet, acc, nacc
     b += 8 * W + 8 * 5;                              // V_L sums, pressure output
     const size_t Kr = p->n_twist > 0 ? p->n_twist : 1;
@@ -355,7 +355,7 @@ void measure(qmc_system* h, const SysView<float>& s, double* el, double* lnpsi, 
     prof_end(h, ep);
     const bool split = h->use_tc && h->use_tc_adj;
     prof_begin(h, KC_MEASURE, ep);
-    launch_measure(s, h->d_X, (const float*)h->d_D, (const float*)h->d_Lp, (const float*)h->d_Gt, h->d_logdet, h->d_acc,
+    launch_measure(s, h->nktask, h->d_ktask, h->d_X, (const float*)h->d_D, (const float*)h->d_Lp, (const float*)h->d_Gt, h->d_logdet, h->d_acc,
                    el, lnpsi, dl, de, split ? h->d_Kt : nullptr, split ? h->d_eg : nullptr,
                    split ? h->d_elw : nullptr, split ? h->d_rk : nullptr, h->stream);
     prof_end(h, ep);
@@ -696,15 +696,15 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
     }
     std::vector<int4> ktask;
     std::vector<double> kxyz;
+    enumerate_ktask(kv, ktask);
+    h->nktask = (int)ktask.size();
+    h->d_ktask = dalloc<int4>(h, ktask.size(), &rc);
     if (!h->mixed) {
-        enumerate_ktask(kv, ktask);
-        h->nktask = (int)ktask.size();
         kxyz.resize(3 * (size_t)nk);
         for (int k = 0; k < nk; ++k) {
             const double tp = 2.0 * kPi / p->L;
             kxyz[k] = tp * kv[k].x; kxyz[nk + k] = tp * kv[k].y; kxyz[2 * nk + k] = tp * kv[k].z;
         }
-        h->d_ktask = dalloc<int4>(h, ktask.size(), &rc);
         h->d_kxyz = dalloc<double>(h, kxyz.size(), &rc);
     }
     if (!h->mixed && p->ewald_kappa * p->L <= kEwMaxKL) h->d_ewt = dalloc<double>(h, 2 * kEwNodes * kEwTerms, &rc);
@@ -725,10 +725,9 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
     cudaMemcpyAsync(h->d_C32, c32.data(), sizeof(float) * B * n, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(h->d_zeta32, z32.data(), sizeof(float) * h->G, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(h->d_kvec, kv.data(), sizeof(int4) * nk, cudaMemcpyHostToDevice, st);
-    if (!h->mixed) {
-        cudaMemcpyAsync(h->d_ktask, ktask.data(), sizeof(int4) * ktask.size(), cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(h->d_ktask, ktask.data(), sizeof(int4) * ktask.size(), cudaMemcpyHostToDevice, st);
+    if (h->d_kxyz)
         cudaMemcpyAsync(h->d_kxyz, kxyz.data(), sizeof(double) * kxyz.size(), cudaMemcpyHostToDevice, st);
-    }
     cudaMemsetAsync(h->d_err, 0, sizeof(int), st);
     cudaMemsetAsync(h->d_nacc, 0, sizeof(unsigned long long) * W, st);
     if (h->d_chat) prepare_tc_coeff(h->d_C32, B, n, h->d_chat, st);

@@ -168,7 +168,8 @@ __device__ __forceinline__ T jas34_orbital(const T* ei, const T* pa, T ell, T ze
 // Without the bound the unsplit instance took 143 registers, one CTA an SM:
 // 3.14 ms for 4096 walkers of N = 64, now 1.53 ms.
 template <bool kSplit>
-__global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax, const double* __restrict__ X,
+__global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax, int ntask,
+                                                      const int4* __restrict__ ktask, const double* __restrict__ X,
                                                       const T* __restrict__ D, const T* __restrict__ Lp,
                                                       const T* __restrict__ Gt, const double* __restrict__ logdet,
                                                       double* __restrict__ acc, double* __restrict__ out_el,
@@ -492,6 +493,7 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
     double vee_p = 0.0;
     const T Lt = (T)L;
     const float iLt = 1.f / (float)Lt, rc2 = kRealCut2Mixed * (float)Lt * (float)Lt;
+    const bool fast = kap * Lt >= kImageKLMin && kap * Lt <= kImageKLMax;
     // balanced cyclic pairing: electron i with i+d (mod N), d = 1..N/2 (d = N/2 only for i < N/2),
     // the distance range split into nparts slices
     for (int tt = tid; tt < nparts * N; tt += nt) {
@@ -503,7 +505,7 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
             const int j = i + d < N ? i + d : i + d - N;      // (i + d) mod N, d < N
             if (skip) continue;
             v += ewald_real_cut<false>(xt[3 * i] - xt[3 * j], xt[3 * i + 1] - xt[3 * j + 1],
-                                       xt[3 * i + 2] - xt[3 * j + 2], false, Lt, iLt, rc2, kap, nullptr);
+                                       xt[3 * i + 2] - xt[3 * j + 2], false, fast, Lt, iLt, rc2, kap, nullptr);
         }
         vee_p += (double)v;
     }
@@ -539,8 +541,8 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
                 ep_jastrow_f32(sd, cd, ell, k2, bep, Zj, vv, pl, pe);
                 for (int mu = 0; mu < 3; ++mu) { dl[mu] += pl[mu]; de[mu] += pe[mu]; }
             }
-            v += ewald_real_cut<true>(xt[3 * i] - ra[0], xt[3 * i + 1] - ra[1], xt[3 * i + 2] - ra[2], close, Lt, iLt,
-                                      rc2, kap, gv);
+            v += ewald_real_cut<true>(xt[3 * i] - ra[0], xt[3 * i + 1] - ra[1], xt[3 * i + 2] - ra[2], close, fast, Lt,
+                                      iLt, rc2, kap, gv);
         }
         v = warp_sum(v);
 #pragma unroll
@@ -656,26 +658,43 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
     __syncthreads();
     double vrec_p = 0.0;
     T vrec_t = 0;
-    for (int k = tid; k < nk; k += nt) {
-        const int4 m = s.kvec[k];
-        T re = 0, im = 0;
+    // A task is two |m_z| of one (m_x, m_y): with ab the x y phase and c the z
+    // phase, the four sums of ab.x c.x, ab.y c.y, ab.x c.y, ab.y c.x give rho at
+    // both signs of m_z, 12 operations an electron for four vectors (32 one by one).
+    for (int tk = tid; tk < ntask; tk += nt) {
+        const int4 m = ktask[tk];                 // m_x >= 0, m_y, first |m_z|, index of (m_x, m_y, 0)
+        const int my = m.y < 0 ? -m.y : m.y, z1 = m.z + 1 <= mmax ? m.z + 1 : mmax;
+        const T sy = m.y < 0 ? T(-1) : T(1);
+        T q[2][4] = {};
         for (int i = 0; i < N; ++i) {
-            const V2<T> a = etab[(3 * i) * nm + m.x];   // m.x >= 0 in the half space
-            V2<T> b = etab[(3 * i + 1) * nm + (m.y < 0 ? -m.y : m.y)], c = etab[(3 * i + 2) * nm + (m.z < 0 ? -m.z : m.z)];
-            if (m.y < 0) b.y = -b.y;
-            if (m.z < 0) c.y = -c.y;
-            const T abx = a.x * b.x - a.y * b.y, aby = a.x * b.y + a.y * b.x;
-            re += abx * c.x - aby * c.y;
-            im += abx * c.y + aby * c.x;
+            const V2<T>* e = etab + (size_t)3 * i * nm;
+            const V2<T> a = e[m.x], b = e[nm + my], c0 = e[2 * nm + m.z], c1 = e[2 * nm + z1];
+            const T by = sy * b.y;
+            const T x = a.x * b.x - a.y * by, y = a.x * by + a.y * b.x;
+            q[0][0] += x * c0.x; q[0][1] += y * c0.y; q[0][2] += x * c0.y; q[0][3] += y * c0.x;
+            q[1][0] += x * c1.x; q[1][1] += y * c1.y; q[1][2] += x * c1.y; q[1][3] += y * c1.x;
         }
-        const double2 rp = s.rho_p[k];
-        const T rr = (T)rp.x - re, ri = (T)rp.y - im;   // electrons carry -1
-        rhot[k] = V2<T>{rr, ri};
-        if constexpr (kSplit) {
-            rk_out[(size_t)w * 2 * nk + 2 * k] = (float)rr;
-            rk_out[(size_t)w * 2 * nk + 2 * k + 1] = (float)ri;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int mz = m.z + h;
+            if (m.x * m.x + m.y * m.y + mz * mz > mmax * mmax) continue;
+#pragma unroll
+            for (int sg = 0; sg < 2; ++sg) {      // +m_z, -m_z
+                if (mz == 0 && (sg || (m.x == 0 && m.y == 0))) continue;
+                if (sg && m.x == 0 && m.y == 0) continue;
+                const int k = m.w + (sg ? -mz : mz);
+                const T re = sg ? q[h][0] + q[h][1] : q[h][0] - q[h][1];
+                const T im = sg ? q[h][3] - q[h][2] : q[h][3] + q[h][2];
+                const double2 rp = s.rho_p[k];
+                const T rr = (T)rp.x - re, ri = (T)rp.y - im;   // electrons carry -1
+                rhot[k] = V2<T>{rr, ri};
+                if constexpr (kSplit) {
+                    rk_out[(size_t)w * 2 * nk + 2 * k] = (float)rr;
+                    rk_out[(size_t)w * 2 * nk + 2 * k + 1] = (float)ri;
+                }
+                vrec_t += s.kwt[k] * (rr * rr + ri * ri);
+            }
         }
-        vrec_t += s.kwt[k] * (rr * rr + ri * ri);
     }
     vrec_p += (double)vrec_t;
     __syncthreads();
@@ -984,7 +1003,7 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
 
 }  // namespace
 
-void launch_measure(const SysView<float>& s, const double* X, const float* D, const float* Lp, const float* Gt,
+void launch_measure(const SysView<float>& s, int ntask, const int4* ktask, const double* X, const float* D, const float* Lp, const float* Gt,
                     const double* logdet, double* acc, double* out_el, double* out_lnpsi, double* out_dl,
                     double* out_de, float* kt_out, float* eg_out, double* elw, float* rk_out, cudaStream_t st) {
     const bool split = kt_out != nullptr;
@@ -998,10 +1017,10 @@ void launch_measure(const SysView<float>& s, const double* X, const float* D, co
         attr_set[split] = true;
     }
     if (split)
-        measure_kernel<true><<<s.W, 256, smem, st>>>(s, s.mmax, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
+        measure_kernel<true><<<s.W, 256, smem, st>>>(s, s.mmax, ntask, ktask, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
                                                      out_de, kt_out, eg_out, elw, rk_out);
     else
-        measure_kernel<false><<<s.W, 256, smem, st>>>(s, s.mmax, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
+        measure_kernel<false><<<s.W, 256, smem, st>>>(s, s.mmax, ntask, ktask, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
                                                       out_de, nullptr, nullptr, nullptr, nullptr);
 }
 

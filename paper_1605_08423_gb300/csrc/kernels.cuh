@@ -48,14 +48,15 @@ void launch_sweep(const SysView<double>& s, double* X, const double* Xp, const d
 int walkers_per_cta(int W, int most);
 
 // k_measure.cu: local energy, d ln psi / dR and dE_L / dR per walker, mixed form.
-void launch_measure(const SysView<float>& s, const double* X, const float* D, const float* Lp, const float* Gt,
+// ktask [ntask]: structure-factor tasks, (m_x, m_y, first of two |m_z|, index of
+// (m_x, m_y, 0)).
+void launch_measure(const SysView<float>& s, int ntask, const int4* ktask, const double* X, const float* D, const float* Lp, const float* Gt,
                     const double* logdet, double* acc, double* out_el, double* out_lnpsi, double* out_dl,
                     double* out_de, float* kt_out, float* eg_out, double* elw, float* rk_out, cudaStream_t st);
 
 // k_measure64.cu: the same in the FP64 form, straight from the inverses.  gl [W][N][4]:
 // g_i and l_i given (twisted orbitals; the orbital force terms are then left out), or
-// null.  ktask [ntask]: (m_x, m_y, first of two |m_z|, index of (m_x, m_y, 0)); kxyz
-// [3][nk]: the reciprocal vectors.
+// null.  kxyz [3][nk]: the reciprocal vectors.
 void launch_measure64(const SysView<double>& s, int ntask, const int4* ktask, const double* kxyz, const double* X,
                       const double* Gt, const double* gl, const double* logdet, double* acc, double* out_el,
                       double* out_lnpsi, double* out_dl, double* out_de, cudaStream_t st);

@@ -12,6 +12,8 @@ order first) and the relative error of their FP32 Horner evaluation.
 """
 from __future__ import annotations
 
+import math
+
 import numpy as np
 
 X_MAX = 4.1
@@ -50,7 +52,31 @@ def fp32_max_rel_error(coef, n: int = 40001) -> float:
     return float(np.max(np.abs(approx - g) / g))
 
 
+# Images other than the nearest one (csrc/common.cuh, ewald_real_cut): with
+# y = (kappa r)^2 and t = 1/y,
+#   erfc(sqrt y)/sqrt y         = exp(-y) t P0(t),
+#   -d/dy [erfc(sqrt y)/sqrt y] = exp(-y) t P1(t),   Y_MIN <= y <= Y_MAX,
+# P0 of degree 5 and P1 of degree 4 (Chebyshev interpolation in t).
+Y_MIN, Y_MAX = 4.0, 30.0
+IMAGE_DEGREES = (5, 4)
+
+
+def image_target(which: int, y):
+    from scipy.special import erfcx
+    r = np.sqrt(y)
+    g0 = 0.5 * math.sqrt(math.pi) * erfcx(r) / r
+    return 2.0 / math.sqrt(math.pi) * (g0 if which == 0 else (1.0 + g0) / (2.0 * y))
+
+
+def fit_image(which: int, n: int = 400) -> np.ndarray:
+    x = np.cos(np.pi * (np.arange(n) + 0.5) / n)
+    t = 0.5 * (x + 1.0) * (1.0 / Y_MIN - 1.0 / Y_MAX) + 1.0 / Y_MAX
+    return np.polyfit(t, image_target(which, 1.0 / t) / t, IMAGE_DEGREES[which])[::-1]
+
+
 if __name__ == "__main__":
+    for k in (0, 1):
+        print("image", k, [f"{float(np.float32(v)):.9e}" for v in fit_image(k)])
     cf = fit()
     print([f"{float(np.float32(v)):.9e}" for v in cf])
     print("max relative error (FP32 evaluation):", fp32_max_rel_error(cf))
