@@ -485,7 +485,7 @@ double run_sampling_twist(qmc_system* h) {
         prof_end(h, ep);
         prof_begin(h, KC_SWEEP, ep);
         launch_twist_sweep(s, h->tv, h->d_X, h->d_Xp, (const double*)h->d_ptp, (const double*)h->d_uacc,
-                           (const double2*)h->d_Phi, (double2*)h->d_Gt, h->d_nacc, h->stream);
+                           (const double2*)h->d_Phi, (double2*)h->d_Gt, h->d_nacc, (double*)h->d_vep, sw == 0, h->stream);
         prof_end(h, ep);
         if ((sw + 1) % h->p.recompute_every == 0) recompute_twist(h, W);
         if (sw >= nw && ((sw - nw + 1) % h->p.measure_every) == 0) measure_twist(h, W, nullptr, nullptr, nullptr, nullptr);

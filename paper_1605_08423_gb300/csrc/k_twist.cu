@@ -286,7 +286,8 @@ void launch_twist_invert(int W, int N, int n, const double2* Phi, double2* Gt, d
 // Slater block at the stored positions.
 // ---------------------------------------------------------------------------
 __host__ __device__ inline size_t twist_sweep_warp_bytes(int N, int n, bool j34) {
-    const size_t b = ((size_t)n * (n + 1) + 2 * (size_t)n) * sizeof(double2) + (size_t)(j34 ? 9 : 6) * N * sizeof(double);
+    const size_t b = ((size_t)n * (n + 1) + 2 * (size_t)n) * sizeof(double2) +
+                     ((size_t)(j34 ? 10 : 7) * N + 6) * sizeof(double);
     return (b + 15) & ~size_t(15);
 }
 
@@ -309,7 +310,13 @@ __device__ __forceinline__ double tw_pair_dist(const double* a, const double* b,
         const double sd = a[mu] * b[3 + mu] - a[3 + mu] * b[mu];
         t += sd * sd;
     }
-    return ell * sqrt(t);
+    return ell * qsqrt_pair(t);
+}
+
+// Pade pair term cu r / (1 + cb r) (cu = 1/2: e-e, cu = -Zj: e-n)
+__device__ __forceinline__ double tw_pade_u(const double* a, const double* b, double ell, double cb, double cu) {
+    const double r = tw_pair_dist(a, b, ell);
+    return cu * r * qrcp(fma(cb, r, 1.0));
 }
 
 __global__ void __launch_bounds__(256) twist_sweep_kernel(SysView<double> s, TwistView tv, double* __restrict__ X,
@@ -317,7 +324,8 @@ __global__ void __launch_bounds__(256) twist_sweep_kernel(SysView<double> s, Twi
                                                           const double* __restrict__ ptp,
                                                           const double* __restrict__ uacc,
                                                           const double2* __restrict__ Phi, double2* __restrict__ Gt,
-                                                          unsigned long long* __restrict__ nacc) {
+                                                          unsigned long long* __restrict__ nacc,
+                                                          double* __restrict__ Vep, int vep_init) {
     extern __shared__ __align__(16) unsigned char smraw[];
     const int N = s.N, n = s.n, ld = n + 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
@@ -328,8 +336,10 @@ __global__ void __launch_bounds__(256) twist_sweep_kernel(SysView<double> s, Twi
     double2* Gs = (double2*)mine;            // [n][ld]
     double2* rowb = Gs + (size_t)n * ld;     // [n]
     double2* phi = rowb + n;                 // [n]
-    double* et = (double*)(phi + n);         // [N][6] electron trig
-    double* c34 = et + 6 * N;                // [N] sum over electrons of chi_a (e-e-n-n term)
+    double* ptb = (double*)(phi + n);        // [6] the proposal's trig
+    double* et = ptb + 6;                    // [N][6] electron trig
+    double* vj = et + 6 * N;                 // [N] V_i = sum_a u_en(r_i, R_a), carried as in sweep_kernel
+    double* c34 = vj + N;                    // [N] sum over electrons of chi_a (e-e-n-n term)
     double* cho = c34 + N;                   // [N] chi_a at the moving electron
     double* chn = cho + N;                   // [N] chi_a at its proposal
     for (int idx = threadIdx.x; idx < 6 * N; idx += blockDim.x) ptr_s[idx] = s.ptrig[idx];
@@ -347,6 +357,14 @@ __global__ void __launch_bounds__(256) twist_sweep_kernel(SysView<double> s, Twi
         et[6 * i + 3 + mu] = cs;
     }
     __syncwarp();
+    for (int i = lane; i < N; i += 32) {
+        double v = 0;
+        if (vep_init)
+            for (int a = 0; a < N; ++a) v += tw_pade_u(et + 6 * i, ptr_s + 6 * a, ell, bep, -Zj);
+        else
+            v = Vep[(size_t)w * N + i];
+        vj[i] = v;
+    }
     const double zj = s.zeta_j;
     if (j34) {
         for (int a = lane; a < N; a += 32) {
@@ -354,8 +372,8 @@ __global__ void __launch_bounds__(256) twist_sweep_kernel(SysView<double> s, Twi
             for (int j = 0; j < N; ++j) c += tw_jas_orbital(et + 6 * j, ptr_s + 6 * a, ell, zj);
             c34[a] = c;
         }
-        __syncwarp();
     }
+    __syncwarp();
     const double* th = tv.theta + 3 * (w / tv.Wk);
     unsigned long long naccept = 0;
     for (int sp = 0; sp < 2; ++sp) {
@@ -366,34 +384,25 @@ __global__ void __launch_bounds__(256) twist_sweep_kernel(SysView<double> s, Twi
         for (int il = 0; il < n; ++il) {
             const int i = sp * n + il;
             const size_t row = (size_t)w * N + i;
-            double pt[6];
-#pragma unroll
-            for (int mu = 0; mu < 6; ++mu) pt[mu] = ptp[row * 6 + mu];
+            if (lane < 6) ptb[lane] = ptp[row * 6 + lane];
             for (int j = lane; j < n; j += 32) phi[j] = Phi[row * n + j];
             const double u = uacc[row];
             __syncwarp();
             double2 part = czero();
             for (int j = lane; j < n; j += 32) part = cadd(part, cmul(phi[j], Gs[il * ld + j]));
-            const double2 ratio = make_double2(warp_sum(part.x), warp_sum(part.y));
-            double du = 0;
             const double* ei = et + 6 * i;
-            for (int j = lane; j < N; j += 32) {
-                const double* ej = et + 6 * j;
-                double u1, u0, d1, d2;
-                pade_ee(bee, tw_pair_dist(pt, ej, ell), u1, d1, d2);
-                pade_ee(bee, tw_pair_dist(ei, ej, ell), u0, d1, d2);
-                du += (j != i) ? u1 - u0 : 0.0;
+            // items 0..N-1: u_ee at the proposal, N..2N-1: minus u_ee at the old position
+            double du = 0, vnew = 0;
+            for (int k = lane; k < 2 * N; k += 32) {
+                const bool old = k >= N;
+                const int j = old ? k - N : k;
+                const double v = tw_pade_u(old ? ei : ptb, et + 6 * j, ell, bee, old ? -0.5 : 0.5);
+                du += j != i ? v : 0.0;
             }
-            for (int a = lane; a < N; a += 32) {
-                const double* pa = ptr_s + 6 * a;
-                double u1, u0, d1, d2, d3;
-                pade_ep(bep, Zj, tw_pair_dist(pt, pa, ell), u1, d1, d2, d3);
-                pade_ep(bep, Zj, tw_pair_dist(ei, pa, ell), u0, d1, d2, d3);
-                du += u1 - u0;
-            }
+            for (int a = lane; a < N; a += 32) vnew += tw_pade_u(ptb, ptr_s + 6 * a, ell, bep, -Zj);
             if (j34) {
                 for (int a = lane; a < N; a += 32) {
-                    chn[a] = tw_jas_orbital(pt, ptr_s + 6 * a, ell, zj);
+                    chn[a] = tw_jas_orbital(ptb, ptr_s + 6 * a, ell, zj);
                     cho[a] = tw_jas_orbital(ei, ptr_s + 6 * a, ell, zj);
                 }
                 __syncwarp();
@@ -404,7 +413,23 @@ __global__ void __launch_bounds__(256) twist_sweep_kernel(SysView<double> s, Twi
                     du += (chn[a] - cho[a]) * wa;
                 }
             }
-            du = warp_sum(du);
+            // the four warp sums in seven additions: each half of the warp keeps two
+            // quantities, then each quarter one
+            double2 ratio;
+            {
+                const bool hi = lane & 16, q = lane & 8;
+                double a0 = hi ? du : part.x, a1 = hi ? vnew : part.y;
+                a0 += __shfl_xor_sync(0xffffffffu, hi ? part.x : du, 16);
+                a1 += __shfl_xor_sync(0xffffffffu, hi ? part.y : vnew, 16);
+                double x = q ? a1 : a0;
+                x += __shfl_xor_sync(0xffffffffu, q ? a0 : a1, 8);
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                ratio = make_double2(__shfl_sync(0xffffffffu, x, 0), __shfl_sync(0xffffffffu, x, 8));
+                du = __shfl_sync(0xffffffffu, x, 16);
+                vnew = __shfl_sync(0xffffffffu, x, 24);
+            }
+            du += vnew - vj[i];
             const double prob = (ratio.x * ratio.x + ratio.y * ratio.y) * exp(2.0 * du);
             if (u < prob) {
                 for (int j = lane; j < n; j += 32) rowb[j] = Gs[il * ld + j];
@@ -426,13 +451,11 @@ __global__ void __launch_bounds__(256) twist_sweep_kernel(SysView<double> s, Twi
                 }
                 if (lane < 3) {
                     const double xpl = Xp[row * 3 + lane];
-                    const double x = xpl - L * floor(xpl / L);
-                    Xw[3 * i + lane] = x;
-                    double sn, cs;
-                    sincospi(x / L, &sn, &cs);
-                    et[6 * i + lane] = sn;
-                    et[6 * i + 3 + lane] = cs;
+                    Xw[3 * i + lane] = xpl - L * floor(xpl / L);
                 }
+                // every use of the trig triple is even in its sign, which is all that wrapping changes
+                if (lane < 6) et[6 * i + lane] = ptb[lane];
+                if (lane == 0) vj[i] = vnew;
                 if (kth != 0.0) {
                     double sn, cs;
                     sincos(sg * kth, &sn, &cs);
@@ -448,22 +471,25 @@ __global__ void __launch_bounds__(256) twist_sweep_kernel(SysView<double> s, Twi
         for (int idx = lane; idx < n * n; idx += 32) G[idx] = Gs[(idx / n) * ld + idx % n];
         __syncwarp();
     }
+    for (int i = lane; i < N; i += 32) Vep[(size_t)w * N + i] = vj[i];
     if (lane == 0) nacc[w] += naccept;
 }
 
 void launch_twist_sweep(const SysView<double>& s, const TwistView& tv, double* X, const double* Xp, const double* ptp,
-                        const double* uacc, const double2* Phi, double2* Gt, unsigned long long* nacc,
-                        cudaStream_t st) {
+                        const double* uacc, const double2* Phi, double2* Gt, unsigned long long* nacc, double* vep,
+                        bool vep_init, cudaStream_t st) {
     const size_t wb = twist_sweep_warp_bytes(s.N, s.n, s.fj != nullptr);
     const size_t base = ((size_t)6 * s.N * sizeof(double) + 15) & ~size_t(15);
     int wpb = (int)((200u * 1024u - base) / wb);
-    wpb = wpb < 1 ? 1 : (wpb > 8 ? 8 : wpb);
+    // spread over the SMs: 512 walkers of N = 64 at 8 a CTA filled 64 of 152 (2.70 ms a sweep)
+    wpb = walkers_per_cta(s.W, wpb < 1 ? 1 : (wpb > 8 ? 8 : wpb));
     const size_t smem = base + (size_t)wpb * wb;
     static size_t attr = 0;
     if (smem > attr &&
         cudaFuncSetAttribute(twist_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)
         attr = smem;
-    twist_sweep_kernel<<<(s.W + wpb - 1) / wpb, 32 * wpb, smem, st>>>(s, tv, X, Xp, ptp, uacc, Phi, Gt, nacc);
+    twist_sweep_kernel<<<(s.W + wpb - 1) / wpb, 32 * wpb, smem, st>>>(s, tv, X, Xp, ptp, uacc, Phi, Gt, nacc, vep,
+                                                                               vep_init ? 1 : 0);
 }
 
 // ---------------------------------------------------------------------------

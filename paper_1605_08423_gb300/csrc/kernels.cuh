@@ -98,8 +98,8 @@ void launch_twist_orbitals(const SysView<double>& s, const TwistView& tv, const 
 void launch_twist_invert(int W, int N, int n, const double2* Phi, double2* Gt, double* logdet, int* err,
                          cudaStream_t st);
 void launch_twist_sweep(const SysView<double>& s, const TwistView& tv, double* X, const double* Xp, const double* ptp,
-                        const double* uacc, const double2* Phi, double2* Gt, unsigned long long* nacc,
-                        cudaStream_t st);
+                        const double* uacc, const double2* Phi, double2* Gt, unsigned long long* nacc, double* vep,
+                        bool vep_init, cudaStream_t st);
 void launch_twist_gl(int rows, int N, int n, const double2* D, const double2* Lp, const double2* Gt, double* gl,
                      cudaStream_t st);
 void launch_twist_pulay(const SysView<double>& s, const TwistView& tv, const double* X, const double2* D,
