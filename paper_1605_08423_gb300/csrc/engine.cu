@@ -302,14 +302,16 @@ void setup_tables(qmc_system* h) {
                  h->stream);
 }
 
-// Orbital rows at `pos`: tensor-core kernel in the mixed form, SIMT otherwise.
-template <typename T>
-void orbitals(qmc_system* h, const SysView<T>& s, const double* pos, int nrows, T* val, T* grad, T* lap) {
-    if (sizeof(T) == 4 && h->use_tc)
-        launch_orbitals_tc(*(const SysView<float>*)&s, h->d_chat, pos, nrows, (float*)val, (float*)grad, (float*)lap,
-                           h->stream);
-    else
-        launch_orbitals<T>(s, pos, nrows, val, grad, lap, h->stream);
+// Orbital rows at `pos`: mixed form, tensor-core or SIMT kernel; FP64 form, values
+// only (ptp: the positions' trig, where the proposal kernel has written it).
+void orbitals(qmc_system* h, const SysView<float>& s, const double* pos, const float*, int nrows, float* val, float* grad,
+              float* lap) {
+    if (h->use_tc) launch_orbitals_tc(s, h->d_chat, pos, nrows, val, grad, lap, h->stream);
+    else launch_orbitals(s, pos, nrows, val, grad, lap, h->stream);
+}
+void orbitals(qmc_system* h, const SysView<double>& s, const double* pos, const double* ptp, int nrows, double* val,
+              double*, double*) {
+    launch_orbitals(s, pos, ptp, nrows, val, h->stream);
 }
 
 // Slater matrices at the current walker positions and their FP64 inverse.
@@ -319,7 +321,7 @@ void recompute(qmc_system* h, int W) {
     prof_begin(h, KC_RECOMPUTE, ep);
     SysView<T> s = view<T>(h, W);
     h->nlaunch += 2;
-    orbitals<T>(h, s, h->d_X, W * h->N, (T*)h->d_Phi, nullptr, nullptr);
+    orbitals(h, s, h->d_X, (const T*)nullptr, W * h->N, (T*)h->d_Phi, nullptr, nullptr);
     launch_invert<T>(W, h->N, h->n, (const T*)h->d_Phi, (T*)h->d_Gt, h->d_logdet, h->d_err, h->stream);
     prof_end(h, ep);
 }
@@ -338,7 +340,7 @@ void recompute_in_call(qmc_system* h, int W) {
             prof_begin(h, KC_RECOMPUTE, ep);
             SysView<T> s = view<T>(h, W);
             h->nlaunch += 2;
-            orbitals<T>(h, s, h->d_X, W * h->N, (T*)h->d_Phi, nullptr, nullptr);
+            orbitals(h, s, h->d_X, (const T*)nullptr, W * h->N, (T*)h->d_Phi, nullptr, nullptr);
             launch_refine(W, h->N, h->n, (const float*)h->d_Phi, (float*)h->d_Gt, h->d_logdet, h->d_err, h->stream);
             prof_end(h, ep);
             return;
@@ -351,7 +353,7 @@ void measure(qmc_system* h, const SysView<float>& s, double* el, double* lnpsi, 
     EventPair ep;
     h->nlaunch += 2;
     prof_begin(h, KC_ORB_MEAS, ep);
-    orbitals<float>(h, s, h->d_X, s.W * h->N, (float*)h->d_Phi, (float*)h->d_D, (float*)h->d_Lp);
+    orbitals(h, s, h->d_X, nullptr, s.W * h->N, (float*)h->d_Phi, (float*)h->d_D, (float*)h->d_Lp);
     prof_end(h, ep);
     const bool split = h->use_tc && h->use_tc_adj;
     prof_begin(h, KC_MEASURE, ep);
@@ -409,7 +411,7 @@ double run_sampling(qmc_system* h) {
                           h->p.sigma, h->w0, h->stream);
         prof_end(h, ep);
         prof_begin(h, KC_ORB_PROP, ep);
-        orbitals<T>(h, s, h->d_Xp, W * N, (T*)h->d_Phi, nullptr, nullptr);
+        orbitals(h, s, h->d_Xp, (const T*)h->d_ptp, W * N, (T*)h->d_Phi, nullptr, nullptr);
         prof_end(h, ep);
         prof_begin(h, KC_SWEEP, ep);
         launch_sweep(s, h->d_X, h->d_Xp, (const T*)h->d_ptp, (const T*)h->d_uacc, (const T*)h->d_Phi, (T*)h->d_Gt,

@@ -89,25 +89,6 @@ __device__ __forceinline__ Geo geometry(const double* e, const double* a, double
     return g;
 }
 
-// Radial factors of the Pade terms u = c r / (1 + b r) in t = r^2, from one
-// reciprocal square root and one reciprocal: with iq = 1/(1 + b r), ir = 1/r,
-//   2 f1 = c iq^2 ir,  4 f2 = -c iq^2 ir^2 (2 b iq + ir),
-//   8 f3 = 3 c iq^2 ir^3 (2 b^2 iq^2 + (2 b iq + ir) ir).
-__device__ __forceinline__ void pade_factors(double t, double b, double c, double& u, double& c2, double& c4) {
-    const double ir = qrsqrt(t), r = t * ir, iq = qrcp(fma(b, r, 1.0));
-    const double A = c * iq * iq;
-    u = c * r * iq;
-    c2 = A * ir;
-    c4 = -(c2 * ir) * fma(2.0 * b, iq, ir);
-}
-__device__ __forceinline__ void pade_factors3(double t, double b, double c, double& c2, double& c4, double& c8) {
-    const double ir = qrsqrt(t), r = t * ir, iq = qrcp(fma(b, r, 1.0));
-    const double bq = b * iq, h = fma(2.0, bq, ir), C = c * iq * iq * ir * ir;
-    c2 = c * iq * iq * ir;
-    c4 = -C * h;
-    c8 = 3.0 * (C * ir) * fma(h, ir, 2.0 * bq * bq);
-}
-
 // Sums of eight values over the warp in nine additions: lane l returns the sum of
 // value (l >> 2) (the halves exchange what the other keeps).
 __device__ __forceinline__ double warp_sum8(double v[8], int lane) {
@@ -204,7 +185,7 @@ __device__ __forceinline__ void gram_store(int np, const double* acc, double* M,
 __device__ __forceinline__ double jas34(const double* ei, const double* pa, double ell, double zeta, double k2,
                                         RadialDerivs<double>& rd) {
     const Geo g = geometry(ei, pa, ell);
-    const double e = exp(-zeta * g.t);
+    const double e = qexp(-zeta * g.t);
     radial_chain(g.p, g.q, -zeta * e, zeta * zeta * e, -zeta * zeta * zeta * e, k2, rd);
     return e;
 }
@@ -411,7 +392,7 @@ __global__ void __launch_bounds__(kThreads, 2) measure64_kernel(SysView<double> 
                                     double s1 = 0, s2 = 0, s3 = 0;   // sum_g Z zeta^q chi
                                     for (int g = 0; g < G; ++g) {
                                         const double z = s.zeta[g];
-                                        const double w1 = z * exp(-z * o.t), w2 = z * w1;
+                                        const double w1 = z * qexp(-z * o.t), w2 = z * w1;
                                         const double Z = Zs[base + g * ld];
                                         Cs[base + g * ld] = 2.0 * w1;
                                         Ys[base + g * ld] = fma(w1, sp2, -(w2 * pp2));
@@ -434,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, 2) measure64_kernel(SysView<double> 
                                     } else {
                                         for (int g = 0; g < G; ++g) {
                                             const double z = s.zeta[g];
-                                            pc = fma(Ys[base + g * ld], 2.0 * z * exp(-z * o.t), pc);
+                                            pc = fma(Ys[base + g * ld], 2.0 * z * qexp(-z * o.t), pc);
                                         }
                                     }
 #pragma unroll

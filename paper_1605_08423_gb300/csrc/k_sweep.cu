@@ -164,7 +164,6 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* _
             __syncwarp();
             double part = 0;
             for (int j = lane; j < n; j += 32) part += phi[j] * Gs[il * ld + j];
-            const double ratio = warp_sum(part);
             const double* ei = et + 6 * i;
             // items 0..N-1: u_ee at the proposal, N..2N-1: minus u_ee at the old position
             double du = 0, vnew = 0;
@@ -192,18 +191,28 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* _
                     du += (chn[a] - cho[a]) * wa;
                 }
             }
-            // both warp sums in five additions: lanes 0-15 reduce du, 16-31 vnew
-            double x = lane < 16 ? du : vnew;
-            x += __shfl_xor_sync(0xffffffffu, lane < 16 ? vnew : du, 16);
+            // the three warp sums in seven additions: the halves of the warp exchange
+            // (ratio, du) for (vnew, 0), then the quarters
+            double ratio;
+            {
+                const bool hi = lane & 16, qr = lane & 8;
+                double a0 = hi ? vnew : part, a1 = hi ? 0.0 : du;
+                a0 += __shfl_xor_sync(0xffffffffu, hi ? part : vnew, 16);
+                a1 += __shfl_xor_sync(0xffffffffu, hi ? du : 0.0, 16);
+                double x = qr ? a1 : a0;
+                x += __shfl_xor_sync(0xffffffffu, qr ? a0 : a1, 8);
 #pragma unroll
-            for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            vnew = __shfl_sync(0xffffffffu, x, 16);
-            du = __shfl_sync(0xffffffffu, x, 0) + (vnew - vj[i]);
-            const double prob = ratio * ratio * exp(2.0 * du);
+                for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                ratio = __shfl_sync(0xffffffffu, x, 0);
+                du = __shfl_sync(0xffffffffu, x, 8);
+                vnew = __shfl_sync(0xffffffffu, x, 16);
+            }
+            du += vnew - vj[i];
+            const double prob = ratio * ratio * qexp(2.0 * du);
             if (u < prob) {
                 for (int j = lane; j < nv; j += 32) rowb[j] = Gs[il * ld + j];
                 __syncwarp();
-                const double ir = 1.0 / ratio;
+                const double ir = qrcp(ratio);
                 const double2* phv = (const double2*)phi;
                 const double2* rbv = (const double2*)rowb;
                 for (int l = lane; l < n; l += 32) {
@@ -221,7 +230,9 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* _
                 }
                 if (lane < 3) {   // wrap into [0, L) at once (as the reference chain does)
                     const double xpl = Xp[row * 3 + lane];
-                    Xw[3 * i + lane] = xpl - L * floor(xpl / L);
+                    const double q = xpl * iL, f = floor(q);
+                    // the division only where the product's rounding could decide
+                    Xw[3 * i + lane] = xpl - L * (fabs(q - rint(q)) > 1e-12 ? f : floor(xpl / L));
                 }
                 // the trig triple of the unwrapped proposal: wrapping flips the
                 // signs of a component's sine and cosine together, and every use

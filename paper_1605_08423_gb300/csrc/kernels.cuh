@@ -5,8 +5,11 @@
 namespace qmc {
 
 // k_orbitals.cu
-template <typename T>
-void launch_orbitals(const SysView<T>& s, const double* pos, int nrows, T* val, T* grad, T* lap, cudaStream_t st);
+void launch_orbitals(const SysView<float>& s, const double* pos, int nrows, float* val, float* grad, float* lap,
+                     cudaStream_t st);
+// FP64 form, values only; trig: (sin, cos)(pi x / L) [rows][6] of the positions, or null
+void launch_orbitals(const SysView<double>& s, const double* pos, const double* trig, int nrows, double* val,
+                     cudaStream_t st);
 template <typename T>
 void launch_propose(int W, int N, double L, double* X, double* Xp, T* ptp, T* uacc, Key key, uint32_t md,
                     uint32_t sweep, double sigma, uint32_t w0, cudaStream_t st);
