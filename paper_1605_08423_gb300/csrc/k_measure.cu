@@ -118,27 +118,92 @@ __device__ __forceinline__ void ep_jastrow_f32(const float sd[3], const float cd
     }
 }
 
-// The same in FP64, for the close pairs.
-__device__ __forceinline__ void ep_jastrow(const double sd[3], const double cd[3], double ell, double k2, double bep,
-                                           double Zj, const double vv[3], double dl[3], double de[3]) {
-    double p[3], q[3], t = 0;
+// sin and cos of |x| <= 1/2 in FP64 by their Taylor series (terms to x^15, x^16:
+// remainder below 1e-19).
+__device__ __forceinline__ void sincos_half(double x, double& sn, double& cs) {
+    const double y = x * x;
+    double p = fma(y, -7.6471637318198164759e-13, 1.6059043836821614599e-10);   // -1/15!, 1/13!
+    p = fma(p, y, -2.5052108385441718775e-08);
+    p = fma(p, y, 2.7557319223985890653e-06);
+    p = fma(p, y, -1.9841269841269841270e-04);
+    p = fma(p, y, 8.3333333333333333333e-03);
+    p = fma(p, y, -1.6666666666666666667e-01);
+    sn = fma(p * y, x, x);
+    double q = fma(y, 4.7794773323873852974e-14, -1.1470745597729724714e-11);   // 1/16!, -1/14!
+    q = fma(q, y, 2.0876756987868098979e-09);
+    q = fma(q, y, -2.7557319223985890653e-07);
+    q = fma(q, y, 2.4801587301587301587e-05);
+    q = fma(q, y, -1.3888888888888888889e-03);
+    q = fma(q, y, 4.1666666666666666667e-02);
+    q = fma(q, y, -0.5);
+    cs = fma(q, y, 1.0);
+}
+
+// erf(kappa r)/r = kappa 2/sqrt(pi) sum_n (-x)^n / (n! (2n + 1)), x = (kappa r)^2 <= 2/3,
+// to n = 12 (remainder 1e-14), with its derivative in x, both over kappa 2/sqrt(pi).
+__device__ __forceinline__ double erf_over_r_series(double x, double& d) {
+    constexpr double c[13] = {1.0,            -1.0 / 3.0,         1.0 / 10.0,           -1.0 / 42.0,        1.0 / 216.0,
+                              -1.0 / 1320.0,  1.0 / 9360.0,       -1.0 / 75600.0,       1.0 / 685440.0,     -1.0 / 6894720.0,
+                              1.0 / 76204800.0, -1.0 / 918086400.0, 1.0 / 11975040000.0};
+    double v = c[12];
+    d = 0.0;
+#pragma unroll
+    for (int n = 11; n >= 0; --n) {
+        d = fma(d, x, v);
+        v = fma(v, x, c[n]);
+    }
+    return v;
+}
+
+// Close electron-proton pair (mixed form, FP64): the e-n Jastrow terms dl (to
+// d ln psi/dR_a) and de (to dE_L/dR_a, given vv = g_i + grad_i U), and the nearest
+// image's phi(r) = erfc(kappa r)/r with its gradient, for d = r_i - R_a.  The pairs
+// are closer than 0.3 bohr, so short series give the trig and the smooth part
+// erf(kappa r)/r: some 170 FP64 operations a pair (450 with the library's sincospi,
+// erfc, exp and divisions).  Cells and splittings outside the series' range
+// (L < 2.1, kappa > 2.5) take the library calls.
+__device__ __forceinline__ void close_pair(const double d[3], double L, double iL, double ell, double kappa, double k2,
+                                           double bep, double Zj, const double vv[3], double& v, double g[3],
+                                           double dl[3], double de[3]) {
+    double m[3], p[3], q[3], s2 = 0, r2 = 0;
+    const bool small = ell > 0.66;      // |pi m / L| <= asin(0.3 / ell) < 1/2
 #pragma unroll
     for (int mu = 0; mu < 3; ++mu) {
-        p[mu] = ell * sd[mu] * cd[mu];
-        q[mu] = cd[mu] * cd[mu] - sd[mu] * sd[mu];
-        t += sd[mu] * sd[mu];
+        m[mu] = d[mu] - L * rint(d[mu] * iL);
+        double sn, cs;
+        if (small) sincos_half(m[mu] * (kPi * iL), sn, cs);
+        else sincospi(m[mu] * iL, &sn, &cs);
+        const double ss = sn * sn;
+        p[mu] = ell * sn * cs;
+        q[mu] = fma(-2.0, ss, 1.0);
+        s2 += ss;
+        r2 += m[mu] * m[mu];
     }
-    t *= ell * ell;
-    const double r = qsqrt_pair(t);
-    double u, u1, u2, u3, f1, f2, f3;
-    pade_ep(bep, Zj, r, u, u1, u2, u3);
-    rho_to_t(r, u1, u2, u3, f1, f2, f3);
-    RadialDerivs<double> rd;
-    radial_chain(p, q, f1, f2, f3, k2, rd);
-    double hv[3];
-    hess_mul(rd.h, vv, hv);
+    double c2, c4, c8;
+    pade_factors3(ell * ell * s2, bep, -Zj, c2, c4, c8);
+    const double pp = p[0] * p[0] + p[1] * p[1] + p[2] * p[2];
+    const double pv = p[0] * vv[0] + p[1] * vv[1] + p[2] * vv[2];
+    const double c0 = fma(c4, pv, 0.5 * fma(c8, pp, fma(c4, q[0] + q[1] + q[2], -k2 * c2)));
 #pragma unroll
-    for (int mu = 0; mu < 3; ++mu) { dl[mu] = -rd.g[mu]; de[mu] = hv[mu] + 0.5 * rd.tl[mu]; }
+    for (int mu = 0; mu < 3; ++mu) {
+        dl[mu] = -c2 * p[mu];
+        de[mu] = fma(p[mu], fma(c4, q[mu], c0), c2 * (q[mu] * vv[mu]));
+    }
+    const double ir = qrsqrt(r2), x = kappa * kappa * r2;
+    double sg;
+    if (kappa <= 2.5 && small) {
+        const double ck = 1.1283791670955126 * kappa;
+        double dx;
+        const double e = ck * erf_over_r_series(x, dx);
+        v = ir - e;
+        sg = -(ir * ir * ir) - 2.0 * ck * kappa * kappa * dx;
+    } else {
+        const double ec = erfc(kappa * (r2 * ir));
+        v = ec * ir;
+        sg = -(ec * ir + 1.1283791670955126 * kappa * exp(-x)) * ir * ir;
+    }
+#pragma unroll
+    for (int mu = 0; mu < 3; ++mu) g[mu] = sg * m[mu];
 }
 
 // e-e-n-n Jastrow orbital chi_a(r_i) = exp(-zeta |d|^2) of electron trig ei and
@@ -606,19 +671,13 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
                 }
                 const double dx = xs[3 * i] - s.R[3 * a], dy = xs[3 * i + 1] - s.R[3 * a + 1],
                              dz = xs[3 * i + 2] - s.R[3 * a + 2];
-                double sdd[3], cdd[3], vv[3], pl[3], pe[3];
-                sincospi(dx * iL, &sdd[0], &cdd[0]);
-                sincospi(dy * iL, &sdd[1], &cdd[1]);
-                sincospi(dz * iL, &sdd[2], &cdd[2]);
+                const double dd[3] = {dx, dy, dz};
+                double vv[3], pl[3], pe[3], pv, pg[3];
                 for (int mu = 0; mu < 3; ++mu) vv[mu] = (double)gi[3 * i + mu] + (double)gU[3 * i + mu];
-                ep_jastrow(sdd, cdd, s.ell, k2d, s.b_ep, s.Zj, vv, pl, pe);
-                const double mx = dx - L * rint(dx * iL), my = dy - L * rint(dy * iL), mz = dz - L * rint(dz * iL);
-                const double r2 = mx * mx + my * my + mz * mz, r = sqrt(r2), ir = 1.0 / r;
-                const double ec = erfc(s.kappa * r);
-                const double sg = -(ec * ir + 1.1283791670955126 * s.kappa * exp(-s.kappa * s.kappa * r2)) * ir * ir;
+                close_pair(dd, L, iL, s.ell, s.kappa, k2d, s.b_ep, s.Zj, vv, pv, pg, pl, pe);
                 double* o = slot + (size_t)(t - base) * 10;
-                o[0] = ec * ir;
-                o[1] = sg * mx; o[2] = sg * my; o[3] = sg * mz;
+                o[0] = pv;
+                o[1] = pg[0]; o[2] = pg[1]; o[3] = pg[2];
                 for (int mu = 0; mu < 3; ++mu) { o[4 + mu] = pl[mu]; o[7 + mu] = pe[mu]; }
             }
             __syncthreads();
