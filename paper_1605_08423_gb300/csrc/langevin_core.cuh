@@ -4,10 +4,10 @@
 // so that all compute the step with the same code.
 //
 // One thread-block cluster of P CTAs (P = 1 for small n) takes the step.  The
-// Cholesky factorisation is blocked: per block column of 32, one warp factors
-// the diagonal tile in registers (shuffles, L D L^T order so that one
-// reciprocal and no square root is on the chain), the rows below are solved
-// against it (a row per lane), and the trailing 32 x 32 tiles are updated by
+// Cholesky factorisation is blocked: per block column of 32, four warps factor
+// the diagonal tile in registers (L D L^T order so that one reciprocal and no
+// square root is on the chain), the rows below are solved against it, four warps
+// a row tile, and the trailing 32 x 32 tiles are updated by
 // all CTAs; the first CTA updates the next diagonal tile first and factors it
 // while the others work on the rest.  The matrix stays in L2 (Lc, read and
 // written with .cg accesses); the cluster barrier orders the phases.
@@ -33,6 +33,7 @@ struct LvSmem {
     double A[kLvTb][kLvTb + 1];   // operand tiles (A also stages a row tile)
     double B[kLvTb][kLvTb + 1];
     double inv[kLvTb];            // reciprocal diagonal of D
+    double col[2][kLvTb];         // column being eliminated of a diagonal tile (alternating)
     double yk[2][kLvTb];          // solved block of up to two right-hand sides
     int fail;                     // set by the first CTA: not positive definite
 };
@@ -51,58 +52,76 @@ __device__ inline void lv_load_diag(int n, const double* Lc, int k, LvSmem& sm) 
         const int r = idx >> 5, c = idx & 31, i = k0 + r, j = k0 + c;
         const double v = (i < n && j <= i) ? __ldcg(Lc + (size_t)i * n + j) : (r == c ? 1.0 : 0.0);
         sm.D[r][c] = v;
-        if (r == c) sm.inv[r] = 1.0 / v;
     }
+    __syncthreads();
+    if (threadIdx.x < kLvTb) sm.inv[threadIdx.x] = 1.0 / sm.D[threadIdx.x][threadIdx.x];
     __syncthreads();
 }
 
-// One warp: Cholesky factor of diagonal tile k in place (lane = row).  Returns
-// false (on every lane) at a pivot that is not positive.
-__device__ inline bool lv_factor_tile(int n, double* Lc, int k) {
-    const int lane = threadIdx.x & 31, k0 = k * kLvTb, row = k0 + lane;
-    double a[kLvTb];
+// Four warps (threads 0-127): Cholesky factor of diagonal tile k in place.  Lane =
+// row, warp q holds columns q, q + 4, ...: the column being eliminated goes through
+// shared memory, one named barrier a column, so that the four FP64 issue ports
+// share the updates (a lone warp issues one FP64 instruction in 64 clocks; one warp
+// for the whole tile took some 50 k clocks).  Returns false on all four warps at a
+// pivot that is not positive.
+__device__ inline bool lv_factor_tile(int n, double* Lc, int k, LvSmem& sm) {
+    constexpr int Q = kLvTb / 4;
+    const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5, k0 = k * kLvTb, row = k0 + lane;
+    double a[Q];
 #pragma unroll
-    for (int c = 0; c < kLvTb; ++c)
-        a[c] = (c <= lane && row < n) ? __ldcg(Lc + (size_t)row * n + k0 + c) : (c == lane ? 1.0 : 0.0);
+    for (int q = 0; q < Q; ++q) {
+        const int c = 4 * q + wq;
+        a[q] = (c <= lane && row < n) ? __ldcg(Lc + (size_t)row * n + k0 + c) : (c == lane ? 1.0 : 0.0);
+    }
     double dl = 1.0;
     bool ok = true;
 #pragma unroll
     for (int c = 0; c < kLvTb; ++c) {
-        const double d = __shfl_sync(0xffffffffu, a[c], c);
+        if (wq == (c & 3)) sm.col[c & 1][lane] = a[c >> 2];
+        asm volatile("bar.sync 1, 128;\n" ::: "memory");
+        const double* col = sm.col[c & 1];
+        const double d = col[c];
         ok = ok && d > 0.0;
         const double y = (d > 1e-280 && d < 1e280) ? qrcp(d) : 1.0 / d;
         if (lane == c) dl = d;
-        const double l = a[c] * y;     // unit-triangular entry; a[c] keeps l d
+        const double l = col[lane] * y;     // unit-triangular entry; the stored column keeps l d
 #pragma unroll
-        for (int j = c + 1; j < kLvTb; ++j) a[j] -= l * __shfl_sync(0xffffffffu, a[c], j);
+        for (int q = 0; q < Q; ++q) {
+            const int j = 4 * q + wq;
+            if (j > c) a[q] -= l * col[j];
+        }
     }
     if (!ok) return false;
     const double rs = 1.0 / sqrt(dl);
 #pragma unroll
-    for (int c = 0; c < kLvTb; ++c) {
-        const double v = a[c] * __shfl_sync(0xffffffffu, rs, c);
+    for (int q = 0; q < Q; ++q) {
+        const int c = 4 * q + wq;
+        const double v = a[q] * __shfl_sync(0xffffffffu, rs, c);
         if (c <= lane && row < n) __stcg(Lc + (size_t)row * n + k0 + c, v);
     }
     return true;
 }
 
-// One warp: row tile I of block column k solved against sm.D, X = A L_kk^-T
-// (lane = row).  st: this warp's staging tile.
-__device__ inline void lv_solve_rows(int n, double* Lc, int k, int I, const LvSmem& sm) {
-    const int lane = threadIdx.x & 31, k0 = k * kLvTb, row = I * kLvTb + lane;
-    if (row >= n) return;
+// Four warps (wq = 0..3 of them): row tile I of block column k solved against sm.D,
+// X = A L_kk^-T; a warp takes 8 rows, its lane 4 r + g row r and columns g, g + 4, ...
+__device__ inline void lv_solve_rows(int n, double* Lc, int k, int I, int wq, const LvSmem& sm) {
+    constexpr int Q = kLvTb / 4;
+    const int lane = threadIdx.x & 31, g = lane & 3, k0 = k * kLvTb, row = I * kLvTb + wq * 8 + (lane >> 2);
     double* p = Lc + (size_t)row * n + k0;
-    double b[kLvTb];
+    double b[Q];
 #pragma unroll
-    for (int c = 0; c < kLvTb; ++c) b[c] = __ldcg(p + c);
+    for (int q = 0; q < Q; ++q) b[q] = row < n ? __ldcg(p + 4 * q + g) : 0.0;
 #pragma unroll
     for (int c = 0; c < kLvTb; ++c) {
-        b[c] *= sm.inv[c];
+        const double x = __shfl_sync(0xffffffffu, b[c >> 2] * sm.inv[c], (lane & 28) | (c & 3));
+        if (g == (c & 3)) b[c >> 2] = x;
 #pragma unroll
-        for (int j = c + 1; j < kLvTb; ++j) b[j] -= b[c] * sm.D[j][c];
+        for (int q = c >> 2; q < Q; ++q)
+            if (4 * q + g > c) b[q] -= x * sm.D[4 * q + g][c];
     }
+    if (row < n)
 #pragma unroll
-    for (int c = 0; c < kLvTb; ++c) __stcg(p + c, b[c]);
+        for (int q = 0; q < Q; ++q) __stcg(p + 4 * q + g, b[q]);
 }
 
 // The CTA: tile (I, J) -= L_Ik L_Jk^T.
@@ -214,21 +233,22 @@ __device__ inline bool lv_cholesky(cg::cluster_group& cl, int n, const double* _
         for (int j = lane; j <= i; j += 32) __stcg(Lc + (size_t)i * n + j, S[(size_t)i * n + j]);
     if (tid == 0) sm.fail = 0;
     cl.sync();
-    if (rank == 0 && warp == 0 && !lv_factor_tile(n, Lc, 0) && lane == 0) sm.fail = 1;
+    if (rank == 0 && warp < 4 && !lv_factor_tile(n, Lc, 0, sm) && tid == 0) sm.fail = 1;
     cl.sync();
     const int* fail = cl.map_shared_rank(&sm.fail, 0);
     for (int k = 0; k < nt; ++k) {
         if (*(volatile const int*)fail) return false;   // written before the last barrier: the same for all
         lv_load_diag(n, Lc, k, sm);
         const int m = nt - 1 - k;                       // row tiles below
-        for (int q = rank + P * warp; q < m; q += P * (kLvThreads / 32)) lv_solve_rows(n, Lc, k, k + 1 + q, sm);
+        for (int q = rank + P * (warp >> 2); q < m; q += P * (kLvThreads / 128))
+            lv_solve_rows(n, Lc, k, k + 1 + q, warp & 3, sm);
         cl.sync();
         // trailing tiles in column order; the first CTA takes (k+1, k+1) and
         // its factorisation (about a tile's time), the others go round
         if (rank == 0 && m > 0) {
             lv_update_tile(n, Lc, k, k + 1, k + 1, sm);
             __syncthreads();
-            if (warp == 0 && !lv_factor_tile(n, Lc, k + 1) && lane == 0) sm.fail = 1;
+            if (warp < 4 && !lv_factor_tile(n, Lc, k + 1, sm) && tid == 0) sm.fail = 1;
         }
         const int total = m * (m + 1) / 2;
         int t = 1, J = 0, base = 0;                      // tile t of column J starts at base
