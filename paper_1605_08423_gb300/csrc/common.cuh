@@ -164,6 +164,26 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
+// Sums of eight values over the warp in nine additions: lane l returns the sum of
+// value (l >> 2) (the halves exchange what the
+// other keeps).  Each value is added up in the order of warp_sum.
+template <typename T>
+__device__ __forceinline__ T warp_sum8(T v[8], int lane) {
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+        const int o = 16 >> s, w = 4 >> s;
+        const bool up = lane & o;
+#pragma unroll
+        for (int k = 0; k < w; ++k) {
+            const T keep = up ? v[k + w] : v[k], give = up ? v[k] : v[k + w];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    T x = v[0];
+    x += __shfl_xor_sync(0xffffffffu, x, 2);
+    x += __shfl_xor_sync(0xffffffffu, x, 1);
+    return x;
+}
 // Deterministic block reduction (fixed tree) of one value per thread; result
 // valid in all threads.  `scratch` holds >= 32 elements.
 template <typename T>

@@ -41,10 +41,12 @@ struct qmc_system {
     float *d_C32 = nullptr, *d_ptrig32 = nullptr;
     int4* d_kvec = nullptr;
     double* d_ewt = nullptr;   // real-space Ewald table (FP64 form)
-    // structure-factor tasks of the measure kernels; reciprocal vectors [3][nk] (FP64 form)
+    // structure-factor tasks of the measure kernels; reciprocal vectors [3][nk] (FP64
+    // form) and their integer vectors (mixed form)
     int nktask = 0;
     int4* d_ktask = nullptr;
     double* d_kxyz = nullptr;
+    float* d_kint = nullptr;
     double2 *d_eikR = nullptr, *d_rhop = nullptr;
     double *d_vconst = nullptr, *d_dvpp = nullptr, *d_vpp = nullptr;
     float *d_R32 = nullptr, *d_kw32 = nullptr, *d_zeta32 = nullptr;
@@ -225,7 +227,7 @@ size_t footprint(const qmc_params* p) {
     const size_t tc = p->n_twist > 0 ? 16 : t;     // complex orbitals of the twisted form
     b += t * W * N + tc * (W * N * n + 2 * W * n * n);   // uacc, Phi, Gt
     if (t == 4 || p->n_twist > 0) b += tc * 4 * W * N * n;   // D, Lp
-    b += 16 * nk + (t == 8 ? 24 * nk : 0);           // structure-factor tasks (at most nk), reciprocal vectors
+    b += 16 * nk + 3 * t * nk;                       // structure-factor tasks (at most nk), reciprocal vectors
     b += 8 * 2 * W + 8 * W * (3 + 9 * N) + 8 * W;   // logdet, acc, nacc
     b += 8 * W + 8 * 5;                              // V_L sums, pressure output
     const size_t Kr = p->n_twist > 0 ? p->n_twist : 1;
@@ -357,7 +359,7 @@ void measure(qmc_system* h, const SysView<float>& s, double* el, double* lnpsi, 
     prof_end(h, ep);
     const bool split = h->use_tc && h->use_tc_adj;
     prof_begin(h, KC_MEASURE, ep);
-    launch_measure(s, h->nktask, h->d_ktask, h->d_X, (const float*)h->d_D, (const float*)h->d_Lp, (const float*)h->d_Gt, h->d_logdet, h->d_acc,
+    launch_measure(s, h->nktask, h->d_ktask, h->d_kint, h->d_X, (const float*)h->d_D, (const float*)h->d_Lp, (const float*)h->d_Gt, h->d_logdet, h->d_acc,
                    el, lnpsi, dl, de, split ? h->d_Kt : nullptr, split ? h->d_eg : nullptr,
                    split ? h->d_elw : nullptr, split ? h->d_rk : nullptr, h->stream);
     prof_end(h, ep);
@@ -698,6 +700,7 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
     }
     std::vector<int4> ktask;
     std::vector<double> kxyz;
+    std::vector<float> kint;
     enumerate_ktask(kv, ktask);
     h->nktask = (int)ktask.size();
     h->d_ktask = dalloc<int4>(h, ktask.size(), &rc);
@@ -708,6 +711,12 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
             kxyz[k] = tp * kv[k].x; kxyz[nk + k] = tp * kv[k].y; kxyz[2 * nk + k] = tp * kv[k].z;
         }
         h->d_kxyz = dalloc<double>(h, kxyz.size(), &rc);
+    } else {
+        kint.resize(3 * (size_t)nk);
+        for (int k = 0; k < nk; ++k) {
+            kint[k] = (float)kv[k].x; kint[nk + k] = (float)kv[k].y; kint[2 * nk + k] = (float)kv[k].z;
+        }
+        h->d_kint = dalloc<float>(h, kint.size(), &rc);
     }
     if (!h->mixed && p->ewald_kappa * p->L <= kEwMaxKL) h->d_ewt = dalloc<double>(h, 2 * kEwNodes * kEwTerms, &rc);
     if (rc != QMC_OK) { qmc_destroy(h); return rc; }
@@ -728,6 +737,7 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
     cudaMemcpyAsync(h->d_zeta32, z32.data(), sizeof(float) * h->G, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(h->d_kvec, kv.data(), sizeof(int4) * nk, cudaMemcpyHostToDevice, st);
     cudaMemcpyAsync(h->d_ktask, ktask.data(), sizeof(int4) * ktask.size(), cudaMemcpyHostToDevice, st);
+    if (h->d_kint) cudaMemcpyAsync(h->d_kint, kint.data(), sizeof(float) * kint.size(), cudaMemcpyHostToDevice, st);
     if (h->d_kxyz)
         cudaMemcpyAsync(h->d_kxyz, kxyz.data(), sizeof(double) * kxyz.size(), cudaMemcpyHostToDevice, st);
     cudaMemsetAsync(h->d_err, 0, sizeof(int), st);

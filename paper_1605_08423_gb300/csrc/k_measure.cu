@@ -18,6 +18,8 @@
 // is assembled later from the per-walker sums accumulated here:
 //   [count, sum E_L, sum E_L^2, sum dlnpsi (3N), sum E_L dlnpsi (3N), sum dE_L (3N)].
 // Every reduction is a fixed-order warp or block tree (bitwise reproducible).
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -26,6 +28,10 @@ namespace qmc {
 namespace {
 
 using T = float;   // working precision of this kernel
+
+// Basis rows per tile of the orbital force products where n <= 32 (64 above): with
+// 4 x 4 outputs a thread 128 rows occupy all 256 threads, 64 rows only half.
+constexpr int kPulayRows = 128;
 
 struct MLayout {
     size_t xs, xt, et, gU, lU, Ui, gi, vv, li, facc, gacc, rhot, red, stage, cmask, uni, total;
@@ -47,18 +53,18 @@ struct MLayout {
         gacc = take(sizeof(T) * 9 * N);
         rhot = take(sizeof(V2<T>) * nk);
         red = take(sizeof(double) * 64);
-        stage = take(split ? 0 : sizeof(double) * 64 * 6);
+        stage = take(split ? 0 : sizeof(double) * kPulayRows * 6);
         cmask = take(sizeof(unsigned) * (size_t)N * ((N + 31) / 32));
         // phase table e^{i m theta}, m = 0..mmax (negative m by conjugation)
         const size_t etab = sizeof(V2<T>) * (size_t)N * 3 * (mmax + 1);
         int np = 4;
         while (np < n) np *= 2;
-        const size_t spin = split ? sizeof(T) * 2 * (size_t)np * (np + 4) : sizeof(T) * (size_t)np * (3 * (np + 4) + 68);
+        const size_t spin = split ? sizeof(T) * 2 * (size_t)np * (np + 4) : sizeof(T) * (size_t)np * (3 * (np + 4) + (np <= 32 ? kPulayRows : 64) + 4);
         // P1 partials: nparts * N <= 256 rows of 5, and (mixed form, N a
         // multiple of 32) the e-e tiles' rows of 5 per electron and partner block
         const size_t jpart = sizeof(T) * 5 * (256 + (size_t)(N / 32) * N);
-        // e-e-n-n Jastrow work space: c [N], S [N][3], 8 warps x 5N
-        const size_t j34 = sizeof(T) * 44 * (size_t)N;
+        // e-e-n-n Jastrow work space: c [N], S [N][3], 8 warps x 5N per electron in hand
+        const size_t j34 = sizeof(T) * (split ? 44 : 84) * (size_t)N;
         size_t u = etab > spin ? etab : spin;
         u = u > j34 ? u : j34;
         uni = take(u > jpart ? u : jpart);
@@ -223,6 +229,19 @@ __device__ __forceinline__ T jas34_orbital(const T* ei, const T* pa, T ell, T ze
     return e;
 }
 
+// Running sum of FP32 terms to FP64-like accuracy without the FP64 pipe: hi + lo,
+// each addition's rounding error kept exactly by Knuth's TwoSum (a conversion and
+// an FP64 addition take 38 clocks of an SM per warp, these seven FP32 ones two).
+struct Sum2 {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float t = __fadd_rn(h, x), z = __fsub_rn(t, h);
+        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(t, z)), __fsub_rn(x, z)));
+        h = t;
+    }
+    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+};
+
 // kSplit: the B x n orbital contractions and their basis-derivative epilogue
 // are left to the tensor-core adjoint kernel; this kernel then writes what
 // that kernel needs: K^T per spin block (kt_out), the electrons' (sin, cos)
@@ -234,7 +253,8 @@ __device__ __forceinline__ T jas34_orbital(const T* ei, const T* pa, T ell, T ze
 // 3.14 ms for 4096 walkers of N = 64, now 1.53 ms.
 template <bool kSplit>
 __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax, int ntask,
-                                                      const int4* __restrict__ ktask, const double* __restrict__ X,
+                                                      const int4* __restrict__ ktask, const T* __restrict__ kint,
+                                                      const double* __restrict__ X,
                                                       const T* __restrict__ D, const T* __restrict__ Lp,
                                                       const T* __restrict__ Gt, const double* __restrict__ logdet,
                                                       double* __restrict__ acc, double* __restrict__ out_el,
@@ -420,74 +440,113 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
 
     // ---- P2: g_i = sum_j D_ij G_ji, l_i = sum_j Lp_ij G_ji (warp per electron,
     // lanes over the orbitals: coalesced rows of D, Lp and G^T)
-    for (int i = warp; i < N; i += nw) {
-        const int sp = i / n, il = i - sp * n;
-        const T* grow = Gt + (((size_t)w * 2 + sp) * n + il) * n;
-        const T* drow = D + ((size_t)w * N + i) * 3 * n;
-        const T* lrow = Lp + ((size_t)w * N + i) * n;
-        T g0 = 0, g1 = 0, g2 = 0, l = 0;
-        for (int j = lane; j < n; j += 32) {
-            const T gj = grow[j];
-            g0 += drow[j] * gj; g1 += drow[n + j] * gj; g2 += drow[2 * n + j] * gj;
-            l += lrow[j] * gj;
+    // Two electrons at a time: twice the loads in flight, and one packed sum.
+    for (int i0 = warp; i0 < N; i0 += 2 * nw) {
+        T v[8] = {};
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int i = i0 + e * nw < N ? i0 + e * nw : i0;
+            const int sp = i / n, il = i - sp * n;
+            const T* grow = Gt + (((size_t)w * 2 + sp) * n + il) * n;
+            const T* drow = D + ((size_t)w * N + i) * 3 * n;
+            const T* lrow = Lp + ((size_t)w * N + i) * n;
+            for (int j = lane; j < n; j += 32) {
+                const T gj = grow[j];
+                v[4 * e] += drow[j] * gj; v[4 * e + 1] += drow[n + j] * gj; v[4 * e + 2] += drow[2 * n + j] * gj;
+                v[4 * e + 3] += lrow[j] * gj;
+            }
         }
-        g0 = warp_sum(g0); g1 = warp_sum(g1); g2 = warp_sum(g2); l = warp_sum(l);
-        if (lane == 0) { gi[3 * i] = g0; gi[3 * i + 1] = g1; gi[3 * i + 2] = g2; li[i] = l; }
+        const T x = warp_sum8(v, lane);
+        const int q = lane >> 2, i = i0 + (q >> 2) * nw, c = q & 3;
+        if ((lane & 3) == 0 && i < N) {
+            if (c < 3) gi[3 * i + c] = x;
+            else li[i] = x;
+        }
     }
     __syncthreads();
 
-    // ---- P2b (FP64 form with the e-e-n-n Jastrow term):
+    // ---- P2b (with the e-e-n-n Jastrow term):
     //   U34 = sum_{i<j} chi_i^T F chi_j = 1/2 sum_i chi_i . w_i,  w_i = F (c - chi_i),  c = sum_j chi_j,
     //   grad_i U34 = sum_a grad chi_a(r_i) w_ia,  lap_i U34 = sum_a lap chi_a(r_i) w_ia,
     // added to grad U, lap U and the per-electron U sums.  c and S_a = sum_j grad chi_a(r_j)
-    // stay in the work space for the force terms after P3.
+    // stay in the work space for the force terms after P3.  The N^3 sums over b are bound
+    // by their loads, so a warp takes several electrons at once: an element of F (global)
+    // and one vector of shared memory serve four (here) or two (P3b) of them.
     T* j34c = (T*)uni;               // [N]
     T* j34S = j34c + N;              // [N][3]
-    T* j34w = j34S + 3 * N;          // per warp: chi_i [N], grad chi_i [N][3], lap chi_i [N]
-    {
-        if (s.fjt) {
-            const T zj = (T)s.zeta_j;
-            for (int a = tid; a < N; a += nt) {
-                T c = 0, g[3] = {0, 0, 0};
-                for (int j = 0; j < N; ++j) {
-                    RadialDerivs<T> rd;
-                    c += jas34_orbital(et + 6 * j, s.ptrig + 6 * a, ell, zj, k2, rd);
-                    for (int mu = 0; mu < 3; ++mu) g[mu] += rd.g[mu];
-                }
-                j34c[a] = c;
-                for (int mu = 0; mu < 3; ++mu) j34S[3 * a + mu] = g[mu];
+    T* j34w = j34S + 3 * N;          // per warp: here c - chi_i of up to four electrons; P3b below
+    if (s.fjt) {
+        const T zj = (T)s.zeta_j;
+        // c and S, the electrons in nparts slices (partials in the warps' work space), summed in order
+        for (int tt = tid; tt < nparts * N; tt += nt) {
+            const int a = tt % N, pi = tt / N, j0 = (N * pi) / nparts, j1 = (N * (pi + 1)) / nparts;
+            T c = 0, g[3] = {0, 0, 0};
+            for (int j = j0; j < j1; ++j) {
+                RadialDerivs<T> rd;
+                c += jas34_orbital(et + 6 * j, s.ptrig + 6 * a, ell, zj, k2, rd);
+                for (int mu = 0; mu < 3; ++mu) g[mu] += rd.g[mu];
             }
-            __syncthreads();
-            T* stc = j34w + (size_t)warp * 5 * N;
-            for (int i = warp; i < N; i += nw) {
-                for (int a = lane; a < N; a += 32) {
-                    RadialDerivs<T> rd;
-                    stc[a] = jas34_orbital(et + 6 * i, s.ptrig + 6 * a, ell, zj, k2, rd);
-                }
-                __syncwarp();
-                T g[3] = {0, 0, 0}, l = 0, u = 0;
-                for (int a = lane; a < N; a += 32) {
-                    RadialDerivs<T> rd;
-                    const T chi = jas34_orbital(et + 6 * i, s.ptrig + 6 * a, ell, zj, k2, rd);
-                    const T* fa = s.fjt + a;   // column a = row a (f symmetric): coalesced over lanes
-                    T w = 0;
-                    for (int b = 0; b < N; ++b) w += fa[(size_t)b * N] * (j34c[b] - stc[b]);
-                    for (int mu = 0; mu < 3; ++mu) g[mu] += rd.g[mu] * w;
-                    l += rd.lap * w;
-                    u += chi * w;
-                }
-                for (int mu = 0; mu < 3; ++mu) g[mu] = warp_sum(g[mu]);
-                l = warp_sum(l);
-                u = warp_sum(u);
-                if (lane == 0) {
-                    for (int mu = 0; mu < 3; ++mu) gU[3 * i + mu] += g[mu];
-                    lU[i] += l;
-                    Ui[i] += T(0.5) * u;
-                }
-                __syncwarp();
-            }
-            __syncthreads();
+            T* o = j34w + 4 * (size_t)tt;
+            o[0] = c; o[1] = g[0]; o[2] = g[1]; o[3] = g[2];
         }
+        __syncthreads();
+        for (int idx = tid; idx < 4 * N; idx += nt) {
+            T v = 0;
+            for (int pi = 0; pi < nparts; ++pi) v += j34w[4 * (size_t)pi * N + idx];
+            if (idx & 3) j34S[3 * (idx >> 2) + (idx & 3) - 1] = v;
+            else j34c[idx >> 2] = v;
+        }
+        __syncthreads();
+        float4* d4 = (float4*)(j34w + (size_t)warp * 4 * N);     // c_b - chi_b(r_i) of four electrons
+        for (int i0 = 4 * warp; i0 < N; i0 += 4 * nw) {
+            const int ne = N - i0 < 4 ? N - i0 : 4;
+            for (int b = lane; b < N; b += 32) {
+                T d[4] = {0, 0, 0, 0};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (e < ne) {
+                        T sd[3], cd[3], t;
+                        disp_trig(et + 6 * (i0 + e), s.ptrig + 6 * b, ell, sd, cd, t);
+                        d[e] = j34c[b] - qexp(-zj * t);
+                    }
+                d4[b] = make_float4(d[0], d[1], d[2], d[3]);
+            }
+            __syncwarp();
+            T acc[4][5] = {};
+            for (int a = lane; a < N; a += 32) {
+                const T* fa = s.fjt + a;   // column a = row a (f symmetric): coalesced over lanes
+                T wv[4] = {0, 0, 0, 0};
+#pragma unroll 4
+                for (int b = 0; b < N; ++b) {
+                    const T f = fa[(size_t)b * N];
+                    const float4 d = d4[b];
+                    wv[0] += f * d.x; wv[1] += f * d.y; wv[2] += f * d.z; wv[3] += f * d.w;
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (e < ne) {
+                        RadialDerivs<T> rd;
+                        const T chi = jas34_orbital(et + 6 * (i0 + e), s.ptrig + 6 * a, ell, zj, k2, rd);
+                        for (int mu = 0; mu < 3; ++mu) acc[e][mu] += rd.g[mu] * wv[e];
+                        acc[e][3] += rd.lap * wv[e];
+                        acc[e][4] += chi * wv[e];
+                    }
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (e < ne) {
+#pragma unroll
+                    for (int c = 0; c < 5; ++c) acc[e][c] = warp_sum(acc[e][c]);
+                    if (lane == 0) {
+                        const int i = i0 + e;
+                        for (int mu = 0; mu < 3; ++mu) gU[3 * i + mu] += acc[e][mu];
+                        lU[i] += acc[e][3];
+                        Ui[i] += T(0.5) * acc[e][4];
+                    }
+                }
+            __syncwarp();
+        }
+        __syncthreads();
     }
 
     // ---- P3: kinetic energy and U
@@ -513,45 +572,64 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
     //   dE_L/dR_a   += sum_i [ 1/2 (grad lap chi_a(r_i) w_ia + lam_ia s_a^(i))
     //                          + (Hess chi_a(r_i) vv_i) w_ia + (vv_i . v_ia) s_a^(i) ]
     // (the R_a-derivative of -1/2 sum_i [lap_i U34 + 2 vv_i . grad_i U34]).
-    {
-        if (s.fjt) {
-            const T zj = (T)s.zeta_j;
-            T* st = j34w + (size_t)warp * 5 * N;   // chi_i [N], grad chi_i [N][3], lap chi_i [N]
-            for (int i = warp; i < N; i += nw) {
-                for (int a = lane; a < N; a += 32) {
-                    RadialDerivs<T> rd;
-                    st[a] = jas34_orbital(et + 6 * i, s.ptrig + 6 * a, ell, zj, k2, rd);
-                    for (int mu = 0; mu < 3; ++mu) st[N + 3 * a + mu] = rd.g[mu];
-                    st[4 * N + a] = rd.lap;
-                }
+    if (s.fjt) {
+        constexpr int EW = kSplit ? 1 : 2;   // electrons a warp has in hand (shared memory: the split form keeps 3 CTAs)
+        const T zj = (T)s.zeta_j;
+        // per warp and electron: (grad chi_b, lap chi_b) [N], c_b - chi_b [N]
+        float4* gl4 = (float4*)(j34w + (size_t)warp * 5 * EW * N);
+        T* df = (T*)(gl4 + EW * N);
+        for (int ac = 0; ac < N; ac += 32) {     // a lane's nucleus keeps its sums over the warp's electrons
+            const int a = ac + lane < N ? ac + lane : N - 1;
+            Sum2 dl[3], de[3];
+            for (int i0 = EW * warp; i0 < N; i0 += EW * nw) {
                 __syncwarp();
-                T vv[3];
-                for (int mu = 0; mu < 3; ++mu) vv[mu] = gi[3 * i + mu] + gU[3 * i + mu];
-                for (int a = lane; a < N; a += 32) {
+                for (int b = lane; b < N; b += 32)
+#pragma unroll
+                    for (int e = 0; e < EW; ++e) {
+                        const int i = i0 + e < N ? i0 + e : N - 1;
+                        RadialDerivs<T> rd;
+                        df[e * N + b] = j34c[b] - jas34_orbital(et + 6 * i, s.ptrig + 6 * b, ell, zj, k2, rd);
+                        gl4[e * N + b] = make_float4(rd.g[0], rd.g[1], rd.g[2], rd.lap);
+                    }
+                __syncwarp();
+                const T* fa = s.fjt + a;   // column a = row a (f symmetric): coalesced over lanes
+                T wv[EW] = {}, v[EW][4] = {};
+#pragma unroll 2
+                for (int b = 0; b < N; ++b) {
+                    const T f = fa[(size_t)b * N];
+#pragma unroll
+                    for (int e = 0; e < EW; ++e) {
+                        const float4 q = gl4[e * N + b];
+                        wv[e] += f * df[e * N + b];
+                        v[e][0] += q.x * f; v[e][1] += q.y * f; v[e][2] += q.z * f; v[e][3] += q.w * f;
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < EW; ++e) {
+                    const int i = i0 + e;
+                    if (i >= N) continue;
                     RadialDerivs<T> rd;
                     jas34_orbital(et + 6 * i, s.ptrig + 6 * a, ell, zj, k2, rd);
-                    const T* fa = s.fjt + a;   // column a = row a (f symmetric): coalesced over lanes
-                    T w = 0, v[3] = {0, 0, 0}, lam = 0;
-                    for (int b = 0; b < N; ++b) {
-                        const T f = fa[(size_t)b * N];
-                        w += f * (j34c[b] - st[b]);
-                        for (int mu = 0; mu < 3; ++mu) v[mu] += st[N + 3 * b + mu] * f;
-                        lam += st[4 * N + b] * f;
-                    }
-                    T hv[3];
+                    T vv[3], hv[3];
+                    for (int mu = 0; mu < 3; ++mu) vv[mu] = vvs[3 * i + mu];
                     hess_mul(rd.h, vv, hv);
-                    const T vvv = vv[0] * v[0] + vv[1] * v[1] + vv[2] * v[2];
+                    const T vvv = vv[0] * v[e][0] + vv[1] * v[e][1] + vv[2] * v[e][2];
+#pragma unroll
                     for (int mu = 0; mu < 3; ++mu) {
                         const T sa = j34S[3 * a + mu] - rd.g[mu];
-                        atomicAdd(&f_dl[3 * a + mu], (double)(-rd.g[mu] * w));
-                        atomicAdd(&f_de[3 * a + mu],
-                                  (double)(T(0.5) * (rd.tl[mu] * w + lam * sa) + hv[mu] * w + vvv * sa));
+                        dl[mu].add(-rd.g[mu] * wv[e]);
+                        de[mu].add(T(0.5) * (rd.tl[mu] * wv[e] + v[e][3] * sa) + hv[mu] * wv[e] + vvv * sa);
                     }
                 }
-                __syncwarp();
             }
-            __syncthreads();
+            if (ac + lane < N)
+#pragma unroll
+                for (int mu = 0; mu < 3; ++mu) {
+                    atomicAdd(&f_dl[3 * a + mu], dl[mu].value());
+                    atomicAdd(&f_de[3 * a + mu], de[mu].value());
+                }
         }
+        __syncthreads();
     }
 
     // ---- P4a: electron-electron real-space Ewald
@@ -609,15 +687,20 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
             v += ewald_real_cut<true>(xt[3 * i] - ra[0], xt[3 * i + 1] - ra[1], xt[3 * i + 2] - ra[2], close, fast, Lt,
                                       iLt, rc2, kap, gv);
         }
-        v = warp_sum(v);
-#pragma unroll
-        for (int mu = 0; mu < 3; ++mu) { gv[mu] = warp_sum(gv[mu]); dl[mu] = warp_sum(dl[mu]); de[mu] = warp_sum(de[mu]); }
-        if (lane == 0) {   // FP32 partials; FP64 only where the sample is accumulated
-            vep_t += -(T)Zn * v;
-            for (int mu = 0; mu < 3; ++mu) {
-                g_dv[3 * a + mu] = (T)Zn * gv[mu];
-                g_dl[3 * a + mu] = dl[mu];
-                g_de[3 * a + mu] = de[mu];
+        T r[8] = {v, gv[0], gv[1], gv[2], dl[0], dl[1], dl[2], de[0]};
+        const T x = warp_sum8(r, lane), d1 = warp_sum(de[1]), d2 = warp_sum(de[2]);
+        const int q = lane >> 2;
+        if ((lane & 3) == 0) {   // FP32 partials; FP64 only where the sample is accumulated
+            if (q == 0) {
+                vep_t += -(T)Zn * x;
+                g_de[3 * a + 1] = d1;
+                g_de[3 * a + 2] = d2;
+            } else if (q < 4) {
+                g_dv[3 * a + q - 1] = (T)Zn * x;
+            } else if (q < 7) {
+                g_dl[3 * a + q - 4] = x;
+            } else {
+                g_de[3 * a] = x;
             }
         }
     }
@@ -746,12 +829,15 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
                 const T im = sg ? q[h][3] - q[h][2] : q[h][3] + q[h][2];
                 const double2 rp = s.rho_p[k];
                 const T rr = (T)rp.x - re, ri = (T)rp.y - im;   // electrons carry -1
-                rhot[k] = V2<T>{rr, ri};
-                if constexpr (kSplit) {
+                const T kw = s.kwt[k];
+                if constexpr (!kSplit) {          // proton charge 1
+                    const T f = T(2) * kw * twopiL;
+                    rhot[k] = V2<T>{f * rr, f * ri};
+                } else {
                     rk_out[(size_t)w * 2 * nk + 2 * k] = (float)rr;
                     rk_out[(size_t)w * 2 * nk + 2 * k + 1] = (float)ri;
                 }
-                vrec_t += s.kwt[k] * (rr * rr + ri * ri);
+                vrec_t += kw * (rr * rr + ri * ri);
             }
         }
     }
@@ -759,18 +845,32 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
     __syncthreads();
     // ---- P4d: reciprocal-space force on the protons (warp per proton; the
     // split path leaves it to the GEMM)
-    for (int a = warp; a < (kSplit ? 0 : N); a += nw) {
-        T gx = 0, gy = 0, gz = 0;
-#pragma unroll 4
-        for (int k = lane; k < nk; k += 32) {
-            const V2<T> e = s.eikRt[(size_t)a * nk + k];
-            const V2<T> rd = rhot[k];
-            const T c = T(2) * (T)Zn * s.kwt[k] * (rd.y * e.x - rd.x * e.y);
-            const int4 m = s.kvec[k];
-            gx += c * twopiL * (T)m.x; gy += c * twopiL * (T)m.y; gz += c * twopiL * (T)m.z;
+    if constexpr (!kSplit) {
+        // four protons at a time share the loads of rho(k) (scaled by 2 w_k 2 pi / L
+        // above) and of the integer vectors
+        for (int a0 = 4 * warp; a0 < N; a0 += 4 * nw) {
+            T gx[4] = {}, gy[4] = {}, gz[4] = {};
+#pragma unroll 2
+            for (int k = lane; k < nk; k += 32) {
+                const V2<T> rd = rhot[k];
+                const T mx = kint[k], my = kint[nk + k], mz = kint[2 * nk + k];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int a = a0 + q < N ? a0 + q : N - 1;
+                    const V2<T> e = s.eikRt[(size_t)a * nk + k];
+                    const T c = rd.y * e.x - rd.x * e.y;
+                    gx[q] += c * mx; gy[q] += c * my; gz[q] += c * mz;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                gx[q] = warp_sum(gx[q]); gy[q] = warp_sum(gy[q]); gz[q] = warp_sum(gz[q]);
+                if (lane == 0 && a0 + q < N) {
+                    const int a = a0 + q;
+                    g_dv[3 * a] += gx[q]; g_dv[3 * a + 1] += gy[q]; g_dv[3 * a + 2] += gz[q];
+                }
+            }
         }
-        gx = warp_sum(gx); gy = warp_sum(gy); gz = warp_sum(gz);
-        if (lane == 0) { g_dv[3 * a] += gx; g_dv[3 * a + 1] += gy; g_dv[3 * a + 2] += gz; }
     }
     vep_p += (double)vep_t;
     const double vee = block_sum(vee_p, red);
@@ -780,9 +880,9 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
     __syncthreads();
 
     // ---- P6: orbital (Pulay) terms, one spin block at a time.  All n x n and
-    // B x n products are register-tiled 4 x 4 per thread on a zero-padded
-    // np x np block (np = padded n, a power of two >= 4):
-    //   M1 = Y G,  K = G M1  (= G Y G),  Z = C G,  P = C K  (per 64-row tile of C)
+    // B x n products are register-tiled on a zero-padded np x np block (np =
+    // padded n, a power of two >= 4):
+    //   M1 = Y G,  K = G M1  (= G Y G),  Z = C G,  P = C K  (per tile of C rows)
     // and the basis-derivative contraction is fused onto each Z/P tile.
     const int np = s.np, ldt = np + 4, ng = np / 4;
     const int lnp = __ffs(np) - 1;   // np is a power of two: index arithmetic by shifts (no integer division)
@@ -861,10 +961,47 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
             __syncthreads();
         }
     } else {
+    // Rows of C per tile and its stride; the n x n products take 2 x 2 outputs a
+    // thread up to n = 32 (256 threads busy; 4 x 4 keeps 64) and 4 x 4 above.  Every
+    // sum runs over j in order, whatever the tiling.
+    const int RB = np <= 32 ? kPulayRows : 64, ldc = RB + 4;
     T* bufA = (T*)uni;                       // Y^T [j][i], later K [j][i]
     T* bufG = bufA + (size_t)np * ldt;       // G   [j][i] = G_{j,i}
-    T* bufS = bufG + (size_t)np * ldt;       // G^T [i][j], later C^T tile [j][b] (stride 68)
-    T* bufM = bufS + (size_t)np * 68;        // M1  [i][i']
+    T* bufM = bufG + (size_t)np * ldt;       // M1  [i][i']
+    T* bufS = bufM + (size_t)np * ldt;       // G^T [i][j], later C^T tile [j][b] (stride ldc)
+    // out[r][c] = sum_j A[j][r] B[j][c] for TT x TT outputs a thread
+    auto square = [&](const T* A, const T* Bm, T* out, auto tile) {
+        constexpr int TT = decltype(tile)::value;
+        const int ngt = np / TT;
+        T acc[TT][TT] = {};
+        const int r0 = TT * (tid / ngt), c0 = TT * (tid % ngt);
+        const bool on = tid < ngt * ngt;
+        if (on)
+            for (int j = 0; j < np; ++j) {
+                T av[TT], bv[TT];
+                if constexpr (TT == 4) {
+                    load4(A + j * ldt + r0, av);
+                    load4(Bm + j * ldt + c0, bv);
+                } else {
+                    const float2 a2 = *(const float2*)(A + j * ldt + r0), b2 = *(const float2*)(Bm + j * ldt + c0);
+                    av[0] = a2.x; av[1] = a2.y; bv[0] = b2.x; bv[1] = b2.y;
+                }
+#pragma unroll
+                for (int a_ = 0; a_ < TT; ++a_)
+#pragma unroll
+                    for (int b_ = 0; b_ < TT; ++b_) acc[a_][b_] += av[a_] * bv[b_];
+            }
+        if (on)
+#pragma unroll
+            for (int a_ = 0; a_ < TT; ++a_)
+#pragma unroll
+                for (int b_ = 0; b_ < TT; ++b_) out[(r0 + a_) * ldt + c0 + b_] = acc[a_][b_];
+        __syncthreads();
+    };
+    auto product = [&](const T* A, const T* Bm, T* out) {
+        if (np <= 32) square(A, Bm, out, std::integral_constant<int, 2>{});
+        else square(A, Bm, out, std::integral_constant<int, 4>{});
+    };
     for (int sp = 0; sp < 2; ++sp) {
         const T* Gsp = Gt + ((size_t)w * 2 + sp) * n * n;
         for (int idx = tid; idx < np * np; idx += nt) {
@@ -882,56 +1019,22 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
             bufA[j * ldt + il] = y;
         }
         __syncthreads();
-        if (tid < ng * ng) {                     // M1[i][i'] = sum_j Y[i][j] G[j][i']
-            const int r0 = 4 * (tid / ng), c0 = 4 * (tid % ng);
-            T acc4[4][4] = {};
-            for (int j = 0; j < np; ++j) {
-                T y4[4], g4[4];
-                load4(bufA + j * ldt + r0, y4);
-                load4(bufG + j * ldt + c0, g4);
-#pragma unroll
-                for (int a_ = 0; a_ < 4; ++a_)
-#pragma unroll
-                    for (int b_ = 0; b_ < 4; ++b_) acc4[a_][b_] += y4[a_] * g4[b_];
-            }
-#pragma unroll
-            for (int a_ = 0; a_ < 4; ++a_)
-#pragma unroll
-                for (int b_ = 0; b_ < 4; ++b_) bufM[(r0 + a_) * ldt + c0 + b_] = acc4[a_][b_];
-        }
-        __syncthreads();
-        if (tid < ng * ng) {                     // K[j][i'] = sum_i G[j][i] M1[i][i']
-            const int r0 = 4 * (tid / ng), c0 = 4 * (tid % ng);
-            T acc4[4][4] = {};
-            for (int i = 0; i < np; ++i) {
-                T g4[4], m4[4];
-                load4(bufS + i * ldt + r0, g4);
-                load4(bufM + i * ldt + c0, m4);
-#pragma unroll
-                for (int a_ = 0; a_ < 4; ++a_)
-#pragma unroll
-                    for (int b_ = 0; b_ < 4; ++b_) acc4[a_][b_] += g4[a_] * m4[b_];
-            }
-#pragma unroll
-            for (int a_ = 0; a_ < 4; ++a_)
-#pragma unroll
-                for (int b_ = 0; b_ < 4; ++b_) bufA[(r0 + a_) * ldt + c0 + b_] = acc4[a_][b_];
-        }
-        __syncthreads();
+        product(bufA, bufG, bufM);               // M1[i][i'] = sum_j Y[i][j] G[j][i']
+        product(bufS, bufM, bufA);               // K[j][i'] = sum_i G[j][i] M1[i][i']
         const int B = s.B;
-        for (int b0 = 0; b0 < B; b0 += 64) {
-            for (int idx = tid; idx < 64 * np; idx += nt) {   // C^T tile
+        for (int b0 = 0; b0 < B; b0 += RB) {
+            for (int idx = tid; idx < RB * np; idx += nt) {   // C^T tile
                 const int bl = idx >> lnp, j = idx & (np - 1);
-                bufS[j * 68 + bl] = (b0 + bl < B && j < n) ? s.C[(size_t)(b0 + bl) * n + j] : T(0);
+                bufS[j * ldc + bl] = (b0 + bl < B && j < n) ? s.C[(size_t)(b0 + bl) * n + j] : T(0);
             }
             __syncthreads();
-            const bool act = tid < 16 * ng;
             const int bg = tid / ng, ig = tid % ng;
+            const bool act = bg < RB / 4 && b0 + 4 * bg < B;
             T z4[4][4] = {}, p4[4][4] = {};
             if (act) {
                 for (int j = 0; j < np; ++j) {
                     T c4[4], g4[4], k4[4];
-                    load4(bufS + j * 68 + 4 * bg, c4);
+                    load4(bufS + j * ldc + 4 * bg, c4);
                     load4(bufG + j * ldt + 4 * ig, g4);
                     load4(bufA + j * ldt + 4 * ig, k4);
 #pragma unroll
@@ -949,7 +1052,7 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
             //   grad lap chi = p o (8 f''' |p|^2 + 4 f'' sum q - 2 k^2 f' + 8 f'' q),
             // so the geometry (p, q, p.gU, q o gU) is computed once per
             // (nucleus, electron) and shared by that nucleus' Gaussians.
-            T fl[4][3] = {}, fe[4][3] = {};
+            T f[24] = {};   // per basis function of the thread: dl (3), de (3)
 #pragma unroll
             for (int ii = 0; ii < 4; ++ii) {
                 const int il = 4 * ig + ii;
@@ -990,29 +1093,39 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
 #pragma unroll
                     for (int mu = 0; mu < 3; ++mu) {
                         // dl -= zb grad chi;  de += pb grad chi + zb (H gU + 1/2 grad lap chi)
-                        fl[bb][mu] -= zb * g1 * pv[mu];
-                        fe[bb][mu] += cp * pv[mu] + cq * qg[mu] + hz * pv[mu] * (A + T(8) * f2 * qv[mu]);
+                        f[6 * bb + mu] -= zb * g1 * pv[mu];
+                        f[6 * bb + 3 + mu] += cp * pv[mu] + cq * qg[mu] + hz * pv[mu] * (A + T(8) * f2 * qv[mu]);
                     }
                 }
             }
-            // reduce over the ng threads that share these four basis functions
+            // Reduce over the ng threads that share these four basis functions: at each
+            // step the pair of threads splits the values between them while they divide
+            // (21 exchanges for the 72 of whole values), in the order 1, 2, 4, 8.
+            int base = 0;
+            auto halve = [&](auto cnt, int o) {
+                constexpr int H = decltype(cnt)::value;
+                const bool up = ig & o;
 #pragma unroll
-            for (int bb = 0; bb < 4; ++bb)
+                for (int k = 0; k < H; ++k) {
+                    const T keep = up ? f[k + H] : f[k], give = up ? f[k] : f[k + H];
+                    f[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                }
+                base += up ? H : 0;
+            };
+            int left = 24;
+            if (ng > 1) { halve(std::integral_constant<int, 12>{}, 1); left = 12; }
+            if (ng > 2) { halve(std::integral_constant<int, 6>{}, 2); left = 6; }
+            if (ng > 4) { halve(std::integral_constant<int, 3>{}, 4); left = 3; }
+            if (ng > 8)
 #pragma unroll
-                for (int mu = 0; mu < 3; ++mu)
-                    for (int o = 1; o < ng; o <<= 1) {
-                        fl[bb][mu] += __shfl_xor_sync(0xffffffffu, fl[bb][mu], o);
-                        fe[bb][mu] += __shfl_xor_sync(0xffffffffu, fe[bb][mu], o);
-                    }
-            if (act && ig == 0)
-                for (int bb = 0; bb < 4; ++bb)
-                    for (int mu = 0; mu < 3; ++mu) {
-                        stage[(4 * bg + bb) * 6 + mu] = (double)fl[bb][mu];
-                        stage[(4 * bg + bb) * 6 + 3 + mu] = (double)fe[bb][mu];
-                    }
+                for (int k = 0; k < 3; ++k) f[k] += __shfl_xor_sync(0xffffffffu, f[k], 8);
+            if (act && ig < 8)
+#pragma unroll
+                for (int k = 0; k < 24; ++k)
+                    if (k < left) stage[24 * bg + base + k] = (double)f[k];
             __syncthreads();
             {   // one thread per nucleus of this tile sums its basis functions in order
-                const int bend = (b0 + 64 < B) ? b0 + 64 : B;
+                const int bend = (b0 + RB < B) ? b0 + RB : B;
                 const int a_first = b0 / G, a_last = (bend - 1) / G;
                 const int a = a_first + tid;
                 if (a <= a_last) {
@@ -1062,7 +1175,8 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
 
 }  // namespace
 
-void launch_measure(const SysView<float>& s, int ntask, const int4* ktask, const double* X, const float* D, const float* Lp, const float* Gt,
+void launch_measure(const SysView<float>& s, int ntask, const int4* ktask, const float* kint,
+                    const double* X, const float* D, const float* Lp, const float* Gt,
                     const double* logdet, double* acc, double* out_el, double* out_lnpsi, double* out_dl,
                     double* out_de, float* kt_out, float* eg_out, double* elw, float* rk_out, cudaStream_t st) {
     const bool split = kt_out != nullptr;
@@ -1076,10 +1190,10 @@ void launch_measure(const SysView<float>& s, int ntask, const int4* ktask, const
         attr_set[split] = true;
     }
     if (split)
-        measure_kernel<true><<<s.W, 256, smem, st>>>(s, s.mmax, ntask, ktask, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
+        measure_kernel<true><<<s.W, 256, smem, st>>>(s, s.mmax, ntask, ktask, kint, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
                                                      out_de, kt_out, eg_out, elw, rk_out);
     else
-        measure_kernel<false><<<s.W, 256, smem, st>>>(s, s.mmax, ntask, ktask, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
+        measure_kernel<false><<<s.W, 256, smem, st>>>(s, s.mmax, ntask, ktask, kint, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
                                                       out_de, nullptr, nullptr, nullptr, nullptr);
 }
 

@@ -89,26 +89,7 @@ __device__ __forceinline__ Geo geometry(const double* e, const double* a, double
     return g;
 }
 
-// Sums of eight values over the warp in nine additions: lane l returns the sum of
-// value (l >> 2) (the halves exchange what the other keeps).
-__device__ __forceinline__ double warp_sum8(double v[8], int lane) {
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-        const int o = 16 >> s, w = 4 >> s;
-        const bool up = lane & o;
-#pragma unroll
-        for (int k = 0; k < w; ++k) {
-            const double keep = up ? v[k + w] : v[k], give = up ? v[k] : v[k + w];
-            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-        }
-    }
-    double x = v[0];
-    x += __shfl_xor_sync(0xffffffffu, x, 2);
-    x += __shfl_xor_sync(0xffffffffu, x, 1);
-    return x;
-}
-// The same within segments of seg < 32 lanes (a power of two), plain: lane l of a
-// segment returns the sum of value min(l, 7)... for seg < 8 the caller loops.
+// Sums of nv values within segments of seg < 32 lanes (a power of two).
 __device__ __forceinline__ void seg_sum(double* v, int nv, int seg) {
     for (int k = 0; k < nv; ++k)
         for (int o = seg >> 1; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
