@@ -98,16 +98,13 @@ struct qmc_system {
     uint32_t langevin_step_no = 0;
     double last_Nc = 0.0;
     // twisted boundary conditions (FP64 form): K twists, walker blocks of W/K;
-    // the twist vectors and their phase table; (Re g, Re l) of every electron
-    // for the FP64 measure kernel; E_L and ln|psi| per walker; the per-twist
-    // results before the average
+    // the twist vectors and their phase table; the per-twist results before the average
     int K = 0;
     TwistView tv{};
     std::vector<double> twist_h;
     double* d_theta = nullptr;
     double2* d_tph = nullptr;
-    double* d_gl = nullptr;
-    double *d_elt = nullptr, *d_lpt = nullptr, *d_tout = nullptr;
+    double* d_tout = nullptr;
     long long nlaunch = 0;  // kernels launched by this handle
     bool profiling = false;
     std::vector<EventPair> events, free_events;
@@ -226,7 +223,7 @@ size_t footprint(const qmc_params* p) {
     b += t * W * N;                                  // carried e-n Jastrow sums of the sweep
     const size_t tc = p->n_twist > 0 ? 16 : t;     // complex orbitals of the twisted form
     b += t * W * N + tc * (W * N * n + 2 * W * n * n);   // uacc, Phi, Gt
-    if (t == 4 || p->n_twist > 0) b += tc * 4 * W * N * n;   // D, Lp
+    if (t == 4) b += tc * 4 * W * N * n;             // D, Lp
     b += 16 * nk + 3 * t * nk;                       // structure-factor tasks (at most nk), reciprocal vectors
     b += 8 * 2 * W + 8 * W * (3 + 9 * N) + 8 * W;   // logdet, acc, nacc
     b += 8 * W + 8 * 5;                              // V_L sums, pressure output
@@ -239,10 +236,9 @@ size_t footprint(const qmc_params* p) {
     if (t == 8) b += 8 * 2 * kEwNodes * kEwTerms;    // real-space Ewald table
     if (p->fj) b += (t == 4 ? 12 : 8) * N * N;       // e-e-n-n Jastrow coefficients (+ FP32 copy)
     if (p->n_twist > 0) {
-        // twists, phase table, Re g and Re l, E_L and ln|psi|, per-twist results
+        // twists, phase table, per-twist results
         const size_t K = p->n_twist, M = bloch_images(p);
-        b += 8 * 3 * K + 16 * 3 * K * (2 * M + 1) + 8 * W * N * 4 + 8 * 2 * W +
-             8 * K * (4 + 3 * N + 9 * N * N);
+        b += 8 * 3 * K + 16 * 3 * K * (2 * M + 1) + 8 * K * (4 + 3 * N + 9 * N * N);
     }
     b += (size_t)kPoolAllocs * kPoolAlign;           // alignment slack of a carved handle
     if (t == 4) {                                    // tensor-core operands (mixed form)
@@ -380,7 +376,7 @@ void measure(qmc_system* h, const SysView<double>& s, double* el, double* lnpsi,
     EventPair ep;
     h->nlaunch += 1;
     prof_begin(h, KC_MEASURE, ep);
-    launch_measure64(s, h->nktask, h->d_ktask, h->d_kxyz, h->d_X, (const double*)h->d_Gt, nullptr, h->d_logdet, h->d_acc,
+    launch_measure64(s, nullptr, h->nktask, h->d_ktask, h->d_kxyz, h->d_X, (const double*)h->d_Gt, h->d_logdet, h->d_acc,
                      el, lnpsi, dl, de, h->stream);
     prof_end(h, ep);
 }
@@ -435,34 +431,19 @@ void recompute_twist(qmc_system* h, int W) {
     prof_begin(h, KC_RECOMPUTE, ep);
     SysView<double> s = view<double>(h, W);
     h->nlaunch += 2;
-    launch_twist_orbitals(s, h->tv, h->d_X, W * h->N, (double2*)h->d_Phi, nullptr, nullptr, h->stream);
+    launch_twist_orbitals(s, h->tv, h->d_X, W * h->N, (double2*)h->d_Phi, h->stream);
     launch_twist_invert(W, h->N, h->n, (const double2*)h->d_Phi, (double2*)h->d_Gt, h->d_logdet, h->d_err, h->stream);
     prof_end(h, ep);
 }
 
-// Local energy and force sample of every walker: complex orbital rows; Re g and
-// Re l; the FP64 measure kernel on them (E_L = Re(H psi / psi), the Jastrow and
-// Ewald force terms with vv = Re g + grad U); then the complex orbital (Pulay)
-// force terms.
+// Local energy and force sample of every walker from the complex inverses (real
+// parts of the estimators).
 void measure_twist(qmc_system* h, int W, double* el, double* lnpsi, double* dl, double* de) {
-    SysView<double> s = view<double>(h, W);
-    const int N = h->N, n = h->n;
     EventPair ep;
-    h->nlaunch += 4;
-    prof_begin(h, KC_ORB_MEAS, ep);
-    launch_twist_orbitals(s, h->tv, h->d_X, W * N, (double2*)h->d_Phi, (double2*)h->d_D, (double2*)h->d_Lp,
-                          h->stream);
-    launch_twist_gl(W * N, N, n, (const double2*)h->d_D, (const double2*)h->d_Lp, (const double2*)h->d_Gt, h->d_gl,
-                    h->stream);
-    prof_end(h, ep);
-    double* elw = el ? el : h->d_elt;
+    h->nlaunch += 1;
     prof_begin(h, KC_MEASURE, ep);
-    launch_measure64(s, h->nktask, h->d_ktask, h->d_kxyz, h->d_X, nullptr, h->d_gl, h->d_logdet, h->d_acc, elw,
-                     lnpsi ? lnpsi : h->d_lpt, dl, de, h->stream);
-    prof_end(h, ep);
-    prof_begin(h, KC_ADJOINT, ep);
-    launch_twist_pulay(s, h->tv, h->d_X, (const double2*)h->d_D, (const double2*)h->d_Lp, (const double2*)h->d_Gt,
-                       elw, h->d_acc, dl, de, h->stream);
+    launch_measure64(view<double>(h, W), &h->tv, h->nktask, h->d_ktask, h->d_kxyz, h->d_X, (const double*)h->d_Gt,
+                     h->d_logdet, h->d_acc, el, lnpsi, dl, de, h->stream);
     prof_end(h, ep);
 }
 
@@ -485,7 +466,7 @@ double run_sampling_twist(qmc_system* h) {
                                (uint32_t)sw, h->p.sigma, h->w0, h->stream);
         prof_end(h, ep);
         prof_begin(h, KC_ORB_PROP, ep);
-        launch_twist_orbitals(s, h->tv, h->d_Xp, W * N, (double2*)h->d_Phi, nullptr, nullptr, h->stream);
+        launch_twist_orbitals(s, h->tv, h->d_Xp, W * N, (double2*)h->d_Phi, h->stream);
         prof_end(h, ep);
         prof_begin(h, KC_SWEEP, ep);
         launch_twist_sweep(s, h->tv, h->d_X, h->d_Xp, (const double*)h->d_ptp, (const double*)h->d_uacc,
@@ -627,7 +608,7 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
     h->d_uacc = dalloc<unsigned char>(h, t * W * N, &rc);
     h->d_Phi = dalloc<unsigned char>(h, tc * W * N * n, &rc);
     h->d_Gt = dalloc<unsigned char>(h, tc * W * 2 * n * n, &rc);
-    if (h->mixed || h->K) {   // the FP64 form at the Gamma point needs no derivative rows
+    if (h->mixed) {   // the FP64 form needs no derivative rows
         h->d_D = dalloc<unsigned char>(h, tc * W * N * 3 * n, &rc);
         h->d_Lp = dalloc<unsigned char>(h, tc * W * N * n, &rc);
     }
@@ -663,9 +644,6 @@ int init_handle(const qmc_params* p, const double* R, void* block, size_t block_
         const int K = h->K, M = bloch_images(p);
         h->d_theta = dalloc<double>(h, 3 * (size_t)K, &rc);
         h->d_tph = dalloc<double2>(h, (size_t)K * 3 * (2 * M + 1), &rc);
-        h->d_gl = dalloc<double>(h, (size_t)W * N * 4, &rc);
-        h->d_elt = dalloc<double>(h, W, &rc);
-        h->d_lpt = dalloc<double>(h, W, &rc);
         h->d_tout = dalloc<double>(h, (size_t)K * (4 + 3 * N + 9 * (size_t)N * N), &rc);
         // exp(i theta_mu m), m = -M..M, per twist and axis
         for (int k = 0; k < K; ++k)

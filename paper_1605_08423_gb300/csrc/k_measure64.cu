@@ -16,7 +16,18 @@
 // done once per (nucleus, electron):
 //   grad: 2 s1 p;   lap: 4 s2 |p|^2 + 2 s1 sum q;
 //   H gU + 1/2 grad lap:  p (4 s2 p.gU + 4 s3 |p|^2 + 2 s2 sum q - k2 s1 + 4 s2 q) + 2 s1 q o gU.
-// N = 64, 1024 walkers: orbital rows + sample 12.1 ms before, 7.3 ms now.
+// N = 64, 1024 walkers: orbital rows + sample 12.1 ms before, 7.2 ms now.
+//
+// Twisted form (complex Bloch-summed orbitals, k_twist.cu): the same with complex
+// G, y and real C, so there Y_ij = sum_b y_bi C_bj, K = G Y G and P = C K are the
+// cheaper products (6 B n^2 + 8 n^3 real multiply-adds a spin, 10 B n^2 through M).
+// The orbitals factorise over the axes, chi = e^{i theta.k} s_x s_y s_z, and with
+// D = grad_i U . grad + 1/2 lap = D_x + D_y + D_z,
+//   y = -D chi,   H gU + 1/2 grad lap = grad (D chi),
+// everything follows from s_q = d^q s, t = D_mu s and t' = d D_mu s of each axis.
+// N = 64, 512 walkers: rows + g, l + sample + force terms 15.5 ms before in four
+// kernels, 9.4 ms now in one.
+#include "bloch.cuh"
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -32,12 +43,13 @@ int pad_pow2(int n) {
     return p;
 }
 
-// Shared memory of one CTA.  orb: the orbital products run here (false: g_i and
-// l_i are given, as for the twisted orbitals).  tb: basis rows per tile; with
-// tb >= B the Z and chi rows of a spin block stay for the second pass.
+// Shared memory of one CTA.  tb: basis rows per tile; in the real form with tb >= B
+// the Z and chi rows of a spin block stay for the second pass.  The twisted form
+// keeps G in shared memory up to n = 32 (np <= 32) and reads it from global memory above.
 struct M64Layout {
     size_t xs, et, gU, lU, Ui, gi, vv, li, facc, rhot, red, part, uni, total;
-    __host__ __device__ M64Layout(int N, int n, int np, int nk, int mmax, bool orb, bool j34, int tb) {
+    __host__ __device__ static size_t square2(int np) { return (size_t)np * (2 * np + 4); }   // complex np x np, planar
+    __host__ __device__ M64Layout(int N, int n, int np, int nk, int mmax, bool tw, bool j34, int tb) {
         size_t o = 0;
         auto take = [&](size_t doubles) { const size_t r = o; o = (o + 8 * doubles + 15) & ~size_t(15); return r; };
         xs = take(3 * N); et = take(6 * N); gU = take(3 * N); lU = take(N); Ui = take(N);
@@ -49,7 +61,11 @@ struct M64Layout {
         const size_t jp = 5 * (size_t)(kThreads > N ? kThreads : N), gp = 4 * (size_t)kWarps * n;
         part = take(jp > gp ? jp : gp);
         size_t u = 2 * (size_t)N * 3 * (mmax + 1);                            // phase table
-        if (orb) {
+        if (tw) {
+            const size_t sq = square2(np), tile = (size_t)tb * (2 * np + 2);
+            const size_t s = (np <= 32 ? 2 : 1) * sq + (sq > tile ? sq : tile);       // G, Y / K, then T or the tile
+            u = u > s ? u : s;
+        } else {
             const size_t s = 2 * (size_t)np * (np + 2) + 3 * (size_t)tb * (np + 2);   // G, M, Z, chi, y / P
             u = u > s ? u : s;
         }
@@ -61,12 +77,11 @@ struct M64Layout {
 
 // Basis rows per tile: the whole spin block if it fits (one tile, nothing
 // evaluated twice), else as many whole nuclei as do.
-int tile_rows(int N, int n, int G, int nk, int mmax, bool j34) {
-    const int B = N * G, np = pad_pow2(n);
+int tile_rows(int N, int n, int G, int nk, int mmax, bool tw, bool j34) {
+    const int np = pad_pow2(n);
     const size_t most = 225 * 1024;
-    if (M64Layout(N, n, np, nk, mmax, true, j34, B).total <= most) return B;
-    int rows = B;
-    while (rows > G && M64Layout(N, n, np, nk, mmax, true, j34, rows).total > most) rows -= G;
+    int rows = N * G;
+    while (rows > G && M64Layout(N, n, np, nk, mmax, tw, j34, rows).total > most) rows -= G;
     return rows;
 }
 
@@ -161,6 +176,131 @@ __device__ __forceinline__ void gram_store(int np, const double* acc, double* M,
         for (int c = 0; c < TT; ++c) M[(r0 + a) * ld + c0 + c] = acc[a * TT + c];
 }
 
+// ---- twisted form: complex matrices are planar (real columns, then imaginary ones)
+
+// Element (j, i) of the inverse G of a spin block: real part at p[j sj + i si],
+// imaginary part `im` further on.
+struct GView {
+    const double* p;
+    int sj, si, im;
+    __device__ __forceinline__ double2 at(int j, int i) const {
+        const double* q = p + (size_t)j * sj + (size_t)i * si;
+        return make_double2(q[0], q[im]);
+    }
+};
+
+// Z[r][i] = sum_j C[r][j] G[j][i] for `rows` rows of C, 4 x 2 complex outputs a thread.
+__device__ __forceinline__ void tw_z(int rows, int n, int np, const double* __restrict__ C, const GView& G, double* out,
+                                     int ld) {
+    const int ncg = np / 2, tasks = (rows + 3) / 4 * ncg;
+    for (int task = threadIdx.x; task < tasks; task += kThreads) {
+        const int r0 = task / ncg * 4, c0 = task % ncg * 2;
+        const int i0 = c0 < n ? c0 : n - 1, i1 = c0 + 1 < n ? c0 + 1 : n - 1;
+        const double* ar[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) ar[a] = C + (size_t)(r0 + a < rows ? r0 + a : rows - 1) * n;
+        double acc[4][4] = {};
+        for (int j = 0; j < n; ++j) {
+            const double2 g0 = G.at(j, i0), g1 = G.at(j, i1);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const double c = ar[a][j];
+                acc[a][0] += c * g0.x; acc[a][1] += c * g1.x; acc[a][2] += c * g0.y; acc[a][3] += c * g1.y;
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            if (r0 + a < rows) {
+                double* o = out + (size_t)(r0 + a) * ld + c0;
+                o[0] = acc[a][0]; o[1] = acc[a][1]; o[np] = acc[a][2]; o[np + 1] = acc[a][3];
+            }
+    }
+}
+
+// Y[r][j] += sum_{b < rows} y[b][r] C[b][j], r over the 2 np planar columns of y
+// (real, then imaginary part of electron i), 2 x 4 outputs a thread.
+__device__ __forceinline__ void tw_y(int rows, int n, int np, const double* y, int ld, const double* __restrict__ C,
+                                     double* Y, int ldy) {
+    const int ncg = np / 4, tasks = np * ncg;
+    for (int task = threadIdx.x; task < tasks; task += kThreads) {
+        const int r0 = task / ncg * 2, j0 = task % ncg * 4;
+        double acc[2][4] = {};
+        for (int b = 0; b < rows; ++b) {
+            const double y0 = y[b * ld + r0], y1 = y[b * ld + r0 + 1];
+            const double* c = C + (size_t)b * n;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const double cv = c[j0 + k < n ? j0 + k : n - 1];
+                acc[0][k] += y0 * cv;
+                acc[1][k] += y1 * cv;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            Y[(size_t)r0 * ldy + j0 + k] += acc[0][k];
+            Y[(size_t)(r0 + 1) * ldy + j0 + k] += acc[1][k];
+        }
+    }
+}
+
+// T[i][c] = sum_j Y[i][j] G[j][c], 2 x 2 complex outputs a thread.
+__device__ __forceinline__ void tw_yg(int n, int np, const double* Y, int ldy, const GView& G, double* T, int ld) {
+    const int ng = np / 2;
+    for (int task = threadIdx.x; task < ng * ng; task += kThreads) {
+        const int i0 = task / ng * 2, c0 = task % ng * 2;
+        const int ca = c0 < n ? c0 : n - 1, cb = c0 + 1 < n ? c0 + 1 : n - 1;
+        double2 acc[2][2] = {};
+        for (int j = 0; j < n; ++j) {
+            const double2 g[2] = {G.at(j, ca), G.at(j, cb)};
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                const double re = Y[(size_t)(i0 + a) * ldy + j], im = Y[(size_t)(np + i0 + a) * ldy + j];
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    acc[a][c].x += re * g[c].x - im * g[c].y;
+                    acc[a][c].y += re * g[c].y + im * g[c].x;
+                }
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                T[(size_t)(i0 + a) * ld + c0 + c] = acc[a][c].x;
+                T[(size_t)(i0 + a) * ld + np + c0 + c] = acc[a][c].y;
+            }
+    }
+}
+
+// K[j][c] = sum_i G[j][i] T[i][c], 2 x 2 complex outputs a thread.
+__device__ __forceinline__ void tw_gt(int n, int np, const GView& G, const double* T, int ld, double* K) {
+    const int ng = np / 2;
+    for (int task = threadIdx.x; task < ng * ng; task += kThreads) {
+        const int j0 = task / ng * 2, c0 = task % ng * 2;
+        const int ja = j0 < n ? j0 : n - 1, jb = j0 + 1 < n ? j0 + 1 : n - 1;
+        double2 acc[2][2] = {};
+        for (int i = 0; i < n; ++i) {
+            const double2 g[2] = {G.at(ja, i), G.at(jb, i)};
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const double re = T[(size_t)i * ld + c0 + c], im = T[(size_t)i * ld + np + c0 + c];
+#pragma unroll
+                for (int a = 0; a < 2; ++a) {
+                    acc[a][c].x += g[a].x * re - g[a].y * im;
+                    acc[a][c].y += g[a].x * im + g[a].y * re;
+                }
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                K[(size_t)(j0 + a) * ld + c0 + c] = acc[a][c].x;
+                K[(size_t)(j0 + a) * ld + np + c0 + c] = acc[a][c].y;
+            }
+    }
+}
+
 // e-e-n-n Jastrow orbital chi_a(r_i) = exp(-zeta |d|^2) with its gradient, Hessian,
 // Laplacian and gradient of the Laplacian in the electron coordinate.
 __device__ __forceinline__ double jas34(const double* ei, const double* pa, double ell, double zeta, double k2,
@@ -171,23 +311,24 @@ __device__ __forceinline__ double jas34(const double* ei, const double* pa, doub
     return e;
 }
 
-// TM: outputs a side per thread of the np x np products (np / TM squared <= 256 threads).
+// TM: outputs a side per thread of the real form's np x np products (np / TM squared
+// <= 256 threads); 0: the twisted form (its shared memory allows one CTA an SM).
 template <int TM>
-__global__ void __launch_bounds__(kThreads, 2) measure64_kernel(SysView<double> s, int mmax, int tb, int ntask,
+__global__ void __launch_bounds__(kThreads, TM ? 2 : 1) measure64_kernel(SysView<double> s, TwistView tv, int mmax, int tb,
+                                                                int ntask,
                                                                 const int4* __restrict__ ktask,
                                                                 const double* __restrict__ kxyz,
                                                                 const double* __restrict__ X,
                                                                 const double* __restrict__ Gt,
-                                                                const double* __restrict__ gl,
                                                                 const double* __restrict__ logdet,
                                                                 double* __restrict__ acc, double* __restrict__ out_el,
                                                                 double* __restrict__ out_lnpsi,
                                                                 double* __restrict__ out_dl,
                                                                 double* __restrict__ out_de) {
     extern __shared__ __align__(16) unsigned char sm[];
-    const int N = s.N, n = s.n, G = s.G, B = s.B, nk = s.nk, np = s.np;
-    const bool orb = gl == nullptr, j34 = s.fj != nullptr;
-    const M64Layout lay(N, n, np, nk, mmax, orb, j34, tb);
+    const int N = s.N, n = s.n, Gn = s.G, B = s.B, nk = s.nk, np = s.np;
+    const bool j34 = s.fj != nullptr;
+    const M64Layout lay(N, n, np, nk, mmax, TM == 0, j34, tb);
     double* xs = (double*)(sm + lay.xs);
     double* et = (double*)(sm + lay.et);
     double* gU = (double*)(sm + lay.gU);
@@ -320,9 +461,44 @@ __global__ void __launch_bounds__(kThreads, 2) measure64_kernel(SysView<double> 
     }
 
     // ---- orbital terms, one spin block at a time
-    if (orb) {
-        const int ld = np + 2, seg = np < 32 ? np : 32, apw = 32 / seg;   // lanes per nucleus, nuclei per warp
-        const int sub = lane / seg, sl = lane - sub * seg;
+    const int seg = np < 32 ? np : 32, apw = 32 / seg;   // lanes per nucleus, nuclei per warp
+    const int sub = lane / seg, sl = lane - sub * seg;
+    // a nucleus' sums over its lanes: v = dl (3), de (3)
+    auto add_forces = [&](double v[8], int a, bool on) {
+        if (seg == 32) {
+            const double x = warp_sum8(v, lane);
+            const int q = lane >> 2;
+            if ((lane & 3) == 0 && q < 6) (q < 3 ? f_dl : f_de)[3 * a + q % 3] += x;
+        } else {
+            seg_sum(v, 6, seg);
+            if (sl == 0 && on)
+#pragma unroll
+                for (int mu = 0; mu < 3; ++mu) { f_dl[3 * a + mu] += v[mu]; f_de[3 * a + mu] += v[3 + mu]; }
+        }
+    };
+    // g_i, l_i of spin block sp from the lanes' sums: the segments of a warp, then the warps in order
+    auto gather_gl = [&](double ga[2][4], int sp) {
+        for (int o = seg; o < 32; o <<= 1)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) ga[0][c] += __shfl_xor_sync(0xffffffffu, ga[0][c], o);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int il = sl + 32 * h;
+            if (sub == 0 && il < n)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) part[((size_t)warp * n + il) * 4 + c] = ga[h][c];
+        }
+        __syncthreads();
+        for (int idx = tid; idx < 4 * n; idx += kThreads) {
+            double v = 0;
+            for (int q = 0; q < kWarps; ++q) v += part[(size_t)q * n * 4 + idx];
+            const int i = sp * n + (idx >> 2), c = idx & 3;
+            if (c < 3) gi[3 * i + c] = v;
+            else li[i] = v;
+        }
+    };
+    if constexpr (TM != 0) {
+        const int ld = np + 2;
         double* Gm = uni;                         // G[j][i]
         double* Mm = Gm + (size_t)np * ld;        // M[i'][i]
         double* Zs = Mm + (size_t)np * ld;        // [tb][ld] Z
@@ -340,7 +516,7 @@ __global__ void __launch_bounds__(kThreads, 2) measure64_kernel(SysView<double> 
             __syncthreads();
             for (int pass = 0; pass < 2; ++pass) {
                 for (int b0 = 0; b0 < B; b0 += tb) {
-                    const int rows = B - b0 < tb ? B - b0 : tb, a0 = b0 / G, na = rows / G;
+                    const int rows = B - b0 < tb ? B - b0 : tb, a0 = b0 / Gn, na = rows / Gn;
                     if (pass == 0 || !whole) {
                         product_any(rows, np, n, s.C + (size_t)b0 * n, n, rows, Gm, ld, Zs, ld);
                         __syncthreads();
@@ -363,7 +539,7 @@ __global__ void __launch_bounds__(kThreads, 2) measure64_kernel(SysView<double> 
                                 if (il >= n) continue;
                                 const int i = sp * n + il;
                                 const Geo o = geometry(et + 6 * i, pa, ell);
-                                const int base = al * G * ld + il;
+                                const int base = al * Gn * ld + il;
                                 if (pass == 0) {
                                     const double* gu = gU + 3 * i;
                                     const double pp = o.p[0] * o.p[0] + o.p[1] * o.p[1] + o.p[2] * o.p[2];
@@ -371,7 +547,7 @@ __global__ void __launch_bounds__(kThreads, 2) measure64_kernel(SysView<double> 
                                     const double pg = o.p[0] * gu[0] + o.p[1] * gu[1] + o.p[2] * gu[2];
                                     const double sp2 = fma(2.0, pg, sq), pp2 = 2.0 * pp;
                                     double s1 = 0, s2 = 0, s3 = 0;   // sum_g Z zeta^q chi
-                                    for (int g = 0; g < G; ++g) {
+                                    for (int g = 0; g < Gn; ++g) {
                                         const double z = s.zeta[g];
                                         const double w1 = z * qexp(-z * o.t), w2 = z * w1;
                                         const double Z = Zs[base + g * ld];
@@ -392,9 +568,9 @@ __global__ void __launch_bounds__(kThreads, 2) measure64_kernel(SysView<double> 
                                 } else {
                                     double pc = 0;                   // -sum_g P_bi 2 zeta chi
                                     if (whole) {
-                                        for (int g = 0; g < G; ++g) pc = fma(Ys[base + g * ld], Cs[base + g * ld], pc);
+                                        for (int g = 0; g < Gn; ++g) pc = fma(Ys[base + g * ld], Cs[base + g * ld], pc);
                                     } else {
-                                        for (int g = 0; g < G; ++g) {
+                                        for (int g = 0; g < Gn; ++g) {
                                             const double z = s.zeta[g];
                                             pc = fma(Ys[base + g * ld], 2.0 * z * qexp(-z * o.t), pc);
                                         }
@@ -404,16 +580,7 @@ __global__ void __launch_bounds__(kThreads, 2) measure64_kernel(SysView<double> 
                                 }
                             }
                         }
-                        if (seg == 32) {
-                            const double x = warp_sum8(v, lane);
-                            const int q = lane >> 2;
-                            if ((lane & 3) == 0 && q < 6) (q < 3 ? f_dl : f_de)[3 * a + q % 3] += x;
-                        } else {
-                            seg_sum(v, 6, seg);
-                            if (sl == 0 && al < na)
-#pragma unroll
-                                for (int mu = 0; mu < 3; ++mu) { f_dl[3 * a + mu] += v[mu]; f_de[3 * a + mu] += v[3 + mu]; }
-                        }
+                        add_forces(v, a, al < na);
                     }
                     __syncthreads();
                     if (pass == 0) {
@@ -423,36 +590,119 @@ __global__ void __launch_bounds__(kThreads, 2) measure64_kernel(SysView<double> 
                 }
                 if (pass == 0) {
                     gram_store<TM>(np, macc, Mm, ld);
-                    // g_i, l_i: the segments of a warp, then the warps in order
-                    for (int o = seg; o < 32; o <<= 1)
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) ga[0][c] += __shfl_xor_sync(0xffffffffu, ga[0][c], o);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int il = sl + 32 * h;
-                        if (sub == 0 && il < n)
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) part[((size_t)warp * n + il) * 4 + c] = ga[h][c];
-                    }
-                    __syncthreads();
-                    for (int idx = tid; idx < 4 * n; idx += kThreads) {
-                        double v = 0;
-                        for (int q = 0; q < kWarps; ++q) v += part[(size_t)q * n * 4 + idx];
-                        const int i = sp * n + (idx >> 2), c = idx & 3;
-                        if (c < 3) gi[3 * i + c] = v;
-                        else li[i] = v;
-                    }
+                    gather_gl(ga, sp);
                 }
             }
             __syncthreads();
         }
     } else {
-        for (int idx = tid; idx < 4 * N; idx += kThreads) {
-            const double v = gl[(size_t)w * 4 * N + idx];
-            if ((idx & 3) < 3) gi[3 * (idx >> 2) + (idx & 3)] = v;
-            else li[idx >> 2] = v;
+        const int ld2 = 2 * np + 2, ldy = np + 2, M = tv.M, t = w / tv.Wk;
+        const size_t sq = M64Layout::square2(np);
+        double* Gs = uni;                                   // G (np <= 32)
+        double* YK = Gs + (np <= 32 ? sq : 0);              // Y [2 np][ldy], then K [np][ld2]
+        double* tile = YK + sq;                             // [tb][ld2]: Z, overwritten by y; P.  T [np][ld2] in between
+        const double2* ph = tv.ph + (size_t)t * 3 * (2 * M + 1);
+        const double* th = tv.theta + 3 * t;
+        __shared__ int images[8][2];                        // per Gaussian: near and far images (n_gauss <= 8)
+        if (tid < Gn) {
+            images[tid][0] = bloch_near(s.zeta[tid], L, M);
+            images[tid][1] = bloch_far(s.zeta[tid], L, M);
         }
-        __syncthreads();
+        for (int sp = 0; sp < 2; ++sp) {
+            const double sg = sp == 0 ? 1.0 : -1.0;
+            const double2* Gsp = (const double2*)Gt + ((size_t)w * 2 + sp) * n * n;   // G^T[i][j] = G[j][i]
+            GView G{(const double*)Gsp, 2, 2 * n, 1};
+            if (np <= 32) {
+                for (int idx = tid; idx < n * n; idx += kThreads) {
+                    const int i = idx / n, j = idx - i * n;
+                    const double2 g = Gsp[idx];
+                    Gs[(size_t)j * ld2 + i] = g.x;
+                    Gs[(size_t)j * ld2 + np + i] = g.y;
+                }
+                G = GView{Gs, ld2, 1, np};
+            }
+            for (int idx = tid; idx < 2 * np * ldy; idx += kThreads) YK[idx] = 0.0;
+            double ga[2][4] = {};
+            __syncthreads();
+            for (int pass = 0; pass < 2; ++pass) {
+                for (int b0 = 0; b0 < B; b0 += tb) {
+                    const int rows = B - b0 < tb ? B - b0 : tb, a0 = b0 / Gn, na = rows / Gn;
+                    const double* Ct = s.C + (size_t)b0 * n;
+                    if (pass == 0) tw_z(rows, n, np, Ct, G, tile, ld2);
+                    else product_any(rows, 2 * np, n, Ct, n, rows, YK, ld2, tile, ld2);    // P = C K
+                    __syncthreads();
+                    for (int ab = warp * apw; ab < na; ab += kWarps * apw) {
+                        const int al = ab + sub, a = a0 + al;
+                        double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // dl, de
+                        if (al < na) {
+#pragma unroll 1
+                            for (int h = 0; h < 2; ++h) {
+                                const int il = sl + 32 * h;
+                                if (il >= n) continue;
+                                const int i = sp * n + il;
+                                double d0[3];
+                                const double2 P = bloch_min_image(xs + 3 * i, s.R + 3 * a, L, iL, M, ph, th, sg, d0);
+                                double* zt = tile + (size_t)al * Gn * ld2 + il;
+                                const double* gu = gU + 3 * i;
+#pragma unroll 1
+                                for (int g = 0; g < Gn; ++g, zt += ld2) {
+                                    const double z = s.zeta[g];
+                                    const int near = images[g][0], far = images[g][1];
+                                    const double2 zp = cmul(make_double2(zt[0], zt[np]), P);
+                                    if (pass == 0) {
+                                        double2 sx[4], sy[4], sz[4];
+                                        bloch_axis<3>(d0[0], z, L, near, far, M, ph, sg, sx);
+                                        bloch_axis<3>(d0[1], z, L, near, far, M, ph + (2 * M + 1), sg, sy);
+                                        bloch_axis<3>(d0[2], z, L, near, far, M, ph + 2 * (2 * M + 1), sg, sz);
+                                        const double2 tx = caxpy(gu[0], sx[1], 0.5, sx[2]), ty = caxpy(gu[1], sy[1], 0.5, sy[2]),
+                                                      tz = caxpy(gu[2], sz[1], 0.5, sz[2]);
+                                        const double2 ux = caxpy(gu[0], sx[2], 0.5, sx[3]), uy = caxpy(gu[1], sy[2], 0.5, sy[3]),
+                                                      uz = caxpy(gu[2], sz[2], 0.5, sz[3]);
+                                        const double2 yz = cmul(sy[0], sz[0]), xz = cmul(sx[0], sz[0]), xy = cmul(sx[0], sy[0]);
+                                        const double2 ayz = cadd(cmul(ty, sz[0]), cmul(sy[0], tz)),
+                                                      axz = cadd(cmul(tx, sz[0]), cmul(sx[0], tz)),
+                                                      axy = cadd(cmul(tx, sy[0]), cmul(sx[0], ty));
+                                        const double2 y = cmul(P, cadd(cmul(tx, yz), cmul(sx[0], ayz)));
+                                        zt[0] = -y.x;
+                                        zt[np] = -y.y;
+                                        const double gr[3] = {cre(zp, cmul(sx[1], yz)), cre(zp, cmul(sy[1], xz)),
+                                                              cre(zp, cmul(sz[1], xy))};
+                                        ga[h][3] += cre(zp, cadd(cadd(cmul(sx[2], yz), cmul(sy[2], xz)), cmul(sz[2], xy)));
+                                        v[3] += cre(zp, cadd(cmul(ux, yz), cmul(sx[1], ayz)));
+                                        v[4] += cre(zp, cadd(cmul(uy, xz), cmul(sy[1], axz)));
+                                        v[5] += cre(zp, cadd(cmul(uz, xy), cmul(sz[1], axy)));
+#pragma unroll
+                                        for (int mu = 0; mu < 3; ++mu) { ga[h][mu] += gr[mu]; v[mu] -= gr[mu]; }
+                                    } else {
+                                        double2 sx[2], sy[2], sz[2];
+                                        bloch_axis<1>(d0[0], z, L, near, far, M, ph, sg, sx);
+                                        bloch_axis<1>(d0[1], z, L, near, far, M, ph + (2 * M + 1), sg, sy);
+                                        bloch_axis<1>(d0[2], z, L, near, far, M, ph + 2 * (2 * M + 1), sg, sz);
+                                        const double2 px = cmul(zp, sx[0]);
+                                        v[3] += cre(cmul(zp, sx[1]), cmul(sy[0], sz[0]));
+                                        v[4] += cre(cmul(px, sy[1]), sz[0]);
+                                        v[5] += cre(cmul(px, sy[0]), sz[1]);
+                                    }
+                                }
+                            }
+                        }
+                        add_forces(v, a, al < na);
+                    }
+                    __syncthreads();
+                    if (pass == 0) {
+                        tw_y(rows, n, np, tile, ld2, Ct, YK, ldy);
+                        __syncthreads();
+                    }
+                }
+                if (pass == 0) {
+                    tw_yg(n, np, YK, ldy, G, tile, ld2);   // T = Y G
+                    __syncthreads();
+                    tw_gt(n, np, G, tile, ld2, YK);        // K = G T over Y
+                    gather_gl(ga, sp);                     // (its barrier ends the reads of T too)
+                }
+            }
+            __syncthreads();
+        }
     }
 
     // ---- kinetic energy and U
@@ -688,29 +938,29 @@ __global__ void __launch_bounds__(kThreads, 2) measure64_kernel(SysView<double> 
 }
 
 template <int TM>
-void launch(const SysView<double>& s, int tb, size_t smem, int ntask, const int4* ktask, const double* kxyz,
-            const double* X, const double* Gt, const double* gl, const double* logdet, double* acc, double* out_el,
+void launch(const SysView<double>& s, const TwistView& tv, int tb, size_t smem, int ntask, const int4* ktask,
+            const double* kxyz, const double* X, const double* Gt, const double* logdet, double* acc, double* out_el,
             double* out_lnpsi, double* out_dl, double* out_de, cudaStream_t st) {
     static bool set = false;
     if (!set) {
-        cudaFuncSetAttribute(measure64_kernel<TM>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        cudaFuncSetAttribute(measure64_kernel<TM>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
         set = true;
     }
-    measure64_kernel<TM><<<s.W, kThreads, smem, st>>>(s, s.mmax, tb, ntask, ktask, kxyz, X, Gt, gl, logdet, acc, out_el,
+    measure64_kernel<TM><<<s.W, kThreads, smem, st>>>(s, tv, s.mmax, tb, ntask, ktask, kxyz, X, Gt, logdet, acc, out_el,
                                                       out_lnpsi, out_dl, out_de);
 }
 
 }  // namespace
 
-void launch_measure64(const SysView<double>& s, int ntask, const int4* ktask, const double* kxyz, const double* X,
-                      const double* Gt, const double* gl, const double* logdet, double* acc, double* out_el,
+void launch_measure64(const SysView<double>& s, const TwistView* tv, int ntask, const int4* ktask, const double* kxyz,
+                      const double* X, const double* Gt, const double* logdet, double* acc, double* out_el,
                       double* out_lnpsi, double* out_dl, double* out_de, cudaStream_t st) {
-    const bool orb = gl == nullptr, j34 = s.fj != nullptr;
-    const int tb = orb ? tile_rows(s.N, s.n, s.G, s.nk, s.mmax, j34) : 0;
-    const size_t smem = M64Layout(s.N, s.n, s.np, s.nk, s.mmax, orb, j34, tb).total;
+    const bool j34 = s.fj != nullptr;
+    const int tb = tile_rows(s.N, s.n, s.G, s.nk, s.mmax, tv != nullptr, j34);
+    const size_t smem = M64Layout(s.N, s.n, s.np, s.nk, s.mmax, tv != nullptr, j34, tb).total;
     // np x np outputs over 256 threads: one, 2 x 2 or 4 x 4 each
-    auto go = s.np <= 16 ? launch<1> : s.np <= 32 ? launch<2> : launch<4>;
-    go(s, tb, smem, ntask, ktask, kxyz, X, Gt, gl, logdet, acc, out_el, out_lnpsi, out_dl, out_de, st);
+    auto go = tv ? launch<0> : s.np <= 16 ? launch<1> : s.np <= 32 ? launch<2> : launch<4>;
+    go(s, tv ? *tv : TwistView{}, tb, smem, ntask, ktask, kxyz, X, Gt, logdet, acc, out_el, out_lnpsi, out_dl, out_de, st);
 }
 
 }  // namespace qmc

@@ -1,6 +1,6 @@
 // k_twist.cu -- twisted boundary conditions in the FP64 form: Bloch-summed
-// Gaussian orbitals, complex Slater inverses, complex Sherman-Morrison sweeps,
-// the orbital parts of E_L and of the force estimators, and the twist average.
+// Gaussian orbitals, complex Slater inverses, complex Sherman-Morrison sweeps and
+// the twist average (the samples are in k_measure64.cu).
 //
 // SI, basis section: orbitals with phi(r + nL) = exp(i theta.n) phi(r) for
 // integer vectors n.  The Gaussians become Bloch functions by the lattice sum
@@ -17,150 +17,109 @@
 // sampled density is |psi|^2 and the estimators take real parts:
 //   E_L = Re(H psi / psi),  d ln|psi| / dR = Re(d ln psi / dR),  dE_L / dR = Re(d (H psi / psi) / dR).
 // Complex values are double2 (x = real, y = imaginary part).
+#include "bloch.cuh"
 #include "common.cuh"
 #include "kernels.cuh"
 
 namespace qmc {
 
-__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
-    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ double2 cscale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
-__device__ __forceinline__ double2 cinv(double2 a) {
-    const double q = a.x * a.x + a.y * a.y;
-    return make_double2(a.x / q, -a.y / q);
-}
-__device__ __forceinline__ double2 czero() { return make_double2(0.0, 0.0); }
-
-// One axis of a Bloch-summed Gaussian at the minimum-image coordinate d0:
-// s[q] = d^q s / dx^q for q = 0..ND, with the phases ph[m + M] = exp(i theta_mu m)
-// (conjugated when sg < 0, the spin-down twist).
-//   g = e^{-zeta u^2}: g' = -2 zeta u g,  g'' = (4 zeta^2 u^2 - 2 zeta) g,  g''' = (12 zeta^2 u - 8 zeta^3 u^3) g.
-template <int ND>
-__device__ __forceinline__ void axis_sums(double d0, double zeta, double L, int M, const double2* __restrict__ ph,
-                                          double sg, double2 s[ND + 1]) {
-#pragma unroll
-    for (int q = 0; q <= ND; ++q) s[q] = czero();
-    for (int m = -M; m <= M; ++m) {
-        const double u = d0 - m * L;
-        const double e = exp(-zeta * u * u);
-        double2 p = ph[m + M];
-        p.y *= sg;
-        const double2 pe = cscale(p, e);
-        s[0] = cadd(s[0], pe);
-        if (ND >= 1) s[1] = cadd(s[1], cscale(pe, -2.0 * zeta * u));
-        if (ND >= 2) s[2] = cadd(s[2], cscale(pe, 4.0 * zeta * zeta * u * u - 2.0 * zeta));
-        if (ND >= 3) s[3] = cadd(s[3], cscale(pe, 12.0 * zeta * zeta * u - 8.0 * zeta * zeta * zeta * u * u * u));
-    }
-}
-
-// Minimum-image split of r - R_a and the Bloch phase exp(i sg theta.k) of the
-// nearest image k.
-__device__ __forceinline__ double2 min_image(const double x[3], const double* __restrict__ Ra, double L, double iL,
-                                             const double* __restrict__ th, double sg, double d0[3]) {
-    double kth = 0.0;
-#pragma unroll
-    for (int mu = 0; mu < 3; ++mu) {
-        const double d = x[mu] - Ra[mu];
-        const double k = rint(d * iL);
-        d0[mu] = d - k * L;
-        kth += th[mu] * k;
-    }
-    double sn, cs;
-    sincos(sg * kth, &sn, &cs);
-    return make_double2(cs, sn);
-}
-
 // ---------------------------------------------------------------------------
-// Orbital rows: one warp per row (walker w = row / N, electron i = row % N).
-// The warp first evaluates the B Bloch-summed basis functions (lanes over the
-// basis; Q = 1: values, Q = 5: value, gradient, Laplacian) into its slice of
-// shared memory, then contracts them with the real coefficients (lanes over
-// the orbitals).  Same layouts as the real kernels: val [rows][n], grad
-// [rows][3][n], lap [rows][n], complex.
+// Orbital rows (walker w = row / N, electron i = row % N): values phi_j(r) [rows][n],
+// complex; nothing needs the derivative rows (k_measure64.cu).  The FP64 pipe bounds
+// it, mostly by the exponentials: two or three per axis and Gaussian (bloch_near,
+// bloch_far), where a sum over all 2M + 1 images and a sincos per pair took 2.29 ms
+// for 32768 rows of N = 64 (1.36 ms now).  256 threads take 32 rows and 8 nuclei at a
+// time: one (row, nucleus) each for the basis, TR x TC complex outputs for the product
+// with the real coefficients.
 // ---------------------------------------------------------------------------
-template <int Q>
+template <int NP, int TR, int TC>
 __global__ void __launch_bounds__(256) twist_orbitals_kernel(SysView<double> s, TwistView tv,
                                                              const double* __restrict__ pos, int nrows,
-                                                             double2* __restrict__ val, double2* __restrict__ grad,
-                                                             double2* __restrict__ lap) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    const int row = blockIdx.x * wpb + warp;
-    if (row >= nrows) return;   // whole warps leave; the kernel has no block-wide barrier
-    const int N = s.N, n = s.n, B = s.B, G = s.G, M = tv.M;
-    double2* chi = (double2*)smraw + (size_t)warp * B * Q;   // [B][Q]
-    const int w = row / N, i = row - w * N, t = w / tv.Wk;
-    const double sg = i < n ? 1.0 : -1.0;
+                                                             double2* __restrict__ val) {
+    constexpr int RT = 32, NA = 8, CG = NP / TC;
+    static_assert(RT / TR * CG == 256, "one output tile per thread");
+    extern __shared__ __align__(16) double smem[];
+    const int n = s.n, Gn = s.G, N = s.N, M = tv.M, KC = NA * Gn;
+    double2* chi = (double2*)smem;                   // [KC][RT]
+    double* csm = smem + 2 * (size_t)KC * RT;        // [KC][NP]
+    const int tid = threadIdx.x, row0 = blockIdx.x * RT;
+    const int al = tid >> 5, r = tid & 31, row = row0 + r < nrows ? row0 + r : nrows - 1;
+    const int w = row / N, t = w / tv.Wk;
+    const double sg = row - w * N < n ? 1.0 : -1.0;
     const double* th = tv.theta + 3 * t;
     const double2* ph = tv.ph + (size_t)t * 3 * (2 * M + 1);
     const double x[3] = {pos[(size_t)row * 3], pos[(size_t)row * 3 + 1], pos[(size_t)row * 3 + 2]};
-    constexpr int ND = Q == 1 ? 0 : 2;
-    for (int b = lane; b < B; b += 32) {
-        const int a = b / G, g = b - a * G;
-        double d0[3];
-        const double2 P = min_image(x, s.R + 3 * a, s.L, s.iL, th, sg, d0);
-        const double z = s.zeta[g];
-        double2 sa[3][ND + 1];
+    __shared__ int images[8][2];                     // per Gaussian: near and far images (n_gauss <= 8)
+    if (tid < Gn) {
+        images[tid][0] = bloch_near(s.zeta[tid], s.L, M);
+        images[tid][1] = bloch_far(s.zeta[tid], s.L, M);
+    }
+    const int r0 = tid / CG * TR, c0 = tid % CG * TC;
+    double2 acc[TR][TC] = {};
+    for (int a0 = 0; a0 < N; a0 += NA) {
+        const int na = N - a0 < NA ? N - a0 : NA, rows = na * Gn;
+        __syncthreads();
+        for (int idx = tid; idx < rows * NP; idx += 256) {
+            const int k = idx / NP, j = idx % NP;
+            csm[idx] = j < n ? s.C[(size_t)(a0 * Gn + k) * n + j] : 0.0;
+        }
+        if (al < na) {
+            double d0[3];
+            const double2 P = bloch_min_image(x, s.R + 3 * (a0 + al), s.L, s.iL, M, ph, th, sg, d0);
+            for (int g = 0; g < Gn; ++g) {
+                const double z = s.zeta[g];
+                const int near = images[g][0], far = images[g][1];
+                double2 c = P, sa[1];
 #pragma unroll
-        for (int mu = 0; mu < 3; ++mu) axis_sums<ND>(d0[mu], z, s.L, M, ph + mu * (2 * M + 1), sg, sa[mu]);
-        const double2 yz = cmul(sa[1][0], sa[2][0]);
-        chi[(size_t)b * Q] = cmul(P, cmul(sa[0][0], yz));
-        if constexpr (Q == 5) {
-            const double2 xz = cmul(sa[0][0], sa[2][0]), xy = cmul(sa[0][0], sa[1][0]);
-            chi[(size_t)b * Q + 1] = cmul(P, cmul(sa[0][1], yz));
-            chi[(size_t)b * Q + 2] = cmul(P, cmul(sa[1][1], xz));
-            chi[(size_t)b * Q + 3] = cmul(P, cmul(sa[2][1], xy));
-            chi[(size_t)b * Q + 4] = cmul(P, cadd(cadd(cmul(sa[0][2], yz), cmul(sa[1][2], xz)), cmul(sa[2][2], xy)));
+                for (int mu = 0; mu < 3; ++mu) {
+                    bloch_axis<0>(d0[mu], z, s.L, near, far, M, ph + mu * (2 * M + 1), sg, sa);
+                    c = cmul(c, sa[0]);
+                }
+                chi[(al * Gn + g) * RT + r] = c;
+            }
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int k = 0; k < rows; ++k) {
+            double2 xv[TR];
+            double c[TC];
+#pragma unroll
+            for (int a = 0; a < TR; ++a) xv[a] = chi[k * RT + r0 + a];
+#pragma unroll
+            for (int m = 0; m < TC; ++m) c[m] = csm[k * NP + c0 + m];
+#pragma unroll
+            for (int a = 0; a < TR; ++a)
+#pragma unroll
+                for (int m = 0; m < TC; ++m) {
+                    acc[a][m].x += xv[a].x * c[m];
+                    acc[a][m].y += xv[a].y * c[m];
+                }
         }
     }
-    __syncwarp();
-    for (int j = lane; j < n; j += 32) {
-        double2 acc[Q];
 #pragma unroll
-        for (int q = 0; q < Q; ++q) acc[q] = czero();
-        for (int b = 0; b < B; ++b) {
-            const double c = s.C[(size_t)b * n + j];
+    for (int a = 0; a < TR; ++a)
 #pragma unroll
-            for (int q = 0; q < Q; ++q) acc[q] = cadd(acc[q], cscale(chi[(size_t)b * Q + q], c));
-        }
-        val[(size_t)row * n + j] = acc[0];
-        if constexpr (Q == 5) {
-#pragma unroll
-            for (int mu = 0; mu < 3; ++mu) grad[((size_t)row * 3 + mu) * n + j] = acc[1 + mu];
-            lap[(size_t)row * n + j] = acc[4];
-        }
-    }
+        for (int m = 0; m < TC; ++m)
+            if (row0 + r0 + a < nrows && c0 + m < n) val[(size_t)(row0 + r0 + a) * n + c0 + m] = acc[a][m];
 }
 
-// Warps per CTA of the orbital kernel: as many [B][Q] slices as fit in 200 KB, at most 8.
-static int twist_orb_warps(int B, int Q) {
-    const size_t per = (size_t)B * Q * sizeof(double2);
-    size_t w = (200u * 1024u) / per;
-    return (int)(w < 1 ? 1 : (w > 8 ? 8 : w));
+template <int NP, int TR, int TC>
+static void launch_tw_orb(const SysView<double>& s, const TwistView& tv, const double* pos, int nrows, double2* val,
+                          cudaStream_t st) {
+    const size_t smem = (size_t)8 * s.G * (2 * 32 + NP) * sizeof(double);   // at most 64 KB (n_gauss = 8, n > 32)
+    static size_t attr = 48 * 1024;
+    if (smem > attr && cudaFuncSetAttribute(twist_orbitals_kernel<NP, TR, TC>,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)
+        attr = smem;
+    twist_orbitals_kernel<NP, TR, TC><<<(nrows + 31) / 32, 256, smem, st>>>(s, tv, pos, nrows, val);
 }
 
-void launch_twist_orbitals(const SysView<double>& s, const TwistView& tv, const double* pos, int nrows,
-                           double2* val, double2* grad, double2* lap, cudaStream_t st) {
-    const int Q = grad ? 5 : 1;
-    const int wpb = twist_orb_warps(s.B, Q);
-    const size_t smem = (size_t)wpb * s.B * Q * sizeof(double2);
-    const int grid = (nrows + wpb - 1) / wpb;
-    if (Q == 5) {
-        static size_t attr = 0;
-        if (smem > attr && cudaFuncSetAttribute(twist_orbitals_kernel<5>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)smem) == cudaSuccess)
-            attr = smem;
-        twist_orbitals_kernel<5><<<grid, 32 * wpb, smem, st>>>(s, tv, pos, nrows, val, grad, lap);
-    } else {
-        static size_t attr = 0;
-        if (smem > attr && cudaFuncSetAttribute(twist_orbitals_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)smem) == cudaSuccess)
-            attr = smem;
-        twist_orbitals_kernel<1><<<grid, 32 * wpb, smem, st>>>(s, tv, pos, nrows, val, nullptr, nullptr);
-    }
+void launch_twist_orbitals(const SysView<double>& s, const TwistView& tv, const double* pos, int nrows, double2* val,
+                           cudaStream_t st) {
+    if (s.n <= 8) launch_tw_orb<8, 1, 1>(s, tv, pos, nrows, val, st);
+    else if (s.n <= 16) launch_tw_orb<16, 1, 2>(s, tv, pos, nrows, val, st);
+    else if (s.n <= 32) launch_tw_orb<32, 1, 4>(s, tv, pos, nrows, val, st);
+    else launch_tw_orb<64, 2, 4>(s, tv, pos, nrows, val, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -490,255 +449,6 @@ void launch_twist_sweep(const SysView<double>& s, const TwistView& tv, double* X
         attr = smem;
     twist_sweep_kernel<<<(s.W + wpb - 1) / wpb, 32 * wpb, smem, st>>>(s, tv, X, Xp, ptp, uacc, Phi, Gt, nacc, vep,
                                                                                vep_init ? 1 : 0);
-}
-
-// ---------------------------------------------------------------------------
-// g_i = sum_j D_ij G^T[i][j] and l_i = sum_j Lp_ij G^T[i][j] of every electron.
-// Their real parts are the only way the complex determinant enters E_L:
-//   Re(H psi / psi) = -1/2 sum_i [ Re l_i + 2 Re g_i . grad_i U + lap_i U + |grad_i U|^2 ] + V,
-// and the e-n Jastrow force terms take vv_i = Re g_i + grad_i U.  The FP64
-// measure kernel computes all of that from gl [rows][4] = (Re g_i, Re l_i).  One
-// warp per electron.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) twist_gl_kernel(int rows, int n, const double2* __restrict__ D,
-                                                       const double2* __restrict__ Lp, const double2* __restrict__ Gt,
-                                                       int N, double* __restrict__ gl) {
-    const int lane = threadIdx.x & 31, r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (r >= rows) return;
-    const int w = r / N, i = r - w * N, sp = i / n, il = i - sp * n;
-    const double2* grow = Gt + (((size_t)w * 2 + sp) * n + il) * n;
-    const double2* drow = D + (size_t)r * 3 * n;
-    const double2* lrow = Lp + (size_t)r * n;
-    double g0 = 0, g1 = 0, g2 = 0, l = 0;
-    for (int j = lane; j < n; j += 32) {
-        const double2 gj = grow[j];
-        const double2 d0 = drow[j], d1 = drow[n + j], d2 = drow[2 * n + j], lj = lrow[j];
-        g0 += d0.x * gj.x - d0.y * gj.y;
-        g1 += d1.x * gj.x - d1.y * gj.y;
-        g2 += d2.x * gj.x - d2.y * gj.y;
-        l += lj.x * gj.x - lj.y * gj.y;
-    }
-    g0 = warp_sum(g0); g1 = warp_sum(g1); g2 = warp_sum(g2); l = warp_sum(l);
-    if (lane == 0) {
-        double* o = gl + 4 * (size_t)r;
-        o[0] = g0; o[1] = g1; o[2] = g2; o[3] = l;
-    }
-}
-
-void launch_twist_gl(int rows, int N, int n, const double2* D, const double2* Lp, const double2* Gt, double* gl,
-                     cudaStream_t st) {
-    twist_gl_kernel<<<(rows + 7) / 8, 256, 0, st>>>(rows, n, D, Lp, Gt, N, gl);
-}
-
-// ---------------------------------------------------------------------------
-// Orbital (Pulay) terms of the force estimators with complex orbitals, one CTA
-// per walker, after the measure kernel has accumulated everything else of the
-// sample (the Jastrow and Ewald terms) and written E_L.  grad_i U (the Pade e-e and
-// e-n terms of the sin-periodised Jastrow, and with s.fj the e-e-n-n term
-// grad_i U34 = sum_a grad chi_a(r_i) w_ia, w_ia = sum_b f_ab (c_b - chi_b(r_i)),
-// c = sum_j chi(r_j)) is formed here again.  Per spin
-// block, with G the inverse (G[j][i] = G^T[i][j]),
-//   Y_ij = -1/2 Lp_ij - grad_i U . D_ij,  K = G Y G,  Z_bi = sum_j C_bj G_ji,  P_bi = sum_j C_bj K_ji,
-//   d ln|psi| / dR_a += -Re sum_i sum_{b in a} Z_bi grad chi_b(r_i)
-//   dE_L / dR_a      +=  Re sum_i sum_{b in a} [ P_bi grad chi_b + Z_bi (H_b grad_i U + 1/2 grad lap chi_b) ]
-// (chi depends on r - R_a, so d/dR_a = -grad; the Hermitian H makes the R-
-// derivative of E the real part).  The sample adds dl, E_L dl and de to the
-// walker's accumulators like the measure kernel does.  A warp handles one
-// nucleus at a time, lanes over its (Gaussian, electron) pairs: fixed order.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) twist_pulay_kernel(SysView<double> s, TwistView tv,
-                                                          const double* __restrict__ X,
-                                                          const double2* __restrict__ D,
-                                                          const double2* __restrict__ Lp,
-                                                          const double2* __restrict__ Gt,
-                                                          const double* __restrict__ elw, double* __restrict__ acc,
-                                                          double* __restrict__ out_dl, double* __restrict__ out_de) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    const int N = s.N, n = s.n, G = s.G, M = tv.M, N3 = 3 * N;
-    const int w = blockIdx.x, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-    double2* Gm = (double2*)smraw;              // [n][n]  G[j][i]
-    double2* YK = Gm + (size_t)n * n;           // [n][n]  Y[i][j], then K[j][i]
-    double2* T1 = YK + (size_t)n * n;           // [n][n]  (Y G)[i][i']
-    double* fdl = (double*)(T1 + (size_t)n * n); // [3N]
-    double* fde = fdl + N3;                      // [3N]
-    double* et = fde + N3;                       // [N][6] (sin, cos)(pi x / L) of the electrons
-    double* gUw = et + 6 * N;                    // [N][3] grad_i U
-    double* c34 = gUw + 3 * N;                   // [N] sum over electrons of chi_a (e-e-n-n term)
-    double* rows = c34 + N;                      // per warp [N]: chi_b(r_i)
-    const double* th = tv.theta + 3 * (w / tv.Wk);
-    const double2* ph = tv.ph + (size_t)(w / tv.Wk) * 3 * (2 * M + 1);
-    for (int c = tid; c < N3; c += nt) {
-        fdl[c] = 0.0; fde[c] = 0.0;
-        double sn, cs;
-        sincospi(X[(size_t)w * N3 + c] * s.iL, &sn, &cs);
-        et[6 * (c / 3) + c % 3] = sn;
-        et[6 * (c / 3) + 3 + c % 3] = cs;
-    }
-    __syncthreads();
-    for (int i = tid; i < N; i += nt) {          // grad_i U: d t / dx = 2 p, p = (L/pi) sin cos
-        double g[3] = {0, 0, 0};
-        const double* ei = et + 6 * i;
-        for (int j = 0; j < N; ++j) {
-            if (j == i) continue;
-            double sd[3], cd[3], t;
-            disp_trig(ei, et + 6 * j, s.ell, sd, cd, t);
-            const double r = qsqrt_pair(t);
-            double u, u1, u2, f1, f2, f3;
-            pade_ee(s.b_ee, r, u, u1, u2);
-            rho_to_t(r, u1, u2, 0.0, f1, f2, f3);
-#pragma unroll
-            for (int mu = 0; mu < 3; ++mu) g[mu] += 2.0 * f1 * (s.ell * sd[mu] * cd[mu]);
-        }
-        for (int a = 0; a < N; ++a) {
-            double sd[3], cd[3], t;
-            disp_trig(ei, s.ptrig + 6 * a, s.ell, sd, cd, t);
-            const double r = qsqrt_pair(t);
-            double u, u1, u2, u3, f1, f2, f3;
-            pade_ep(s.b_ep, s.Zj, r, u, u1, u2, u3);
-            rho_to_t(r, u1, u2, 0.0, f1, f2, f3);
-#pragma unroll
-            for (int mu = 0; mu < 3; ++mu) g[mu] += 2.0 * f1 * (s.ell * sd[mu] * cd[mu]);
-        }
-#pragma unroll
-        for (int mu = 0; mu < 3; ++mu) gUw[3 * i + mu] = g[mu];
-    }
-    __syncthreads();
-    if (s.fj) {   // grad chi = -zeta chi grad t, grad t = 2 p, p = (L/pi) sin cos
-        const double zj = s.zeta_j;
-        for (int a = tid; a < N; a += nt) {
-            double c = 0;
-            for (int j = 0; j < N; ++j) c += tw_jas_orbital(et + 6 * j, s.ptrig + 6 * a, s.ell, zj);
-            c34[a] = c;
-        }
-        __syncthreads();
-        double* row = rows + (size_t)warp * N;
-        for (int i = warp; i < N; i += nw) {
-            for (int b = lane; b < N; b += 32) row[b] = tw_jas_orbital(et + 6 * i, s.ptrig + 6 * b, s.ell, zj);
-            __syncwarp();
-            double g[3] = {0, 0, 0};
-            for (int a = lane; a < N; a += 32) {
-                const double* fa = s.fj + a;   // f symmetric: column a = row a
-                double wa = 0;
-                for (int b = 0; b < N; ++b) wa += fa[(size_t)b * N] * (c34[b] - row[b]);
-                double sd[3], cd[3], t;
-                disp_trig(et + 6 * i, s.ptrig + 6 * a, s.ell, sd, cd, t);
-#pragma unroll
-                for (int mu = 0; mu < 3; ++mu) g[mu] += -2.0 * zj * row[a] * (s.ell * sd[mu] * cd[mu]) * wa;
-            }
-#pragma unroll
-            for (int mu = 0; mu < 3; ++mu) g[mu] = warp_sum(g[mu]);
-            if (lane == 0)
-#pragma unroll
-                for (int mu = 0; mu < 3; ++mu) gUw[3 * i + mu] += g[mu];
-            __syncwarp();
-        }
-        __syncthreads();
-    }
-    for (int sp = 0; sp < 2; ++sp) {
-        const double sg = sp == 0 ? 1.0 : -1.0;
-        const double2* Gsp = Gt + ((size_t)w * 2 + sp) * n * n;
-        for (int idx = tid; idx < n * n; idx += nt) {
-            const int i = idx / n, j = idx - i * n;
-            Gm[j * n + i] = Gsp[idx];                     // G[j][i] = G^T[i][j]
-            const int e = sp * n + i;
-            const size_t r = (size_t)w * N + e;
-            const double2* dr = D + r * 3 * n;
-            const double2 lp = Lp[r * n + j];
-            const double gx = gUw[3 * e], gy = gUw[3 * e + 1], gz = gUw[3 * e + 2];
-            YK[idx] = make_double2(-0.5 * lp.x - (gx * dr[j].x + gy * dr[n + j].x + gz * dr[2 * n + j].x),
-                                   -0.5 * lp.y - (gx * dr[j].y + gy * dr[n + j].y + gz * dr[2 * n + j].y));
-        }
-        __syncthreads();
-        for (int idx = tid; idx < n * n; idx += nt) {     // T1 = Y G
-            const int i = idx / n, c = idx - i * n;
-            double2 a = czero();
-            for (int j = 0; j < n; ++j) a = cadd(a, cmul(YK[i * n + j], Gm[j * n + c]));
-            T1[idx] = a;
-        }
-        __syncthreads();
-        for (int idx = tid; idx < n * n; idx += nt) {     // K = G T1 (over Y)
-            const int j = idx / n, c = idx - j * n;
-            double2 a = czero();
-            for (int i = 0; i < n; ++i) a = cadd(a, cmul(Gm[j * n + i], T1[i * n + c]));
-            YK[idx] = a;
-        }
-        __syncthreads();
-        for (int a = warp; a < N; a += nw) {
-            double dl[3] = {0, 0, 0}, de[3] = {0, 0, 0};
-            for (int pr = lane; pr < G * n; pr += 32) {
-                const int g = pr / n, il = pr - g * n, b = a * G + g, e = sp * n + il;
-                double2 z = czero(), p = czero();
-                for (int j = 0; j < n; ++j) {
-                    const double c = s.C[(size_t)b * n + j];
-                    z = cadd(z, cscale(Gm[j * n + il], c));
-                    p = cadd(p, cscale(YK[j * n + il], c));
-                }
-                const double x[3] = {X[((size_t)w * N + e) * 3], X[((size_t)w * N + e) * 3 + 1],
-                                     X[((size_t)w * N + e) * 3 + 2]};
-                double d0[3];
-                const double2 P = min_image(x, s.R + 3 * a, s.L, s.iL, th, sg, d0);
-                double2 sa[3][4];
-#pragma unroll
-                for (int mu = 0; mu < 3; ++mu) axis_sums<3>(d0[mu], s.zeta[g], s.L, M, ph + mu * (2 * M + 1), sg, sa[mu]);
-                // grad chi, Hessian, grad lap chi of the Bloch Gaussian (each times P)
-                double2 gr[3], hs[3][3], tl[3];
-#pragma unroll
-                for (int mu = 0; mu < 3; ++mu) {
-                    const int m1 = (mu + 1) % 3, m2 = (mu + 2) % 3;
-                    gr[mu] = cmul(P, cmul(sa[mu][1], cmul(sa[m1][0], sa[m2][0])));
-                    hs[mu][mu] = cmul(P, cmul(sa[mu][2], cmul(sa[m1][0], sa[m2][0])));
-                    hs[mu][m1] = cmul(P, cmul(cmul(sa[mu][1], sa[m1][1]), sa[m2][0]));
-                    hs[mu][m2] = cmul(P, cmul(cmul(sa[mu][1], sa[m2][1]), sa[m1][0]));
-                    tl[mu] = cmul(P, cadd(cmul(sa[mu][3], cmul(sa[m1][0], sa[m2][0])),
-                                          cmul(sa[mu][1], cadd(cmul(sa[m1][2], sa[m2][0]), cmul(sa[m1][0], sa[m2][2])))));
-                }
-                const double* gu = gUw + 3 * e;
-#pragma unroll
-                for (int mu = 0; mu < 3; ++mu) {
-                    const double2 hg = cadd(cadd(cscale(hs[mu][0], gu[0]), cscale(hs[mu][1], gu[1])),
-                                            cscale(hs[mu][2], gu[2]));
-                    const double2 zt = cmul(z, cadd(hg, cscale(tl[mu], 0.5)));
-                    const double2 pg = cmul(p, gr[mu]);
-                    dl[mu] -= cmul(z, gr[mu]).x;
-                    de[mu] += pg.x + zt.x;
-                }
-            }
-#pragma unroll
-            for (int mu = 0; mu < 3; ++mu) { dl[mu] = warp_sum(dl[mu]); de[mu] = warp_sum(de[mu]); }
-            if (lane == 0)
-#pragma unroll
-                for (int mu = 0; mu < 3; ++mu) { fdl[3 * a + mu] += dl[mu]; fde[3 * a + mu] += de[mu]; }
-        }
-        __syncthreads();
-    }
-    const double EL = elw[w];
-    const size_t stride = 3 + 9 * (size_t)N;
-    double* aw = acc + (size_t)w * stride;
-    bool bad = false;
-    for (int c = tid; c < N3; c += nt) {
-        const double dl = fdl[c], de = fde[c];
-        if (!isfinite(dl) || !isfinite(de)) bad = true;
-        aw[3 + c] += dl;
-        aw[3 + N3 + c] += EL * dl;
-        aw[3 + 2 * N3 + c] += de;
-        if (out_dl) { out_dl[(size_t)w * N3 + c] += dl; out_de[(size_t)w * N3 + c] += de; }
-    }
-    if (bad) raise_err(s.err, kErrNonfinite);
-}
-
-size_t twist_pulay_smem_bytes(int N, int n, bool j34) {
-    return (size_t)3 * n * n * sizeof(double2) + (size_t)(j34 ? 15 + 1 + 8 : 15) * N * sizeof(double);
-}
-
-void launch_twist_pulay(const SysView<double>& s, const TwistView& tv, const double* X, const double2* D,
-                        const double2* Lp, const double2* Gt, const double* elw, double* acc, double* out_dl,
-                        double* out_de, cudaStream_t st) {
-    const size_t smem = twist_pulay_smem_bytes(s.N, s.n, s.fj != nullptr);
-    static size_t attr = 0;
-    if (smem > attr &&
-        cudaFuncSetAttribute(twist_pulay_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)
-        attr = smem;
-    twist_pulay_kernel<<<s.W, 256, smem, st>>>(s, tv, X, D, Lp, Gt, elw, acc, out_dl, out_de);
 }
 
 // ---------------------------------------------------------------------------

@@ -58,11 +58,10 @@ void launch_measure(const SysView<float>& s, int ntask, const int4* ktask, const
                     const float* D, const float* Lp, const float* Gt, const double* logdet, double* acc, double* out_el, double* out_lnpsi, double* out_dl,
                     double* out_de, float* kt_out, float* eg_out, double* elw, float* rk_out, cudaStream_t st);
 
-// k_measure64.cu: the same in the FP64 form, straight from the inverses.  gl [W][N][4]:
-// g_i and l_i given (twisted orbitals; the orbital force terms are then left out), or
-// null.  kxyz [3][nk]: the reciprocal vectors.
-void launch_measure64(const SysView<double>& s, int ntask, const int4* ktask, const double* kxyz, const double* X,
-                      const double* Gt, const double* gl, const double* logdet, double* acc, double* out_el,
+// k_measure64.cu: the same in the FP64 form, straight from the inverses (complex
+// ones where tv is given: twisted orbitals).  kxyz [3][nk]: the reciprocal vectors.
+void launch_measure64(const SysView<double>& s, const TwistView* tv, int ntask, const int4* ktask, const double* kxyz,
+                      const double* X, const double* Gt, const double* logdet, double* acc, double* out_el,
                       double* out_lnpsi, double* out_dl, double* out_de, cudaStream_t st);
 
 // k_setup.cu: per-R tables (proton trig, structure factors, p-p Ewald terms; vpp is
@@ -97,19 +96,13 @@ void launch_shard_reduce(int W, int N, const double* acc, const double* sums, do
 void launch_shard_finish(int N, const double* sums, const double* gram, double* out, cudaStream_t st);
 
 // k_twist.cu: twisted boundary conditions (FP64 form, complex orbitals).
-void launch_twist_orbitals(const SysView<double>& s, const TwistView& tv, const double* pos, int nrows,
-                           double2* val, double2* grad, double2* lap, cudaStream_t st);
+void launch_twist_orbitals(const SysView<double>& s, const TwistView& tv, const double* pos, int nrows, double2* val,
+                           cudaStream_t st);
 void launch_twist_invert(int W, int N, int n, const double2* Phi, double2* Gt, double* logdet, int* err,
                          cudaStream_t st);
 void launch_twist_sweep(const SysView<double>& s, const TwistView& tv, double* X, const double* Xp, const double* ptp,
                         const double* uacc, const double2* Phi, double2* Gt, unsigned long long* nacc, double* vep,
                         bool vep_init, cudaStream_t st);
-void launch_twist_gl(int rows, int N, int n, const double2* D, const double2* Lp, const double2* Gt, double* gl,
-                     cudaStream_t st);
-void launch_twist_pulay(const SysView<double>& s, const TwistView& tv, const double* X, const double2* D,
-                        const double2* Lp, const double2* Gt, const double* elw, double* acc, double* out_dl,
-                        double* out_de, cudaStream_t st);
-size_t twist_pulay_smem_bytes(int N, int n, bool j34);
 void launch_twist_average(int K, int N, const double* tout, double* out, cudaStream_t st);
 void launch_twist_partial(int Kr, int N, const double* out, double* part, cudaStream_t st);
 void launch_twist_combine(int K, int N, const double* part, double* out, cudaStream_t st);
