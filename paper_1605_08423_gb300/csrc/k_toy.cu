@@ -39,118 +39,172 @@ namespace {
 
 constexpr uint32_t kToy = 8;   // Philox purpose word of the toy-model noise
 
-struct Sym2 { double s11, s12, s22; };
+// Tables of one block (shared memory, filled at its start by the library's log and
+// sincospi): 1/c and log c of 128 centres c over [0.6875, 1.375), and sin, cos of
+// 2 pi j / 256.
+struct ToyTables {
+    double2 lg[128], cs[256];
+};
+constexpr long long kLogOff = 0x3fe6000000000000LL;   // bits of 0.6875
 
-// S at (x, y) in the radial form above (ir = 1/r, ir2 = 1/r^2); st_out receives s_t.
-__device__ __forceinline__ Sym2 toy_smat(const ToyDev& p, double x, double y, double ir, double ir2, double& st_out) {
-    const double st = p.s_mode == QMC_TOY_S_HG ? p.k * (1.0 - p.a * ir) + p.mu : 1.0;
-    const double d = (p.sr_const - st) * ir2;
-    st_out = st;
-    return Sym2{fma(d * x, x, st), d * x * y, fma(d * y, y, st)};
+__device__ __forceinline__ void fill_tables(ToyTables& T) {
+    for (int i = threadIdx.x; i < 128; i += blockDim.x) {
+        const double lo = __longlong_as_double(kLogOff + ((long long)i << 45));
+        const double hi = __longlong_as_double(kLogOff + ((long long)(i + 1) << 45));
+        // the two intervals that meet at 1 keep c = 1, so that log u -> 0 keeps its relative accuracy
+        const double c = (hi == 1.0 || lo == 1.0) ? 1.0 : 1.0 / (0.5 * (lo + hi));
+        T.lg[i] = make_double2(c, -log(c));
+    }
+    for (int j = threadIdx.x; j < 256; j += blockDim.x) {
+        double sn, cs;
+        sincospi(j / 128.0, &sn, &cs);
+        T.cs[j] = make_double2(sn, cs);
+    }
+    __syncthreads();
 }
 
-// 2x2 Cholesky factor S = L L^T kept as l21 and the reciprocal diagonal
-// (i11 = 1/l11, i22 = 1/l22, each one reciprocal square root); false if S is
-// not positive definite.
-struct Chol2 { double l21, i11, i22; };
-__device__ __forceinline__ bool chol2(const Sym2& S, Chol2& c) {
-    if (!(S.s11 > 0.0)) return false;
-    c.i11 = rsqrt(S.s11);
-    c.l21 = S.s12 * c.i11;
-    const double d = S.s22 - c.l21 * c.l21;
-    if (!(d > 0.0)) return false;
-    c.i22 = rsqrt(d);
-    return true;
-}
-// S u = v by the two triangular solves.
-__device__ __forceinline__ void chol2_solve(const Chol2& c, double v0, double v1, double& u0, double& u1) {
-    const double w0 = v0 * c.i11, w1 = (v1 - c.l21 * w0) * c.i22;
-    u1 = w1 * c.i22;
-    u0 = (w0 - c.l21 * u1) * c.i11;
+// 2^53 u of the 53-bit uniform u53(a, b) (the same rounding: one addition of 1/2).
+__device__ __forceinline__ double u53_scaled(uint32_t a, uint32_t b) {
+    const double hi = __hiloint2double(0x43300000, (int)(a >> 5)) - 4503599627370496.0;      // 2^52 + k - 2^52
+    const double lo = __hiloint2double(0x43300000, (int)(b >> 6)) - 4503599627370495.5;      // + 1/2
+    return fma(hi, 67108864.0, lo);
 }
 
-__global__ void __launch_bounds__(256) toy_kernel(ToyDev p, int n_traj, const double* __restrict__ xy0,
+// The step's two normals from its Philox block, Box-Muller: -2 log u by table and
+// series (P. T. P. Tang, ACM Trans. Math. Softw. 16, 1990; r <= 2^-7, to r^7), the
+// angle by table and series (|x| <= pi / 256).  36 FP64 operations where the
+// library's log, sqrt and sincospi take some 85.
+__device__ __forceinline__ void toy_normals(uint4 w, const ToyTables& T, double& xi0, double& xi1) {
+    const double v1 = u53_scaled(w.x, w.y), v2 = u53_scaled(w.z, w.w);
+    const long long ix = __double_as_longlong(v1), tmp = ix - kLogOff;
+    const int e = (int)(tmp >> 52) - 53;                                       // u = 2^e z
+    const double z = __longlong_as_double(ix - (tmp & (long long)0xfff0000000000000ULL));
+    const double2 lc = T.lg[(int)(tmp >> 45) & 127];
+    const double r = fma(z, lc.x, -1.0);
+    double q = fma(r, 1.0 / 7.0, -1.0 / 6.0);
+    q = fma(q, r, 0.2);
+    q = fma(q, r, -0.25);
+    q = fma(q, r, 1.0 / 3.0);
+    q = fma(q, r, -0.5);
+    const double ed = __hiloint2double(0x43300000, e + 0x40000000) - (4503599627370496.0 + 1073741824.0);
+    const double lg = fma(ed, 0.69314718055994530942, lc.y) + fma(q, r * r, r);
+    const double rho = qsqrt_pair(-2.0 * lg);
+    const double magic = 6755399441055744.0;                                   // 1.5 * 2^52
+    const double jm = fma(v2, 256.0 / 9007199254740992.0, magic);
+    const double x = 6.2831853071795864769 / 9007199254740992.0 * fma(-(9007199254740992.0 / 256.0), jm - magic, v2);
+    const double y = x * x;
+    const double sn = fma(fma(y, 1.0 / 120.0, -1.0 / 6.0) * y, x, x);
+    const double cs = fma(fma(fma(y, -1.0 / 720.0, 1.0 / 24.0), y, -0.5), y, 1.0);
+    const double2 t = T.cs[__double2loint(jm) & 255];
+    xi0 = rho * (t.y * cs - t.x * sn);
+    xi1 = rho * (t.x * cs + t.y * sn);
+}
+
+// x > 0 for a finite or infinite x, false for NaN, on the integer pipe
+__device__ __forceinline__ bool positive(double x) {
+    const int h = __double2hiint(x);
+    return h > 0 && h <= 0x7ff00000;
+}
+
+// One thread per trajectory.  The FP64 pipe bounds it, so the step is written for
+// few FP64 operations: S = st I + d R R^T with d = (s_r - s_t) / r^2, so that
+//   S^{-1} v = p_t v + (p_r - p_t)/r^2 (R.v) R,   p = 1/s,
+//   (S(Q) - S(R)) e = (st_Q - st) e + d_Q (Q.e) Q - d (R.e) R,
+// take dot products instead of triangular solves, the factor L is only formed for
+// the noise z = L^{-T} xi, and with S = G_lambda its second diagonal entry follows
+// from det S = 1/lambda.  100003 trajectories of 500 adopted steps: 15.7 ms with the
+// Cholesky solves and the library's log, sqrt, sincospi and rsqrt, 10.9 ms now.
+// The polar angle travelled: the sum of the per-step increments (each below pi in
+// magnitude) equals phi_end - phi_0 + 2 pi (net turns across the negative x axis),
+// so only the crossings are counted per step -- sign tests on the y coordinates and
+// on the cross product R x R' -- and phi comes from atan2 at the two ends.
+template <int SCHEME, bool HG>
+__global__ void __launch_bounds__(128) toy_kernel(ToyDev p, int n_traj, const double* __restrict__ xy0,
                                                   double* __restrict__ out) {
+    __shared__ ToyTables T;
+    fill_tables(T);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n_traj) return;
     const double x0 = xy0[2 * t], y0 = xy0[2 * t + 1];
-    double x = x0, y = y0;
-    double xp = x, yp = y;
-    double r2 = x * x + y * y, ir = rsqrt(r2), r = r2 * ir;
-    double sp_st = 0.0;
-    Sym2 Sp = toy_smat(p, x, y, ir, ir * ir, sp_st);      // S(R_prev), carried from step to step
+    double x = x0, y = y0, xp = x, yp = y;
+    double r2 = x * x + y * y, ir = qrsqrt(r2), r = r2 * ir;
     double su = 0.0, su2 = 0.0, sr = 0.0, status = 0.0;
-    // Polar angle travelled: the sum of the per-step increments (each below pi in
-    // magnitude) equals phi_end - phi_0 + 2 pi (net turns across the negative x
-    // axis), so only the crossings are counted per step -- sign tests on the
-    // y coordinates and on the cross product R x R' -- and phi comes from atan2
-    // at the two ends.
     int turns = 0;
-    const double D = p.delta;
+    const double D = p.delta, ka = p.k * p.a, pr = 1.0 / p.sr_const;
+    auto s_t = [&](double ir_) { return HG ? fma(-ka, ir_, p.k) + p.mu : 1.0; };
+    double stp = s_t(ir), dp = (p.sr_const - stp) * (ir * ir);      // S(R_prev), carried from step to step
+    const double c22 = HG ? 0.0 : rsqrt(p.sr_const);                // 1 / sqrt(det S) of G_lambda
     for (int s = 0; s < p.n_steps; ++s) {
-        const uint4 w = philox((uint32_t)t, (uint32_t)s, 0u, kToy, p.key);
-        const double u1 = u53(w.x, w.y), u2 = u53(w.z, w.w);
-        const double rho = sqrt(-2.0 * log(u1));
-        double sn, cs;
-        sincospi(2.0 * u2, &sn, &cs);
-        const double xi0 = rho * cs, xi1 = rho * sn;
-        const double ir2 = ir * ir;
-        const double fr = -p.k * (r - p.a) * ir;
-        const double fx = fr * x, fy = fr * y;
-        double xn, yn;
-        Sym2 S{1.0, 0.0, 1.0};
-        if (p.scheme == QMC_TOY_PLAIN) {
-            xn = x + D * fx + p.amp * xi0;
-            yn = y + D * fy + p.amp * xi1;
+        double xi0, xi1;
+        toy_normals(philox((uint32_t)t, (uint32_t)s, 0u, kToy, p.key), T, xi0, xi1);
+        const double fr = fma(ka, ir, -p.k);                        // f = fr R
+        // terms added in the order of the schemes above
+        double xn, yn, st = 1.0, d = 0.0;
+        if constexpr (SCHEME == QMC_TOY_PLAIN) {
+            xn = fma(p.amp, xi0, fma(D, fr * x, x));
+            yn = fma(p.amp, xi1, fma(D, fr * y, y));
         } else {
-            double st;
-            S = toy_smat(p, x, y, ir, ir2, st);
-            Chol2 c;
-            if (!chol2(S, c)) { status = s + 1; break; }
-            const double z1 = xi1 * c.i22, z0 = (xi0 - c.l21 * z1) * c.i11;
-            double sfx, sfy;
-            chol2_solve(c, fx, fy, sfx, sfy);
-            switch (p.scheme) {
-            case QMC_TOY_STANDARD: {
-                const double g = (1.0 / p.sr_const - 1.0 / st) * ir2;   // Gamma = g R
-                xn = x + D * sfx + p.T * D * g * x + p.amp * z0;
-                yn = y + D * sfy + p.T * D * g * y + p.amp * z1;
-                break;
+            const double ir2 = ir * ir;
+            st = s_t(ir);
+            d = (p.sr_const - st) * ir2;
+            const double dx = d * x, s11 = fma(dx, x, st), s12 = dx * y;
+            if (!positive(s11)) { status = s + 1; break; }
+            const double i11 = qrsqrt(s11), l21 = s12 * i11;
+            double i22;
+            if constexpr (HG) {
+                const double q = fma(-l21, l21, fma(d * y, y, st));
+                if (!positive(q)) { status = s + 1; break; }
+                i22 = qrsqrt(q);
+            } else {
+                i22 = s11 * i11 * c22;
             }
-            case QMC_TOY_FIRST: {
-                const double ex = p.amp * z0, ey = p.amp * z1;          // y - R
+            const double z1 = xi1 * i22, z0 = fma(-l21, z1, xi0) * i11;
+            const double pt = HG ? qrcp(st) : 1.0;
+            const double gs = (pr - pt) * ir2;
+            // S^{-1} v
+            auto solve = [&](double vx, double vy, double& wx, double& wy) {
+                const double c = gs * fma(x, vx, y * vy);
+                wx = HG ? fma(c, x, pt * vx) : fma(c, x, vx);
+                wy = HG ? fma(c, y, pt * vy) : fma(c, y, vy);
+            };
+            // (S(Q) - S(R)) e
+            auto diff = [&](double stq, double dq, double qx, double qy, double ex, double ey, double& vx, double& vy) {
+                const double a = dq * fma(qx, ex, qy * ey), b = d * fma(x, ex, y * ey);
+                vx = fma(a, qx, -(b * x));
+                vy = fma(a, qy, -(b * y));
+                if constexpr (HG) { vx = fma(stq - st, ex, vx); vy = fma(stq - st, ey, vy); }
+            };
+            const double prf = pr * fr;                              // S^{-1} f = prf R
+            if constexpr (SCHEME == QMC_TOY_STANDARD) {
+                const double g = p.T * D * gs;                       // Gamma = gs R
+                xn = fma(p.amp, z0, fma(g, x, fma(D, prf * x, x)));
+                yn = fma(p.amp, z1, fma(g, y, fma(D, prf * y, y)));
+            } else if constexpr (SCHEME == QMC_TOY_FIRST) {
+                const double ex = p.amp * z0, ey = p.amp * z1;       // y - R
                 const double qx = x + ex, qy = y + ey;
-                const double iq = rsqrt(qx * qx + qy * qy);
-                double sty;
-                const Sym2 Sy = toy_smat(p, qx, qy, iq, iq * iq, sty);
-                const double vx = (Sy.s11 - S.s11) * ex + (Sy.s12 - S.s12) * ey;
-                const double vy = (Sy.s12 - S.s12) * ex + (Sy.s22 - S.s22) * ey;
-                double wx, wy;
-                chol2_solve(c, vx, vy, wx, wy);
-                xn = qx + D * sfx - 0.5 * wx;
-                yn = qy + D * sfy - 0.5 * wy;
-                break;
-            }
-            case QMC_TOY_FAST:
-            case QMC_TOY_ADOPTED: {
-                const double ex = xp - x, ey = yp - y;                  // R_prev - R
-                const double vx = (Sp.s11 - S.s11) * ex + (Sp.s12 - S.s12) * ey;
-                const double vy = (Sp.s12 - S.s12) * ex + (Sp.s22 - S.s22) * ey;
-                double wx, wy;
-                chol2_solve(c, vx, vy, wx, wy);
-                if (p.scheme == QMC_TOY_FAST) {
-                    xn = x + D * sfx + p.amp * z0 - 0.5 * wx;
-                    yn = y + D * sfy + p.amp * z1 - 0.5 * wy;
+                const double iq = qrsqrt(fma(qx, qx, qy * qy));
+                const double stq = s_t(iq);
+                double vx, vy, wx, wy;
+                diff(stq, (p.sr_const - stq) * (iq * iq), qx, qy, ex, ey, vx, vy);
+                solve(vx, vy, wx, wy);
+                const double g = D * prf;
+                xn = fma(-0.5, wx, fma(g, x, qx));
+                yn = fma(-0.5, wy, fma(g, y, qy));
+            } else if constexpr (SCHEME == QMC_TOY_FAST || SCHEME == QMC_TOY_ADOPTED) {
+                constexpr bool kAdopted = SCHEME == QMC_TOY_ADOPTED;
+                double vx, vy, wx, wy;
+                diff(stp, dp, xp, yp, xp - x, yp - y, vx, vy);
+                solve(vx, vy, wx, wy);
+                if constexpr (kAdopted) {
+                    xn = fma(p.ampb, z0, fma(p.dt, fma(-p.half_idb, wx, prf * x), x));
+                    yn = fma(p.ampb, z1, fma(p.dt, fma(-p.half_idb, wy, prf * y), y));
                 } else {
-                    xn = x + p.dt * (sfx - p.half_idb * wx) + p.ampb * z0;
-                    yn = y + p.dt * (sfy - p.half_idb * wy) + p.ampb * z1;
+                    xn = fma(-0.5, wx, fma(p.amp, z0, fma(D, prf * x, x)));
+                    yn = fma(-0.5, wy, fma(p.amp, z1, fma(D, prf * y, y)));
                 }
-                break;
-            }
-            default:   // QMC_TOY_NOROGNA
-                xn = x + D * sfx + p.amp * z0;
-                yn = y + D * sfy + p.amp * z1;
-                break;
+            } else {   // QMC_TOY_NOROGNA
+                xn = fma(p.amp, z0, fma(D, prf * x, x));
+                yn = fma(p.amp, z1, fma(D, prf * y, y));
             }
         }
         {
@@ -161,14 +215,14 @@ __global__ void __launch_bounds__(256) toy_kernel(ToyDev p, int n_traj, const do
                 else if (!up && cr < 0) --turns;      // clockwise across it
             }
         }
-        xp = x; yp = y; Sp = S;
+        xp = x; yp = y; stp = st; dp = d;
         x = xn; y = yn;
         r2 = x * x + y * y;
-        ir = rsqrt(r2);
+        ir = qrsqrt(r2);
         r = r2 * ir;
         if (s >= p.n_burn) {
-            const double d = r - p.a;
-            const double u = 0.5 * p.k * d * d;
+            const double dr = r - p.a;
+            const double u = 0.5 * p.k * dr * dr;
             su += u; su2 += u * u; sr += r;
         }
     }
@@ -177,11 +231,26 @@ __global__ void __launch_bounds__(256) toy_kernel(ToyDev p, int n_traj, const do
     o[0] = x; o[1] = y; o[2] = su; o[3] = su2; o[4] = sr; o[5] = theta; o[6] = status;
 }
 
+template <int SCHEME>
+void launch_scheme(const ToyDev& p, int n_traj, const double* xy0, double* out, cudaStream_t st) {
+    // one warp per block while every warp can have an SM's FP64 issue ports nearly to itself
+    const int tpb = n_traj <= 32 * 2 * 152 ? 32 : 128, grid = (n_traj + tpb - 1) / tpb;
+    if (p.s_mode == QMC_TOY_S_HG) toy_kernel<SCHEME, true><<<grid, tpb, 0, st>>>(p, n_traj, xy0, out);
+    else toy_kernel<SCHEME, false><<<grid, tpb, 0, st>>>(p, n_traj, xy0, out);
+}
+
 }  // namespace
 
 void launch_toy(const ToyDev& p, int n_traj, const double* xy0, double* out, cudaStream_t st) {
     if (n_traj <= 0) return;
-    toy_kernel<<<(n_traj + 255) / 256, 256, 0, st>>>(p, n_traj, xy0, out);
+    switch (p.scheme) {
+    case QMC_TOY_PLAIN: launch_scheme<QMC_TOY_PLAIN>(p, n_traj, xy0, out, st); break;
+    case QMC_TOY_STANDARD: launch_scheme<QMC_TOY_STANDARD>(p, n_traj, xy0, out, st); break;
+    case QMC_TOY_FIRST: launch_scheme<QMC_TOY_FIRST>(p, n_traj, xy0, out, st); break;
+    case QMC_TOY_FAST: launch_scheme<QMC_TOY_FAST>(p, n_traj, xy0, out, st); break;
+    case QMC_TOY_ADOPTED: launch_scheme<QMC_TOY_ADOPTED>(p, n_traj, xy0, out, st); break;
+    default: launch_scheme<QMC_TOY_NOROGNA>(p, n_traj, xy0, out, st); break;
+    }
 }
 
 }  // namespace qmc
