@@ -12,8 +12,8 @@
 
 namespace qmc {
 
-// Mixed form.  Q = 1: values only (proposal rows / Slater matrix).
-// Q = 5: value, d/dx, d/dy, d/dz, Laplacian (local energy).
+// Mixed form.  Q = 1: values (proposal rows / Slater matrix).
+// Q = 4: d/dx, d/dy, d/dz, Laplacian (local energy; it needs no values).
 template <typename T, int Q, int NP>
 __global__ void __launch_bounds__(512) orbitals_simt(SysView<T> s, const double* __restrict__ pos, int nrows,
                                                      T* __restrict__ val, T* __restrict__ grad, T* __restrict__ lap) {
@@ -68,14 +68,15 @@ __global__ void __launch_bounds__(512) orbitals_simt(SysView<T> s, const double*
                 t *= ell * ell;
                 const T z = s.zetat[g];
                 const T e = qexp(-z * t);
-                v[0] = e;
-                if (Q == 5) {
+                if constexpr (Q == 1) {
+                    v[0] = e;
+                } else {
                     const T f1 = -z * e, f2 = z * z * e;
                     T pp = 0, sq = 0;
 #pragma unroll
                     for (int mu = 0; mu < 3; ++mu) {
                         const T p = ell * sd[mu] * cd[mu], qq = cd[mu] * cd[mu] - sd[mu] * sd[mu];
-                        v[1 + mu] = T(2) * f1 * p;
+                        v[mu] = T(2) * f1 * p;
                         pp += p * p; sq += qq;
                     }
                     v[Q - 1] = T(4) * f2 * pp + T(2) * f1 * sq;
@@ -112,10 +113,11 @@ __global__ void __launch_bounds__(512) orbitals_simt(SysView<T> s, const double*
         for (int m = 0; m < 4; ++m) {
             const int j = c0 + m;
             if (j >= n) continue;
-            val[(size_t)row * n + j] = acc[0][a][m];
-            if (Q == 5) {
+            if constexpr (Q == 1) {
+                val[(size_t)row * n + j] = acc[0][a][m];
+            } else {
 #pragma unroll
-                for (int mu = 0; mu < 3; ++mu) grad[((size_t)row * 3 + mu) * n + j] = acc[1 + mu][a][m];
+                for (int mu = 0; mu < 3; ++mu) grad[((size_t)row * 3 + mu) * n + j] = acc[mu][a][m];
                 lap[(size_t)row * n + j] = acc[Q - 1][a][m];
             }
         }
@@ -234,7 +236,7 @@ static void launch_orb(const SysView<float>& s, const double* pos, int nrows, fl
 
 void launch_orbitals(const SysView<float>& s, const double* pos, int nrows, float* val, float* grad, float* lap,
                      cudaStream_t st) {
-    if (grad) launch_orb<5>(s, pos, nrows, val, grad, lap, st);
+    if (grad) launch_orb<4>(s, pos, nrows, nullptr, grad, lap, st);
     else launch_orb<1>(s, pos, nrows, val, nullptr, nullptr, st);
 }
 
