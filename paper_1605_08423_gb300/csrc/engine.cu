@@ -355,7 +355,7 @@ void measure(qmc_system* h, const SysView<float>& s, double* el, double* lnpsi, 
     prof_end(h, ep);
     const bool split = h->use_tc && h->use_tc_adj;
     prof_begin(h, KC_MEASURE, ep);
-    launch_measure(s, h->nktask, h->d_ktask, h->d_kint, h->d_X, (const float*)h->d_D, (const float*)h->d_Lp, (const float*)h->d_Gt, h->d_logdet, h->d_acc,
+    launch_measure(s, h->nktask, h->d_ktask, h->d_kint, h->d_X, (const float*)h->d_D, (float*)h->d_Lp, (const float*)h->d_Gt, h->d_logdet, h->d_acc,
                    el, lnpsi, dl, de, split ? h->d_Kt : nullptr, split ? h->d_eg : nullptr,
                    split ? h->d_elw : nullptr, split ? h->d_rk : nullptr, h->stream);
     prof_end(h, ep);

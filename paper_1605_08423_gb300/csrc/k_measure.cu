@@ -255,7 +255,7 @@ template <bool kSplit>
 __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax, int ntask,
                                                       const int4* __restrict__ ktask, const T* __restrict__ kint,
                                                       const double* __restrict__ X,
-                                                      const T* __restrict__ D, const T* __restrict__ Lp,
+                                                      const T* __restrict__ D, T* LpY,
                                                       const T* __restrict__ Gt, const double* __restrict__ logdet,
                                                       double* __restrict__ acc, double* __restrict__ out_el,
                                                       double* __restrict__ out_lnpsi, double* __restrict__ out_dl,
@@ -437,32 +437,6 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
         gU[3 * i] = v[0]; gU[3 * i + 1] = v[1]; gU[3 * i + 2] = v[2];
         lU[i] = v[3]; Ui[i] = v[4];
     }
-
-    // ---- P2: g_i = sum_j D_ij G_ji, l_i = sum_j Lp_ij G_ji (warp per electron,
-    // lanes over the orbitals: coalesced rows of D, Lp and G^T)
-    // Two electrons at a time: twice the loads in flight, and one packed sum.
-    for (int i0 = warp; i0 < N; i0 += 2 * nw) {
-        T v[8] = {};
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int i = i0 + e * nw < N ? i0 + e * nw : i0;
-            const int sp = i / n, il = i - sp * n;
-            const T* grow = Gt + (((size_t)w * 2 + sp) * n + il) * n;
-            const T* drow = D + ((size_t)w * N + i) * 3 * n;
-            const T* lrow = Lp + ((size_t)w * N + i) * n;
-            for (int j = lane; j < n; j += 32) {
-                const T gj = grow[j];
-                v[4 * e] += drow[j] * gj; v[4 * e + 1] += drow[n + j] * gj; v[4 * e + 2] += drow[2 * n + j] * gj;
-                v[4 * e + 3] += lrow[j] * gj;
-            }
-        }
-        const T x = warp_sum8(v, lane);
-        const int q = lane >> 2, i = i0 + (q >> 2) * nw, c = q & 3;
-        if ((lane & 3) == 0 && i < N) {
-            if (c < 3) gi[3 * i + c] = x;
-            else li[i] = x;
-        }
-    }
     __syncthreads();
 
     // ---- P2b (with the e-e-n-n Jastrow term):
@@ -548,6 +522,54 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
         }
         __syncthreads();
     }
+
+    // ---- P2: g_i = sum_j D_ij G_ji, l_i = sum_j Lp_ij G_ji (warp per electron,
+    // lanes over the orbitals: coalesced rows of D, Lp and G^T)
+    // Two electrons at a time: twice the loads in flight, and one packed sum.  The
+    // same pass over D and Lp forms Y_ij = -1/2 Lp_ij - grad_i U . D_ij for the
+    // orbital force terms, which go into Lp's place (P6 read D and Lp once more
+    // before: 4 n values an electron from memory where it now reads n).
+    for (int i0 = warp; i0 < N; i0 += 2 * nw) {
+        T v[8] = {}, r[2][2][5];                 // [electron][j = lane, lane + 32]: G, D (3), Lp
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int i = i0 + e * nw, sp = i / n, il = i - sp * n;
+            const T* grow = Gt + (((size_t)w * 2 + sp) * n + il) * n;
+            const T* drow = D + ((size_t)w * N + i) * 3 * n;
+            const T* lrow = LpY + ((size_t)w * N + i) * n;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int j = lane + 32 * h;
+                const bool on = i < N && j < n;
+                r[e][h][0] = on ? grow[j] : T(0);
+                r[e][h][1] = on ? drow[j] : T(0);
+                r[e][h][2] = on ? drow[n + j] : T(0);
+                r[e][h][3] = on ? drow[2 * n + j] : T(0);
+                r[e][h][4] = on ? lrow[j] : T(0);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int i = i0 + e * nw;
+            if (i >= N) continue;
+            T* lrow = LpY + ((size_t)w * N + i) * n;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int j = lane + 32 * h;
+                const T gj = r[e][h][0], dx = r[e][h][1], dy = r[e][h][2], dz = r[e][h][3], lp = r[e][h][4];
+                v[4 * e] += dx * gj; v[4 * e + 1] += dy * gj; v[4 * e + 2] += dz * gj;
+                v[4 * e + 3] += lp * gj;
+                if (j < n) lrow[j] = T(-0.5) * lp - (gU[3 * i] * dx + gU[3 * i + 1] * dy + gU[3 * i + 2] * dz);
+            }
+        }
+        const T x = warp_sum8(v, lane);
+        const int q = lane >> 2, i = i0 + (q >> 2) * nw, c = q & 3;
+        if ((lane & 3) == 0 && i < N) {
+            if (c < 3) gi[3 * i + c] = x;
+            else li[i] = x;
+        }
+    }
+    __syncthreads();
 
     // ---- P3: kinetic energy and U
     double kin_p = 0.0, u_p = 0.0;
@@ -900,12 +922,8 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
                 const int il = idx >> lnp, j = idx & (np - 1);
                 T g = 0, y = 0;
                 if (il < n && j < n) {
-                    const int i = sp * n + il;
                     g = Gsp[il * n + j];
-                    const size_t rr = (size_t)w * N + i;
-                    const T* dr = D + rr * 3 * n;
-                    y = T(-0.5) * Lp[rr * n + j] -
-                        (gU[3 * i] * dr[j] + gU[3 * i + 1] * dr[n + j] + gU[3 * i + 2] * dr[2 * n + j]);
+                    y = LpY[((size_t)w * N + sp * n + il) * n + j];
                 }
                 bufG2[j * ldt + il] = g;
                 bufY[j * ldt + il] = y;
@@ -1008,11 +1026,8 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
             const int il = idx >> lnp, j = idx & (np - 1);
             T g = 0, y = 0;
             if (il < n && j < n) {
-                const int i = sp * n + il;
                 g = Gsp[il * n + j];
-                const size_t rr = (size_t)w * N + i;
-                const T* dr = D + rr * 3 * n;
-                y = T(-0.5) * Lp[rr * n + j] - (gU[3 * i] * dr[j] + gU[3 * i + 1] * dr[n + j] + gU[3 * i + 2] * dr[2 * n + j]);
+                y = LpY[((size_t)w * N + sp * n + il) * n + j];
             }
             bufS[il * ldt + j] = g;
             bufG[j * ldt + il] = g;
@@ -1176,7 +1191,7 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
 }  // namespace
 
 void launch_measure(const SysView<float>& s, int ntask, const int4* ktask, const float* kint,
-                    const double* X, const float* D, const float* Lp, const float* Gt,
+                    const double* X, const float* D, float* LpY, const float* Gt,
                     const double* logdet, double* acc, double* out_el, double* out_lnpsi, double* out_dl,
                     double* out_de, float* kt_out, float* eg_out, double* elw, float* rk_out, cudaStream_t st) {
     const bool split = kt_out != nullptr;
@@ -1190,10 +1205,10 @@ void launch_measure(const SysView<float>& s, int ntask, const int4* ktask, const
         attr_set[split] = true;
     }
     if (split)
-        measure_kernel<true><<<s.W, 256, smem, st>>>(s, s.mmax, ntask, ktask, kint, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
+        measure_kernel<true><<<s.W, 256, smem, st>>>(s, s.mmax, ntask, ktask, kint, X, D, LpY, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
                                                      out_de, kt_out, eg_out, elw, rk_out);
     else
-        measure_kernel<false><<<s.W, 256, smem, st>>>(s, s.mmax, ntask, ktask, kint, X, D, Lp, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
+        measure_kernel<false><<<s.W, 256, smem, st>>>(s, s.mmax, ntask, ktask, kint, X, D, LpY, Gt, logdet, acc, out_el, out_lnpsi, out_dl,
                                                       out_de, nullptr, nullptr, nullptr, nullptr);
 }
 

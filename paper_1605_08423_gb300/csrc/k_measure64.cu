@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(kThreads, TM ? 2 : 1) measure64_kernel(SysView
     // (the orbital products use the work space in between).
     double* j34c = uni;              // [N]
     double* j34S = j34c + N;         // [N][3]
-    double* st = j34S + 3 * N + (size_t)warp * 5 * N;   // per warp: chi_i [N], grad chi_i [N][3], lap chi_i [N]
+    double* st = j34S + 3 * N + (size_t)warp * 5 * N;   // per warp: c - chi_i [N], grad chi_i [N][3], lap chi_i [N]
     const double zj = s.zeta_j;
     auto j34_sums = [&]() {
         for (int a = tid; a < N; a += kThreads) {
@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(kThreads, TM ? 2 : 1) measure64_kernel(SysView
         for (int i = warp; i < N; i += kWarps) {
             for (int a = lane; a < N; a += 32) {
                 RadialDerivs<double> rd;
-                st[a] = jas34(et + 6 * i, s.ptrig + 6 * a, ell, zj, k2, rd);
+                st[a] = j34c[a] - jas34(et + 6 * i, s.ptrig + 6 * a, ell, zj, k2, rd);
             }
             __syncwarp();
             double g[3] = {0, 0, 0}, l = 0, u = 0;
@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(kThreads, TM ? 2 : 1) measure64_kernel(SysView
                 const double chi = jas34(et + 6 * i, s.ptrig + 6 * a, ell, zj, k2, rd);
                 const double* fa = s.fj + a;   // column a = row a (f symmetric): coalesced over lanes
                 double wa = 0;
-                for (int b = 0; b < N; ++b) wa += fa[(size_t)b * N] * (j34c[b] - st[b]);
+                for (int b = 0; b < N; ++b) wa += fa[(size_t)b * N] * st[b];
                 for (int mu = 0; mu < 3; ++mu) g[mu] += rd.g[mu] * wa;
                 l += rd.lap * wa;
                 u += chi * wa;
@@ -733,7 +733,7 @@ __global__ void __launch_bounds__(kThreads, TM ? 2 : 1) measure64_kernel(SysView
         for (int i = warp; i < N; i += kWarps) {
             for (int a = lane; a < N; a += 32) {
                 RadialDerivs<double> rd;
-                st[a] = jas34(et + 6 * i, s.ptrig + 6 * a, ell, zj, k2, rd);
+                st[a] = j34c[a] - jas34(et + 6 * i, s.ptrig + 6 * a, ell, zj, k2, rd);
                 for (int mu = 0; mu < 3; ++mu) st[N + 3 * a + mu] = rd.g[mu];
                 st[4 * N + a] = rd.lap;
             }
@@ -747,7 +747,7 @@ __global__ void __launch_bounds__(kThreads, TM ? 2 : 1) measure64_kernel(SysView
                 double wa = 0, v[3] = {0, 0, 0}, lam = 0;
                 for (int b = 0; b < N; ++b) {
                     const double f = fa[(size_t)b * N];
-                    wa += f * (j34c[b] - st[b]);
+                    wa += f * st[b];
                     for (int mu = 0; mu < 3; ++mu) v[mu] += st[N + 3 * b + mu] * f;
                     lam += st[4 * N + b] * f;
                 }

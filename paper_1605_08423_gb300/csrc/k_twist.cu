@@ -299,8 +299,8 @@ __global__ void __launch_bounds__(256) twist_sweep_kernel(SysView<double> s, Twi
     double* et = ptb + 6;                    // [N][6] electron trig
     double* vj = et + 6 * N;                 // [N] V_i = sum_a u_en(r_i, R_a), carried as in sweep_kernel
     double* c34 = vj + N;                    // [N] sum over electrons of chi_a (e-e-n-n term)
-    double* cho = c34 + N;                   // [N] chi_a at the moving electron
-    double* chn = cho + N;                   // [N] chi_a at its proposal
+    double* dif = c34 + N;                   // [N] c_a - chi_a at the moving electron
+    double* dch = dif + N;                   // [N] change of chi_a at its proposal
     for (int idx = threadIdx.x; idx < 6 * N; idx += blockDim.x) ptr_s[idx] = s.ptrig[idx];
     __syncthreads();
     const int w = blockIdx.x * wpb + warp;
@@ -361,15 +361,16 @@ __global__ void __launch_bounds__(256) twist_sweep_kernel(SysView<double> s, Twi
             for (int a = lane; a < N; a += 32) vnew += tw_pade_u(ptb, ptr_s + 6 * a, ell, bep, -Zj);
             if (j34) {
                 for (int a = lane; a < N; a += 32) {
-                    chn[a] = tw_jas_orbital(ptb, ptr_s + 6 * a, ell, zj);
-                    cho[a] = tw_jas_orbital(ei, ptr_s + 6 * a, ell, zj);
+                    const double old = tw_jas_orbital(ei, ptr_s + 6 * a, ell, zj);
+                    dch[a] = tw_jas_orbital(ptb, ptr_s + 6 * a, ell, zj) - old;
+                    dif[a] = c34[a] - old;
                 }
                 __syncwarp();
                 for (int a = lane; a < N; a += 32) {
                     const double* fa = s.fj + a;   // f symmetric: column a = row a, consecutive over lanes
                     double wa = 0;
-                    for (int b = 0; b < N; ++b) wa += fa[(size_t)b * N] * (c34[b] - cho[b]);
-                    du += (chn[a] - cho[a]) * wa;
+                    for (int b = 0; b < N; ++b) wa += fa[(size_t)b * N] * dif[b];
+                    du += dch[a] * wa;
                 }
             }
             // the four warp sums in seven additions: each half of the warp keeps two
@@ -422,7 +423,7 @@ __global__ void __launch_bounds__(256) twist_sweep_kernel(SysView<double> s, Twi
                     for (int j = lane; j < n; j += 32) Gs[il * ld + j] = cmul(Gs[il * ld + j], f);
                 }
                 if (j34)
-                    for (int a = lane; a < N; a += 32) c34[a] += chn[a] - cho[a];
+                    for (int a = lane; a < N; a += 32) c34[a] += dch[a];
                 ++naccept;
             }
             __syncwarp();

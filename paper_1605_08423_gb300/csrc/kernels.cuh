@@ -54,9 +54,10 @@ int walkers_per_cta(int W, int most);
 // k_measure.cu: local energy, d ln psi / dR and dE_L / dR per walker, mixed form.
 // ktask [ntask]: structure-factor tasks, (m_x, m_y, first of two |m_z|, index of
 // (m_x, m_y, 0)).
+// LpY: lap phi rows, overwritten with Y.
 // kint [3][nk]: the integer vectors (m_x, m_y, m_z) of the reciprocal vectors.
 void launch_measure(const SysView<float>& s, int ntask, const int4* ktask, const float* kint, const double* X,
-                    const float* D, const float* Lp, const float* Gt, const double* logdet, double* acc, double* out_el, double* out_lnpsi, double* out_dl,
+                    const float* D, float* LpY, const float* Gt, const double* logdet, double* acc, double* out_el, double* out_lnpsi, double* out_dl,
                     double* out_de, float* kt_out, float* eg_out, double* elw, float* rk_out, cudaStream_t st);
 
 // k_measure64.cu: the same in the FP64 form, straight from the inverses (complex
