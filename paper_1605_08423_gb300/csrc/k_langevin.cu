@@ -93,7 +93,9 @@ __global__ void __launch_bounds__(kLvThreads) first_correct_kernel(int n, double
     __syncthreads();
     for (int k = 0; k < (n + kLvTb - 1) / kLvTb; ++k) {
         lv_load_diag(n, Lc, k, sm);
-        lv_forward_block(n, Lc, k, g, sm);
+        lv_forward_diag(n, k, g, sm);
+        __syncthreads();
+        lv_forward_rows(n, Lc, k, g, sm);
     }
     double* const w[2] = {g, g};
     lv_backward(n, Lc, w, 1, sm);

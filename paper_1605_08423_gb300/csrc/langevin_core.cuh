@@ -15,7 +15,7 @@
 // What bounds it: an SM issues two FP64 multiply-adds a clock, so the n^3/6 of
 // n = 384 take 2.3 ms on one SM; 16 SMs bring that under the chain of diagonal
 // tiles and barriers.  One CTA, column by column, took 11.5 ms at n = 384 and
-// 0.77 ms at n = 48 (1.03 and 0.15 ms in this form).
+// 0.77 ms at n = 48 (0.68 and 0.10 ms in this form).
 #pragma once
 #include <cooperative_groups.h>
 
@@ -157,10 +157,9 @@ __device__ inline void lv_update_tile(int n, double* Lc, int k, int I, int J, Lv
         }
 }
 
-// The CTA: block k of the forward solve L y = g (g in shared memory, solved in
-// place), sm.D holding diagonal tile k: the block itself by one warp, then the
-// rows below, one per thread.
-__device__ inline void lv_forward_block(int n, const double* Lc, int k, double* g, LvSmem& sm) {
+// Block k of the forward solve L y = g (g in shared memory, solved in place), sm.D
+// holding diagonal tile k: the block itself by warp 0 (y_k also to sm.yk[0]) ...
+__device__ inline void lv_forward_diag(int n, int k, double* g, LvSmem& sm) {
     const int tid = threadIdx.x, k0 = k * kLvTb;
     if (tid < 32) {
         double v = k0 + tid < n ? g[k0 + tid] : 0.0;
@@ -172,8 +171,11 @@ __device__ inline void lv_forward_block(int n, const double* Lc, int k, double* 
         sm.yk[0][tid] = v;
         if (k0 + tid < n) g[k0 + tid] = v;
     }
-    __syncthreads();
-    for (int i = k0 + kLvTb + tid; i < n; i += kLvThreads) {
+}
+// ... then the rows below, one per thread.
+__device__ inline void lv_forward_rows(int n, const double* Lc, int k, double* g, const LvSmem& sm) {
+    const int k0 = k * kLvTb;
+    for (int i = k0 + kLvTb + threadIdx.x; i < n; i += kLvThreads) {
         const double* p = Lc + (size_t)i * n + k0;
         double s0 = 0, s1 = 0;
 #pragma unroll 8
@@ -242,25 +244,25 @@ __device__ inline bool lv_cholesky(cg::cluster_group& cl, int n, const double* _
         const int m = nt - 1 - k;                       // row tiles below
         for (int q = rank + P * (warp >> 2); q < m; q += P * (kLvThreads / 128))
             lv_solve_rows(n, Lc, k, k + 1 + q, warp & 3, sm);
+        if (g) lv_forward_diag(n, k, g, sm);            // the last CTA has no row tile when P > m
         cl.sync();
-        // trailing tiles in column order; the first CTA takes (k+1, k+1) and
-        // its factorisation (about a tile's time), the others go round
+        // trailing tiles in column order; the first CTA takes (k+1, k+1) and its
+        // factorisation (about a tile's time) and joins once the others have two each
+        // (half tiles balance the end better but load as much each: 0.72 ms for 0.68)
         if (rank == 0 && m > 0) {
             lv_update_tile(n, Lc, k, k + 1, k + 1, sm);
             __syncthreads();
             if (warp < 4 && !lv_factor_tile(n, Lc, k + 1, sm) && tid == 0) sm.fail = 1;
         }
-        const int total = m * (m + 1) / 2;
-        int t = 1, J = 0, base = 0;                      // tile t of column J starts at base
-        for (; t < total; ++t) {
-            const int slot = t + (t >= P ? 1 : 0);       // slot P (the first CTA's second turn) is the factorisation
-            if (slot % P != rank) continue;
+        if (g) lv_forward_rows(n, Lc, k, g, sm);
+        const int total = m * (m + 1) / 2, head = 2 * (P - 1);
+        int J = 0, base = 0;                            // tile t of column J starts at base
+        for (int t = 1; t < total; ++t) {
+            const int q = t - 1;
+            const int owner = P == 1 ? 0 : q < head ? 1 + q % (P - 1) : (q - head) % P;
+            if (owner != rank) continue;
             while (t >= base + (m - J)) { base += m - J; ++J; }
             lv_update_tile(n, Lc, k, k + 1 + J + (t - base), k + 1 + J, sm);
-        }
-        if (g) {
-            __syncthreads();
-            lv_forward_block(n, Lc, k, g, sm);
         }
         cl.sync();
     }
