@@ -436,12 +436,12 @@ __device__ __forceinline__ double ewald_table(double dx, double dy, double dz, c
     // moving component m of the minimum image by L away from zero adds L (L - 2 |d_m|) to r^2
     const double e0 = fma(-2.0 * L, fabs(dx), T.LL), e1 = fma(-2.0 * L, fabs(dy), T.LL),
                  e2 = fma(-2.0 * L, fabs(dz), T.LL);
-    const double r1 = r0 + e0, r2 = r0 + e1, r3 = r1 + e1, r4 = r0 + e2;
+    const double r1 = r0 + e0, r2 = r0 + e1, r3 = r1 + e1, r4 = r0 + e2, r5 = r1 + e2, r6 = r2 + e2, r7 = r3 + e2;
     // positive doubles compare as their bit patterns (integer pipe)
     const long long lim = __double_as_longlong(T.LL);
     auto in = [&](double r) { return __double_as_longlong(r) < lim; };
     unsigned mask = (in(r1) ? 2u : 0u) | (in(r2) ? 4u : 0u) | (in(r3) ? 8u : 0u) | (in(r4) ? 16u : 0u) |
-                    (in(r1 + e2) ? 32u : 0u) | (in(r2 + e2) ? 64u : 0u) | (in(r3 + e2) ? 128u : 0u);
+                    (in(r5) ? 32u : 0u) | (in(r6) ? 64u : 0u) | (in(r7) ? 128u : 0u);
     double v = 0, s = 0, s0 = 0, s1 = 0, s2 = 0, d;
     if (__double_as_longlong(r0) > 0) {
         const double ir = qrsqrt(r0);
@@ -451,8 +451,10 @@ __device__ __forceinline__ double ewald_table(double dx, double dy, double dz, c
     while (mask) {
         const int c = __ffs(mask) - 1;
         mask &= mask - 1;
-        const double ra = (c & 1) ? e0 : 0.0, rb = (c & 2) ? e1 : 0.0, rc = (c & 4) ? e2 : 0.0;
-        v += ew_eval<kGrad>(T, 1, r0 + ra + rb + rc, &d);
+        // selected, not summed again: selects run on the integer pipe
+        const double lo = (c & 2) ? ((c & 1) ? r3 : r2) : r1;                               // c = 1..3
+        const double hi = (c & 2) ? ((c & 1) ? r7 : r6) : ((c & 1) ? r5 : r4);               // c = 4..7
+        v += ew_eval<kGrad>(T, 1, (c & 4) ? hi : lo, &d);
         if (kGrad) {
             s += d;
             s0 += (c & 1) ? d : 0.0; s1 += (c & 2) ? d : 0.0; s2 += (c & 4) ? d : 0.0;

@@ -16,7 +16,8 @@
 // done once per (nucleus, electron):
 //   grad: 2 s1 p;   lap: 4 s2 |p|^2 + 2 s1 sum q;
 //   H gU + 1/2 grad lap:  p (4 s2 p.gU + 4 s3 |p|^2 + 2 s2 sum q - k2 s1 + 4 s2 q) + 2 s1 q o gU.
-// N = 64, 1024 walkers: orbital rows + sample 12.1 ms before, 7.2 ms now.
+// N = 64, 1024 walkers: orbital rows + sample 12.1 ms before, 6.8 ms now (7.2 with the
+// e-e Jastrow pairs evaluated from both ends).
 //
 // Twisted form (complex Bloch-summed orbitals, k_twist.cu): the same with complex
 // G, y and real C, so there Y_ij = sum_b y_bi C_bj, K = G Y G and P = C K are the
@@ -26,7 +27,7 @@
 //   y = -D chi,   H gU + 1/2 grad lap = grad (D chi),
 // everything follows from s_q = d^q s, t = D_mu s and t' = d D_mu s of each axis.
 // N = 64, 512 walkers: rows + g, l + sample + force terms 15.5 ms before in four
-// kernels, 9.4 ms now in one.
+// kernels, 9.2 ms now in one.
 #include "bloch.cuh"
 #include "common.cuh"
 #include "kernels.cuh"
@@ -57,8 +58,8 @@ struct M64Layout {
         facc = take(9 * N);
         rhot = take(2 * nk);
         red = take(64);
-        // slices of the Jastrow sums (5 per electron), then the warps' g_i, l_i sums
-        const size_t jp = 5 * (size_t)(kThreads > N ? kThreads : N), gp = 4 * (size_t)kWarps * n;
+        // slices of the Jastrow sums (5 + 4 per electron; N <= kThreads), then the warps' g_i, l_i sums
+        const size_t jp = 9 * (size_t)kThreads, gp = 4 * (size_t)kWarps * n;
         part = take(jp > gp ? jp : gp);
         size_t u = 2 * (size_t)N * 3 * (mmax + 1);                            // phase table
         if (tw) {
@@ -362,27 +363,46 @@ __global__ void __launch_bounds__(kThreads, TM ? 2 : 1) measure64_kernel(SysView
     __syncthreads();
 
     // ---- Jastrow gradient / Laplacian per electron and U, the partner range cut
-    // into nparts slices so that every thread works, the slices summed in order
-    const int nparts = kThreads >= N ? kThreads / N : 1;
-    for (int tt = tid; tt < nparts * N; tt += kThreads) {
-        const int i = tt % N, pi = tt / N;
-        const int j0 = (N * pi) / nparts, j1 = (N * (pi + 1)) / nparts;
+    // into nparts slices so that every thread works, the slices summed in order.  An
+    // e-e pair is evaluated once: electron i with i + d (mod N), d = 1..N/2 (d = N/2
+    // only for i < N/2); at each distance every electron of a slice is one pair's
+    // partner, whose share goes to its slot of the slice (a barrier per distance).
+    const int nparts = kThreads >= N ? kThreads / N : 1, half = N / 2;
+    double* partner = part + (size_t)5 * nparts * N;      // [nparts][N][4]
+    for (int idx = tid; idx < 4 * nparts * N; idx += kThreads) partner[idx] = 0.0;
+    __syncthreads();
+    {
+        const int i = tid % N, pi = tid / N;
+        const bool on = pi < nparts;
+        const int d0 = 1 + (half * pi) / nparts, d1 = 1 + (half * (pi + 1)) / nparts;
+        const int j0 = (N * pi) / nparts, j1 = (N * (pi + 1)) / nparts, steps = (half + nparts - 1) / nparts;
         double g[3] = {0, 0, 0}, lp = 0, ui = 0;
         double ei[6];
 #pragma unroll
         for (int c = 0; c < 6; ++c) ei[c] = et[6 * i + c];
-        for (int j = j0; j < j1; ++j) {
-            if (j == i) continue;
-            const Geo o = geometry(ei, et + 6 * j, ell);
-            double u, c2, c4;
-            pade_factors(o.t, bee, 0.5, u, c2, c4);
-            const double pp = o.p[0] * o.p[0] + o.p[1] * o.p[1] + o.p[2] * o.p[2];
-            lp += c4 * pp + c2 * (o.q[0] + o.q[1] + o.q[2]);
+        for (int q = 0; q < steps; ++q) {
+            const int d = d0 + q;
+            if (on && d < d1 && !(2 * d == N && i >= half)) {
+                const int j = i + d < N ? i + d : i + d - N;
+                const Geo o = geometry(ei, et + 6 * j, ell);
+                double u, c2, c4;
+                pade_factors(o.t, bee, 0.5, u, c2, c4);
+                const double pp = o.p[0] * o.p[0] + o.p[1] * o.p[1] + o.p[2] * o.p[2];
+                const double lv = c4 * pp + c2 * (o.q[0] + o.q[1] + o.q[2]);
+                double* pj = partner + 4 * ((size_t)pi * N + j);
 #pragma unroll
-            for (int mu = 0; mu < 3; ++mu) g[mu] += c2 * o.p[mu];
-            if (j > i) ui += u;
+                for (int mu = 0; mu < 3; ++mu) {
+                    const double gm = c2 * o.p[mu];       // odd under the exchange of the pair
+                    g[mu] += gm;
+                    pj[mu] -= gm;
+                }
+                lp += lv;
+                pj[3] += lv;
+                ui += u;
+            }
+            __syncthreads();
         }
-        for (int a = j0; a < j1; ++a) {
+        for (int a = j0; on && a < j1; ++a) {
             const Geo o = geometry(ei, s.ptrig + 6 * a, ell);
             double u, c2, c4;
             pade_factors(o.t, bep, -Zj, u, c2, c4);
@@ -392,8 +412,11 @@ __global__ void __launch_bounds__(kThreads, TM ? 2 : 1) measure64_kernel(SysView
             for (int mu = 0; mu < 3; ++mu) g[mu] += c2 * o.p[mu];
             ui += u;
         }
-        double* o = part + ((size_t)pi * N + i) * 5;
-        o[0] = g[0]; o[1] = g[1]; o[2] = g[2]; o[3] = lp; o[4] = ui;
+        if (on) {
+            double* o = part + 5 * ((size_t)pi * N + i);
+            const double* pj = partner + 4 * ((size_t)pi * N + i);
+            o[0] = g[0] + pj[0]; o[1] = g[1] + pj[1]; o[2] = g[2] + pj[2]; o[3] = lp + pj[3]; o[4] = ui;
+        }
     }
     __syncthreads();
     for (int i = tid; i < N; i += kThreads) {
@@ -770,7 +793,7 @@ __global__ void __launch_bounds__(kThreads, TM ? 2 : 1) measure64_kernel(SysView
     const EwTable ewt{s.ewt, s.ew_h, s.ew_ih, L, iL, L * L};
     double vee_p = 0.0;
     for (int tt = tid; tt < nparts * N; tt += kThreads) {
-        const int i = tt % N, pi = tt / N, half = N / 2;
+        const int i = tt % N, pi = tt / N;
         const int d0 = 1 + (half * pi) / nparts, d1 = 1 + (half * (pi + 1)) / nparts;
         double v = 0;
         for (int d = d0; d < d1; ++d) {
