@@ -146,18 +146,25 @@ __global__ void __launch_bounds__(256) invert_kernel(int N, int n, const T* __re
 //     between FP32 numbers (about one in 10^4), so that the pair cannot tell its
 //     rounding, its column gets one Newton correction X r with the residual r = e_c -
 //     A x_c in FP64, and those elements are rounded anew.
-// So the result is the rounded inverse but where the FP64 elimination's own error
-// (10^-14) decides.  Blocks with a zero pivot or more than kPairColumns such columns
-// (nearly singular ones) go to FP64 Gauss-Jordan.  ln|det A| is the FP64 sum of the
+//  3. Where the corrected element still lies within kExactMargin 2^-53 (same scale) of
+//     the midpoint, the FP64 elimination's own error decides its rounding: the block
+//     goes to FP64 Gauss-Jordan, as do blocks with a zero pivot or more than kPairColumns
+//     columns of step 2 (nearly singular ones).  The FP64 error, in units of 2^-53 of that
+//     scale against an extended-precision inverse, exceeds 20 in one undecided element of
+//     a thousand (n = 64; at most 46, and less for smaller n); a margin of 24 takes some 4 %
+//     of the blocks of n = 64, one of 64 took 11 % and 2 ms more per recompute.
+// So the result is FP64 Gauss-Jordan's to the bit: the walkers of 44 starts of N = 128
+// (16384 each, five calls) had the same accumulators with either; without step 3 some
+// 3600 in 2 x 10^6 differed, one by a whole move.  ln|det A| is the FP64 sum of the
 // pivots' logarithms.
 //
 // Layout: g x g threads (g = ceil(n / 4)) with a 4 x 4 tile of the block each in
 // registers; no row moves: the pivot rows are marked and the permutation applied when
 // the inverse is written.  Per column two barriers: the column (with the pivot search
 // by every warp on its own), then the pivot row.
-// 32768 blocks of n = 64: 17.5 ms in FP64, 8.4 ms so.
+// 32768 blocks of n = 64: 17.5 ms in FP64, 9.3 ms so (8.4 without step 3).
 // ---------------------------------------------------------------------------
-constexpr float kPairMargin = 48.f;
+constexpr float kPairMargin = 48.f, kExactMargin = 24.f;
 constexpr int kPairColumns = 16;
 
 struct PairF { float h, l; };
@@ -187,6 +194,7 @@ struct PairShared {
     int perm[64], kof[64];    // pivot row of step k; step of pivot row i
     float rmax[64], cmax[64], amax, wmax[8], res[64], corr[64];
     unsigned mark[2];         // columns with an element whose rounding is open
+    int open;                 // an element's rounding depends on the FP64 elimination's own error
 };
 
 // Column k = 4 kb + kk of the elimination (kk a constant: the tile m stays in
@@ -298,6 +306,7 @@ __global__ void __launch_bounds__(256, 3) invert_pair_kernel(int N, int n, int g
         for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
         if (lane == 0) sh.wmax[tid >> 5] = v;
         if (tid < 2) sh.mark[tid] = 0u;
+        if (tid == 0) sh.open = 0;
         __syncthreads();
         if (tid == 0) {
             for (int q = 1; q < nt / 32; ++q) v = fmaxf(v, sh.wmax[q]);
@@ -379,11 +388,21 @@ __global__ void __launch_bounds__(256, 3) invert_pair_kernel(int N, int n, int g
                 __syncthreads();
                 for (int l = tid; l < n; l += nt)
                     if (undecided(l, c)) {
-                        Xh[l * ld + c] = (float)((double)Xh[l * ld + c] + ((double)Xl[l * ld + c] + (double)sh.corr[l]));
+                        const double v = (double)Xh[l * ld + c] + ((double)Xl[l * ld + c] + (double)sh.corr[l]);
+                        const float f = (float)v;
+                        // distance to f against half an ulp of f (a quarter below a power of two)
+                        const unsigned fb = __float_as_uint(f);
+                        const double half = (double)(__uint_as_float(fb & 0x7f800000u) * 5.9604644775390625e-08f);
+                        const double off = fabs(v - (double)f);
+                        const double d = (double)(kExactMargin / kPairMargin / 64.f * scale * sh.rmax[l] * sh.cmax[c]);
+                        if (!(fabs(off - half) >= d) || ((fb & 0x7fffffu) == 0u && fabs(off - 0.5 * half) < d))
+                            sh.open = 1;
+                        Xh[l * ld + c] = f;
                         Xl[l * ld + c] = 0.f;
                     }
                 __syncthreads();
             }
+        if (fine && sh.open) fine = false;
     }
     if (!fine) {
         __syncthreads();
