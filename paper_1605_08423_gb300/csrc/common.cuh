@@ -239,6 +239,7 @@ struct SysView {
     double zeta_j;          // their Gaussians' exponent
     const double* ewt;      // real-space Ewald table (FP64 form, kappa L <= kEwMaxKL), or null: see EwTable
     double ew_h, ew_ih;     // its node spacing in r^2 and the inverse
+    bool served;            // the handle's kernels overlap other trajectories' (see launch_sweep)
 };
 
 // Twisted boundary conditions: walker w samples twist t = w / Wk (K contiguous

@@ -288,7 +288,7 @@ SysView<T> view(qmc_system* h, int W) {
     s.kvec = h->d_kvec; s.kw = h->d_kw; s.eikR = h->d_eikR; s.rho_p = h->d_rhop;
     s.vconst = h->d_vconst; s.dvpp = h->d_dvpp; s.err = h->d_err; s.vacc = h->d_vacc;
     s.ewt = h->d_ewt; s.ew_h = 0.75 * h->p.L * h->p.L / (kEwNodes - 1); s.ew_ih = 1.0 / s.ew_h;
-    s.fj = h->d_fj; s.zeta_j = h->p.zeta_j;
+    s.fj = h->d_fj; s.zeta_j = h->p.zeta_j; s.served = h->pool != nullptr;
     s.fjt = (const T*)(sizeof(T) == 8 ? (const void*)h->d_fj : (const void*)h->d_fj32);
     return s;
 }

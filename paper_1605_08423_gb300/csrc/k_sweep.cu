@@ -30,10 +30,10 @@ struct SweepSmem {
     // per warp: G^T [n][ld], old row [nv], phi' [nv], proposal trig [6], trig
     // [6N], V [N], and only with the e-e-n-n Jastrow term (j34) three [N]
     // vectors (sum over electrons of chi_a, the same less the moving electron's,
-    // and the change at its proposal)
+    // and the change at its proposal); last the sums of two warps, [2][4]
     __host__ __device__ static size_t warp_bytes(int N, int n, bool j34) {
         size_t b = ((size_t)n * ld(n) + 2 * (size_t)nv(n) + 6) * sizeof(double);
-        b += (size_t)(j34 ? 10 : 7) * N * sizeof(double);
+        b += (size_t)(j34 ? 10 : 7) * N * sizeof(double) + 8 * sizeof(double);
         return (b + 15) & ~size_t(15);
     }
 };
@@ -75,6 +75,14 @@ __device__ __forceinline__ double pade_u(const double* a, const double* b, doubl
 // of N = 64 costs 3 N Pade pairs of 22 operations and the rank-1 update.  The
 // new and old e-e terms share one lane loop of 2 N items, so that small N
 // fills the warp; walkers are spread evenly over the SMs by the launcher.
+// WW warps take a walker: one, or two where the walkers are so few that half of the
+// SMs' four issue ports would idle (a port issues an FP64 instruction in 64 clocks,
+// so a lone warp's move is a chain of some 90 of them at N = 16).  With two, the first
+// takes the e-e terms, the second the ratio and the e-n terms, each summed in the order
+// of the lone warp, and a row's update is cut over up to four threads: a walker's chain
+// is the same to the bit whatever the number of walkers.  256 walkers of N = 16: 63 us a
+// sweep, 80 with one warp.
+template <int WW>
 __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* __restrict__ X,
                                                     const double* __restrict__ Xp, const double* __restrict__ ptp,
                                                     const double* __restrict__ uacc, const double* __restrict__ Phi,
@@ -83,7 +91,12 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* _
     extern __shared__ __align__(16) unsigned char smraw[];
     constexpr int VE = SweepSmem::VE;
     const int N = s.N, n = s.n, nv = SweepSmem::nv(n), ld = SweepSmem::ld(n), nvv = nv / VE;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    constexpr int T = 32 * WW;
+    const int lane = threadIdx.x & (T - 1), warp = threadIdx.x / T, wpb = blockDim.x / T;   // thread of the walker
+    auto sync = [&]() {
+        if (WW == 1) __syncwarp();
+        else asm volatile("bar.sync %0, %1;\n" ::"r"(1 + warp), "n"(T) : "memory");
+    };
     double* ptr_s = (double*)smraw;                          // [N][6] proton trig
     const size_t off = ((size_t)6 * N * sizeof(double) + 15) & ~size_t(15);
     const bool j34 = s.fjt != nullptr;
@@ -97,6 +110,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* _
     double* c34 = vj + N;         // [N] sum over electrons of chi_a (e-e-n-n Jastrow term)
     double* dif = c34 + N;        // [N] c_a - chi_a at the moving electron
     double* dch = dif + N;        // [N] change of chi_a at its proposal
+    double* red = (double*)(mine + SweepSmem::warp_bytes(N, n, j34)) - 8;   // the warps' sums
 
     for (int idx = threadIdx.x; idx < 6 * N; idx += blockDim.x) ptr_s[idx] = s.ptrig[idx];
     __syncthreads();
@@ -106,15 +120,15 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* _
     const double ell = s.ell, bee = s.b_ee, bep = s.b_ep, Zj = s.Zj;
     const double L = s.L, iL = s.iL;
     double* Xw = X + (size_t)w * 3 * N;   // positions stay in HBM; accepted moves are written through
-    for (int idx = lane; idx < 3 * N; idx += 32) {
+    for (int idx = lane; idx < 3 * N; idx += T) {
         const int i = idx / 3, mu = idx % 3;
         double sn, cs;
         sincospi(Xw[idx] * iL, &sn, &cs);
         et[6 * i + mu] = sn;
         et[6 * i + 3 + mu] = cs;
     }
-    __syncwarp();
-    for (int i = lane; i < N; i += 32) {
+    sync();
+    for (int i = lane; i < N; i += T) {
         double v = 0;
         if (vep_init)
             for (int a = 0; a < N; ++a) v += pade_u(et + 6 * i, ptr_s + 6 * a, ell, bep, -Zj);
@@ -124,14 +138,14 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* _
     }
     const double zj = s.zeta_j;
     if (j34) {
-        for (int a = lane; a < N; a += 32) {
+        for (int a = lane; a < N; a += T) {
             double c = 0;
             for (int j = 0; j < N; ++j) c += jas_orbital(et + 6 * j, ptr_s + 6 * a, ell, zj);
             c34[a] = c;
         }
     }
-    __syncwarp();
-    for (int j = n + lane; j < nv; j += 32) phi[j] = 0.0;   // padding stays zero
+    sync();
+    for (int j = n + lane; j < nv; j += T) phi[j] = 0.0;   // padding stays zero
     unsigned long long naccept = 0;
     // the next move's proposal trig (lanes 0-5), orbital row (n <= 64: two per
     // lane) and uniform are loaded one move ahead, so their HBM latency
@@ -141,49 +155,52 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* _
         const size_t row = (size_t)w * N + i;
         pt_nx = lane < 6 ? ptp[row * 6 + lane] : 0.0;
 #pragma unroll
-        for (int k = 0; k < 2; ++k) ph_nx[k] = (lane + 32 * k < n) ? Phi[row * n + lane + 32 * k] : 0.0;
+        for (int k = 0; k < 2; ++k) ph_nx[k] = (lane + T * k < n) ? Phi[row * n + lane + T * k] : 0.0;
         u_nx = uacc[row];
     };
     fetch(0);
     for (int sp = 0; sp < 2; ++sp) {
         double* G = Gt + ((size_t)w * 2 + sp) * n * n;
-        for (int idx = lane; idx < n * nv; idx += 32) {
+        for (int idx = lane; idx < n * nv; idx += T) {
             const int r = idx / nv, c = idx - r * nv;
             Gs[r * ld + c] = c < n ? G[r * n + c] : 0.0;
         }
-        __syncwarp();
+        sync();
         for (int il = 0; il < n; ++il) {
             const int i = sp * n + il;
             const size_t row = (size_t)w * N + i;
             if (lane < 6) ptb[lane] = pt_nx;
 #pragma unroll
             for (int k = 0; k < 2; ++k)
-                if (lane + 32 * k < n) phi[lane + 32 * k] = ph_nx[k];
+                if (lane + T * k < n) phi[lane + T * k] = ph_nx[k];
             const double u = u_nx;
             if (i + 1 < N) fetch(i + 1);
-            __syncwarp();
-            double part = 0;
-            for (int j = lane; j < n; j += 32) part += phi[j] * Gs[il * ld + j];
-            const double* ei = et + 6 * i;
+            sync();
             // items 0..N-1: u_ee at the proposal, N..2N-1: minus u_ee at the old position
-            double du = 0, vnew = 0;
-            for (int k = lane; k < 2 * N; k += 32) {
-                const bool old = k >= N;
-                const int j = old ? k - N : k;
-                const double v = pade_u(old ? ei : ptb, et + 6 * j, ell, bee, old ? -0.5 : 0.5);
-                du += j != i ? v : 0.0;
+            const double* ei = et + 6 * i;
+            const int ln = lane & 31;
+            double part = 0, du = 0, vnew = 0;
+            if (WW == 1 || lane < 32)
+                for (int k = ln; k < 2 * N; k += 32) {
+                    const bool old = k >= N;
+                    const int j = old ? k - N : k;
+                    const double v = pade_u(old ? ei : ptb, et + 6 * j, ell, bee, old ? -0.5 : 0.5);
+                    du += j != i ? v : 0.0;
+                }
+            if (WW == 1 || lane >= 32) {
+                for (int j = ln; j < n; j += 32) part += phi[j] * Gs[il * ld + j];
+                for (int a = ln; a < N; a += 32) vnew += pade_u(ptb, ptr_s + 6 * a, ell, bep, -Zj);
             }
-            for (int a = lane; a < N; a += 32) vnew += pade_u(ptb, ptr_s + 6 * a, ell, bep, -Zj);
             if (j34) {
                 // e-e-n-n term: the pairs (i, j != i) change by
                 // sum_a (chi_a(r'_i) - chi_a(r_i)) sum_b f_ab (c_b - chi_b(r_i))
-                for (int a = lane; a < N; a += 32) {
+                for (int a = lane; a < N; a += T) {
                     const double old = jas_orbital(ei, ptr_s + 6 * a, ell, zj);
                     dch[a] = jas_orbital(ptb, ptr_s + 6 * a, ell, zj) - old;
                     dif[a] = c34[a] - old;
                 }
-                __syncwarp();
-                for (int a = lane; a < N; a += 32) {
+                sync();
+                for (int a = lane; a < N; a += T) {
                     // f is symmetric (checked at qmc_init): column a = row a,
                     // and the lanes' loads of a column element are consecutive
                     const double* fa = s.fjt + a;
@@ -195,7 +212,7 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* _
             // the three warp sums in seven additions: the halves of the warp exchange
             // (ratio, du) for (vnew, 0), then the quarters
             double ratio;
-            {
+            if (WW == 1) {
                 const bool hi = lane & 16, qr = lane & 8;
                 double a0 = hi ? vnew : part, a1 = hi ? 0.0 : du;
                 a0 += __shfl_xor_sync(0xffffffffu, hi ? part : vnew, 16);
@@ -207,16 +224,30 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* _
                 ratio = __shfl_sync(0xffffffffu, x, 0);
                 du = __shfl_sync(0xffffffffu, x, 8);
                 vnew = __shfl_sync(0xffffffffu, x, 16);
+            } else {         // du is the first warp's, ratio and vnew the second's; each added up in the same order
+                const bool hi = lane & 16, second = lane >= 32;
+                double x = second ? (hi ? vnew : part) : du;
+                x += __shfl_xor_sync(0xffffffffu, second ? (hi ? part : vnew) : du, 16);
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                double* rd = red + 4 * (il & 1);     // alternating: read after the barrier, written a move later
+                if ((lane & 15) == 0) rd[lane >> 4] = x;
+                sync();
+                du = rd[0];
+                ratio = rd[2];
+                vnew = rd[3];
             }
             du += vnew - vj[i];
             const double prob = ratio * ratio * qexp(2.0 * du);
             if (u < prob) {
-                for (int j = lane; j < nv; j += 32) rowb[j] = Gs[il * ld + j];
-                __syncwarp();
+                for (int j = lane; j < nv; j += T) rowb[j] = Gs[il * ld + j];
+                sync();
                 const double ir = qrcp(ratio);
                 const double2* phv = (const double2*)phi;
                 const double2* rbv = (const double2*)rowb;
-                for (int l = lane; l < n; l += 32) {
+                // two warps: S consecutive threads per row, which update every S-th vector each
+                const int S = WW == 1 ? 1 : n <= 16 ? 4 : n <= 32 ? 2 : 1, h = lane & (S - 1);
+                for (int l = lane / S; l < n; l += T / S) {
                     double2* gl = (double2*)(Gs + l * ld);
                     double w0 = 0, w1 = 0;   // two partial sums: short chains
                     for (int jv = 0; jv < nvv; ++jv) {
@@ -224,7 +255,8 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* _
                         w0 += p.x * g.x; w1 += p.y * g.y;
                     }
                     const double coef = ((w0 + w1) - (l == il ? 1.0 : 0.0)) * ir;
-                    for (int jv = 0; jv < nvv; ++jv) {
+                    if (S > 1) __syncwarp(((1u << S) - 1u) << (lane & 31 & ~(S - 1)));   // the row's threads have read it
+                    for (int jv = h; jv < nvv; jv += S) {
                         const double2 g = gl[jv], r = rbv[jv];
                         gl[jv] = make_double2(g.x - coef * r.x, g.y - coef * r.y);
                     }
@@ -241,15 +273,15 @@ __global__ void __launch_bounds__(512) sweep_kernel(SysView<double> s, double* _
                 if (lane < 6) et[6 * i + lane] = ptb[lane];
                 if (lane == 0) vj[i] = vnew;
                 if (j34)
-                    for (int a = lane; a < N; a += 32) c34[a] += dch[a];
+                    for (int a = lane; a < N; a += T) c34[a] += dch[a];
                 ++naccept;
             }
-            __syncwarp();
+            sync();
         }
-        for (int idx = lane; idx < n * n; idx += 32) G[idx] = Gs[(idx / n) * ld + idx % n];
-        __syncwarp();
+        for (int idx = lane; idx < n * n; idx += T) G[idx] = Gs[(idx / n) * ld + idx % n];
+        sync();
     }
-    for (int i = lane; i < N; i += 32) Vep[(size_t)w * N + i] = vj[i];
+    for (int i = lane; i < N; i += T) Vep[(size_t)w * N + i] = vj[i];
     if (lane == 0) nacc[w] += naccept;
 }
 
@@ -518,17 +550,22 @@ __global__ void __launch_bounds__(64 * kSwWalkers) sweep_reg_kernel(SysView<floa
     if (tw == 0) nacc[w] += naccept;
 }
 
-// Walkers per CTA of a kernel that takes one warp per walker: at most `most`
-// (shared memory), and no more than spreads the walkers evenly over the SMs in
-// the fewest rounds.  With 16 walkers a CTA, 1024 walkers sat on 64 of the 152
-// SMs and a sweep of N = 64 took 2.9 ms (0.9 ms with 7 a CTA on 147 of them).
-int walkers_per_cta(int W, int most) {
+static int sm_count() {
     static const int sms = [] {
         int dev = 0, v = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
         return v > 0 ? v : 1;
     }();
+    return sms;
+}
+
+// Walkers per CTA of a kernel that takes one warp per walker: at most `most`
+// (shared memory), and no more than spreads the walkers evenly over the SMs in
+// the fewest rounds.  With 16 walkers a CTA, 1024 walkers sat on 64 of the 152
+// SMs and a sweep of N = 64 took 2.9 ms (0.9 ms with 7 a CTA on 147 of them).
+int walkers_per_cta(int W, int most) {
+    const int sms = sm_count();
     const long long per_round = (long long)sms * most;
     const long long rounds = (W + per_round - 1) / per_round;
     return (int)((W + sms * rounds - 1) / (sms * rounds));
@@ -556,11 +593,19 @@ void launch_sweep(const SysView<double>& s, double* X, const double* Xp, const d
     const int wpb = walkers_per_cta(s.W, std::max(1, std::min(16, fit)));
     static bool attr_set = false;
     if (!attr_set) {
-        cudaFuncSetAttribute(sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        cudaFuncSetAttribute(sweep_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        cudaFuncSetAttribute(sweep_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         attr_set = true;
     }
-    sweep_kernel<<<(s.W + wpb - 1) / wpb, 32 * wpb, head + wpb * wb, st>>>(s, X, Xp, ptp, uacc, Phi, Gt, nacc, vep,
-                                                                           vep_init ? 1 : 0);
+    // two warps a walker while they still find a free issue port each: at most two walkers
+    // an SM, and no other trajectory's kernels beside them (six served trajectories of
+    // 256 walkers: 10.6 ms a step, 10.4 with one warp); the e-e-n-n sums stay with one warp
+    if (wpb <= 2 && s.W <= 2 * sm_count() && !s.served && !s.fj)
+        sweep_kernel<2><<<(s.W + wpb - 1) / wpb, 64 * wpb, head + wpb * wb, st>>>(s, X, Xp, ptp, uacc, Phi, Gt, nacc, vep,
+                                                                                  vep_init ? 1 : 0);
+    else
+        sweep_kernel<1><<<(s.W + wpb - 1) / wpb, 32 * wpb, head + wpb * wb, st>>>(s, X, Xp, ptp, uacc, Phi, Gt, nacc, vep,
+                                                                                  vep_init ? 1 : 0);
 }
 
 }  // namespace qmc

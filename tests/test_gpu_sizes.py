@@ -115,3 +115,18 @@ def test_reductions_match_the_accumulators(N, W, K):
     for key in ("E", "E_err", "f", "S"):
         a, b = np.asarray(g[key]).ravel(), np.asarray(ref[key]).ravel()
         assert np.max(np.abs(a - b)) <= 1e-12 * W * np.max(np.abs(b)), key
+
+
+# FP64 sweep with two warps a walker (few walkers, handle of its own) against one (many
+# walkers): the same walkers' chains, to the bit
+@pytest.mark.parametrize("N", [2, 10, 16, 34, 66, 128])
+def test_sweep_does_not_depend_on_the_number_of_walkers(N):
+    runs = []
+    for W in (24, 640):
+        wl = _workload(N, 2, W, sweeps=2)
+        s = q.QMCSystem(q.Config.from_workload(wl, warmup=1, recompute_every=2), wl.R)
+        g = s.energy_forces(wl.R)
+        runs.append((s.walkers()[:24], s.accumulators()[:24], g["accept"]))
+    assert np.array_equal(runs[0][0], runs[1][0])
+    assert np.array_equal(runs[0][1], runs[1][1])
+    assert runs[0][2] > 0.0
