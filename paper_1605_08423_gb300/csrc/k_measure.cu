@@ -757,6 +757,7 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
         }
         __syncthreads();
         const int total = coff[N];
+        __syncthreads();   // read by every thread before the phase table below takes coff's place (no pair: no other barrier)
         const double k2d = (2.0 * kPi * iL) * (2.0 * kPi * iL);
         for (int base = 0; base < total; base += CH) {
             const int end = base + CH < total ? base + CH : total;

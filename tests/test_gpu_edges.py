@@ -1,0 +1,64 @@
+"""Calls at the edges of what the entry points take: no electron near a proton, the
+largest reciprocal-space cutoff, very large meshes, far electrons, short runs.
+
+Tolerances against the FP64 oracle are those of the parity tests: 1e-10 (FP64 form)
+and 1e-4 (mixed form) relative to the largest magnitude.
+"""
+import numpy as np
+import pytest
+
+from oracle import oracle as orc
+from paper_1605_08423_gb300 import qmcmd as q
+from paper_1605_08423_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+ZETA = {1: (0.7,), 2: synth.ZETA_2, 4: synth.ZETA_4}
+
+
+def _workload(N, G, walkers, rs=1.3, **kw):
+    return synth.Workload(name="edges", N=N, rs=rs, zeta=ZETA[G], walkers=walkers, T_kelvin=1500.0,
+                          **{"seed": 7, "sweeps": 1, **kw})
+
+
+def _osys(wl, **kw):
+    return orc.System(N=wl.N, L=wl.L, zeta=np.array(wl.zeta), coeff=wl.C, **kw)
+
+
+def _sampled(wl, n):
+    """|psi|^2-distributed configurations from the oracle's own chains."""
+    X, _, _ = orc.vmc(_osys(wl), wl.R, W=n, n_sweeps=1, n_warmup=12, sigma=wl.sigma, seed=5, forces=False)
+    return X
+
+
+def _close(g, ref, tol):
+    lp, el, dl, de = ref
+    assert np.max(np.abs(g["el"] - el)) <= tol * np.max(np.abs(el))
+    assert np.all(np.abs(g["lnpsi"] - lp) <= tol * np.maximum(np.abs(lp), 1.0))
+    for key, v in (("dlnpsi", dl), ("del_", de)):
+        rel = np.max(np.abs(g[key] - v), axis=(-1, -2)) / np.max(np.abs(v), axis=(-1, -2))
+        assert np.all(rel <= tol), (key, rel)
+
+
+def _pushed_out(X, R, L, r_min):
+    """X with every electron closer than r_min to its nearest proton moved out to r_min."""
+    d = X[:, :, None, :] - R[None, None]
+    d -= L * np.rint(d / L)
+    r = np.linalg.norm(d, axis=-1)
+    a = np.argmin(r, axis=-1)
+    rmin = np.take_along_axis(r, a[..., None], -1)
+    dmin = np.take_along_axis(d, a[..., None, None], 2)[:, :, 0]
+    return np.where(rmin < r_min, R[a] + dmin * (r_min / rmin), X)
+
+
+# the mixed sample without a single close pair (no electron within 0.3 bohr of a proton):
+# its list of close pairs is empty and shares its place with the phase table built next
+@pytest.mark.parametrize("N,G,W", [(16, 2, 300), (34, 2, 48), (128, 4, 4)])
+def test_mixed_sample_without_close_pairs(N, G, W):
+    wl = _workload(N, G, W)
+    X = _pushed_out(_sampled(wl, 2 * W), wl.R, wl.L, 0.45)
+    X = X[np.argsort([orc.slater_condition(_osys(wl), wl.R, x) for x in X])[:W]]   # FP32: away from the nodes
+    s = q.QMCSystem(q.Config.from_workload(wl, precision=q.QMC_MIXED), wl.R)
+    ref = orc.eval_configs(_osys(wl), wl.R, X, derivs=True)
+    for _ in range(3):
+        _close(s.eval_config(X, wl.R), ref, 1e-4)
