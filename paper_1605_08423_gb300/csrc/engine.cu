@@ -320,7 +320,7 @@ void recompute(qmc_system* h, int W) {
     SysView<T> s = view<T>(h, W);
     h->nlaunch += 2;
     orbitals(h, s, h->d_X, (const T*)nullptr, W * h->N, (T*)h->d_Phi, nullptr, nullptr);
-    launch_invert(W, h->N, h->n, (const T*)h->d_Phi, (T*)h->d_Gt, h->d_logdet, h->d_err, h->stream);
+    launch_invert<T>(W, h->N, h->n, (const T*)h->d_Phi, (T*)h->d_Gt, h->d_logdet, h->d_err, h->stream);
     prof_end(h, ep);
 }
 

@@ -5,8 +5,7 @@
 // turn into column interchanges of the inverse, undone at the end.  Always
 // FP64: this is the periodic recompute that resets the drift of the rank-1
 // (Sherman-Morrison) updates of the sweep kernel.  Output: Gt[i][j] = (A^-1)_{j,i}
-// in the working precision and ln|det A|.  The mixed form reaches FP64's accuracy
-// with pairs of FP32 numbers above n = 16 (invert_pair_kernel).
+// in the working precision, ln|det A| and the pivot sign.
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -130,293 +129,6 @@ __global__ void __launch_bounds__(256) invert_kernel(int N, int n, const T* __re
                                                      double* __restrict__ logdet, int* err) {
     extern __shared__ double sm[];
     gj_invert<T>(N, n, Phi, Gt, logdet, err, blockIdx.x >> 1, blockIdx.x & 1, sm);
-}
-
-// ---------------------------------------------------------------------------
-// Mixed form, n > 16: the inverse of an FP32 Slater block, rounded to FP32 as FP64
-// Gauss-Jordan's is, mostly without the FP64 pipe, which an FP64 warp instruction
-// occupies for 19 clocks of an SM and an FP32 one for a quarter of a clock.
-//  1. Gauss-Jordan with partial pivoting on pairs (hi, lo) of FP32 numbers, each
-//     product split exactly by one FMA and each sum by Knuth's TwoSum (T. J. Dekker,
-//     Numer. Math. 18, 1971): about 47 bits, 12 FP32 operations per update.  Its
-//     error on Slater blocks (n = 20 to 64, cond up to 10^4) stays below
-//     30 2^-47 max_j|X_lj| max_i|X_ic| max|A| per element: 10^-13 to 10^-12 of the
-//     largest, some 10^-5 of the FP32 rounding.
-//  2. Where an element lies within kPairMargin 2^-47 (same scale) of a midpoint
-//     between FP32 numbers (about one in 10^4), so that the pair cannot tell its
-//     rounding, its column gets one Newton correction X r with the residual r = e_c -
-//     A x_c in FP64, and those elements are rounded anew.
-//  3. Where the corrected element still lies within kExactMargin 2^-53 (same scale) of
-//     the midpoint, the FP64 elimination's own error decides its rounding: the block
-//     goes to FP64 Gauss-Jordan, as do blocks with a zero pivot or more than kPairColumns
-//     columns of step 2 (nearly singular ones).  The FP64 error, in units of 2^-53 of that
-//     scale against an extended-precision inverse, exceeds 20 in one undecided element of
-//     a thousand (n = 64; at most 46, and less for smaller n); a margin of 24 takes some 4 %
-//     of the blocks of n = 64, one of 64 took 11 % and 2 ms more per recompute.
-// So the result is FP64 Gauss-Jordan's to the bit: the walkers of 44 starts of N = 128
-// (16384 each, five calls) had the same accumulators with either; without step 3 some
-// 3600 in 2 x 10^6 differed, one by a whole move.  ln|det A| is the FP64 sum of the
-// pivots' logarithms.
-//
-// Layout: g x g threads (g = ceil(n / 4)) with a 4 x 4 tile of the block each in
-// registers; no row moves: the pivot rows are marked and the permutation applied when
-// the inverse is written.  Per column two barriers: the column (with the pivot search
-// by every warp on its own), then the pivot row.
-// 32768 blocks of n = 64: 17.5 ms in FP64, 9.3 ms so (8.4 without step 3).
-// ---------------------------------------------------------------------------
-constexpr float kPairMargin = 48.f, kExactMargin = 24.f;
-constexpr int kPairColumns = 16;
-
-struct PairF { float h, l; };
-__device__ __forceinline__ PairF two_sum(float a, float b) {
-    const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
-    return PairF{s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z))};
-}
-__device__ __forceinline__ PairF pair_mul(PairF a, PairF b) {
-    const float p = __fmul_rn(a.h, b.h);
-    float e = __fmaf_rn(a.h, b.h, -p);
-    e = __fmaf_rn(a.h, b.l, e);
-    e = __fmaf_rn(a.l, b.h, e);
-    const float h = __fadd_rn(p, e);
-    return PairF{h, __fsub_rn(e, __fsub_rn(h, p))};
-}
-// 1 / a: the hardware's approximation y, then y (1 + r + r^2), r = 1 - a y exactly formed
-__device__ __forceinline__ PairF pair_rcp(PairF a) {
-    const float y = __frcp_rn(a.h);
-    const float r = __fmaf_rn(-a.l, y, __fmaf_rn(-a.h, y, 1.f));
-    const float l = __fmul_rn(y, __fmaf_rn(r, r, r)), h = __fadd_rn(y, l);
-    return PairF{h, __fsub_rn(l, __fsub_rn(h, y))};
-}
-
-struct PairShared {
-    __align__(16) float colh[2][64], coll[2][64], rowh[64], rowl[64];
-    PairF piv[64];
-    int perm[64], kof[64];    // pivot row of step k; step of pivot row i
-    float rmax[64], cmax[64], amax, wmax[8], res[64], corr[64];
-    unsigned mark[2];         // columns with an element whose rounding is open
-    int open;                 // an element's rounding depends on the FP64 elimination's own error
-};
-
-// Column k = 4 kb + kk of the elimination (kk a constant: the tile m stays in
-// registers).  used: rows pivoted so far and the padding, per 32.
-template <int kk>
-__device__ __forceinline__ void pair_column(int n, int kb, int tr, int tc, bool act, PairF (&m)[4][4],
-                                            unsigned (&used)[2], bool& fine, PairShared& sh) {
-    constexpr int buf = kk & 1;
-    const int k = 4 * kb + kk, lane = threadIdx.x & 31, r0 = 4 * tr, c0 = 4 * tc;
-    if (k >= n || !fine) return;     // the same on every thread
-    if (tc == kb)
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const PairF v = two_sum(m[a][kk].h, m[a][kk].l);
-            sh.colh[buf][r0 + a] = v.h;
-            sh.coll[buf][r0 + a] = v.l;
-        }
-    __syncthreads();
-    // largest |column| among the free rows, the lowest row of equals (every warp for itself)
-    const unsigned b0 = (used[0] >> lane) & 1u ? 0u : __float_as_uint(sh.colh[buf][lane]) & 0x7fffffffu;
-    const unsigned b1 = (used[1] >> lane) & 1u ? 0u : __float_as_uint(sh.colh[buf][lane + 32]) & 0x7fffffffu;
-    const unsigned best = __reduce_max_sync(0xffffffffu, b0 > b1 ? b0 : b1);
-    const unsigned e0 = __ballot_sync(0xffffffffu, b0 == best), e1 = __ballot_sync(0xffffffffu, b1 == best);
-    const int p = e0 ? __ffs(e0) - 1 : 31 + __ffs(e1);
-    fine = best != 0u;
-    if (p < 32) used[0] |= 1u << p;
-    else used[1] |= 1u << (p - 32);
-    const int pa = p & 3;
-    if (tr == (p >> 2)) {
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const float h = pa == 0 ? m[0][b].h : pa == 1 ? m[1][b].h : pa == 2 ? m[2][b].h : m[3][b].h;
-            const float l = pa == 0 ? m[0][b].l : pa == 1 ? m[1][b].l : pa == 2 ? m[2][b].l : m[3][b].l;
-            const PairF v = two_sum(h, l);
-            sh.rowh[c0 + b] = v.h;
-            sh.rowl[c0 + b] = v.l;
-        }
-    }
-    __syncthreads();
-    if (act && fine) {
-        const PairF pv{sh.colh[buf][p], sh.coll[buf][p]}, ip = pair_rcp(pv);
-        if (threadIdx.x == 0) {
-            sh.piv[k] = pv;
-            sh.perm[k] = p;
-            sh.kof[p] = k;
-        }
-        PairF r[4], c[4];
-        const float4 rh = *(const float4*)(sh.rowh + c0), rl = *(const float4*)(sh.rowl + c0);
-        const float4 ch = *(const float4*)(sh.colh[buf] + r0), cl = *(const float4*)(sh.coll[buf] + r0);
-        r[0] = PairF{rh.x, rl.x}; r[1] = PairF{rh.y, rl.y}; r[2] = PairF{rh.z, rl.z}; r[3] = PairF{rh.w, rl.w};
-        c[0] = PairF{ch.x, cl.x}; c[1] = PairF{ch.y, cl.y}; c[2] = PairF{ch.z, cl.z}; c[3] = PairF{ch.w, cl.w};
-#pragma unroll
-        for (int b = 0; b < 4; ++b) r[b] = pair_mul(r[b], ip);
-        if (tc == kb) {      // the pivot column becomes -c / pivot
-            r[kk] = ip;
-#pragma unroll
-            for (int a = 0; a < 4; ++a) m[a][kk] = PairF{0.f, 0.f};
-        }
-        if (tr == (p >> 2)) {  // the pivot row becomes row / pivot
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                const bool on = a == pa;
-                c[a].h = on ? -1.f : c[a].h;
-                c[a].l = on ? 0.f : c[a].l;
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    m[a][b].h = on ? 0.f : m[a][b].h;
-                    m[a][b].l = on ? 0.f : m[a][b].l;
-                }
-            }
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {     // m -= c r; low parts renormalised when published
-                const float q = __fmul_rn(c[a].h, r[b].h);
-                float e = __fmaf_rn(c[a].h, r[b].h, -q);
-                e = __fmaf_rn(c[a].h, r[b].l, e);
-                e = __fmaf_rn(c[a].l, r[b].h, e);
-                const PairF t = two_sum(m[a][b].h, -q);
-                m[a][b].h = t.h;
-                m[a][b].l = __fadd_rn(m[a][b].l, __fsub_rn(t.l, e));
-            }
-    }
-}
-
-__global__ void __launch_bounds__(256, 3) invert_pair_kernel(int N, int n, int g, const float* __restrict__ Phi,
-                                                             float* __restrict__ Gt, double* __restrict__ logdet,
-                                                             int* err) {
-    extern __shared__ double sm[];
-    __shared__ PairShared sh;
-    const int w = blockIdx.x >> 1, sp = blockIdx.x & 1;
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-    const bool act = tid < g * g;
-    const int tr = act ? tid / g : g, tc = act ? tid - tr * g : g, r0 = 4 * tr, c0 = 4 * tc;
-    const float* A = Phi + ((size_t)w * N + (size_t)sp * n) * n;
-    PairF m[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) m[a][b] = PairF{(r0 + a < n && c0 + b < n) ? A[(r0 + a) * n + c0 + b] : 0.f, 0.f};
-    {
-        float v = 0.f;
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) v = fmaxf(v, fabsf(m[a][b].h));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-        if (lane == 0) sh.wmax[tid >> 5] = v;
-        if (tid < 2) sh.mark[tid] = 0u;
-        if (tid == 0) sh.open = 0;
-        __syncthreads();
-        if (tid == 0) {
-            for (int q = 1; q < nt / 32; ++q) v = fmaxf(v, sh.wmax[q]);
-            sh.amax = v;
-        }
-    }
-    unsigned used[2] = {0u, 0u};         // rows pivoted so far (and the padding), per 32
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-        if (n < 32 * (q + 1)) used[q] = n <= 32 * q ? 0xffffffffu : 0xffffffffu << (n - 32 * q);
-    bool fine = true;
-    for (int kb = 0; kb < g; ++kb) {
-        pair_column<0>(n, kb, tr, tc, act, m, used, fine, sh);
-        pair_column<1>(n, kb, tr, tc, act, m, used, fine, sh);
-        pair_column<2>(n, kb, tr, tc, act, m, used, fine, sh);
-        pair_column<3>(n, kb, tr, tc, act, m, used, fine, sh);
-    }
-    __syncthreads();
-    const int ld = n + 1;
-    float* Xh = (float*)sm;              // X[l][c], high parts, then the rounded inverse
-    float* Xl = Xh + n * ld;             // low parts
-    if (fine) {
-        if (act)                         // X[k][p_j] = M[p_k][j]
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    const int i = r0 + a, j = c0 + b;
-                    if (i < n && j < n) {
-                        const PairF v = two_sum(m[a][b].h, m[a][b].l);
-                        Xh[sh.kof[i] * ld + sh.perm[j]] = v.h;
-                        Xl[sh.kof[i] * ld + sh.perm[j]] = v.l;
-                    }
-                }
-        __syncthreads();
-        for (int t = tid; t < 2 * n; t += nt) {     // row and column maxima
-            const float* q = t < n ? Xh + t * ld : Xh + (t - n);
-            const int step = t < n ? 1 : ld;
-            float v = 0.f;
-            for (int k = 0; k < n; ++k) v = fmaxf(v, fabsf(q[k * step]));
-            (t < n ? sh.rmax : sh.cmax)[t < n ? t : t - n] = v;
-        }
-        __syncthreads();
-        const float scale = kPairMargin * 7.105427357601002e-15f * sh.amax;     // 2^-47
-        auto undecided = [&](int l, int c) {
-            const unsigned hb = __float_as_uint(Xh[l * ld + c]);
-            const float half = __uint_as_float(hb & 0x7f800000u) * 5.9604644775390625e-08f;   // half an ulp: 2^(e - 24)
-            const float lo = fabsf(Xl[l * ld + c]), d = scale * sh.rmax[l] * sh.cmax[c];
-            return fabsf(lo - half) < d || ((hb & 0x7fffffu) == 0u && fabsf(lo - 0.5f * half) < d);
-        };
-        for (int idx = tid; idx < n * n; idx += nt) {
-            const int l = idx / n, c = idx - l * n;
-            if (undecided(l, c)) atomicOr(&sh.mark[c >> 5], 1u << (c & 31));
-        }
-        __syncthreads();
-        unsigned mk[2] = {sh.mark[0], sh.mark[1]};
-        fine = __popc(mk[0]) + __popc(mk[1]) <= kPairColumns;
-        // the marked columns: eight threads per row of A, then per row of X
-        for (int h = 0; h < 2 && fine; ++h)
-            while (mk[h]) {
-                const int c = 32 * h + __ffs(mk[h]) - 1, sub = tid & 7;
-                mk[h] &= mk[h] - 1;
-                for (int r = tid >> 3; r < (n + 3) / 4 * 4; r += nt >> 3) {    // whole warps (4 rows each) go round
-                    double t = 0.0;
-                    if (r < n)
-                        for (int l = sub; l < n; l += 8)
-                            t = fma((double)A[r * n + l], (double)Xh[l * ld + c] + (double)Xl[l * ld + c], t);
-                    t += __shfl_xor_sync(0xffffffffu, t, 4);
-                    t += __shfl_xor_sync(0xffffffffu, t, 2);
-                    t += __shfl_xor_sync(0xffffffffu, t, 1);
-                    if (sub == 0 && r < n) sh.res[r] = (float)((r == c ? 1.0 : 0.0) - t);
-                }
-                __syncthreads();
-                for (int l = tid; l < n; l += nt) {
-                    float v = 0.f;
-                    for (int r = 0; r < n; ++r) v += Xh[l * ld + r] * sh.res[r];
-                    sh.corr[l] = v;
-                }
-                __syncthreads();
-                for (int l = tid; l < n; l += nt)
-                    if (undecided(l, c)) {
-                        const double v = (double)Xh[l * ld + c] + ((double)Xl[l * ld + c] + (double)sh.corr[l]);
-                        const float f = (float)v;
-                        // distance to f against half an ulp of f (a quarter below a power of two)
-                        const unsigned fb = __float_as_uint(f);
-                        const double half = (double)(__uint_as_float(fb & 0x7f800000u) * 5.9604644775390625e-08f);
-                        const double off = fabs(v - (double)f);
-                        const double d = (double)(kExactMargin / kPairMargin / 64.f * scale * sh.rmax[l] * sh.cmax[c]);
-                        if (!(fabs(off - half) >= d) || ((fb & 0x7fffffu) == 0u && fabs(off - 0.5 * half) < d))
-                            sh.open = 1;
-                        Xh[l * ld + c] = f;
-                        Xl[l * ld + c] = 0.f;
-                    }
-                __syncthreads();
-            }
-        if (fine && sh.open) fine = false;
-    }
-    if (!fine) {
-        __syncthreads();
-        gj_invert<float>(N, n, Phi, Gt, logdet, err, w, sp, sm);
-        return;
-    }
-    float* out = Gt + ((size_t)w * 2 + sp) * n * n;
-    for (int idx = tid; idx < n * n; idx += nt) out[idx] = Xh[idx % n * ld + idx / n];     // Gt[i][j] = X[j][i]
-    if (tid < 32) {
-        double lsum = 0.0;
-        for (int k = lane; k < n; k += 32) lsum += log(fabs((double)sh.piv[k].h + (double)sh.piv[k].l));
-        lsum = warp_sum(lsum);
-        if (lane == 0) logdet[2 * w + sp] = lsum;
-    }
 }
 
 // Mixed form, periodic recompute inside a call: one Newton-Schulz step
@@ -548,25 +260,13 @@ void launch_refine(int W, int N, int n, const float* Phi, float* Gt, double* log
 }
 
 template <typename T>
-static void launch_gj(int W, int N, int n, const T* Phi, T* Gt, double* logdet, int* err, cudaStream_t st) {
+void launch_invert(int W, int N, int n, const T* Phi, T* Gt, double* logdet, int* err, cudaStream_t st) {
     const size_t smem = (size_t)n * (n + 1) * sizeof(double) + n * sizeof(double) + n * sizeof(int);
     const int threads = n >= 32 ? 256 : 64;
     invert_kernel<T><<<2 * W, threads, smem, st>>>(N, n, Phi, Gt, logdet, err);
 }
 
-void launch_invert(int W, int N, int n, const double* Phi, double* Gt, double* logdet, int* err, cudaStream_t st) {
-    launch_gj(W, N, n, Phi, Gt, logdet, err, st);
-}
-
-void launch_invert(int W, int N, int n, const float* Phi, float* Gt, double* logdet, int* err, cudaStream_t st) {
-    if (n <= 16) {       // a few thousand FP64 operations: the pair kernel's barriers would cost more
-        launch_gj(W, N, n, Phi, Gt, logdet, err, st);
-        return;
-    }
-    const int g = (n + 3) / 4, threads = (g * g + 31) / 32 * 32;
-    // the pair inverse and what the FP64 fallback needs are within a few bytes of each other
-    const size_t smem = (size_t)n * (n + 1) * sizeof(double) + n * sizeof(double) + n * sizeof(int);
-    invert_pair_kernel<<<2 * W, threads, smem, st>>>(N, n, g, Phi, Gt, logdet, err);
-}
+template void launch_invert<double>(int, int, int, const double*, double*, double*, int*, cudaStream_t);
+template void launch_invert<float>(int, int, int, const float*, float*, double*, int*, cudaStream_t);
 
 }  // namespace qmc

@@ -31,10 +31,9 @@ void launch_adjoint_tc(const SysView<float>& s, const void* ahat, const float* G
                        const double* elw, const float* frec, double* acc, double* out_dl, double* out_de,
                        cudaStream_t st);
 
-// k_invert.cu: inverse of each walker's two Slater blocks, to FP64 accuracy (mixed
-// form: of the FP32 blocks, rounded to FP32).
-void launch_invert(int W, int N, int n, const double* Phi, double* Gt, double* logdet, int* err, cudaStream_t st);
-void launch_invert(int W, int N, int n, const float* Phi, float* Gt, double* logdet, int* err, cudaStream_t st);
+// k_invert.cu: FP64 Gauss-Jordan inverse of each walker's two Slater blocks.
+template <typename T>
+void launch_invert(int W, int N, int n, const T* Phi, T* Gt, double* logdet, int* err, cudaStream_t st);
 
 // k_invert.cu: mixed-form periodic recompute (one Newton-Schulz step, FP64
 // Gauss-Jordan where the carried inverse is too far off).

@@ -62,3 +62,22 @@ def test_mixed_sample_without_close_pairs(N, G, W):
     ref = orc.eval_configs(_osys(wl), wl.R, X, derivs=True)
     for _ in range(3):
         _close(s.eval_config(X, wl.R), ref, 1e-4)
+
+
+# The order of the orbitals does not change |det|, only the order of the elimination: ln|psi|
+# of two handles whose coefficients are column permutations of each other differs by the
+# elimination's rounding.  First order, delta ln|det| = tr(A^-1 E) with rounding errors
+# E_ij of random sign, some u sqrt(n) max|A| each after n steps: |delta| <~ u sqrt(n)
+# |A^-1|_F max|A|; three times that per block (u = 2^-53), and the result's own last place.
+@pytest.mark.parametrize("N", [34, 64, 126])
+def test_mixed_determinant_is_eliminated_in_fp64(N):
+    wl = _workload(N, 2, 24)
+    X, n = _sampled(wl, 24), N // 2
+    perm = np.random.default_rng(1).permutation(n)
+    lp = [q.QMCSystem(q.Config.from_workload(wl, precision=q.QMC_MIXED, coeff=C), wl.R).eval_config(X, wl.R)["lnpsi"]
+          for C in (wl.C, np.ascontiguousarray(wl.C[:, perm]))]
+    u = 2.0 ** -53
+    for k, x in enumerate(X):
+        A = np.asarray(orc.slater_matrices(_osys(wl), wl.R, x)).reshape(2, n, n)
+        tol = sum(3 * u * np.sqrt(n) * np.linalg.norm(np.linalg.inv(a)) * np.max(np.abs(a)) for a in A)
+        assert abs(lp[0][k] - lp[1][k]) <= tol + 4 * u * abs(lp[0][k]), (k, lp[0][k] - lp[1][k], tol)
