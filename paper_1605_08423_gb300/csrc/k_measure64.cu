@@ -47,6 +47,9 @@ int pad_pow2(int n) {
 // Shared memory of one CTA.  tb: basis rows per tile; in the real form with tb >= B
 // the Z and chi rows of a spin block stay for the second pass.  The twisted form
 // keeps G in shared memory up to n = 32 (np <= 32) and reads it from global memory above.
+// rho(k) stands behind the phase table in the work space of the orbital products, which
+// are done by then: at the largest cutoff (ewald_mmax = 12, 3576 vectors) its 57 KB beside
+// them left no launch for twisted cells of N >= 84 (every accepted cell fits 225 KB now).
 struct M64Layout {
     size_t xs, et, gU, lU, Ui, gi, vv, li, facc, rhot, red, part, uni, total;
     __host__ __device__ static size_t square2(int np) { return (size_t)np * (2 * np + 4); }   // complex np x np, planar
@@ -56,12 +59,12 @@ struct M64Layout {
         xs = take(3 * N); et = take(6 * N); gU = take(3 * N); lU = take(N); Ui = take(N);
         gi = take(3 * N); vv = take(3 * N); li = take(N);
         facc = take(9 * N);
-        rhot = take(2 * nk);
         red = take(64);
         // slices of the Jastrow sums (5 + 4 per electron; N <= kThreads), then the warps' g_i, l_i sums
         const size_t jp = 9 * (size_t)kThreads, gp = 4 * (size_t)kWarps * n;
         part = take(jp > gp ? jp : gp);
-        size_t u = 2 * (size_t)N * 3 * (mmax + 1);                            // phase table
+        const size_t table = 2 * (size_t)N * 3 * (mmax + 1);                  // phase table
+        size_t u = table + 2 * (size_t)nk;
         if (tw) {
             const size_t sq = square2(np), tile = (size_t)tb * (2 * np + 2);
             const size_t s = (np <= 32 ? 2 : 1) * sq + (sq > tile ? sq : tile);       // G, Y / K, then T or the tile
@@ -72,6 +75,7 @@ struct M64Layout {
         }
         if (j34 && 44 * (size_t)N > u) u = 44 * (size_t)N;
         uni = take(u);
+        rhot = uni + 8 * table;
         total = o;
     }
 };

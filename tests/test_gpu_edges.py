@@ -81,3 +81,17 @@ def test_mixed_determinant_is_eliminated_in_fp64(N):
         A = np.asarray(orc.slater_matrices(_osys(wl), wl.R, x)).reshape(2, n, n)
         tol = sum(3 * u * np.sqrt(n) * np.linalg.norm(np.linalg.inv(a)) * np.max(np.abs(a)) for a in A)
         assert abs(lp[0][k] - lp[1][k]) <= tol + 4 * u * abs(lp[0][k]), (k, lp[0][k] - lp[1][k], tol)
+
+
+# the largest cutoff: 3576 reciprocal vectors beside the sample's work space in shared memory
+@pytest.mark.parametrize("N,G,twisted", [(84, 2, True), (94, 1, True), (128, 4, True), (94, 2, False), (128, 4, False)])
+def test_sample_at_the_largest_reciprocal_cutoff(N, G, twisted):
+    wl = _workload(N, G, 2)
+    tw = synth.monkhorst_pack(4)[[11]] if twisted else None
+    X = _sampled(wl, 2)
+    g = q.QMCSystem(q.Config.from_workload(wl, twists=tw, mmax=12), wl.R).eval_config(X, wl.R)
+    if twisted:
+        ref = orc.eval_configs_twist(_osys(wl, twist=np.asarray(tw[0]), mmax=12), wl.R, X, tw)
+    else:
+        ref = orc.eval_configs(_osys(wl, mmax=12), wl.R, X, derivs=True)
+    _close(g, ref, 1e-10)
