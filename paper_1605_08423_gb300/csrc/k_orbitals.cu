@@ -275,26 +275,25 @@ template <typename T>
 __global__ void propose_kernel(int W, int N, double L, double* __restrict__ X, double* __restrict__ Xp,
                                T* __restrict__ ptp, T* __restrict__ uacc, Key key, uint32_t md, uint32_t sweep,
                                double sigma, uint32_t w0) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x, rows = W * N;
-    const bool uniform = sizeof(T) == 4 ? k < rows : k >= 3 * rows;
-    const int t = sizeof(T) == 4 ? k : (uniform ? k - 3 * rows : k / 3);
-    if (t >= rows) return;
-    const int w = t / N, i = t - w * N;
+    const int rows = W * N;
+    const ProposeTask task = propose_task((long long)blockIdx.x * blockDim.x + threadIdx.x, rows, sizeof(T) == 8);
+    if (task.t < 0) return;
+    const int t = task.t, w = t / N, i = t - w * N;
     const uint32_t idx = sweep * (uint32_t)N + (uint32_t)i;
     if constexpr (sizeof(T) == 4) {
 #pragma unroll
         for (int mu = 0; mu < 3; ++mu) propose_coordinate<T>(t, mu, w, idx, L, X, Xp, ptp, key, md, sigma, w0);
-    } else if (!uniform) {
-        propose_coordinate<T>(t, k - 3 * t, w, idx, L, X, Xp, ptp, key, md, sigma, w0);
+    } else if (task.mu < 3) {
+        propose_coordinate<T>(t, task.mu, w, idx, L, X, Xp, ptp, key, md, sigma, w0);
     }
-    if (uniform) uacc[t] = Draw<T>::uniform(philox(w0 + (uint32_t)w, md, idx, kAccept, key));
+    if (task.mu == 3) uacc[t] = Draw<T>::uniform(philox(w0 + (uint32_t)w, md, idx, kAccept, key));
 }
 
 template <typename T>
 void launch_propose(int W, int N, double L, double* X, double* Xp, T* ptp, T* uacc, Key key, uint32_t md,
                     uint32_t sweep, double sigma, uint32_t w0, cudaStream_t st) {
-    const int tot = (sizeof(T) == 4 ? 1 : 4) * W * N, tpb = sizeof(T) == 4 ? 256 : 128;
-    propose_kernel<T><<<(tot + tpb - 1) / tpb, tpb, 0, st>>>(W, N, L, X, Xp, ptp, uacc, key, md, sweep, sigma, w0);
+    const int tpb = sizeof(T) == 4 ? 256 : 128;
+    propose_kernel<T><<<propose_blocks(W * N, sizeof(T) == 8, tpb), tpb, 0, st>>>(W, N, L, X, Xp, ptp, uacc, key, md, sweep, sigma, w0);
 }
 
 // Walker start: electron i next to proton i (up electrons on protons 0..N/2-1,

@@ -10,6 +10,24 @@ void launch_orbitals(const SysView<float>& s, const double* pos, int nrows, floa
 // FP64 form, values only; trig: (sin, cos)(pi x / L) [rows][6] of the positions, or null
 void launch_orbitals(const SysView<double>& s, const double* pos, const double* trig, int nrows, double* val,
                      cudaStream_t st);
+// Thread k of the proposal kernel: electron t (of rows = W N) and what it does there,
+// mu = 0..2 a coordinate, 3 the acceptance uniform.  With per_coordinate the 3 rows
+// coordinates come first, then the uniforms; else a thread has an electron's all (mu = 3).
+// t < 0: nothing to do.  Indices in 64 bits: 4 rows exceeds an int from 2^29 electrons on
+// (34 million walkers of N = 16, about 210 GB).
+struct ProposeTask { int t, mu; };
+__host__ __device__ inline ProposeTask propose_task(long long k, int rows, bool per_coordinate) {
+    if (!per_coordinate) return k < rows ? ProposeTask{(int)k, 3} : ProposeTask{-1, 0};
+    const long long r3 = 3LL * rows;
+    if (k < r3) {
+        const long long t = k / 3;
+        return ProposeTask{(int)t, (int)(k - 3 * t)};
+    }
+    return k < r3 + rows ? ProposeTask{(int)(k - r3), 3} : ProposeTask{-1, 0};
+}
+inline unsigned propose_blocks(int rows, bool per_coordinate, int threads) {
+    return (unsigned)(((per_coordinate ? 4LL : 1LL) * rows + threads - 1) / threads);
+}
 template <typename T>
 void launch_propose(int W, int N, double L, double* X, double* Xp, T* ptp, T* uacc, Key key, uint32_t md,
                     uint32_t sweep, double sigma, uint32_t w0, cudaStream_t st);
