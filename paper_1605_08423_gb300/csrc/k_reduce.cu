@@ -21,15 +21,16 @@
 namespace qmc {
 
 // The reductions run for a batch of K walker blocks of W walkers each (the
-// twists of a twisted handle; K = 1 otherwise), batch index blockIdx.y (.z in
-// the Gram kernels): one launch sequence for the whole mesh, where one per
-// twist made 320 launches and 2.25 ms of a 64-twist call at N = 64 (0.29 ms batched).
+// twists of a twisted handle; K = 1 otherwise): one launch sequence for the whole
+// mesh, where one per twist made 320 launches and 2.25 ms of a 64-twist call at N = 64
+// (0.29 ms batched).  The batch is part of blockIdx.x, the one grid dimension that goes
+// beyond 65535: a 41 x 41 x 41 mesh has 68921 twists.
 
 // colsum[c] = sum_w acc[w][c] for c < ncol; colsum[ncol] = sum_w nacc[w].
 __global__ void colsum_kernel(int W, int ncol, const double* __restrict__ acc, const unsigned long long* __restrict__ nacc,
                               double* colsum) {
     __shared__ double red[32];
-    const int c = blockIdx.x, b = blockIdx.y;
+    const int c = blockIdx.x % (ncol + 1), b = blockIdx.x / (ncol + 1);
     acc += (size_t)b * W * ncol;
     nacc += (size_t)b * W;
     colsum += (size_t)b * (ncol + 1);
@@ -64,14 +65,15 @@ __global__ void finalize_kernel(int N, double moves, const double* __restrict__ 
 }
 
 // dev[w][c] = f_w[c] - f[c] (c < 3N), dev[w][3N] = E_w - E.
-__global__ void deviation_kernel(int W, int N, const double* __restrict__ acc, const double* __restrict__ out,
+__global__ void deviation_kernel(int W, int N, int blocks, const double* __restrict__ acc, const double* __restrict__ out,
                                  double* dev) {
     const int N3 = 3 * N, ncol = 3 + 9 * N;
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = blockIdx.x / blocks;                     // `blocks` blocks a batch
+    const size_t t = (size_t)(blockIdx.x - b * blocks) * blockDim.x + threadIdx.x;
     if (t >= (size_t)W * (N3 + 1)) return;
-    acc += (size_t)blockIdx.y * W * ncol;
-    out += (size_t)blockIdx.y * (4 + N3 + (size_t)N3 * N3);
-    dev += (size_t)blockIdx.y * W * (N3 + 1);
+    acc += (size_t)b * W * ncol;
+    out += (size_t)b * (4 + N3 + (size_t)N3 * N3);
+    dev += (size_t)b * W * (N3 + 1);
     const int w = (int)(t / (N3 + 1)), c = (int)(t - (size_t)w * (N3 + 1));
     const double* a = acc + (size_t)w * ncol;
     const double cnt = a[0], E = out[0];
@@ -91,15 +93,15 @@ __global__ void deviation_kernel(int W, int N, const double* __restrict__ acc, c
 // 36 at N = 64: the reduction took 5.5 ms for 16384 walkers and 1.3 ms for 4096,
 // now 2.5 and 0.24 ms).  The slices'
 // partial tiles go to ws [K][nsplit][tiles][256], summed in order by
-// gram_sum_kernel.  Tile index blockIdx.x (the last one is the energy's sum),
-// slice blockIdx.y, batch blockIdx.z.
+// gram_sum_kernel.  blockIdx.x counts tiles (the last one is the energy's sum),
+// then slices, then batches.
 constexpr int kGramTile = 16, kGramRows = 32;
-__global__ void __launch_bounds__(256) gram_kernel(int W, int N, int tiles, const double* __restrict__ dev, double* ws) {
+__global__ void __launch_bounds__(256) gram_kernel(int W, int N, int tiles, int ns, const double* __restrict__ dev, double* ws) {
     __shared__ double A[kGramRows][kGramTile], Bm[kGramRows][kGramTile];
     const int N3 = 3 * N, ld = N3 + 1, tid = threadIdx.x;
-    const int t = blockIdx.x, sl = blockIdx.y, ns = gridDim.y;
-    dev += (size_t)blockIdx.z * W * ld;
-    ws += (((size_t)blockIdx.z * ns + sl) * (tiles + 1) + t) * 256;
+    const int q = blockIdx.x / (tiles + 1), t = blockIdx.x - q * (tiles + 1), b = q / ns, sl = q - b * ns;
+    dev += (size_t)b * W * ld;
+    ws += (size_t)blockIdx.x * 256;
     const int w0 = (int)((long long)W * sl / ns), w1 = (int)((long long)W * (sl + 1) / ns);
     if (t == tiles) {
         double e = 0.0;
@@ -141,10 +143,10 @@ __global__ void __launch_bounds__(256) gram_sum_kernel(int N, int tiles, int ns,
                                                        double* dst_e, double* dst_S, size_t stride, double scale,
                                                        int finish) {
     __shared__ double red[32];
-    const int N3 = 3 * N, tid = threadIdx.x, t = blockIdx.x;
-    dst_e += blockIdx.z * stride;
-    dst_S += blockIdx.z * stride;
-    ws += ((size_t)blockIdx.z * ns * (tiles + 1) + t) * 256 + tid;
+    const int N3 = 3 * N, tid = threadIdx.x, b = blockIdx.x / (tiles + 1), t = blockIdx.x - b * (tiles + 1);
+    dst_e += b * stride;
+    dst_S += b * stride;
+    ws += ((size_t)b * ns * (tiles + 1) + t) * 256 + tid;
     double v = 0.0;
     for (int s = 0; s < ns; ++s) v += ws[(size_t)s * (tiles + 1) * 256];
     if (t == tiles) {
@@ -178,19 +180,20 @@ size_t gram_ws_doubles(int K, int W, int N) {
 static void gram(int K, int W, int N, const double* dev, double* ws, double* dst_e, double* dst_S, size_t stride,
                  double scale, int finish, cudaStream_t st) {
     const int tiles = gram_tiles(N), ns = gram_splits(K, W, N);
-    gram_kernel<<<dim3(tiles + 1, ns, K), 256, 0, st>>>(W, N, tiles, dev, ws);
-    gram_sum_kernel<<<dim3(tiles + 1, 1, K), 256, 0, st>>>(N, tiles, ns, ws, dst_e, dst_S, stride, scale, finish);
+    gram_kernel<<<(unsigned)(tiles + 1) * ns * K, 256, 0, st>>>(W, N, tiles, ns, dev, ws);
+    gram_sum_kernel<<<(unsigned)(tiles + 1) * K, 256, 0, st>>>(N, tiles, ns, ws, dst_e, dst_S, stride, scale, finish);
 }
 
 static void deviations(int K, int W, int N, const double* acc, const double* out, double* dev, cudaStream_t st) {
     const size_t tot = (size_t)W * (3 * N + 1);
-    deviation_kernel<<<dim3((unsigned)((tot + 255) / 256), K), 256, 0, st>>>(W, N, acc, out, dev);
+    const int blocks = (int)((tot + 255) / 256);
+    deviation_kernel<<<(unsigned)blocks * K, 256, 0, st>>>(W, N, blocks, acc, out, dev);
 }
 
 void launch_reduce(int K, int W, int N, double moves, const double* acc, const unsigned long long* nacc, double* colsum,
                    double* dev, double* ws, double* out, int* err, cudaStream_t st) {
     const int ncol = 3 + 9 * N, N3 = 3 * N;
-    colsum_kernel<<<dim3(ncol + 1, K), 256, 0, st>>>(W, ncol, acc, nacc, colsum);
+    colsum_kernel<<<(unsigned)(ncol + 1) * K, 256, 0, st>>>(W, ncol, acc, nacc, colsum);
     finalize_kernel<<<K, 256, 0, st>>>(N, moves, colsum, out, err);
     deviations(K, W, N, acc, out, dev, st);
     gram(K, W, N, dev, ws, out + 1, out + 4 + N3, 4 + N3 + (size_t)N3 * N3, W > 1 ? 1.0 / ((double)W * (W - 1)) : 0.0, 1,

@@ -95,3 +95,16 @@ def test_sample_at_the_largest_reciprocal_cutoff(N, G, twisted):
     else:
         ref = orc.eval_configs(_osys(wl, mmax=12), wl.R, X, derivs=True)
     _close(g, ref, 1e-10)
+
+
+# more twists than a grid's second and third dimensions hold (65535): 65537 points of the
+# 41 x 41 x 41 mesh, two walkers each, reduced on their own and averaged; the tolerance is
+# that of sums taken in another order
+def test_more_twists_than_a_grid_dimension_holds():
+    K = 65537
+    wl = _workload(2, 1, 2 * K)
+    s = q.QMCSystem(q.Config.from_workload(wl, warmup=1, twists=synth.monkhorst_pack(41)[:K]), wl.R)
+    g, ref = s.energy_forces(wl.R), orc.reduce_twists(s.accumulators(), 2, K)
+    for key in ("E", "E_err", "f", "S"):
+        a, b = np.asarray(g[key]).ravel(), np.asarray(ref[key]).ravel()
+        assert np.max(np.abs(a - b)) <= 1e-12 * K * np.max(np.abs(b)), key
