@@ -100,6 +100,15 @@ __device__ __forceinline__ void toy_normals(uint4 w, const ToyTables& T, double&
     xi1 = rho * (t.x * cs + t.y * sn);
 }
 
+// The same from the library's log and sincospi, without the tables.
+__device__ __forceinline__ void toy_normals_library(uint4 w, double& xi0, double& xi1) {
+    const double rho = sqrt(-2.0 * log(u53(w.x, w.y)));
+    double sn, cs;
+    sincospi(2.0 * u53(w.z, w.w), &sn, &cs);
+    xi0 = rho * cs;
+    xi1 = rho * sn;
+}
+
 // x > 0 for a finite or infinite x, false for NaN, on the integer pipe
 __device__ __forceinline__ bool positive(double x) {
     const int h = __double2hiint(x);
@@ -118,11 +127,13 @@ __device__ __forceinline__ bool positive(double x) {
 // magnitude) equals phi_end - phi_0 + 2 pi (net turns across the negative x axis),
 // so only the crossings are counted per step -- sign tests on the y coordinates and
 // on the cross product R x R' -- and phi comes from atan2 at the two ends.
-template <int SCHEME, bool HG>
+// TAB: normals by the tables, which every block fills first; without them (launch_scheme)
+// the library's functions.
+template <int SCHEME, bool HG, bool TAB>
 __global__ void __launch_bounds__(128) toy_kernel(ToyDev p, int n_traj, const double* __restrict__ xy0,
                                                   double* __restrict__ out) {
     __shared__ ToyTables T;
-    fill_tables(T);
+    if constexpr (TAB) fill_tables(T);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n_traj) return;
     const double x0 = xy0[2 * t], y0 = xy0[2 * t + 1];
@@ -136,7 +147,9 @@ __global__ void __launch_bounds__(128) toy_kernel(ToyDev p, int n_traj, const do
     const double c22 = HG ? 0.0 : rsqrt(p.sr_const);                // 1 / sqrt(det S) of G_lambda
     for (int s = 0; s < p.n_steps; ++s) {
         double xi0, xi1;
-        toy_normals(philox((uint32_t)t, (uint32_t)s, 0u, kToy, p.key), T, xi0, xi1);
+        const uint4 w = philox((uint32_t)t, (uint32_t)s, 0u, kToy, p.key);
+        if constexpr (TAB) toy_normals(w, T, xi0, xi1);
+        else toy_normals_library(w, xi0, xi1);
         const double fr = fma(ka, ir, -p.k);                        // f = fr R
         // terms added in the order of the schemes above
         double xn, yn, st = 1.0, d = 0.0;
@@ -235,8 +248,14 @@ template <int SCHEME>
 void launch_scheme(const ToyDev& p, int n_traj, const double* xy0, double* out, cudaStream_t st) {
     // one warp per block while every warp can have an SM's FP64 issue ports nearly to itself
     const int tpb = n_traj <= 32 * 2 * 152 ? 32 : 128, grid = (n_traj + tpb - 1) / tpb;
-    if (p.s_mode == QMC_TOY_S_HG) toy_kernel<SCHEME, true><<<grid, tpb, 0, st>>>(p, n_traj, xy0, out);
-    else toy_kernel<SCHEME, false><<<grid, tpb, 0, st>>>(p, n_traj, xy0, out);
+    // a block's tables (128 logarithms, 256 sincospi) cost more than one or two steps save:
+    // the adopted scheme's 10^6 trajectories take 562 / 749 / 937 / 1124 us for 1 / 2 / 3 / 4
+    // steps with them, 440 / 682 / 925 / 1165 with the library's functions (10^3: 23 / 27 /
+    // 31 / 33 and 12 / 17 / 21 / 25); the other schemes cross between 2 and 4 too.
+    const bool hg = p.s_mode == QMC_TOY_S_HG;
+    const auto kernel = p.n_steps <= 2 ? (hg ? toy_kernel<SCHEME, true, false> : toy_kernel<SCHEME, false, false>)
+                                       : (hg ? toy_kernel<SCHEME, true, true> : toy_kernel<SCHEME, false, true>);
+    kernel<<<grid, tpb, 0, st>>>(p, n_traj, xy0, out);
 }
 
 }  // namespace

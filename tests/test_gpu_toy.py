@@ -92,3 +92,11 @@ def test_toy_full_size_sampled_trajectories():
     # and the whole launch samples the canonical <U> = T/2 (SI: the adopted scheme has no time-step error here)
     mU = g[:, 2].sum() / (n * (steps - cfg["n_burn"]))
     assert abs(mU - synth.TOY_T / 2) < 0.01 * synth.TOY_T / 2, mU
+
+
+# the shortest runs take their normals from the library's functions, longer ones from tables
+@pytest.mark.parametrize("n_steps", [0, 1, 2, 3])
+@pytest.mark.parametrize("scheme", list(q.TOY_SCHEMES.values()))
+def test_toy_shortest_runs_match_oracle(scheme, n_steps):
+    for s_mode, mu in ((q.QMC_TOY_S_G, 0.5), (q.QMC_TOY_S_HG, 2.0)):
+        _close(*_both(scheme, s_mode, mu, n_traj=300, n_steps=n_steps, n_burn=0, delta=0.1))
