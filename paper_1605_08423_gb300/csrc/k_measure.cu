@@ -644,14 +644,16 @@ __global__ void __launch_bounds__(256, 3) measure_kernel(SysView<T> s, int mmax,
                     }
                 }
             }
-            if (ac + lane < N)
+            for (int q = 0; q < nw; ++q) {       // the warps' sums in order
+                if (q == warp && ac + lane < N)
 #pragma unroll
-                for (int mu = 0; mu < 3; ++mu) {
-                    atomicAdd(&f_dl[3 * a + mu], dl[mu].value());
-                    atomicAdd(&f_de[3 * a + mu], de[mu].value());
-                }
+                    for (int mu = 0; mu < 3; ++mu) {
+                        f_dl[3 * a + mu] += dl[mu].value();
+                        f_de[3 * a + mu] += de[mu].value();
+                    }
+                __syncthreads();
+            }
         }
-        __syncthreads();
     }
 
     // ---- P4a: electron-electron real-space Ewald

@@ -73,7 +73,7 @@ struct M64Layout {
             const size_t s = 2 * (size_t)np * (np + 2) + 3 * (size_t)tb * (np + 2);   // G, M, Z, chi, y / P
             u = u > s ? u : s;
         }
-        if (j34 && 44 * (size_t)N > u) u = 44 * (size_t)N;
+        if (j34 && 92 * (size_t)N > u) u = 92 * (size_t)N;   // c, S, 5 a warp, the warps' force terms
         uni = take(u);
         rhot = uni + 8 * table;
         total = o;
@@ -441,6 +441,7 @@ __global__ void __launch_bounds__(kThreads, TM ? 2 : 1) measure64_kernel(SysView
     double* j34c = uni;              // [N]
     double* j34S = j34c + N;         // [N][3]
     double* st = j34S + 3 * N + (size_t)warp * 5 * N;   // per warp: c - chi_i [N], grad chi_i [N][3], lap chi_i [N]
+    double* j34f = j34S + 3 * N + (size_t)kWarps * 5 * N;   // [6][kWarps][N] force terms of the warps' electrons
     const double zj = s.zeta_j;
     auto j34_sums = [&]() {
         for (int a = tid; a < N; a += kThreads) {
@@ -756,6 +757,8 @@ __global__ void __launch_bounds__(kThreads, TM ? 2 : 1) measure64_kernel(SysView
     //                          + (Hess chi_a(r_i) vv_i) w_ia + (vv_i . v_ia) s_a^(i) ]
     // (the R_a-derivative of -1/2 sum_i [lap_i U34 + 2 vv_i . grad_i U34]).
     if (j34) {
+        // a warp adds its electrons' terms up in its own slots, the warps are added in order
+        for (int idx = tid; idx < 6 * kWarps * N; idx += kThreads) j34f[idx] = 0.0;
         j34_sums();
         for (int i = warp; i < N; i += kWarps) {
             for (int a = lane; a < N; a += 32) {
@@ -781,13 +784,21 @@ __global__ void __launch_bounds__(kThreads, TM ? 2 : 1) measure64_kernel(SysView
                 double hv[3];
                 hess_mul(rd.h, vv, hv);
                 const double vvv = vv[0] * v[0] + vv[1] * v[1] + vv[2] * v[2];
+                double* o = j34f + (size_t)warp * N + a;
                 for (int mu = 0; mu < 3; ++mu) {
                     const double sa = j34S[3 * a + mu] - rd.g[mu];
-                    atomicAdd(&f_dl[3 * a + mu], -rd.g[mu] * wa);
-                    atomicAdd(&f_de[3 * a + mu], 0.5 * (rd.tl[mu] * wa + lam * sa) + hv[mu] * wa + vvv * sa);
+                    o[mu * kWarps * N] -= rd.g[mu] * wa;
+                    o[(3 + mu) * kWarps * N] += 0.5 * (rd.tl[mu] * wa + lam * sa) + hv[mu] * wa + vvv * sa;
                 }
             }
             __syncwarp();
+        }
+        __syncthreads();
+        for (int idx = tid; idx < 6 * N; idx += kThreads) {
+            const int c = idx / N, a = idx - c * N;
+            double t = 0;
+            for (int q = 0; q < kWarps; ++q) t += j34f[(size_t)(c * kWarps + q) * N + a];
+            (c < 3 ? f_dl : f_de)[3 * a + c % 3] += t;
         }
         __syncthreads();
     }

@@ -108,3 +108,19 @@ def test_more_twists_than_a_grid_dimension_holds():
     for key in ("E", "E_err", "f", "S"):
         a, b = np.asarray(g[key]).ravel(), np.asarray(ref[key]).ravel()
         assert np.max(np.abs(a - b)) <= 1e-12 * K * np.max(np.abs(b)), key
+
+
+# every sum in a fixed order, also with the e-e-n-n Jastrow term: the same call on two
+# handles gives the same accumulators to the bit
+@pytest.mark.parametrize("N,G,mixed,twisted", [(54, 4, True, False), (128, 4, True, False), (126, 2, True, False),
+                                               (30, 2, False, False), (66, 2, False, False), (22, 2, False, True)])
+def test_eenn_samples_are_reproducible(N, G, mixed, twisted):
+    wl = _workload(N, G, 200, sweeps=2)
+    f = 0.02 * np.random.default_rng(3).standard_normal((N, N))
+    runs = []
+    for _ in range(3):
+        s = q.QMCSystem(q.Config.from_workload(wl, warmup=2, fj=f + f.T, precision=q.QMC_MIXED if mixed else q.QMC_FP64,
+                                               twists=synth.monkhorst_pack(2)[:2] if twisted else None), wl.R)
+        s.energy_forces(wl.R)
+        runs.append(s.accumulators())
+    assert np.array_equal(runs[0], runs[1]) and np.array_equal(runs[0], runs[2])
