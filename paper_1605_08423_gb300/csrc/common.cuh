@@ -67,7 +67,8 @@ template <> struct Draw<float> {
 //   exp(x) = 2^m (2^(j/64) + 2^(j/64) (r + r^2/2 + ... + r^5/120)),
 // 11 FP64 operations (the library's 18 cost 340 clocks of an SM's FP64 pipe per
 // warp); the truncation is below 4e-17, the result within 1 unit in the last
-// place.  Arguments below -690 give 0, above 700 the library's value.
+// place.  From |x| = 690 on, where 2^m (..) leaves the normal range, the library's value
+// (0 below -746: no call where far images and nuclei are evaluated by the thousand).
 static __device__ const double kExp2j64[64] = {
     0x1.0000000000000p+0, 0x1.02c9a3e778061p+0, 0x1.059b0d3158574p+0, 0x1.0874518759bc8p+0,
     0x1.0b5586cf9890fp+0, 0x1.0e3ec32d3d1a2p+0, 0x1.11301d0125b51p+0, 0x1.1429aaea92de0p+0,
@@ -88,7 +89,8 @@ static __device__ const double kExp2j64[64] = {
 __device__ __forceinline__ double qexp(double x) {
     const double magic = 6755399441055744.0;                     // 1.5 * 2^52
     const int hx = __double2hiint(x);
-    if ((hx & 0x7fffffff) >= 0x40859000) return hx < 0 && hx < (int)0xfff00001 ? 0.0 : exp(x);   // |x| >= 690 or NaN
+    if ((hx & 0x7fffffff) >= 0x40859000)                         // |x| >= 690 or NaN; [-inf, -746] on the integer pipe
+        return hx >= (int)0xc0875000 && hx < (int)0xfff00001 ? 0.0 : exp(x);
     const double q = fma(x, 0x1.71547652b82fep+6, magic);                          // 64 / ln 2
     const int k = __double2loint(q);
     const double kd = q - magic;

@@ -124,3 +124,20 @@ def test_eenn_samples_are_reproducible(N, G, mixed, twisted):
         s.energy_forces(wl.R)
         runs.append(s.accumulators())
     assert np.array_equal(runs[0], runs[1]) and np.array_equal(runs[0], runs[2])
+
+
+# an electron so far from every proton that its orbitals are some 1e-302 (still normal numbers):
+# the determinant is not singular and all terms are finite
+def test_fp64_sample_of_a_far_electron():
+    wl = synth.Workload(name="far", N=2, rs=39.0, zeta=(0.8,), walkers=2, sweeps=1, seed=3)
+    X = np.random.default_rng(5).uniform(0.0, wl.L, (200000, 3))
+    d = X[:, None] - wl.R
+    t = np.min((wl.L / np.pi) ** 2 * np.sum(np.sin(np.pi * d / wl.L) ** 2, -1), -1)
+    far = X[(0.8 * t > 691.0) & (0.8 * t < 699.0)][:2]
+    X = np.stack([far, wl.R[1] + [[0.3, 0.2, 0.4], [0.5, -0.2, 0.1]]], 1)
+    g = q.QMCSystem(q.Config.from_workload(wl), wl.R).eval_config(X, wl.R)
+    # the oracle's dual numbers hold 1/phi^2: orbitals scaled by 2^500, which only shifts ln|psi|
+    osys = orc.System(N=2, L=wl.L, zeta=np.array(wl.zeta), coeff=wl.C * 2.0 ** 500)
+    lp, el, dl, de = orc.eval_configs(osys, wl.R, X, derivs=True)
+    assert all(np.all(np.isfinite(v)) for v in (lp, el, dl, de))
+    _close(g, (lp - 1000.0 * np.log(2.0), el, dl, de), 1e-10)
