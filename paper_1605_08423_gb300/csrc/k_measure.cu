@@ -146,15 +146,17 @@ __device__ __forceinline__ void sincos_half(double x, double& sn, double& cs) {
 }
 
 // erf(kappa r)/r = kappa 2/sqrt(pi) sum_n (-x)^n / (n! (2n + 1)), x = (kappa r)^2 <= 2/3,
-// to n = 12 (remainder 1e-14), with its derivative in x, both over kappa 2/sqrt(pi).
+// to n = 15 (remainder below 3e-18), with its derivative in x (below 6e-17), both over
+// kappa 2/sqrt(pi).
 __device__ __forceinline__ double erf_over_r_series(double x, double& d) {
-    constexpr double c[13] = {1.0,            -1.0 / 3.0,         1.0 / 10.0,           -1.0 / 42.0,        1.0 / 216.0,
-                              -1.0 / 1320.0,  1.0 / 9360.0,       -1.0 / 75600.0,       1.0 / 685440.0,     -1.0 / 6894720.0,
-                              1.0 / 76204800.0, -1.0 / 918086400.0, 1.0 / 11975040000.0};
-    double v = c[12];
+    constexpr double c[16] = {1.0, -1.0 / 3.0, 1.0 / 10.0, -1.0 / 42.0, 1.0 / 216.0, -1.0 / 1320.0, 1.0 / 9360.0,
+                              -1.0 / 75600.0, 1.0 / 685440.0, -1.0 / 6894720.0, 1.0 / 76204800.0, -1.0 / 918086400.0,
+                              1.0 / 11975040000.0, -1.0 / 168129561600.0, 1.0 / 2528170444800.0,
+                              -1.0 / 40537905408000.0};
+    double v = c[15];
     d = 0.0;
 #pragma unroll
-    for (int n = 11; n >= 0; --n) {
+    for (int n = 14; n >= 0; --n) {
         d = fma(d, x, v);
         v = fma(v, x, c[n]);
     }
@@ -165,7 +167,7 @@ __device__ __forceinline__ double erf_over_r_series(double x, double& d) {
 // d ln psi/dR_a) and de (to dE_L/dR_a, given vv = g_i + grad_i U), and the nearest
 // image's phi(r) = erfc(kappa r)/r with its gradient, for d = r_i - R_a.  The pairs
 // are closer than 0.3 bohr, so short series give the trig and the smooth part
-// erf(kappa r)/r: some 170 FP64 operations a pair (450 with the library's sincospi,
+// erf(kappa r)/r: some 180 FP64 operations a pair (450 with the library's sincospi,
 // erfc, exp and divisions).  Cells and splittings outside the series' range
 // (L < 2.1, kappa > 2.5) take the library calls.
 __device__ __forceinline__ void close_pair(const double d[3], double L, double iL, double ell, double kappa, double k2,
