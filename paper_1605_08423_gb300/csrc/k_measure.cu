@@ -72,13 +72,9 @@ struct MLayout {
     }
 };
 
-// One electron-proton pair: real-space Ewald value v = phi(r) summed over
-// images and its gradient g with respect to the electron-proton vector; the
-// e-n Jastrow contributions dl (to d ln psi/dR_a) and de (to dE_L/dR_a, given
-// vv = g_i + grad_i U).  sd, cd: sin, cos(pi (x - R_a)/L) per component.
 // FP32 radial factors of the Pade pair functions in t = rho^2, from one
-// reciprocal square root and one reciprocal (the FP64 form goes through
-// pade_* and rho_to_t):  f1 = u'/(2 rho),  f2 = (u''/rho^2 - u'/rho^3)/4,
+// reciprocal square root and one reciprocal (FP64: pade_factors):
+// f1 = u'/(2 rho),  f2 = (u''/rho^2 - u'/rho^3)/4,
 // f3 = (u'''/rho^3 - 3 u''/rho^4 + 3 u'/rho^5)/8.
 __device__ __forceinline__ void jas_ee_f32(float t, float b, float& u, float& f1, float& f2) {
     const float ir = rsqrtf(t), r = t * ir, ir2 = ir * ir;
@@ -98,8 +94,7 @@ __device__ __forceinline__ void jas_ep_f32(float t, float b, float Zj, float& u,
     f3 = 0.125f * (u3 - 3.0f * (u2 - u1 * ir) * ir) * ir2 * ir;
 }
 
-// FP32 e-n pair terms of d ln psi / dR and dE_L / dR (same quantities as
-// ep_jastrow): g = 2 f1 p, H v = 4 f2 p (p.v) + 2 f1 q o v,
+// FP32 e-n pair terms of d ln psi / dR and dE_L / dR: g = 2 f1 p, H v = 4 f2 p (p.v) + 2 f1 q o v,
 // grad lap u = p o (8 f3 |p|^2 + 8 f2 q + 4 f2 sum q - 2 k^2 f1).
 __device__ __forceinline__ void ep_jastrow_f32(const float sd[3], const float cd[3], float ell, float k2, float bep,
                                                float Zj, const float vv[3], float dl[3], float de[3]) {

@@ -131,3 +131,98 @@ def test_table_exponential(run):
         lim = np.array([-747.0, -1e4, -np.inf, 710.0, np.inf])
         assert np.array_equal(run("F_EXP", lim)[0], np.exp(lim))
     assert np.isnan(run("F_EXP", np.array([np.nan]))[0][0])
+
+
+def _positive(rng, n, lo, hi):
+    """Both halves of a binade and its ends, exponents from lo to hi."""
+    m = np.concatenate([rng.uniform(1, 2, n), [1.0, np.nextafter(1.0, 2), np.nextafter(2.0, 1)]])
+    return np.ldexp(m, rng.integers(lo, hi, len(m)))
+
+
+# the last multiply-add's rounding, and of the correction's own 2^-20 of one; the truncation 2^-4 at most
+def test_reciprocal(run):
+    x = _positive(np.random.default_rng(1), 1000000, -1000, 1000)
+    assert _ulps(run("F_RCP", x)[0], 1 / x.astype(LD)) <= 0.57
+
+
+# rsqrt: the last rounding and that of x y (u/2 of the result: at most half a unit); sqrt: times x,
+# whose rounding is another half a unit, on a value at most a unit and a half of the result's off
+def test_reciprocal_square_root(run):
+    x = _positive(np.random.default_rng(2), 1000000, -1000, 1000)
+    assert _ulps(run("F_RSQRT", x)[0], 1 / np.sqrt(x.astype(LD))) <= 1.07
+    assert _ulps(run("F_SQRT_PAIR", x)[0], np.sqrt(x.astype(LD))) <= 2.1
+    assert np.array_equal(run("F_SQRT_PAIR", np.array([0.0, -0.0]))[0], [0.0, 0.0])
+
+
+# the last multiply-add's rounding and those before, scaled by x^2 / 6 and x^2 / 2 <= 1/8
+def test_sine_and_cosine_of_close_pairs(run):
+    x = np.concatenate([np.linspace(-0.5, 0.5, 200001), np.geomspace(1e-12, 0.5, 2000)])
+    sn, cs = run("F_SINCOS_HALF", x)
+    keep = x != 0.0
+    assert _ulps(sn[keep], np.sin(x[keep].astype(LD))) <= 0.75 and np.all(sn[~keep] == 0.0)
+    assert _ulps(cs, np.cos(x.astype(LD))) <= 0.75
+
+
+def _boys(n, x):
+    """F_n(x) = int_0^1 s^2n exp(-x s^2) ds by its series of positive terms."""
+    term, total = np.ones_like(x) / (2 * n + 1), np.zeros_like(x)
+    for j in range(1, 300):
+        total += term
+        term = term * 2 * x / (2 * n + 1 + 2 * j)
+    return np.exp(-x) * total
+
+
+# Real-space Ewald table, L = 1: erf(kappa r)/r on r^2 <= 3/4 and erfc(kappa r)/r on [1/4, 1), and
+# their derivatives in r^2, at nodes, midpoints and between.  erf: exp's unit (2 u), the series and
+# the recurrence's few operations on positive terms, Horner's last step: 8 u.  erfc: the
+# library's five units (10 u), a square root, two divisions, three products: 16 u.  The
+# truncations are the 1e-18 kappa and 2e-16 kappa^3 of common.cuh.
+@pytest.mark.parametrize("kl", [0.01, 1.0, 3.0, 5.0, 6.0])
+def test_ewald_table(run, kl):
+    rng = np.random.default_rng(4)
+    h = 0.75 / 511
+    k, c = LD(kl), 2 / np.sqrt(LD(np.pi) + LD(1.2246467991473531772e-16))
+    for name, lo, hi in (("F_EWALD_ERF", 0.0, 0.75), ("F_EWALD_ERFC", 0.25, 1.0)):
+        i = np.arange(0, 682) * h
+        r2 = np.concatenate([rng.uniform(lo, hi, 20000), i, i + 0.5 * h, i + 0.4999 * h])
+        r2 = r2[(r2 >= lo) & (r2 < hi) | (r2 == lo)]
+        v, d = run(name, r2, kl)
+        x = k * k * r2.astype(LD)
+        f0, f1 = _boys(0, x), _boys(1, x)
+        if name == "F_EWALD_ERFC":           # G_n = int_0^inf - F_n
+            x = np.maximum(x, LD(1e-30))
+            f0 = np.sqrt(1 / (c * c)) / np.sqrt(x) - f0
+            f1 = np.sqrt(1 / (c * c)) / (2 * x * np.sqrt(x)) - f1
+        roundings = (16 if name == "F_EWALD_ERFC" else 8) * U
+        ref, dref = c * k * f0, -c * k ** 3 * f1
+        assert np.max(np.abs(v - ref) - roundings * (np.abs(ref) + kl)) <= 1e-18 * kl
+        assert np.max(np.abs(d - dref) - roundings * (np.abs(dref) + kl ** 3)) <= 2e-16 * kl ** 3
+
+
+# Box-Muller normals by tables: log u is good to 3 u relative (its last sum, the table and the
+# exponent's product), its square root to 1.5 u + 1.5 units more, sine and cosine to 4 u absolute
+# (table, series, and two products): 10 u rho in all.  Words at the log's ends (u next to 0 and
+# to 1, the seams at 1 and 0.6875) and at the angles' table points and midpoints.
+def test_toy_normals(run):
+    rng = np.random.default_rng(6)
+    w = rng.integers(0, 2 ** 32, (400000, 4), dtype=np.uint64)
+
+    def words(v):                            # the two words of 53 bits v
+        v = np.asarray(v, dtype=np.uint64)
+        return np.stack([(v >> np.uint64(26)) << np.uint64(5), (v & np.uint64(2 ** 26 - 1)) << np.uint64(6)], -1)
+    ends = np.concatenate([np.arange(64), 2 ** 53 - 1 - np.arange(4096),
+                           (0.6875 * 2.0 ** (53 - np.arange(20)[:, None]) + np.arange(-3, 4)).ravel(),
+                           (2.0 ** (53 - np.arange(1, 20)[:, None]) + np.arange(-3, 4)).ravel()]).astype(np.uint64)
+    angle = (np.arange(512)[:, None] * 2 ** 44 + np.arange(-3, 4)).ravel() % 2 ** 53
+    edge = np.concatenate([np.concatenate([words(ends), rng.integers(0, 2 ** 32, (len(ends), 2), dtype=np.uint64)], -1),
+                           np.concatenate([rng.integers(0, 2 ** 32, (len(angle), 2), dtype=np.uint64), words(angle)], -1)])
+    w = np.concatenate([w, edge]).astype(np.uint32)
+    g0, g1 = run("F_NORMALS", w)
+    bits = lambda a, b: (a >> 5).astype(LD) * 2 ** 26 + (b >> 6).astype(LD) + LD(0.5)
+
+    def u53(a, b):                           # the kernel's uniform: 53 bits and a half, rounded once to FP64
+        return bits(a, b).astype(np.float64).astype(LD) / LD(2) ** 53
+    u1, u2 = u53(w[:, 0], w[:, 1]), u53(w[:, 2], w[:, 3])
+    rho, th = np.sqrt(-2 * np.log(u1)), 2 * (LD(np.pi) + LD(1.2246467991473531772e-16)) * u2
+    for g, ref in ((g0, rho * np.cos(th)), (g1, rho * np.sin(th))):
+        assert np.max(np.abs(g - ref) - 10 * U * rho) <= 0.0
