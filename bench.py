@@ -175,8 +175,8 @@ def _flops_per_launch(cls: str, W, N, n, B, G, acc_ratio, use_tc, nk=462):
     """Algorithmic FLOPs of one launch of a kernel class (dense multiply-adds x 2)."""
     if cls == "orbitals_prop":
         return 2.0 * W * N * B * n
-    if cls == "orbitals_meas":   # grad (3) + Laplacian on the tensor cores; SIMT also forms the values
-        return (8.0 if use_tc else 10.0) * W * N * B * n
+    if cls == "orbitals_meas":   # grad (3) + Laplacian
+        return 8.0 * W * N * B * n
     if cls == "measure":
         u = MEASURE_UNIT
         # (the mixed form computes the reciprocal-space force, fk, as a GEMM
