@@ -82,3 +82,16 @@ def test_empirical_s_arguments_validated():
     with pytest.raises(q.QMCError):
         sysg.langevin_step(wl.R.ravel(), np.zeros(3 * wl.N), None, 1000.0, 0.1, s_mode=q.QMC_S_EMPIRICAL,
                            alpha=-1.0)
+
+
+def test_bench_leg_keeps_S_positive_definite():
+    """The benchmark's steps with S = H + mu I on the N = 128 protons: H's lowest eigenvalue
+    falls from -1.30 as the protons move, which mu has to outlast."""
+    import torch
+
+    import bench
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        out = bench._empirical_bench(stream)
+    for tag in ("empirical_S", "given_S"):
+        assert out[tag]["R_finite"] and out[tag]["ms_per_step_median"] > 0.0
