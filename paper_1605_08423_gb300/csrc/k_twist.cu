@@ -107,7 +107,8 @@ template <int NP, int TR, int TC>
 static void launch_tw_orb(const SysView<double>& s, const TwistView& tv, const double* pos, int nrows, double2* val,
                           cudaStream_t st) {
     const size_t smem = (size_t)8 * s.G * (2 * 32 + NP) * sizeof(double);   // at most 64 KB (n_gauss = 8, n > 32)
-    static size_t attr = 48 * 1024;
+    // 48 KB less the kernel's static shared memory without asking (n_gauss = 8, 16 < n <= 32 is 48 KB)
+    static size_t attr = 48 * 1024 - 8 * 2 * sizeof(int);
     if (smem > attr && cudaFuncSetAttribute(twist_orbitals_kernel<NP, TR, TC>,
                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)
         attr = smem;

@@ -13,7 +13,7 @@ from paper_1605_08423_gb300 import synth
 
 pytestmark = pytest.mark.gpu
 
-ZETA = {1: (0.7,), 2: synth.ZETA_2, 4: synth.ZETA_4}
+ZETA = {1: (0.7,), 2: synth.ZETA_2, 4: synth.ZETA_4, 8: (0.2, 0.3, 0.45, 0.7, 1.0, 1.5, 2.0, 3.0)}
 
 
 def _workload(N, G, walkers, rs=1.3, **kw):
@@ -141,3 +141,18 @@ def test_fp64_sample_of_a_far_electron():
     lp, el, dl, de = orc.eval_configs(osys, wl.R, X, derivs=True)
     assert all(np.all(np.isfinite(v)) for v in (lp, el, dl, de))
     _close(g, (lp - 1000.0 * np.log(2.0), el, dl, de), 1e-10)
+
+
+# the largest number of Gaussians, whose basis tiles take the most shared memory, at each
+# size of the orbital kernels
+@pytest.mark.parametrize("N,twisted", [(32, True), (34, True), (34, False), (66, False)])
+def test_fp64_sample_with_eight_gaussians(N, twisted):
+    wl = _workload(N, 8, 2)
+    tw = synth.monkhorst_pack(4)[[11]] if twisted else None
+    X = _sampled(wl, 2)[:1]
+    g = q.QMCSystem(q.Config.from_workload(wl, twists=tw), wl.R).eval_config(X, wl.R)
+    if twisted:
+        ref = orc.eval_configs_twist(_osys(wl, twist=np.asarray(tw[0])), wl.R, X, tw)
+    else:
+        ref = orc.eval_configs(_osys(wl), wl.R, X, derivs=True)
+    _close(g, ref, 1e-10)
