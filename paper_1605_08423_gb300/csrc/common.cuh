@@ -67,7 +67,7 @@ template <> struct Draw<float> {
 //   exp(x) = 2^m (2^(j/64) + 2^(j/64) p(r)),  p(r) = r + r^2/2 + ... + r^5/120,
 // the next term r^6/720 (up to 3.5e-17) taken in by economisation (C. Lanczos, Applied
 // Analysis, 1956): r^6 = 3/2 a^2 r^4 - 9/16 a^4 r^2 to a^6/32, which leaves 1.1e-18.
-// 11 FP64 operations (the library's 18 cost 340 clocks of an SM's FP64 pipe per
+// 11 FP64 operations (the library's 18 cost 290 clocks of an SM's FP64 pipe per
 // warp); the result is within 1.01 units in the last place (1.28 without that term).
 // From |x| = 690 on, where 2^m (..) leaves the normal range, the library's value
 // (0 below -746: no call where far images and nuclei are evaluated by the thousand).

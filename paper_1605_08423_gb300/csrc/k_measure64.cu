@@ -2,7 +2,7 @@
 // form (the mixed form's kernel and the estimators are in k_measure.cu).
 //
 // One CTA per walker.  The FP64 pipe bounds everything here (an SM issues a warp's
-// FP64 instruction every 19 clocks), so the kernel is arranged for few FP64
+// FP64 instruction every 16 clocks), so the kernel is arranged for few FP64
 // operations.  The orbital rows D = grad phi and Lp = lap phi are not needed:
 // with C the coefficients, G the inverse of a spin block and Z = C G,
 //   g_i = sum_b Z_bi grad chi_b(r_i),   l_i = sum_b Z_bi lap chi_b(r_i),
@@ -80,13 +80,19 @@ struct M64Layout {
     }
 };
 
-// Basis rows per tile: the whole spin block if it fits (one tile, nothing
-// evaluated twice), else as many whole nuclei as do.
+// Basis rows per tile: the whole spin block if it fits (one tile, nothing evaluated
+// twice), else as many whole nuclei as do, but full rounds of 4 x 4 outputs over the
+// threads (64 rows at n > 32, 128 at n <= 32; half of that in the twisted form).
+// N = 128, four Gaussians, 608 walkers: 29.5 ms so, 36.0 with the 68 rows that fit (272
+// tasks: a second round for 16 of them); one to three Gaussians 15.3, 20.0 and 25.2 where
+// all rows that fit take 16.2, 22.4 and 28.7.
 int tile_rows(int N, int n, int G, int nk, int mmax, bool tw, bool j34) {
     const int np = pad_pow2(n);
     const size_t most = 225 * 1024;
     int rows = N * G;
     while (rows > G && M64Layout(N, n, np, nk, mmax, tw, j34, rows).total > most) rows -= G;
+    const int round = 16 * kThreads / (tw ? 2 * np : np);
+    if (rows < N * G && rows > round) rows = rows / round * round / G * G;
     return rows;
 }
 
