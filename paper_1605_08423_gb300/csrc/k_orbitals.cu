@@ -205,12 +205,12 @@ __global__ void __launch_bounds__(256) orbitals64_kernel(SysView<double> s, cons
 template <int NP, int TR, int TC>
 static void launch_orb64(const SysView<double>& s, const double* pos, const double* trig, int nrows, double* val,
                          cudaStream_t st) {
-    const size_t smem = (32 * 6 + (size_t)8 * s.G * (32 + NP)) * sizeof(double);   // at most 52 KB (n_gauss = 8, n > 32)
-    static size_t attr = 48 * 1024;
-    if (smem > attr &&
-        cudaFuncSetAttribute(orbitals64_kernel<NP, TR, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-            cudaSuccess)
-        attr = smem;
+    const size_t smem = (32 * 6 + (size_t)8 * s.G * (32 + NP)) * sizeof(double);
+    // allowed once, at n_gauss = 8: the same value from every thread that calls
+    static const cudaError_t allowed = cudaFuncSetAttribute(
+        orbitals64_kernel<NP, TR, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        (int)((32 * 6 + 8 * 8 * (32 + NP)) * sizeof(double)));
+    (void)allowed;
     orbitals64_kernel<NP, TR, TC><<<(nrows + 31) / 32, 256, smem, st>>>(s, pos, trig, nrows, val);
 }
 

@@ -106,12 +106,13 @@ __global__ void __launch_bounds__(256) twist_orbitals_kernel(SysView<double> s, 
 template <int NP, int TR, int TC>
 static void launch_tw_orb(const SysView<double>& s, const TwistView& tv, const double* pos, int nrows, double2* val,
                           cudaStream_t st) {
-    const size_t smem = (size_t)8 * s.G * (2 * 32 + NP) * sizeof(double);   // at most 64 KB (n_gauss = 8, n > 32)
-    // 48 KB less the kernel's static shared memory without asking (n_gauss = 8, 16 < n <= 32 is 48 KB)
-    static size_t attr = 48 * 1024 - 8 * 2 * sizeof(int);
-    if (smem > attr && cudaFuncSetAttribute(twist_orbitals_kernel<NP, TR, TC>,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess)
-        attr = smem;
+    const size_t smem = (size_t)8 * s.G * (2 * 32 + NP) * sizeof(double);
+    // allowed once, at n_gauss = 8 (with 16 < n <= 32 that is 48 KB, too much beside the static
+    // shared memory without asking): the same value from every thread that calls
+    static const cudaError_t allowed =
+        cudaFuncSetAttribute(twist_orbitals_kernel<NP, TR, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(8 * 8 * (2 * 32 + NP) * sizeof(double)));
+    (void)allowed;
     twist_orbitals_kernel<NP, TR, TC><<<(nrows + 31) / 32, 256, smem, st>>>(s, tv, pos, nrows, val);
 }
 
